@@ -704,8 +704,11 @@ pcad_status create_common(const uint8_t *g_src, bool g_on_device, int H, int W, 
         e = cudaMemsetAsync(ch->tdev, 0, misc, ch->stream);
     if (e == cudaSuccess && m->L <= kSmallMaxLabels)
         e = launch_ptab(tabs.dm.T, ch->ptab, ch->stream);
-    if (e == cudaSuccess && (pca_tc_eligible(tabs.dm) || pca_win_eligible(tabs.dm)))
-        e = launch_tc_table(tabs.dm, ch->ftab, ch->stream);
+    if (e == cudaSuccess && (pca_tc_eligible(tabs.dm) || pca_win_eligible(tabs.dm))) {
+        DevModel dm = tabs.dm;
+        dm.ta64 = ch->ta64;
+        e = launch_tc_table(dm, ch->ftab, ch->stream);
+    }
     if (e == cudaSuccess && m->L == 2) {
         DevModel dm = tabs.dm;
         dm.ta64 = ch->ta64;

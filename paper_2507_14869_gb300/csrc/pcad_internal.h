@@ -280,7 +280,8 @@ bool pca_tc_auto(const DevModel &m);
 
 // The outside-window chunk sums of a model, as the batched tensor-core
 // sweep reads them: tc_table_floats(L) floats (16-byte aligned), written by
-// launch_tc_table.
+// launch_tc_table (m.ta64 set: the segment draw's prefix tables follow, at
+// kTabF floats, for the models it accepts).
 int tc_table_floats(int L);
 cudaError_t launch_tc_table(const DevModel &m, float *out, cudaStream_t s);
 
@@ -318,6 +319,23 @@ cudaError_t launch_gibbs_winw(const SweepArgs &a, const float *ftab, uint8_t *x,
 // Checkerboard Gibbs colour phase q (0..nbhd/2 - 1) in place on a.xin with
 // the windowed draw; a.last_phase: accumulate the cells after it.
 cudaError_t launch_gibbs_win(const SweepArgs &a, int q, const float *ftab, cudaStream_t s);
+
+// The segment draw (seg_draw.cuh) in the windowed sweeps' launch forms, for
+// the models seg_eligible accepts (a subset of pca_win_eligible's with 4
+// neighbours and c >= 0): launch_pca_win and its siblings hand such models
+// over.  stab: the prefix tables (seg_table_floats() floats, 16-byte aligned,
+// written by launch_seg_table from m.ta64).
+int seg_table_floats();
+bool seg_eligible(const DevModel &m);
+cudaError_t launch_seg_table(const DevModel &m, float *out, cudaStream_t s);
+cudaError_t launch_pca_seg(const SweepArgs &a, const float *stab, uint8_t *x0, uint8_t *x1,
+                           const uint32_t *budget, cudaStream_t s);
+cudaError_t launch_gibbs_seg(const SweepArgs &a, int q, const float *stab, cudaStream_t s);
+cudaError_t launch_pca_segw(const SweepArgs &a, const float *stab, uint8_t *x0, uint8_t *x1, int n,
+                            unsigned int *done, unsigned int *grab, int *err, bool par_from_t,
+                            const uint32_t *budget, cudaStream_t s);
+cudaError_t launch_gibbs_segw(const SweepArgs &a, const float *stab, uint8_t *x, int nsweeps,
+                              unsigned int *done, unsigned int *grab, int *err, cudaStream_t s);
 
 // Batched tensor-core sweeps: nsweeps sweeps of every slot listed in items
 // (tiles of 4 rows x 32 sites of the slot's grid in geom, rows = 4) in one
