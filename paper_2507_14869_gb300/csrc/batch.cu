@@ -1196,8 +1196,8 @@ pcad_status pcad_batch_read_sample(pcad_batch *b, int i, uint8_t *host_out, int 
     const SlotDesc &d = b->desc[i];
     if (out_pitch < d.W)
         return set_error(PCAD_EINVAL, "out_pitch < W");
-    B_TRY(cudaMemcpy2DAsync(host_out, out_pitch, d.x[b->t & 1], d.pitch, d.W, d.H,
-                            cudaMemcpyDeviceToHost, b->stream));
+    B_TRY(read_labels(host_out, out_pitch, d.x[b->t & 1], d.pitch, d.H, d.W, b->d_plane,
+                      b->stream));
     B_TRY(cudaStreamSynchronize(b->stream));
     return PCAD_OK;
 }
@@ -1691,8 +1691,9 @@ pcad_status pcad_server_step(pcad_server *sv, int slice_sweeps, int *n_active, i
             const SlotDesc &d = sv->desc[i];
             rq.sample.resize((size_t)d.H * d.W);
             rq.mean.assign((size_t)d.H * d.W, 0.0f);
-            B_TRY(cudaMemcpy2DAsync(rq.sample.data(), d.W, d.x[rq.t & 1], d.pitch, d.W, d.H,
-                                    cudaMemcpyDeviceToHost, sv->stream));
+            // packed through the plane of the other parity (done with)
+            B_TRY(read_labels(rq.sample.data(), d.W, d.x[rq.t & 1], d.pitch, d.H, d.W,
+                              d.x[(rq.t & 1) ^ 1], sv->stream));
             const uint64_t n_acc = rq.t > (uint64_t)d.burn_in ? rq.t - d.burn_in : 0;
             if (n_acc > 0) {
                 B_TRY(launch_mean(d.acc, (float)n_acc, d.acc, (long)d.H * d.W, sv->stream));

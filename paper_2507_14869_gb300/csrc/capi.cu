@@ -1060,8 +1060,9 @@ pcad_status pcad_chain_read_min_state(pcad_chain *ch, uint8_t *host_out, int out
     CUDA_TRY(cudaMemcpy(&bs, ch->track.best_sweep, sizeof(bs), cudaMemcpyDeviceToHost));
     if (bs == 0)
         return fail(PCAD_ESTATE, "no sweep has been tracked yet");
-    CUDA_TRY(cudaMemcpy2D(host_out, out_pitch, ch->track.xb, ch->pitch, ch->W, ch->H,
-                          cudaMemcpyDeviceToHost));
+    CUDA_TRY(read_labels(host_out, out_pitch, ch->track.xb, ch->pitch, ch->H, ch->W, ch->fplane,
+                         ch->stream));
+    CUDA_TRY(cudaStreamSynchronize(ch->stream));
     if (energy)
         *energy = best;
     if (sweep)
@@ -1212,8 +1213,8 @@ pcad_status pcad_chain_read_sample(pcad_chain *ch, uint8_t *host_out, int out_pi
         return fail(PCAD_EINVAL, "NULL argument");
     if (out_pitch < ch->W)
         return fail(PCAD_EINVAL, "out_pitch < W");
-    CUDA_TRY(cudaMemcpy2DAsync(host_out, out_pitch, ch->x[ch->cur], ch->pitch, ch->W, ch->H,
-                               cudaMemcpyDeviceToHost, ch->stream));
+    CUDA_TRY(read_labels(host_out, out_pitch, ch->x[ch->cur], ch->pitch, ch->H, ch->W, ch->fplane,
+                         ch->stream));
     CUDA_TRY(cudaStreamSynchronize(ch->stream));
     return PCAD_OK;
 }
@@ -1392,10 +1393,10 @@ pcad_status pcad_chain_export(pcad_chain *ch, void *host_blob, size_t *bytes)
     char *b = (char *)host_blob;
     memcpy(b, &h, sizeof(h));
     // layout: header | current labels | observation | accumulator
-    CUDA_TRY(cudaMemcpy2DAsync(b + sizeof(h), ch->W, ch->x[ch->cur], ch->pitch, ch->W, ch->H,
-                               cudaMemcpyDeviceToHost, ch->stream));
-    CUDA_TRY(cudaMemcpy2DAsync(b + sizeof(h) + n, ch->W, ch->g, ch->pitch, ch->W, ch->H,
-                               cudaMemcpyDeviceToHost, ch->stream));
+    uint8_t *hx = (uint8_t *)b + sizeof(h);
+    CUDA_TRY(read_labels(hx, ch->W, ch->x[ch->cur], ch->pitch, ch->H, ch->W, ch->fplane,
+                         ch->stream));
+    CUDA_TRY(read_labels(hx + n, ch->W, ch->g, ch->pitch, ch->H, ch->W, ch->fplane, ch->stream));
     CUDA_TRY(cudaMemcpyAsync(b + sizeof(h) + 2 * n, ch->acc, n * sizeof(float),
                              cudaMemcpyDeviceToHost, ch->stream));
     CUDA_TRY(cudaStreamSynchronize(ch->stream));

@@ -201,6 +201,21 @@ cudaError_t launch_labels_to_float(const uint8_t *x, int pitch, int H, int W, fl
     return cudaGetLastError();
 }
 
+cudaError_t read_labels(uint8_t *host, int host_pitch, const uint8_t *x, int pitch, int H, int W,
+                        void *packed, cudaStream_t s)
+{
+    if (host_pitch != W)
+        return cudaMemcpy2DAsync(host, host_pitch, x, pitch, W, H, cudaMemcpyDeviceToHost, s);
+    if (pitch != W) {
+        const cudaError_t e =
+            cudaMemcpy2DAsync(packed, W, x, pitch, W, H, cudaMemcpyDeviceToDevice, s);
+        if (e != cudaSuccess)
+            return e;
+        x = static_cast<const uint8_t *>(packed);
+    }
+    return cudaMemcpyAsync(host, x, (size_t)H * W, cudaMemcpyDeviceToHost, s);
+}
+
 cudaError_t launch_check_labels(const uint8_t *x, int pitch, int H, int W, int L, int *bad,
                                 cudaStream_t s)
 {

@@ -107,6 +107,14 @@ cudaError_t launch_mean(const float *acc, float n, float *mean, long count, cuda
 cudaError_t launch_labels_to_float(const uint8_t *x, int pitch, int H, int W, float *out,
                                    cudaStream_t s);
 
+// Labels (device rows of `pitch` bytes) to host rows of host_pitch bytes,
+// asynchronous.  Host rows without gaps are read as one linear copy, through
+// `packed` (H W bytes of device memory) when the device rows have gaps: a 2-D
+// copy to pageable memory moves row by row (57 ms for 8192^2 labels, 0.6 ms
+// for 512^2).
+cudaError_t read_labels(uint8_t *host, int host_pitch, const uint8_t *x, int pitch, int H, int W,
+                        void *packed, cudaStream_t s);
+
 // Metrics: est (H x W floats, label units), clean (H x W bytes, contiguous).
 // out[0] = PSNR dB, out[1] = SSIM (device doubles).  scratch: >= 8 doubles.
 cudaError_t launch_metrics(const float *est, const uint8_t *clean, int H, int W, int L,
