@@ -216,6 +216,7 @@ void build_tables(const pcad_model &m, ModelTables &t)
         d.kb0 = (float)(1.5 * (4.0 + 22.0) * u);
         d.kbr = (float)(1.01 * 1.5 * (3.0 * u * ln2 * std::fmax(J, 0.0) + 2.0 * u));
     }
+    d.cbs = seg_offset(d);
     d.ta64 = nullptr;
     d.pr64 = nullptr;
 }

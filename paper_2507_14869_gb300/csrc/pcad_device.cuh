@@ -53,6 +53,7 @@ struct DevModel {
     float eta;         // FP32 error bound of the normalised CDF
     float cb;          // tensor-core sweep: common exponent offset (-mu nbhd T, mu > 0)
     float hb, kb0, kb1, kbr;   // its per-site margin kb1 (hb - log2 Z) + kb0 + kbr delta / Z
+    float cbs;         // segment draw: cb + its scales' offset (NaN: not taken)
     int norm;          // inertia price: 0 L0 (via em1 / el64), 1 or 2 Lp (via kappa / in64)
     float kappa;       // Lp price exponent coefficient, -lambda log2(e) / (L - 1)^p
     const double *ta64;  // [511] data factor exp(-(U(g, g-d) - U(g,g))) at d + 255, FP64

@@ -334,6 +334,7 @@ cudaError_t launch_gibbs_win(const SweepArgs &a, int q, const float *ftab, cudaS
 // over.  stab: the prefix tables (seg_table_floats() floats, 16-byte aligned,
 // written by launch_seg_table from m.ta64).
 int seg_table_floats();
+float seg_offset(const DevModel &m);   // DevModel::cbs of a model's coefficients
 bool seg_eligible(const DevModel &m);
 cudaError_t launch_seg_table(const DevModel &m, float *out, cudaStream_t s);
 cudaError_t launch_pca_seg(const SweepArgs &a, const float *stab, uint8_t *x0, uint8_t *x1,

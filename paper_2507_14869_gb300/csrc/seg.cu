@@ -48,7 +48,8 @@ __global__ void __launch_bounds__(kSegRow) seg_table_kernel(const DevModel m, fl
     const int at = k >= 0 ? j : kSegRow - 1 - j;
     double x = 0.0;
     if (d > -m.L && d < m.L)   // a label's d = s - g; no other entry is read
-        x = m.ta64[kTableOffset + d] * exp2((double)(-m.gam) * (double)k * (double)d);
+        x = m.ta64[kTableOffset + d] *
+            exp2((double)(-m.gam) * (double)k * (double)d - rint((double)m.cbs - (double)m.cb));
     v[0][at] = x;
     __syncthreads();
     int cur = 0;
@@ -419,22 +420,39 @@ int seg_table_floats()
     return kSegFloats;
 }
 
-// c >= 0, Gaussian or no likelihood, and exponents that fit FP32 scales and
-// entries: every line's value at d = 0 within 2^+-125, every row's sum below
-// 2^127.
-bool seg_eligible(const DevModel &m)
+// c >= 0, Gaussian or no likelihood, L0 price, 4 neighbours, and exponents
+// that fit FP32.  A line's value at d = 0 lies within +-B, B = 4 mu (L - 1 + T)
+// + A bits; the scales 2^(c + S) carry an offset S (the tables 2^-S) that
+// keeps them from being flushed below 2^-126, S = 0 for B <= 125 (c_T <=
+// 0.068 at L = 256, T = 30).  A scale above 2^127 turns Z into an infinity or
+// a NaN, which certifies nothing: such a site is re-drawn in FP64.  It takes
+// four neighbours more than (127 - S) / (4 mu) labels away from the
+// observation, so that distance must be one the noise does not reach.  The
+// rows' sums must stay below 2^127.
+float seg_offset(const DevModel &m)
 {
+    const float no = NAN;
     if (m.nbhd != 4 || m.norm != 0 || m.gam > 0.0f || m.alpha > 0.0f || m.T < 1 || m.L < 9 ||
         m.L > 256)
-        return false;
-    const double mu = -(double)m.gam, A = mu * 4.0 * m.T;
-    if (mu * 4.0 * (m.L - 1 + m.T) + A > 125.0)
-        return false;
+        return no;
+    const double mu = -(double)m.gam, A = mu * 4.0 * m.T, range = m.L - 1 + m.T;
+    const double S = std::ceil(std::fmax(0.0, 4.0 * mu * range + A - 125.0));
+    const double sigma = m.alpha < 0.0f ? std::sqrt(0.5 * 1.4426950408889634 / -(double)m.alpha)
+                                        : 1e9;
+    if (S > 0.0 && (127.0 - S) / (4.0 * mu) < std::fmin(range, 5.0 * sigma + m.T))
+        return no;
     // the largest alpha d^2 + 4 mu d over d < L
     double d = m.L - 1;
     if (m.alpha < 0.0f && 2.0 * mu / -(double)m.alpha < d)
         d = 2.0 * mu / -(double)m.alpha;
-    return (double)m.alpha * d * d + 4.0 * mu * d <= 117.0;
+    if ((double)m.alpha * d * d + 4.0 * mu * d - S > 117.0)
+        return no;
+    return (float)((double)m.cb + S);
+}
+
+bool seg_eligible(const DevModel &m)
+{
+    return !std::isnan(m.cbs);
 }
 
 cudaError_t launch_seg_table(const DevModel &m, float *out, cudaStream_t st)

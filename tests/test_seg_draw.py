@@ -22,12 +22,23 @@ def _fma(a, b, c):   # exact product and sum in FP64 for these magnitudes, one r
     return (np.asarray(a, f64) * np.asarray(b, f64) + np.asarray(c, f64)).astype(f32)
 
 
-def _table(alpha64, mu, L):
+def _offset(alpha, mu, L, T):
+    """seg_offset of csrc/seg.cu: the scales' offset S, or None."""
+    A, rng = mu * 4 * T, L - 1 + T
+    S = np.ceil(max(0.0, 4 * mu * rng + A - 125.0))
+    sigma = np.sqrt(0.5 * LOG2E / -alpha) if alpha < 0 else 1e9
+    if S > 0 and (127.0 - S) / (4 * mu) < min(rng, 5 * sigma + T):
+        return None
+    d = L - 1.0 if alpha == 0 else min(L - 1.0, 2 * mu / -alpha)
+    return S if alpha * d * d + 4 * mu * d - S <= 117.0 else None
+
+
+def _table(alpha64, mu, L, S):
     """F_k(i) at [k + 4, i + 256]."""
     d = np.arange(-255, 256, dtype=f64)
     out = np.zeros((9, 512))
     for k in range(-4, 5):
-        e = np.where(np.abs(d) < L, alpha64 * d * d + float(mu) * k * d, -np.inf)
+        e = np.where(np.abs(d) < L, alpha64 * d * d + float(mu) * k * d - S, -np.inf)
         assert e.max() <= 117.5
         v = np.exp2(e)
         if k >= 0:
@@ -59,11 +70,15 @@ def _prepare(mod, x, g, xi, ulp):
     alpha64 = 0.0 if mod["noise"] == 2 else -LOG2E / (2.0 * sig * sig)
     alpha = f32(alpha64)
     cb = f32(float(gam) * 4 * T)
+    S = _offset(float(alpha), -float(gam), L, T)
+    assert S is not None
+    cbs = f32(f64(cb) + S)
     em1 = f32(np.expm1(lam))
-    tab = _table(alpha64, -gam, L).reshape(-1)
+    tab = _table(alpha64, -gam, L, S).reshape(-1)
 
     def ex2(c):
-        e = np.exp2(np.asarray(c, f64)).astype(f32)
+        with np.errstate(over="ignore"):   # beyond 2^128: an infinity
+            e = np.exp2(np.asarray(c, f64)).astype(f32)
         e = (e.astype(f64) * (1.0 + ulp * 2 * U)).astype(f32)
         return np.where(np.asarray(c) < -126.0, f32(0), e)
 
@@ -72,7 +87,8 @@ def _prepare(mod, x, g, xi, ulp):
     assert (np.diff(key, axis=1) >= 0).all()   # the network sorts
     lo, hi = -g, L - g
     Pb = (np.maximum(T - np.abs(xi[:, None] - x), 0)).sum(1)
-    v = _fma(alpha, (xi - g) ** 2, _fma(-gam, Pb, cb))
+    iv = _fma(-gam, Pb, cb)
+    v = _fma(alpha, (xi - g) ** 2, iv)
     delta = (ex2(v).astype(f64) * f64(em1)).astype(f32) if lam > 0 else np.zeros(n, f32)
     row = np.full(n, 4)
     C = np.zeros(n, np.int64)
@@ -80,7 +96,7 @@ def _prepare(mod, x, g, xi, ulp):
     E1, E2 = np.zeros(n, f32), np.zeros(n, f32)
     at = lo + 255 + 512 * row
     p = tab[at]
-    s = ex2(np.full(n, cb))
+    s = ex2(np.full(n, cbs))
     s0, c = s, np.zeros(n, f32)
     Gd, sc, ends = [], [], []
     for i in range(13):
@@ -96,7 +112,7 @@ def _prepare(mod, x, g, xi, ulp):
         q = tab[end]
         D = q - p
         assert (D >= 0).all()
-        w = (D.astype(f64) * s).astype(f32)
+        w = (D.astype(f64) * s).astype(f32)   # 0 times an infinite scale: NaN, uncertain
         E1 = _fma(np.abs(p) + np.abs(q), s, E1)
         E2 = _fma(w, np.abs(c), E2)
         G = w if i == 0 else G + w
@@ -111,13 +127,13 @@ def _prepare(mod, x, g, xi, ulp):
         p = tab[at]
         if i < 11:
             assert (np.abs(4 * C) < 2 ** 22).all()
-            c = _fma(mu4, 4 * C, cb)
-            assert (np.abs(c) <= 126.0).all()   # no scale overflows or is flushed
+            c = _fma(mu4, 4 * C, cbs)
+            assert (c >= -126.0).all()   # no scale is flushed
             s = ex2(c)
         else:
             c, s = np.zeros(n, f32), s0
     return dict(tab=tab, Gd=Gd, sc=sc, ends=ends, G=G, Z=G + delta, delta=delta, E1=E1, E2=E2,
-                av=np.abs(v), cb=cb)
+                av=np.abs(v) + np.abs(iv), cb=cb, kd=6 + f32(0.7) * np.abs(cbs))
 
 
 def _draw(mod, r, g, xi, ub):
@@ -153,7 +169,7 @@ def _draw(mod, r, g, xi, ub):
     loC = np.where(xin & (hi > ax), loC + r["delta"], loC)
     M = (f32(1.25 * U) * (r["E1"] + 2 * np.maximum(np.abs(f1), np.abs(fl)) * scs +
                           f32(0.6931472) * (r["E2"] - r["cb"] * r["Z"]) + 22 * r["Z"] +
-                          (f32(2.08) * r["av"] + 6) * r["delta"])).astype(f32)
+                          (f32(1.39) * r["av"] + r["kd"]) * r["delta"])).astype(f32)
     certain = (t < hiC) & ((sl == L - 1) | (hiC - t > M)) & ((sl == 0) | (t - loC > M))
     return np.clip(sl, 0, L - 1), certain, M
 
@@ -174,6 +190,9 @@ def _exact_cdf(mod, x, g, xi):
 MODELS = [
     dict(L=256, T=30, pair_coef=0.05, sigma=25.0, inertia=2.0, noise=0),
     dict(L=256, T=30, pair_coef=0.068, sigma=40.0, inertia=0.0, noise=0),
+    dict(L=256, T=30, pair_coef=0.08, sigma=39.0, inertia=2.0, noise=0),
+    dict(L=256, T=30, pair_coef=0.08, sigma=6.0, inertia=1.0, noise=0),
+    dict(L=17, T=2, pair_coef=1.27, sigma=0.4, inertia=2.0, noise=0),
     dict(L=256, T=30, pair_coef=0.03, sigma=5.0, inertia=3.0, noise=0),
     dict(L=256, T=1, pair_coef=0.08, sigma=15.0, inertia=1.5, noise=0),
     dict(L=33, T=4, pair_coef=0.5, sigma=2.6, inertia=1.0, noise=0),
@@ -204,7 +223,8 @@ def test_certified_labels_are_the_fp64_labels(mi):
     Zx = C[:, -1]
     total = uncertain = 0
     for ulp in (-1.0, 0.0, 1.0):
-        r = _prepare(mod, x, g, xi, ulp)
+        with np.errstate(invalid="ignore"):
+            r = _prepare(mod, x, g, xi, ulp)
         # uniforms on and around every boundary the FP64 CDF has, and at random
         for k in list(range(0, L, max(1, L // 24))) + [-1]:
             b = np.floor(C[:, k] / Zx * 2.0 ** 24) if k >= 0 else rng.integers(0, 1 << 24, n)
@@ -223,10 +243,11 @@ def test_certified_labels_are_the_fp64_labels(mi):
             lab = (end & 511) - 256 + g                    # last label of the segment
             ok = lab >= 0
             ref = np.where(ok, C[at, np.maximum(lab, 0)], 0.0) / Zx
+            fin = np.isfinite(r["Z"])      # others certify nothing
             err = np.abs(r["Gd"][i].astype(f64) / r["Z"] - ref)
             bound = 1.25 * U * (r["E1"] + 0.6931472 * (r["E2"] - r["cb"] * r["Z"]) +
-                                22 * r["Z"] + (2.08 * r["av"] + 6) * r["delta"]) / r["Z"]
-            assert (err <= bound).all()
+                                22 * r["Z"] + (1.39 * r["av"] + r["kd"]) * r["delta"]) / r["Z"]
+            assert (err <= bound)[fin].all() and fin.mean() > 0.9
     assert uncertain < 0.05 * total
 
 
