@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "pcad_internal.h"
+#include "tile.h"
 
 using namespace pcad;
 
@@ -133,10 +134,43 @@ size_t slot_bytes(const pcad_job &j)
     return job_layout(j, (int)((j.W + 15) / 16 * 16), 0).end;
 }
 
+// Device memory of a slot beside its block: the segment draw's prefix tables
+// and the border exchange of its tile-resident sweeps (null: not its models,
+// or too many sites).  Not part of the HBM accounting: at most 18 KB and 4
+// bytes a site of images up to kTileMaxSites.
+struct SlotSide {
+    float *stab = nullptr;
+    unsigned long long *xch = nullptr;
+};
+
+size_t side_bytes(const pcad_job &j, size_t &stab, size_t &xch)
+{
+    const int T = j.model.pair == PCAD_PAIR_POTTS ? 1 : j.model.pair_T;
+    DevModel m{};
+    m.L = j.model.L;
+    m.nbhd = j.model.nbhd;
+    m.T = T;
+    stab = seg_structure(m) ? al((size_t)seg_table_floats() * sizeof(float)) : 0;
+    xch = (long long)j.H * j.W <= kTileMaxSites ? al(tile_xch_bytes(j.H, j.W)) : 0;
+    return stab + xch;
+}
+
+// A slot's side memory at `mem` (side_bytes of it), exchange words cleared.
+pcad_status side_init(const pcad_job &j, void *mem, cudaStream_t s, SlotSide &sd)
+{
+    size_t stab = 0, xch = 0;
+    side_bytes(j, stab, xch);
+    sd.stab = stab ? (float *)mem : nullptr;
+    sd.xch = xch ? (unsigned long long *)((char *)mem + stab) : nullptr;
+    if (xch)
+        B_TRY(cudaMemsetAsync(sd.xch, 0, xch, s));
+    return PCAD_OK;
+}
+
 // Build a slot: copy g, x0 <- g, acc <- 0, tables; fill the descriptor.
 pcad_status init_slot(const pcad_job &j, char *base, const SlotMem &sm, int pitch,
                       uint32_t *tdev, const uint32_t *budget, unsigned long long *fp64,
-                      cudaStream_t s, SlotDesc &d)
+                      const SlotSide &sd, cudaStream_t s, SlotDesc &d)
 {
     double ta64[511];
     std::vector<double> pr64;
@@ -152,6 +186,9 @@ pcad_status init_slot(const pcad_job &j, char *base, const SlotMem &sm, int pitc
                           cudaMemcpyHostToDevice, s));
     dm.ta64 = (const double *)(base + sm.ta);
     dm.pr64 = (const double *)(base + sm.pr);
+    dm.stab = seg_eligible(dm) ? sd.stab : nullptr;
+    if (dm.stab)
+        B_TRY(launch_seg_table(dm, sd.stab, s));
     d = SlotDesc{};
     d.g = (const uint8_t *)(base + sm.g);
     d.x[0] = (uint8_t *)(base + sm.x0);
@@ -600,6 +637,220 @@ pcad_status small_set_retable(const SmallSet &ss, const SlotDesc &d, int i, cuda
     return PCAD_OK;
 }
 
+// Mid-size chains run tile-resident (tile.cu), several in one cooperative
+// launch: chains of one launch kind share the SMs in proportion to their
+// sites, up to kTilePackSites sites together (more rounds of draws per launch
+// than its exchange costs); planes by the device sweep counter, budget-aware.
+// Segment-draw chains from kWinWaveBlocks blocks per SM on stay with the
+// wavefront (as in capi.cu).  Measured on GB300 against the batched kernels:
+// the design doc's batch and serve rows.
+constexpr long long kTilePackSites = 1ll << 20;
+
+struct TileSet {
+    struct Launch {
+        TileKind kind;
+        TilePack pack;
+        int ctas = 0;
+        size_t smem = 0;
+    };
+    std::vector<Launch> launches;
+    std::vector<int> slots;
+    std::vector<int> table_T;      // T of each pair table
+    uint32_t *tables = nullptr;
+    size_t cap = 0;
+    uint4 *btabs = nullptr;        // threshold tables of the two-label slots
+    size_t bcap = 0;
+};
+
+// CTAs for the jobs of a launch: the fewest rounds of draws per sweep that
+// all jobs reach together on `cap` CTAs.
+bool tile_assign(const TileKind &k, std::vector<TileJob> &jobs, int cap, bool two, int &ctas,
+                 size_t &smem)
+{
+    long long total = 0;
+    for (const TileJob &J : jobs)
+        total += (long long)J.a.H * J.a.W;
+    for (int R = (int)std::max(1ll, total / ((long long)cap * 512)); R <= 16; ++R) {
+        ctas = 0;
+        smem = 0;
+        bool ok = true;
+        for (TileJob &J : jobs) {
+            const int c0 = (int)(((long long)J.a.H * J.a.W + 512ll * R - 1) / (512ll * R));
+            bool got = false;
+            // (a tile grid may not use the CTAs it is offered evenly: a few more)
+            for (int c = c0; c <= c0 + c0 / 2 + 1 && c <= cap && !got; ++c) {
+                size_t b = 0;
+                if (tile_plan_ctas(k, J.a.H, J.a.W, c, two, J.tg, b) && tile_rounds(J.tg) <= R) {
+                    J.cta0 = ctas;
+                    ctas += J.tg.tiles_x * J.tg.tiles_y;
+                    smem = std::max(smem, b);
+                    got = true;
+                }
+            }
+            ok = ok && got;
+        }
+        if (ok && ctas <= cap)
+            return true;
+    }
+    return false;
+}
+
+// Split `in` into the tile-resident slots and the rest; tables and launches.
+pcad_status tile_set_build(TileSet &ts, const std::vector<SlotDesc> &d,
+                           const std::vector<SlotSide> &side, const std::vector<int> &in,
+                           std::vector<int> &rest, int *err, cudaStream_t st)
+{
+    ts.launches.clear();
+    ts.slots.clear();
+    ts.table_T.clear();
+    rest.clear();
+    int sms = 0, dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess)
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    std::vector<std::pair<TileKind, std::vector<int>>> groups;
+    size_t nbin = 0;
+    for (int i : in) {
+        const long long sites = (long long)d[i].H * d[i].W;
+        TileKind k;
+        if (sms <= 0 || !side[i].xch || !tile_kind(d[i].m, false, k) ||
+            (k.draw == TileKind::kSegment &&
+             (!d[i].m.stab || sites >= kWinWaveBlocks * 128 * sms))) {
+            rest.push_back(i);
+            continue;
+        }
+        size_t gi = 0;
+        while (gi < groups.size() && !(groups[gi].first == k))
+            ++gi;
+        if (gi == groups.size())
+            groups.push_back({k, {}});
+        groups[gi].second.push_back(i);
+        nbin += k.draw == TileKind::kBinary;
+        if (k.draw == TileKind::kSmall &&
+            std::find(ts.table_T.begin(), ts.table_T.end(), d[i].m.T) == ts.table_T.end())
+            ts.table_T.push_back(d[i].m.T);
+    }
+    if (ts.table_T.size() > ts.cap) {
+        if (ts.tables)
+            B_TRY(cudaFreeAsync(ts.tables, st));
+        ts.tables = nullptr;
+        ts.cap = std::max(ts.table_T.size(), 2 * ts.cap);
+        B_TRY(cudaMallocAsync((void **)&ts.tables, ts.cap * ptab_words() * sizeof(uint32_t), st));
+    }
+    for (size_t k = 0; k < ts.table_T.size(); ++k)
+        B_TRY(launch_ptab(ts.table_T[k], ts.tables + k * ptab_words(), st));
+    if (nbin > ts.bcap) {
+        if (ts.btabs)
+            B_TRY(cudaFreeAsync(ts.btabs, st));
+        ts.btabs = nullptr;
+        ts.bcap = std::max(nbin, 2 * ts.bcap);
+        B_TRY(cudaMallocAsync((void **)&ts.btabs, ts.bcap * bin_tab_entries() * sizeof(uint4), st));
+    }
+    size_t bin = 0;
+    for (auto &gr : groups) {
+        const TileKind k = gr.first;
+        std::vector<int> &v = gr.second;
+        std::stable_sort(v.begin(), v.end(), [&](int a, int b) {
+            return (long long)d[a].H * d[a].W > (long long)d[b].H * d[b].W;
+        });
+        for (size_t at = 0; at < v.size();) {
+            // the next launch: as many chains as share it
+            std::vector<TileJob> jobs;
+            long long total = 0;
+            const size_t first = at;
+            for (; at < v.size() && jobs.size() < (size_t)kTileJobs; ++at) {
+                const SlotDesc &s = d[v[at]];
+                const long long sites = (long long)s.H * s.W;
+                if (!jobs.empty() && total + sites > kTilePackSites)
+                    break;
+                total += sites;
+                TileJob J{};
+                J.a.g = s.g;
+                J.a.acc = s.acc;
+                J.a.fp64_draws = s.fp64_draws;
+                J.a.sweep_base = s.tdev;
+                J.a.seed = s.seed;
+                J.a.H = s.H;
+                J.a.W = s.W;
+                J.a.pitch = s.pitch;
+                J.a.chain = s.chain;
+                J.a.burn_in = s.burn_in;
+                J.a.m = s.m;
+                J.x0 = s.x[0];
+                J.x1 = s.x[1];
+                J.budget = s.budget;
+                J.par_from_t = 1;
+                J.xch = side[v[at]].xch;
+                if (k.draw == TileKind::kSmall)
+                    J.a.m.ptab = ts.tables + ptab_words() *
+                                                 (std::find(ts.table_T.begin(), ts.table_T.end(),
+                                                            s.m.T) - ts.table_T.begin());
+                jobs.push_back(J);
+            }
+            TileSet::Launch L;
+            L.kind = k;
+            bool fits = false;
+            while (!jobs.empty() && !fits) {
+                total = 0;
+                for (const TileJob &J : jobs)
+                    total += (long long)J.a.H * J.a.W;
+                const bool two = total > 512ll * sms;
+                fits = tile_assign(k, jobs, two ? 2 * sms : sms, two, L.ctas, L.smem);
+                if (!fits) {   // one chain less
+                    jobs.pop_back();
+                    --at;
+                }
+            }
+            if (jobs.empty()) {   // a shape that does not fit at all
+                rest.push_back(v[first]);
+                at = first + 1;
+                continue;
+            }
+            L.pack.njobs = (int)jobs.size();
+            L.pack.err = err;
+            for (size_t q = 0; q < jobs.size(); ++q) {
+                if (k.draw == TileKind::kBinary) {
+                    uint4 *t = ts.btabs + bin++ * bin_tab_entries();
+                    B_TRY(launch_btab(jobs[q].a.m, t, st));
+                    jobs[q].a.m.btab = t;
+                }
+                L.pack.job[q] = jobs[q];
+                ts.slots.push_back(v[first + q]);
+            }
+            ts.launches.push_back(L);
+        }
+    }
+    return PCAD_OK;
+}
+
+// n sweeps of every tile-resident slot.
+pcad_status tile_set_issue(const TileSet &ts, int n, cudaStream_t st)
+{
+    for (const TileSet::Launch &L : ts.launches) {
+        if (L.pack.njobs == 1) {
+            TileLaunch one{};
+            one.nsweeps = n;
+            one.njobs = 1;
+            one.err = L.pack.err;
+            one.job[0] = L.pack.job[0];
+            B_TRY(launch_tile(L.kind, one, L.ctas, L.smem, st));
+        } else {
+            TilePack p = L.pack;
+            p.nsweeps = n;
+            B_TRY(launch_tile(L.kind, p, L.ctas, L.smem, st));
+        }
+    }
+    return PCAD_OK;
+}
+
+void tile_set_free(TileSet &ts, cudaStream_t st)
+{
+    if (ts.tables)
+        cudaFreeAsync(ts.tables, st);
+    if (ts.btabs)
+        cudaFreeAsync(ts.btabs, st);
+    ts = TileSet{};
+}
+
 // Two-label chains small enough to keep their state in one CTA's shared
 // memory (64 x 64 and the like) run the resident kernel: one launch per
 // neighbourhood holds every such chain, one CTA each, for all the sweeps of
@@ -774,6 +1025,10 @@ struct pcad_batch {
     TcSet tc;                        // chains on the tensor-core sweep
     SmallSet small;                  // large small-label chains, launched one at a time
     ResSet res;                      // small two-label chains, one CTA each
+    TileSet tile;                    // mid-size chains, tile-resident
+    std::vector<SlotSide> side;
+    void *side_block = nullptr;
+    bool items_dirty = false;        // a model change may move a slot to another launch
     float tune_ms = 0.0f;
     cudaGraphExec_t graph = nullptr;
 };
@@ -782,15 +1037,19 @@ namespace {
 
 pcad_status batch_set_items(pcad_batch *b, int rows, int lpt, int slice)
 {
-    std::vector<int> all(b->n), not_res, others, active;
+    std::vector<int> all(b->n), not_res, not_tile, others, active;
+    b->items_dirty = false;
     for (int i = 0; i < b->n; ++i)
         all[i] = i;
-    // small two-label chains run resident, chains with a tensor-core table
-    // on the batched tensor-core sweep, large small-label chains on their
-    // own launches; the tiling below applies to the others
+    // small two-label chains run resident, mid-size chains tile-resident,
+    // chains with a tensor-core table on the windowed or batched tensor-core
+    // sweeps, large small-label chains on their own launches; the tiling
+    // below applies to the others
     pcad_status st0 = res_set_build(b->res, b->desc, all, not_res, b->stream);
     if (st0 == PCAD_OK)
-        st0 = tc_set_build(b->tc, b->desc, not_res, others, b->stream);
+        st0 = tile_set_build(b->tile, b->desc, b->side, not_res, not_tile, b->d_err, b->stream);
+    if (st0 == PCAD_OK)
+        st0 = tc_set_build(b->tc, b->desc, not_tile, others, b->stream);
     if (st0 == PCAD_OK)
         st0 = small_set_build(b->small, b->desc, others, active, b->stream);
     if (st0 != PCAD_OK)
@@ -828,6 +1087,8 @@ pcad_status batch_issue_slice(pcad_batch *b, cudaStream_t s)
 {
     const int n = b->slice;
     pcad_status st0 = res_set_issue(b->res, b->d_slots, n, s);
+    if (st0 == PCAD_OK)
+        st0 = tile_set_issue(b->tile, n, s);
     if (st0 == PCAD_OK)
         st0 = tc_set_issue(b->tc, b->desc, b->d_slots, b->d_t, b->d_budget, n, b->d_grab,
                            b->d_err, s);
@@ -875,6 +1136,11 @@ pcad_status batch_graph(pcad_batch *b)
 
 pcad_status batch_run_sweeps(pcad_batch *b, int nsweeps)
 {
+    if (b->items_dirty) {
+        pcad_status st = batch_set_items(b, b->rows, b->lpt, b->slice);
+        if (st != PCAD_OK)
+            return st;
+    }
     std::vector<uint32_t> bud(b->n, (uint32_t)(b->t + nsweeps));
     B_TRY(cudaMemcpyAsync(b->d_budget, bud.data(), bud.size() * sizeof(uint32_t),
                           cudaMemcpyHostToDevice, b->stream));
@@ -897,6 +1163,8 @@ pcad_status batch_reset_state(pcad_batch *b)
         B_TRY(cudaMemcpy2DAsync(d.x[0], d.pitch, d.g, d.pitch, d.W, d.H, cudaMemcpyDeviceToDevice,
                                 b->stream));
         B_TRY(cudaMemsetAsync(d.acc, 0, (size_t)d.H * d.W * sizeof(float), b->stream));
+        if (b->side[i].xch)   // the sweep indices, hence the words' tags, start again
+            B_TRY(cudaMemsetAsync(b->side[i].xch, 0, tile_xch_bytes(d.H, d.W), b->stream));
     }
     B_TRY(cudaMemsetAsync(b->d_t, 0, b->n * sizeof(uint32_t), b->stream));
     B_TRY(cudaMemsetAsync(b->d_fp64, 0, b->n * sizeof(unsigned long long), b->stream));
@@ -1043,11 +1311,29 @@ pcad_status pcad_batch_create(const pcad_job *jobs, int n, int autotune, void *c
         tc_set_free(b->tc, b->stream);
         small_set_free(b->small, b->stream);
         res_set_free(b->res, b->stream);
+        tile_set_free(b->tile, b->stream);
+        if (b->side_block)
+            cudaFreeAsync(b->side_block, b->stream);
         cudaFreeAsync(b->block, b->stream);
         cudaStreamSynchronize(b->stream);
         delete b;
         return st;
     };
+    b->side.resize(n);
+    std::vector<size_t> soff(n);
+    size_t stotal = 0;
+    for (int i = 0; i < n; ++i) {
+        size_t u = 0, v = 0;
+        soff[i] = stotal;
+        stotal += side_bytes(jobs[i], u, v);
+    }
+    if (stotal > 0 &&
+        (e = cudaMallocAsync(&b->side_block, stotal, b->stream)) != cudaSuccess) {
+        b->side_block = nullptr;
+        cudaGetLastError();
+        return bail(set_error(e == cudaErrorMemoryAllocation ? PCAD_ENOMEM : PCAD_ECUDA,
+                              cudaGetErrorString(e)));
+    }
     e = cudaMemsetAsync(base + off_ctr, 0, al(n * 16), b->stream);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(b->d_err, 0, sizeof(int), b->stream);
@@ -1055,8 +1341,11 @@ pcad_status pcad_batch_create(const pcad_job *jobs, int n, int autotune, void *c
         return bail(set_error(PCAD_ECUDA, cudaGetErrorString(e)));
     for (int i = 0; i < n; ++i) {
         const int pitch = (jobs[i].W + 15) / 16 * 16;
-        pcad_status st = init_slot(jobs[i], base, mem[i], pitch, b->d_t + i, b->d_budget + i,
-                                   fp64 + i, b->stream, b->desc[i]);
+        pcad_status st =
+            side_init(jobs[i], (char *)b->side_block + soff[i], b->stream, b->side[i]);
+        if (st == PCAD_OK)
+            st = init_slot(jobs[i], base, mem[i], pitch, b->d_t + i, b->d_budget + i, fp64 + i,
+                           b->side[i], b->stream, b->desc[i]);
         if (st != PCAD_OK)
             return bail(st);
         b->jobs.push_back(jobs[i]);
@@ -1119,7 +1408,12 @@ pcad_status pcad_batch_set_model(pcad_batch *b, int i, const pcad_model *m)
                           cudaMemcpyHostToDevice, b->stream));
     dm.ta64 = (const double *)(base + sm.ta);
     dm.pr64 = (const double *)(base + sm.pr);
+    dm.stab = seg_eligible(dm) ? b->side[i].stab : nullptr;
+    if (dm.stab)
+        B_TRY(launch_seg_table(dm, b->side[i].stab, b->stream));
     b->desc[i].m = dm;
+    if (b->side[i].xch)   // the tile-resident launches carry their chains' models
+        b->items_dirty = true;
     if (b->desc[i].tctab)   // the tensor-core sweep's outside sums follow the model
         B_TRY(launch_tc_table(dm, const_cast<float *>(b->desc[i].tctab), b->stream));
     {
@@ -1260,6 +1554,9 @@ void pcad_batch_destroy(pcad_batch *b)
     tc_set_free(b->tc, b->stream);
     small_set_free(b->small, b->stream);
     res_set_free(b->res, b->stream);
+    tile_set_free(b->tile, b->stream);
+    if (b->side_block)
+        cudaFreeAsync(b->side_block, b->stream);
     cudaFreeAsync(b->block, b->stream);
     cudaStreamSynchronize(b->stream);
     delete b;
@@ -1282,6 +1579,7 @@ struct Request {
     uint64_t t = 0;              // sweeps done (host mirror)
     size_t bytes = 0;
     void *mem = nullptr;
+    void *side = nullptr;        // its slot's side memory
     double t_submit = 0.0;       // seconds (steady clock)
     double unit_cost = 0.0;      // estimated seconds per site-update
     std::vector<uint8_t> sample;
@@ -1320,6 +1618,8 @@ struct pcad_server {
     WaveBuf wb;                   // wavefront work list of the admitted requests
     TcSet tc;                     // requests on the tensor-core sweep
     SmallSet small;               // large small-label requests, launched one at a time
+    TileSet tile;                 // mid-size requests, tile-resident
+    std::vector<SlotSide> side;   // per slot
     bool items_dirty = true;
     int grid = 0;
     int n_active = 0;              // admitted requests (both kinds of launch)
@@ -1359,14 +1659,25 @@ pcad_status admit_one(pcad_server *sv, Request &rq, int slot)
         cudaGetLastError();
         return set_error(PCAD_ENOMEM, cudaGetErrorString(e));
     }
+    size_t u = 0, v = 0;
+    const size_t sbytes = side_bytes(rq.job, u, v);
+    if (sbytes > 0 && (e = cudaMallocAsync(&rq.side, sbytes, sv->stream)) != cudaSuccess) {
+        rq.side = nullptr;
+        cudaGetLastError();
+        cudaFreeAsync(rq.mem, sv->stream);
+        rq.mem = nullptr;
+        return set_error(PCAD_ENOMEM, cudaGetErrorString(e));
+    }
     const int pitch = (rq.job.W + 15) / 16 * 16;
     SlotMem sm = job_layout(rq.job, pitch, 0);
     pcad_job j = rq.job;
     j.g_host = rq.g.data();
     j.g_pitch = rq.job.W;
     SlotDesc d{};
-    pcad_status st = init_slot(j, (char *)rq.mem, sm, pitch, sv->d_t + slot,
-                               sv->d_budget + slot, sv->d_fp64 + slot, sv->stream, d);
+    pcad_status st = side_init(j, rq.side, sv->stream, sv->side[slot]);
+    if (st == PCAD_OK)
+        st = init_slot(j, (char *)rq.mem, sm, pitch, sv->d_t + slot, sv->d_budget + slot,
+                       sv->d_fp64 + slot, sv->side[slot], sv->stream, d);
     if (st != PCAD_OK)
         return st;
     const uint32_t zero = 0, bud = (uint32_t)rq.nsweeps;
@@ -1490,9 +1801,13 @@ pcad_status server_items(pcad_server *sv)
     for (int i = 0; i < sv->max_slots; ++i)
         if (sv->slot_req[i] != 0 && sv->reqs[sv->slot_req[i]].running)
             all.push_back(i);
-    // requests with a tensor-core table run on the batched tensor-core sweep
-    std::vector<int> others;
-    pcad_status st = tc_set_build(sv->tc, sv->desc, all, others, sv->stream);
+    // mid-size requests run tile-resident, those with a tensor-core table on
+    // the windowed or batched tensor-core sweeps
+    std::vector<int> not_tile, others;
+    pcad_status st =
+        tile_set_build(sv->tile, sv->desc, sv->side, all, not_tile, sv->d_err, sv->stream);
+    if (st == PCAD_OK)
+        st = tc_set_build(sv->tc, sv->desc, not_tile, others, sv->stream);
     if (st == PCAD_OK)
         st = small_set_build(sv->small, sv->desc, others, active, sv->stream);
     if (st != PCAD_OK)
@@ -1573,6 +1888,7 @@ pcad_status pcad_server_create(int max_slots, size_t hbm_budget_bytes, void *cud
     }
     sv->h_err[0] = sv->h_err[1] = 0;
     sv->desc.assign(max_slots, SlotDesc{});
+    sv->side.assign(max_slots, SlotSide{});
     sv->slot_req.assign(max_slots, 0);
     sv->grid = wave_grid();
     *out = sv;
@@ -1659,9 +1975,11 @@ pcad_status pcad_server_step(pcad_server *sv, int slice_sweeps, int *n_active, i
     }
     int finished = 0, active = 0;
     if (sv->n_active > 0) {
-        // one wavefront launch per kind runs the slice for every admitted request
-        st = tc_set_issue(sv->tc, sv->desc, sv->d_slots, sv->d_t, sv->d_budget, slice_sweeps,
-                          sv->d_grab, sv->d_err, sv->stream);
+        // one launch per kind runs the slice for every admitted request of it
+        st = tile_set_issue(sv->tile, slice_sweeps, sv->stream);
+        if (st == PCAD_OK)
+            st = tc_set_issue(sv->tc, sv->desc, sv->d_slots, sv->d_t, sv->d_budget, slice_sweeps,
+                              sv->d_grab, sv->d_err, sv->stream);
         if (st == PCAD_OK)
             st = small_set_issue(sv->small, sv->desc, slice_sweeps, sv->stream);
         if (st == PCAD_OK && sv->wb.n_items > 0)
@@ -1707,6 +2025,10 @@ pcad_status pcad_server_step(pcad_server *sv, int slice_sweeps, int *n_active, i
                                   cudaMemcpyHostToDevice, sv->stream));
             B_TRY(cudaFreeAsync(rq.mem, sv->stream));
             rq.mem = nullptr;
+            if (rq.side)
+                B_TRY(cudaFreeAsync(rq.side, sv->stream));
+            rq.side = nullptr;
+            sv->side[i] = SlotSide{};
             sv->used -= rq.bytes;
             sv->active_sites -= (size_t)d.H * d.W;
             sv->slot_req[i] = 0;
@@ -1791,12 +2113,14 @@ void pcad_server_destroy(pcad_server *sv)
         return;
     cudaStreamSynchronize(sv->stream);
     for (auto &kv : sv->reqs)
-        if (kv.second.mem)
-            cudaFreeAsync(kv.second.mem, sv->stream);
+        for (void *q : {kv.second.mem, kv.second.side})
+            if (q)
+                cudaFreeAsync(q, sv->stream);
     if (sv->wb.mem)
         cudaFreeAsync(sv->wb.mem, sv->stream);
     tc_set_free(sv->tc, sv->stream);
     small_set_free(sv->small, sv->stream);
+    tile_set_free(sv->tile, sv->stream);
     cudaFreeAsync(sv->ctl, sv->stream);
     cudaStreamSynchronize(sv->stream);
     for (int k = 0; k < 2; ++k)

@@ -18,6 +18,7 @@
 
 #include "../../include/pcaden.h"
 #include "pcad_internal.h"
+#include "tile.h"
 
 using namespace pcad;
 
@@ -246,6 +247,7 @@ struct pcad_chain {
     uint32_t *ptab = nullptr;     // small-L sweep: pair prior table
     uint4 *btab = nullptr;        // two-label draw thresholds (L = 2)
     float *ftab = nullptr;        // outside-chunk sums of the windowed sweeps
+    float *stab = nullptr;        // prefix tables of the segment draw (nullptr: not its structure)
     DevModel dm{};
     cudaGraphExec_t graph = nullptr;
     int tb_k = 0;                 // sweeps per temporally blocked launch (0: one per launch)
@@ -263,6 +265,10 @@ struct pcad_chain {
     unsigned int *wave = nullptr; // wavefront kernel: per-tile counters + work counter
     int wave_tiles = 0;
     int sms = 0;                  // multiprocessors of the chain's device
+    unsigned long long *xch = nullptr;   // tile-resident sweeps: border exchange (nullptr: not taken)
+    TileKind tkind;
+    TileGeom tgeom{};
+    size_t tsmem = 0;
     void *track_block = nullptr;
 };
 
@@ -360,6 +366,41 @@ bool uses_resident(const pcad_chain *ch)
 }
 
 bool uses_wave(const pcad_chain *ch);
+
+// Whole runs of sweeps of mid-size images in one tile-resident launch, where
+// AUTO (or SMALL) would run the small-label, wavefront, two-label, general or
+// windowed kernels; energy tracking needs every sweep's state.  Measured on
+// GB300, us per sweep (tile-resident / the kernel it replaces):
+//   small labels, to kTileMaxSites sites: 256^2 L = 9, 8 neighbours 2.8 / 6.7,
+//   L = 5 Gibbs 4.3 / 12.3 (four launches); L = 16 300^2 2.7 / 7.0, 512^2
+//   4.8 / 7.0, 1024^2 13.2 / 15.6 (2048^2, on TMA tiles: 45);
+//   two labels: 300^2 1.6 / 3.8, 600^2 2.7 / 4.5, 1000^2 5.1 / 5.8;
+//   segment draw: 256^2 L = 24 3.9 / 6.2, L = 64 4.4 / 8.5; at 512^2 L = 256
+//   the wavefront's 4 x 32-site items pack better (10.5 / 9.5; Gibbs, whose
+//   phases need no exchange here, 13.3 / 14.4; at 720^2 20.5 / 19.6): from 8
+//   blocks of 4 x 32 sites per multiprocessor on, PCA stays with it, from
+//   kTileSegGibbsSites sites on Gibbs too.
+constexpr long long kTileSegGibbsSites = 300000;
+
+bool uses_tile(const pcad_chain *ch)
+{
+    if (!ch->xch || ch->tb_k > 0 || ch->track.trace || uses_resident(ch))
+        return false;
+    const bool gibbs = ch->model.sampler != PCAD_SAMPLER_PCA;
+    TileKind k;   // the coefficients may have changed since the creation
+    if (!tile_kind(ch->dm, gibbs, k) || !(k == ch->tkind))
+        return false;
+    if (ch->kernel == PCAD_KERNEL_SMALL)
+        return k.draw == TileKind::kSmall && !gibbs;
+    if (ch->kernel != PCAD_KERNEL_AUTO)
+        return false;
+    if (k.draw != TileKind::kSegment)
+        return true;
+    if (pca_tc_auto(ch->dm) && win_auto_mode(ch) == 0)
+        return false;   // AUTO's tensor-core images
+    const long long sites = (long long)ch->H * ch->W;
+    return sites < (gibbs ? kTileSegGibbsSites : 8LL * 128 * ch->sms);
+}
 
 // Unblocked sweeps (PCA or Gibbs) on the CUDA-core windowed kernels: on
 // request, or with AUTO where win_auto takes them.
@@ -466,6 +507,23 @@ pcad_status issue_sweeps(pcad_chain *ch, int off0, int n, int &cur, cudaStream_t
         const bool gibbs = ch->model.sampler != PCAD_SAMPLER_PCA;
         const int out = gibbs ? cur : cur ^ (n & 1);
         CUDA_TRY(launch_resident(a, ch->x[cur], ch->x[out], n, gibbs, st));
+        cur = out;
+        return PCAD_OK;
+    }
+    if (uses_tile(ch) && n > 0) {
+        a.sweep_off = (uint32_t)off0;
+        const bool gibbs = ch->model.sampler != PCAD_SAMPLER_PCA;
+        const int out = gibbs ? cur : cur ^ (n & 1);
+        TileLaunch L{};
+        L.nsweeps = n;
+        L.njobs = 1;
+        L.err = ch->err;
+        L.job[0].a = a;
+        L.job[0].x0 = ch->x[cur];
+        L.job[0].x1 = ch->x[out];
+        L.job[0].xch = ch->xch;
+        L.job[0].tg = ch->tgeom;
+        CUDA_TRY(launch_tile(ch->tkind, L, ch->tgeom.tiles_x * ch->tgeom.tiles_y, ch->tsmem, st));
         cur = out;
         return PCAD_OK;
     }
@@ -643,8 +701,22 @@ pcad_status create_common(const uint8_t *g_src, bool g_on_device, int H, int W, 
     const size_t pbytes = align_up((size_t)ptab_words() * sizeof(uint32_t), 256);
     const size_t bbytes = align_up((size_t)btab_bytes(), 256);
     const size_t obytes = align_up((size_t)tc_table_floats(m->L) * sizeof(float), 256);
+    int sms = 0, dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess)
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    // tile-resident sweeps: the models of tile_kind, but those whose small
+    // images AUTO gives the tensor-core sweep
+    const bool gibbs = m->sampler != PCAD_SAMPLER_PCA;
+    TileKind tkind;
+    TileGeom tgeom{};
+    size_t tsmem = 0;
+    const bool tile = (long long)H * W <= kTileMaxSites && tile_kind(tabs.dm, gibbs, tkind) &&
+                      tile_plan(tkind, H, W, sms, tgeom, tsmem);
+    const size_t xbytes = tile ? align_up(tile_xch_bytes(H, W), 256) : 0;
+    const size_t sbytes =
+        seg_structure(tabs.dm) ? align_up(seg_table_floats() * sizeof(float), 256) : 0;
     const size_t total =
-        3 * plane + 2 * fbytes + cbytes + tbytes + wbytes + pbytes + bbytes + obytes + misc;
+        sbytes + xbytes + 3 * plane + 2 * fbytes + cbytes + tbytes + wbytes + pbytes + bbytes + obytes + misc;
     cudaError_t e = cudaMallocAsync(&ch->block, total, ch->stream);
     if (e != cudaSuccess) {
         delete ch;
@@ -667,11 +739,18 @@ pcad_status create_common(const uint8_t *g_src, bool g_on_device, int H, int W, 
     ch->btab = (uint4 *)p; p += bbytes;
     ch->ftab = (float *)p; p += obytes;
     ch->wave_tiles = ntiles;
-    {
-        int dev = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess)
-            cudaDeviceGetAttribute(&ch->sms, cudaDevAttrMultiProcessorCount, dev);
+    if (sbytes) {
+        ch->stab = (float *)p;
+        p += sbytes;
     }
+    if (tile) {
+        ch->xch = (unsigned long long *)p;
+        p += xbytes;
+        ch->tkind = tkind;
+        ch->tgeom = tgeom;
+        ch->tsmem = tsmem;
+    }
+    ch->sms = sms;
     ch->tdev = (uint32_t *)p;
     ch->fp64 = (unsigned long long *)(p + 8);
     ch->mscratch = (double *)(p + 16);
@@ -703,12 +782,16 @@ pcad_status create_common(const uint8_t *g_src, bool g_on_device, int H, int W, 
                             cudaMemcpyHostToDevice, ch->stream);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(ch->tdev, 0, misc, ch->stream);
+    if (e == cudaSuccess && tile)
+        e = cudaMemsetAsync(ch->xch, 0, xbytes, ch->stream);   // no tag is 0
     if (e == cudaSuccess && m->L <= kSmallMaxLabels)
         e = launch_ptab(tabs.dm.T, ch->ptab, ch->stream);
-    if (e == cudaSuccess && (pca_tc_eligible(tabs.dm) || pca_win_eligible(tabs.dm))) {
+    if (e == cudaSuccess && (pca_tc_eligible(tabs.dm) || pca_win_eligible(tabs.dm)))
+        e = launch_tc_table(tabs.dm, ch->ftab, ch->stream);
+    if (e == cudaSuccess && seg_eligible(tabs.dm)) {
         DevModel dm = tabs.dm;
         dm.ta64 = ch->ta64;
-        e = launch_tc_table(dm, ch->ftab, ch->stream);
+        e = launch_seg_table(dm, ch->stab, ch->stream);
     }
     if (e == cudaSuccess && m->L == 2) {
         DevModel dm = tabs.dm;
@@ -736,6 +819,7 @@ pcad_status create_common(const uint8_t *g_src, bool g_on_device, int H, int W, 
     ch->dm.in64 = ch->in64;
     ch->dm.ptab = m->L <= kSmallMaxLabels ? ch->ptab : nullptr;
     ch->dm.btab = m->L == 2 ? ch->btab : nullptr;
+    ch->dm.stab = seg_eligible(ch->dm) ? ch->stab : nullptr;
     // TMA descriptors of the planes for the small-label kernel's tile form
     // (large images; temporal blocking encodes them on demand otherwise)
     if (m->L <= kSmallMaxLabels && (long long)H * W >= kSmallTmaMinSites)
@@ -786,9 +870,9 @@ pcad_status pcad_chain_run(pcad_chain *ch, int nsweeps)
         return fail(PCAD_EINVAL, "accumulator would leave the exact FP32 range");
     int left = nsweeps;
     // Whole captured blocks need the ping-pong parity at 0 (always true for
-    // Gibbs); the resident kernel runs any number of sweeps in one launch.
+    // Gibbs); the resident kernels run any number of sweeps in one launch.
     const bool parity_ok = ch->model.sampler != PCAD_SAMPLER_PCA || ch->cur == 0;
-    if (left >= kGraphSweeps && parity_ok && !uses_resident(ch)) {
+    if (left >= kGraphSweeps && parity_ok && !uses_resident(ch) && !uses_tile(ch)) {
         if (!ch->graph) {
             pcad_status st = build_graph(ch);
             if (st != PCAD_OK)
@@ -842,6 +926,8 @@ pcad_status pcad_chain_reset(pcad_chain *ch)
     CUDA_TRY(cudaMemsetAsync(ch->acc, 0, n * sizeof(float), ch->stream));
     CUDA_TRY(cudaMemsetAsync(ch->tdev, 0, 16, ch->stream));
     CUDA_TRY(cudaMemsetAsync(ch->err, 0, sizeof(int), ch->stream));
+    if (ch->xch)   // the sweep index, hence the border words' tags, starts again
+        CUDA_TRY(cudaMemsetAsync(ch->xch, 0, tile_xch_bytes(ch->H, ch->W), ch->stream));
     ch->cur = 0;
     ch->t = 0;
     ch->n_acc = 0;
@@ -855,7 +941,8 @@ pcad_status pcad_chain_sync(pcad_chain *ch)
     if (!ch)
         return fail(PCAD_EINVAL, "chain is NULL");
     CUDA_TRY(cudaStreamSynchronize(ch->stream));
-    if (ch->tb_k > 0 || uses_tc(ch) || uses_wave(ch) || uses_winw(ch) || small_tma(ch)) {
+    if (ch->tb_k > 0 || uses_tc(ch) || uses_wave(ch) || uses_winw(ch) || small_tma(ch) ||
+        uses_tile(ch)) {
         int e = 0;
         CUDA_TRY(cudaMemcpy(&e, ch->err, sizeof(int), cudaMemcpyDeviceToHost));
         if (e == 2)
@@ -912,10 +999,13 @@ pcad_status pcad_chain_set_model(pcad_chain *ch, const pcad_model *m)
     ch->dm.in64 = ch->in64;
     ch->dm.ptab = m->L <= kSmallMaxLabels ? ch->ptab : nullptr;   // T is unchanged
     ch->dm.btab = m->L == 2 ? ch->btab : nullptr;
+    ch->dm.stab = seg_eligible(ch->dm) ? ch->stab : nullptr;
     if (m->L == 2)   // stream-ordered after the new FP64 tables
         CUDA_TRY(launch_btab(ch->dm, ch->btab, ch->stream));
     if (pca_tc_eligible(ch->dm) || pca_win_eligible(ch->dm))
         CUDA_TRY(launch_tc_table(ch->dm, ch->ftab, ch->stream));
+    if (ch->dm.stab)
+        CUDA_TRY(launch_seg_table(ch->dm, ch->stab, ch->stream));
     ch->ecoef = energy_coef(*m, (long)ch->H * ch->W);
     return PCAD_OK;
 }

@@ -61,6 +61,7 @@ struct DevModel {
     const double *in64;  // [256] Lp price factor exp(-lambda (d / (L - 1))^p), FP64
     double el64;         // e^lambda, FP64
     const uint32_t *ptab;  // small-L sweep: pair prior table (nullptr: not built)
+    const float *stab;     // segment draw: prefix tables (nullptr: not built)
     const uint4 *btab;     // two-label draw thresholds per site configuration (nullptr: not built)
 };
 
@@ -579,17 +580,20 @@ __device__ __forceinline__ double weight64(const DevModel &m, int g, int xi, con
 // set: for each such lane in turn, the 32 lanes compute 8 labels' FP64
 // weights each, an FP64 warp scan gives the CDF, and the lane holding u*Z
 // finds the label.  All 32 lanes of the warp must call this together.
+// Draws of lanes with `count` set are added to *counter.
 template <int NB, int NORM = 0>
 __device__ __forceinline__ int warp_redraw_fp64(const DevModel &m, bool need, const SiteIn<NB> &in,
-                                                int s, unsigned long long *counter)
+                                                int s, unsigned long long *counter,
+                                                bool count = true)
 {
     constexpr unsigned kFull = 0xFFFFFFFFu;
     unsigned todo = __ballot_sync(kFull, need);
     if (todo == 0u)
         return s;
     const int lane = (int)(threadIdx.x & 31u);
-    if (lane == 0)
-        atomicAdd(counter, (unsigned long long)__popc(todo));
+    const unsigned counted = todo & __ballot_sync(kFull, count);
+    if (lane == 0 && counted)
+        atomicAdd(counter, (unsigned long long)__popc(counted));
     while (todo) {
         const int leader = __ffs((int)todo) - 1;
         todo &= todo - 1u;

@@ -288,8 +288,7 @@ bool pca_tc_auto(const DevModel &m);
 
 // The outside-window chunk sums of a model, as the batched tensor-core
 // sweep reads them: tc_table_floats(L) floats (16-byte aligned), written by
-// launch_tc_table (m.ta64 set: the segment draw's prefix tables follow, at
-// kTabF floats, for the models it accepts).
+// launch_tc_table.
 int tc_table_floats(int L);
 cudaError_t launch_tc_table(const DevModel &m, float *out, cudaStream_t s);
 
@@ -331,19 +330,21 @@ cudaError_t launch_gibbs_win(const SweepArgs &a, int q, const float *ftab, cudaS
 // The segment draw (seg_draw.cuh) in the windowed sweeps' launch forms, for
 // the models seg_eligible accepts (a subset of pca_win_eligible's with 4
 // neighbours and c >= 0): launch_pca_win and its siblings hand such models
-// over.  stab: the prefix tables (seg_table_floats() floats, 16-byte aligned,
-// written by launch_seg_table from m.ta64).
+// over once their prefix tables are in place (a.m.stab: seg_table_floats()
+// floats, 16-byte aligned, written by launch_seg_table from m.ta64).
+// seg_structure: the models whose coefficients may make them eligible.
 int seg_table_floats();
 float seg_offset(const DevModel &m);   // DevModel::cbs of a model's coefficients
 bool seg_eligible(const DevModel &m);
+bool seg_structure(const DevModel &m);
 cudaError_t launch_seg_table(const DevModel &m, float *out, cudaStream_t s);
-cudaError_t launch_pca_seg(const SweepArgs &a, const float *stab, uint8_t *x0, uint8_t *x1,
+cudaError_t launch_pca_seg(const SweepArgs &a, uint8_t *x0, uint8_t *x1,
                            const uint32_t *budget, cudaStream_t s);
-cudaError_t launch_gibbs_seg(const SweepArgs &a, int q, const float *stab, cudaStream_t s);
-cudaError_t launch_pca_segw(const SweepArgs &a, const float *stab, uint8_t *x0, uint8_t *x1, int n,
+cudaError_t launch_gibbs_seg(const SweepArgs &a, int q, cudaStream_t s);
+cudaError_t launch_pca_segw(const SweepArgs &a, uint8_t *x0, uint8_t *x1, int n,
                             unsigned int *done, unsigned int *grab, int *err, bool par_from_t,
                             const uint32_t *budget, cudaStream_t s);
-cudaError_t launch_gibbs_segw(const SweepArgs &a, const float *stab, uint8_t *x, int nsweeps,
+cudaError_t launch_gibbs_segw(const SweepArgs &a, uint8_t *x, int nsweeps,
                               unsigned int *done, unsigned int *grab, int *err, cudaStream_t s);
 
 // Batched tensor-core sweeps: nsweeps sweeps of every slot listed in items

@@ -72,7 +72,7 @@ __device__ __forceinline__ void load_tab(float *tab, const float *src, int tid, 
 // One lazy-PCA sweep: a.xin -> a.xout (or the planes x0 / x1 by the parity of
 // the sweep index), skipped at or past *budget.
 __global__ void __launch_bounds__(kSegThreads, 3)
-    pca_seg_kernel(const SweepArgs a, const float *stab, int tiles_x, int ntiles, uint8_t *x0,
+    pca_seg_kernel(const SweepArgs a, int tiles_x, int ntiles, uint8_t *x0,
                    uint8_t *x1, const uint32_t *budget)
 {
     __shared__ __align__(16) float tab[kSegFloats];
@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(kSegThreads, 3)
     const uint8_t *xin = x0 ? ((t & 1u) ? x1 : x0) : a.xin;
     uint8_t *xout = x0 ? ((t & 1u) ? x0 : x1) : a.xout;
     const int lane = (int)threadIdx.x & 31, wp = (int)threadIdx.x >> 5;
-    load_tab(tab, stab, (int)threadIdx.x, kSegThreads);
+    load_tab(tab, a.m.stab, (int)threadIdx.x, kSegThreads);
     __syncthreads();
     const bool acc_on = accumulate_after(a, t);
     const int H = a.H, W = a.W;
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(kSegThreads, 3)
 
 // Wavefront form: items, waits and planes as pca_winw_kernel's.
 __global__ void __launch_bounds__(kSegwThreads, 8)
-    pca_segw_kernel(const SweepArgs a, const float *stab, uint8_t *x0, uint8_t *x1, int nsweeps,
+    pca_segw_kernel(const SweepArgs a, uint8_t *x0, uint8_t *x1, int nsweeps,
                     int tiles_x, int tiles_y, unsigned int *done, unsigned int *grab, int *err,
                     int par_from_t, const uint32_t *budget)
 {
@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(kSegwThreads, 8)
     const unsigned int total = ntiles * (unsigned int)nsweeps;
     const uint32_t t0 = sweep_index(a);
     const long long limit = wait_limit(a.wait_ns);
-    load_tab(tab, stab, tid, kSegwThreads);
+    load_tab(tab, a.m.stab, tid, kSegwThreads);
     if (tid == 0)
         s_next = atomicAdd(grab, 1u);
     __syncthreads();
@@ -264,14 +264,14 @@ __device__ __forceinline__ void gibbs_uniforms(const SweepArgs &a, int row0, int
 // accumulated.  A phase writes one colour and reads the other, but for the
 // site's own label, which only the accumulation reads, after its own write.
 __global__ void __launch_bounds__(kSegThreads, 4)
-    gibbs_seg_kernel(const SweepArgs a, int q, const float *stab, int tiles_x, int ntiles)
+    gibbs_seg_kernel(const SweepArgs a, int q, int tiles_x, int ntiles)
 {
     __shared__ __align__(16) float tab[kSegFloats];
     __shared__ __align__(16) uint32_t U_s[kSegWarps][kSY * 2 * kSX];
     uint8_t *x = const_cast<uint8_t *>(a.xin);
     const uint32_t t = sweep_index(a);
     const int lane = (int)threadIdx.x & 31, wp = (int)threadIdx.x >> 5;
-    load_tab(tab, stab, (int)threadIdx.x, kSegThreads);
+    load_tab(tab, a.m.stab, (int)threadIdx.x, kSegThreads);
     __syncthreads();
     const bool acc_on = a.last_phase && accumulate_after(a, t);
     uint32_t *U = U_s[wp];
@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(kSegThreads, 4)
 
 // Wavefront of colour phases: items and waits as gibbs_winw_kernel's.
 __global__ void __launch_bounds__(kSegwThreads, 7)
-    gibbs_segw_kernel(const SweepArgs a, const float *stab, uint8_t *x, int nphases, int tiles_x,
+    gibbs_segw_kernel(const SweepArgs a, uint8_t *x, int nphases, int tiles_x,
                       int tiles_y, unsigned int *done, unsigned int *grab, int *err)
 {
     __shared__ __align__(16) float tab[kSegFloats];
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(kSegwThreads, 7)
     const unsigned int total = ntiles * (unsigned int)nphases;
     const uint32_t t0 = sweep_index(a);
     const long long limit = wait_limit(a.wait_ns);
-    load_tab(tab, stab, tid, kSegwThreads);
+    load_tab(tab, a.m.stab, tid, kSegwThreads);
     if (tid == 0)
         s_next = atomicAdd(grab, 1u);
     __syncthreads();
@@ -429,11 +429,15 @@ int seg_table_floats()
 // four neighbours more than (127 - S) / (4 mu) labels away from the
 // observation, so that distance must be one the noise does not reach.  The
 // rows' sums must stay below 2^127.
+bool seg_structure(const DevModel &m)
+{
+    return m.nbhd == 4 && m.T >= 1 && m.L >= 9 && m.L <= 256;
+}
+
 float seg_offset(const DevModel &m)
 {
     const float no = NAN;
-    if (m.nbhd != 4 || m.norm != 0 || m.gam > 0.0f || m.alpha > 0.0f || m.T < 1 || m.L < 9 ||
-        m.L > 256)
+    if (!seg_structure(m) || m.norm != 0 || m.gam > 0.0f || m.alpha > 0.0f)
         return no;
     const double mu = -(double)m.gam, A = mu * 4.0 * m.T, range = m.L - 1 + m.T;
     const double S = std::ceil(std::fmax(0.0, 4.0 * mu * range + A - 125.0));
@@ -463,7 +467,7 @@ cudaError_t launch_seg_table(const DevModel &m, float *out, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_pca_seg(const SweepArgs &a, const float *stab, uint8_t *x0, uint8_t *x1,
+cudaError_t launch_pca_seg(const SweepArgs &a, uint8_t *x0, uint8_t *x1,
                            const uint32_t *budget, cudaStream_t st)
 {
     static int per_sm[64] = {};
@@ -477,11 +481,11 @@ cudaError_t launch_pca_seg(const SweepArgs &a, const float *stab, uint8_t *x0, u
         return cudaErrorInvalidValue;
     const long long need = (ntiles + kSegWarps - 1) / kSegWarps;
     pca_seg_kernel<<<(int)(need < cap ? need : cap), kSegThreads, 0, st>>>(
-        a, stab, tiles_x, (int)ntiles, x0, x1, budget);
+        a, tiles_x, (int)ntiles, x0, x1, budget);
     return cudaGetLastError();
 }
 
-cudaError_t launch_gibbs_seg(const SweepArgs &a, int q, const float *stab, cudaStream_t st)
+cudaError_t launch_gibbs_seg(const SweepArgs &a, int q, cudaStream_t st)
 {
     static int per_sm[64] = {};
     int cap = 0;
@@ -493,12 +497,12 @@ cudaError_t launch_gibbs_seg(const SweepArgs &a, int q, const float *stab, cudaS
     if (ntiles >= (1ll << 30))
         return cudaErrorInvalidValue;
     const long long need = (ntiles + kSegWarps - 1) / kSegWarps;
-    gibbs_seg_kernel<<<(int)(need < cap ? need : cap), kSegThreads, 0, st>>>(a, q, stab, tiles_x,
+    gibbs_seg_kernel<<<(int)(need < cap ? need : cap), kSegThreads, 0, st>>>(a, q, tiles_x,
                                                                              (int)ntiles);
     return cudaGetLastError();
 }
 
-cudaError_t launch_pca_segw(const SweepArgs &a, const float *stab, uint8_t *x0, uint8_t *x1, int n,
+cudaError_t launch_pca_segw(const SweepArgs &a, uint8_t *x0, uint8_t *x1, int n,
                             unsigned int *done, unsigned int *grab, int *err, bool par_from_t,
                             const uint32_t *budget, cudaStream_t st)
 {
@@ -513,11 +517,11 @@ cudaError_t launch_pca_segw(const SweepArgs &a, const float *stab, uint8_t *x0, 
         return cudaErrorInvalidValue;
     // at most the resident capacity: every block that takes an item runs
     pca_segw_kernel<<<(int)(items < cap ? items : cap), dim3(kSX, kSY), 0, st>>>(
-        a, stab, x0, x1, n, tiles_x, tiles_y, done, grab, err, par_from_t ? 1 : 0, budget);
+        a, x0, x1, n, tiles_x, tiles_y, done, grab, err, par_from_t ? 1 : 0, budget);
     return cudaGetLastError();
 }
 
-cudaError_t launch_gibbs_segw(const SweepArgs &a, const float *stab, uint8_t *x, int nsweeps,
+cudaError_t launch_gibbs_segw(const SweepArgs &a, uint8_t *x, int nsweeps,
                               unsigned int *done, unsigned int *grab, int *err, cudaStream_t st)
 {
     static int per_sm[64] = {};
@@ -530,7 +534,7 @@ cudaError_t launch_gibbs_segw(const SweepArgs &a, const float *stab, uint8_t *x,
     if (items >= (1ll << 32))
         return cudaErrorInvalidValue;
     gibbs_segw_kernel<<<(int)(items < cap ? items : cap), dim3(kSX, kSY), 0, st>>>(
-        a, stab, x, 2 * nsweeps, tiles_x, tiles_y, done, grab, err);
+        a, x, 2 * nsweeps, tiles_x, tiles_y, done, grab, err);
     return cudaGetLastError();
 }
 

@@ -964,7 +964,7 @@ bool pca_tc_auto(const DevModel &m)
 
 int tc_table_floats(int)
 {
-    return kTabF + seg_table_floats();
+    return kTabF;
 }
 
 cudaError_t launch_tc_table(const DevModel &m, float *out, cudaStream_t st)
@@ -973,8 +973,7 @@ cudaError_t launch_tc_table(const DevModel &m, float *out, cudaStream_t st)
         tc_table_kernel<true><<<(kTabF + 255) / 256, 256, 0, st>>>(m, out);
     else
         tc_table_kernel<false><<<(kTabF + 255) / 256, 256, 0, st>>>(m, out);
-    const cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess && seg_eligible(m) ? launch_seg_table(m, out + kTabF, st) : e;
+    return cudaGetLastError();
 }
 
 cudaError_t launch_pca_tc(const SweepArgs &a, uint8_t *x0, uint8_t *x1, int nsweeps,

@@ -1,0 +1,661 @@
+// Tile-resident sweeps: images of a few hundred to a few thousand sites per
+// SM, whole runs in one cooperative launch (lazy PCA, Section 5.2;
+// checkerboard Gibbs, Section 5.1).
+//
+// A sweep of such an image is shorter than what one launch per sweep costs
+// around it: at 256^2, 9 labels and 8 neighbours, the per-sweep small-label
+// kernel took 6.3 us per sweep (launch gap, tables, tile staging, four draws
+// in a row per thread) and a Gibbs sweep 11.4 us (four launches), for draws
+// that fill the SMs' issue slots for 0.5 us.  Here every CTA owns one tile for
+// all sweeps of a run: labels, observation, accumulator and tables stay in
+// shared memory, and only tile borders travel.
+//
+//   * Exchange.  After a sweep the tile's border words (4 labels) go to an
+//     exchange buffer in global memory as 64-bit stores of (labels, tag = the
+//     sweep's number), and the neighbours' threads poll exactly the words of
+//     their halo until the tag is the sweep's: data and flag are one relaxed
+//     64-bit access, so a sweep waits for one store-to-load trip through L2
+//     and needs no fence.  Two buffers by sweep parity suffice: a tile writes
+//     sweep k + 2 only after its neighbours' words of k + 1 arrived, which
+//     they published after reading this tile's words of k.
+//   * Gibbs.  A sweep's 2 (4) colour phases run without exchange: the halo is
+//     2 (4) sites wide and phase q also updates the sites up to 1 - q (3 - q)
+//     beyond the tile.  Draws are keyed by (sweep, site), so both owners of
+//     such a site draw the same label.
+//   * The next sweep's uniforms are computed while the border words travel.
+//   * A launch holds one chain, or (batches, the server) several small ones,
+//     each on CTAs of its own.
+//
+// The draws are the other kernels': the small-label draw, the segment draw and
+// the two-label threshold table.  The CTAs wait on one another, so the launch is cooperative (all resident);
+// every poll is bounded (elapsed time, or another wait's error flag).
+// Measured times stand at uses_tile in capi.cu.
+#include <type_traits>
+
+#include "async_ptx.cuh"
+#include "seg_draw.cuh"
+#include "small_draw.cuh"
+#include "tile.h"
+
+namespace pcad {
+
+namespace {
+
+using namespace sld;
+
+constexpr int kTlThreads = 512;
+constexpr int kTlMaxSites = 8192;      // sites per tile
+constexpr int kTlMaxSmem = 224 * 1024;    // one CTA per SM
+constexpr int kTlMaxSmem2 = 112 * 1024;   // two
+
+__device__ __forceinline__ unsigned long long ld_word(const unsigned long long *p)
+{
+    unsigned long long v;
+    asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void st_word(unsigned long long *p, unsigned long long v)
+{
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// The labels of an exchange word once its tag is `tag`; false when the wait
+// ran out or another wait of the launch did.
+__device__ __forceinline__ bool poll_word(const unsigned long long *p, uint32_t tag, uint32_t &w,
+                                          const int *err, long long limit_ns)
+{
+    unsigned long long v = ld_word(p);
+    if ((uint32_t)(v >> 32) != tag) {
+        const unsigned long long t0 = globaltimer_ns();
+        for (unsigned int i = 1; (uint32_t)((v = ld_word(p)) >> 32) != tag; ++i)
+            if ((i & 63u) == 0u &&
+                (ld_flag(err) != 0 || (long long)(globaltimer_ns() - t0) > limit_ns))
+                return false;
+    }
+    w = (uint32_t)v;
+    return true;
+}
+
+// Halo width: a PCA sweep reads one site around the tile, a Gibbs sweep as
+// many as it has phases.
+__host__ __device__ constexpr int tile_halo(int nb, bool gibbs)
+{
+    return !gibbs ? 1 : (nb == 4 ? 2 : 4);
+}
+
+// ------------------------------------------------------------------- draws
+// A draw policy: kFill, the staged word outside the image; kTabBytes of
+// shared tables and kRowBytes of shared scratch per thread; load() fills the
+// tables; draw(), called by all lanes of a warp, returns the new label of the
+// site at `me` (rows of SB bytes) at image position (r, c).  Re-draws in FP64
+// are counted for sites of the tile itself (own).
+
+template <int LMAX, int NB_, bool MASK>
+struct SmallPol {
+    static constexpr int NB = NB_;
+    static constexpr uint32_t kFill = 0x10101010u;   // code 16: missing
+    static constexpr int kTabBytes = kPtabWords * 4 + 16 * kAqStride * 4;
+    static constexpr int kRowBytes = kPrefixStride * 4;
+    uint32_t *pt;
+    float *aq, *pre;
+
+    __device__ __forceinline__ void load(const DevModel &m, uint8_t *tab, uint8_t *row, int tid)
+    {
+        pt = reinterpret_cast<uint32_t *>(tab);
+        aq = reinterpret_cast<float *>(tab + kPtabWords * 4);
+        pre = reinterpret_cast<float *>(row);
+        for (int i = tid; i < kPtabWords / 4; i += kTlThreads)
+            reinterpret_cast<uint4 *>(pt)[i] = __ldg(reinterpret_cast<const uint4 *>(m.ptab) + i);
+        fill_aq(m, aq, tid, kTlThreads);
+    }
+
+    __device__ __forceinline__ int draw(const SweepArgs &a, const uint8_t *me, int SB, int g,
+                                        uint32_t ub, int, int, bool valid, bool own)
+    {
+        int nc[NB], xi = 0, s = 0;
+        bool certain = true;
+        if (valid) {
+            nc[0] = me[-SB];
+            nc[1] = me[SB];
+            nc[2] = me[-1];
+            nc[3] = me[1];
+            if constexpr (NB == 8) {
+                nc[4] = me[-SB - 1];
+                nc[5] = me[-SB + 1];
+                nc[6] = me[SB - 1];
+                nc[7] = me[SB + 1];
+            }
+            xi = me[0];
+            s = draw_small<LMAX, NB, MASK, true>(a.m, pt, nc, g, xi, ub, pre, certain, aq);
+        }
+        if (__any_sync(0xFFFFFFFFu, valid && !certain)) {
+            SiteIn<NB> in{};
+            in.g = g;
+            in.xi = xi;
+            in.ub = ub;
+#pragma unroll
+            for (int j = 0; j < NB; ++j)
+                in.xni[j] = valid && nc[j] != 16 ? nc[j] : kMissingLabelI;
+            s = warp_redraw_fp64<NB>(a.m, valid && !certain, in, s, a.fp64_draws, own);
+        }
+        return s;
+    }
+    __device__ __forceinline__ void finish(const SweepArgs &) {}
+};
+
+struct SegPol {
+    static constexpr int NB = 4;
+    static constexpr uint32_t kFill = 0u;
+    static constexpr int kTabBytes = seg::kSegFloats * 4;
+    static constexpr int kRowBytes = 0;
+    float *tab;
+
+    __device__ __forceinline__ void load(const DevModel &m, uint8_t *t, uint8_t *, int tid)
+    {
+        tab = reinterpret_cast<float *>(t);
+        for (int i = tid; i < seg::kSegFloats / 4; i += kTlThreads)
+            reinterpret_cast<float4 *>(tab)[i] =
+                __ldg(reinterpret_cast<const float4 *>(m.stab) + i);
+    }
+
+    __device__ __forceinline__ int draw(const SweepArgs &a, const uint8_t *me, int SB, int g,
+                                        uint32_t ub, int r, int c, bool valid, bool own)
+    {
+        SiteIn<4> in{};
+        bool certain = true;
+        int s = 0;
+        if (valid) {
+            in.g = g;
+            in.xi = me[0];
+            in.ub = ub;
+            in.xni[0] = r > 0 ? (int)me[-SB] : kMissingLabelI;
+            in.xni[1] = r + 1 < a.H ? (int)me[SB] : kMissingLabelI;
+            in.xni[2] = c > 0 ? (int)me[-1] : kMissingLabelI;
+            in.xni[3] = c + 1 < a.W ? (int)me[1] : kMissingLabelI;
+            s = seg::draw_seg(a.m, tab, in, certain);
+        }
+        return warp_redraw_fp64<4>(a.m, valid && !certain, in, s, a.fp64_draws, own);
+    }
+    __device__ __forceinline__ void finish(const SweepArgs &) {}
+};
+
+template <int NB_>
+struct BinPol {
+    static constexpr int NB = NB_;
+    static constexpr uint32_t kFill = 0u;   // a missing neighbour is no label-1 neighbour
+    static constexpr int kEntries = 4 * (NB + 1) * (NB + 1);
+    static constexpr int kTabBytes = kEntries * 16;
+    static constexpr int kRowBytes = 0;
+    const uint4 *tab;
+    uint32_t nre;
+
+    __device__ __forceinline__ void load(const DevModel &m, uint8_t *t, uint8_t *, int tid)
+    {
+        for (int i = tid; i < kEntries; i += kTlThreads)
+            reinterpret_cast<uint4 *>(t)[i] = m.btab[i];
+        tab = reinterpret_cast<const uint4 *>(t);
+        nre = 0u;
+    }
+
+    __device__ __forceinline__ int draw(const SweepArgs &a, const uint8_t *me, int SB, int g,
+                                        uint32_t ub, int r, int c, bool valid, bool own)
+    {
+        if (!valid)
+            return 0;
+        int n1 = me[-SB] + me[SB] + me[-1] + me[1];
+        const int top = r == 0, bot = r + 1 == a.H, le = c == 0, ri = c + 1 == a.W;
+        int nm = top + bot + le + ri;
+        if constexpr (NB == 8) {
+            n1 += me[-SB - 1] + me[-SB + 1] + me[SB - 1] + me[SB + 1];
+            nm += (top | le) + (top | ri) + (bot | le) + (bot | ri);
+        }
+        const uint4 e = tab[((g * (NB + 1) + nm) * (NB + 1) + n1) * 2 + me[0]];
+        nre += own && ub - e.y < e.z ? 1u : 0u;
+        return ub >= e.x ? 1 : 0;
+    }
+    __device__ __forceinline__ void finish(const SweepArgs &a)
+    {
+        const uint32_t n = __reduce_add_sync(0xFFFFFFFFu, nre);
+        if ((threadIdx.x & 31u) == 0u && n != 0u)
+            atomicAdd(a.fp64_draws, (unsigned long long)n);
+    }
+};
+
+// Shared memory of a tile (bytes), in the order of the kernel's pointers:
+// tables, thread scratch, uniforms, label planes, observation, counts.
+template <class P, bool GIBBS>
+size_t tile_smem(int th, int twq)
+{
+    const int h = tile_halo(P::NB, GIBBS);
+    const size_t words = (size_t)(th + 2 * h) * (twq + 2);
+    return (size_t)P::kTabBytes + (size_t)kTlThreads * P::kRowBytes + words * 16 +
+           words * 4 * (GIBBS ? 1 : 2) + words * 4 + (size_t)th * twq * 16;
+}
+
+template <class P, bool GIBBS, int JOBS>
+__global__ void __launch_bounds__(kTlThreads, 2)
+    tile_kernel(const __grid_constant__ TileLaunchT<JOBS> L)
+{
+    constexpr bool MULTI = JOBS > 1;
+    extern __shared__ __align__(16) uint8_t sm[];
+    constexpr int NB = P::NB;
+    constexpr int h = tile_halo(NB, GIBBS);
+    constexpr int kCol = NB == 4 ? 2 : 4;
+    int j = 0;
+    if (MULTI)
+        while (j + 1 < L.njobs && (int)blockIdx.x >= L.job[j + 1].cta0)
+            ++j;
+    const TileJob &J = L.job[MULTI ? j : 0];
+    const SweepArgs &a = J.a;
+    int *const err = L.err;
+    const int cta = (int)blockIdx.x - (MULTI ? J.cta0 : 0);
+    const int tid = (int)threadIdx.x;
+    const int TH = J.tg.th, TWq = J.tg.twq, TW = 4 * TWq;
+    const int SW = TWq + 2, SB = 4 * SW;            // words and bytes per staged row
+    const int words = (TH + 2 * h) * SW;
+    const int H = a.H, W = a.W, Wq = (W + 3) >> 2;
+    const int ty = cta / J.tg.tiles_x, tx = cta - ty * J.tg.tiles_x;
+    const int r0 = ty * TH, q0 = tx * TWq, c0 = 4 * q0;
+    const uint32_t t0 = sweep_index(a);
+    int nsweeps = L.nsweeps;
+    if (J.budget) {   // a slot runs up to its budget (the same for all its CTAs)
+        const uint32_t b = *J.budget;
+        nsweeps = b > t0 ? (int)min((uint32_t)nsweeps, b - t0) : 0;
+    }
+    if (nsweeps == 0)
+        return;
+    // planes: in and out, or those of even and odd sweep indices
+    const uint8_t *xg_in = J.par_from_t && (t0 & 1u) ? J.x1 : J.x0;
+    uint8_t *xg_out = J.par_from_t ? (((t0 + (uint32_t)nsweeps) & 1u) ? J.x1 : J.x0) : J.x1;
+
+    uint8_t *const tab = sm;
+    uint8_t *const row = sm + P::kTabBytes + tid * P::kRowBytes;
+    uint32_t *U = reinterpret_cast<uint32_t *>(sm + P::kTabBytes + kTlThreads * P::kRowBytes);
+    uint32_t *pl0 = U + 4 * words;
+    uint32_t *pl1 = GIBBS ? pl0 : pl0 + words;
+    uint32_t *gw = pl1 + words;
+    uint32_t *cnt = gw + words;                     // [TH][TW] label sums of this launch
+    P pol;
+    pol.load(a.m, tab, row, tid);
+    // labels and observation with the halo
+    for (int i = tid; i < words; i += kTlThreads) {
+        const int sr = i / SW, sq = i - sr * SW;
+        const int r = r0 - h + sr, q = q0 - 1 + sq;
+        uint32_t x = P::kFill, g = 0u;
+        if (r >= 0 && r < H && q >= 0 && q < Wq) {
+            x = *reinterpret_cast<const uint32_t *>(xg_in + (size_t)r * a.pitch + 4 * q);
+            g = *reinterpret_cast<const uint32_t *>(a.g + (size_t)r * a.pitch + 4 * q);
+            const int nv = W - 4 * q;
+            if (nv < 4) {
+                const uint32_t mask = (1u << (8 * nv)) - 1u;
+                x = (x & mask) | (P::kFill & ~mask);
+                g &= mask;
+            }
+        }
+        pl0[i] = x;
+        if (!GIBBS)
+            pl1[i] = P::kFill;
+        gw[i] = g;
+    }
+    for (int i = tid; i < TH * TW; i += kTlThreads)
+        cnt[i] = 0u;
+
+    const long long limit = wait_limit(a.wait_ns);
+    const uint32_t key0 = (uint32_t)(a.seed & 0xFFFFFFFFull), key1 = (uint32_t)(a.seed >> 32);
+    const uint32_t ctr3 = ((GIBBS ? kTagGibbs : kTagPCA) << 24) | (a.chain & 0xFFFFFFu);
+    // the uniforms of a sweep: the tile's quads (Gibbs: with the halo's), at
+    // their staged word
+    const auto uniforms = [&](uint32_t t) {
+        const int nw = GIBBS ? words : TH * TWq;
+        for (int i = tid; i < nw; i += kTlThreads) {
+            int sr, sq;
+            if (GIBBS) {
+                sr = i / SW;
+                sq = i - sr * SW;
+            } else {
+                sr = i / TWq;
+                sq = i - sr * TWq + 1;
+                sr += h;
+            }
+            uint32_t o0, o1, o2, o3;
+            philox4x32_10((uint32_t)(q0 - 1 + sq), (uint32_t)(r0 - h + sr + a.row_off), t, ctr3,
+                          key0, key1, o0, o1, o2, o3);
+            reinterpret_cast<uint4 *>(U)[sr * SW + sq] =
+                make_uint4(o0 >> 8, o1 >> 8, o2 >> 8, o3 >> 8);
+        }
+    };
+    // the draw of the site at local (lr, lc) from plane X
+    const auto draw = [&](const uint32_t *X, int lr, int lc, bool valid, bool own) -> int {
+        const int o = (lr + h) * SB + lc + 4;
+        const int g = valid ? (int)reinterpret_cast<const uint8_t *>(gw)[o] : 0;
+        const uint32_t ub = valid ? U[o] : 0u;
+        return pol.draw(a, reinterpret_cast<const uint8_t *>(X) + o, SB, g, ub, r0 + lr, c0 + lc,
+                        valid, own);
+    };
+    uniforms(t0);
+    bool ok = true;
+    uint32_t *X = pl0;
+    for (int k = 0; k < nsweeps; ++k) {
+        const uint32_t t = t0 + (uint32_t)k;
+        const bool acc_now = accumulate_after(a, t);
+        // halo words and uniforms in place; leave together when a wait gave up
+        if (__syncthreads_or(!ok)) {
+            if (tid == 0)
+                atomicExch(err, 1);
+            return;
+        }
+        if constexpr (!GIBBS) {
+            uint32_t *Y = X == pl0 ? pl1 : pl0;
+            for (int b = 0; b < TH * TW; b += kTlThreads) {
+                const int i = b + tid;
+                const int lr = (int)__umulhi((unsigned int)i, J.tg.inv_tw), lc = i - lr * TW;
+                const bool valid = i < TH * TW && r0 + lr < H && c0 + lc < W;
+                const int s = draw(X, lr, lc, valid, true);
+                if (valid) {
+                    reinterpret_cast<uint8_t *>(Y)[(lr + h) * SB + lc + 4] = (uint8_t)s;
+                    if (acc_now)
+                        cnt[i] += (uint32_t)s;
+                }
+            }
+            X = Y;
+            __syncthreads();
+        } else {
+#pragma unroll 1
+            for (int q = 0; q < kCol; ++q) {
+                // colour q of rows [-e, TH + e), columns [-e, TW + e)
+                const int e = kCol - 1 - q;
+                int nr, per, sr0, sc0;   // rows, sites per row, first row and column
+                if (NB == 4) {
+                    nr = TH + 2 * e;
+                    per = (TW + 2 * e + 1) >> 1;
+                    sr0 = -e;
+                    sc0 = -e;
+                } else {
+                    sr0 = -e + ((r0 - e + (q >> 1)) & 1);
+                    sc0 = -e + ((-e + q) & 1);
+                    nr = (TH + e - sr0 + 1) >> 1;
+                    per = (TW + e - sc0 + 1) >> 1;
+                }
+                const unsigned int inv = 0xFFFFFFFFu / (unsigned int)per + 1u;
+                for (int b = 0; b < nr * per; b += kTlThreads) {
+                    const int i = b + tid;
+                    const int ir = (int)__umulhi((unsigned int)i, inv), ic = i - ir * per;
+                    const int lr = NB == 4 ? sr0 + ir : sr0 + 2 * ir;
+                    int lc = sc0 + 2 * ic;
+                    if (NB == 4)
+                        lc += (r0 + lr + c0 + lc + q) & 1;
+                    const bool valid = ir < nr && lc < TW + e && (unsigned)(r0 + lr) < (unsigned)H &&
+                                       (unsigned)(c0 + lc) < (unsigned)W;
+                    const int s = draw(X, lr, lc, valid,
+                                       (unsigned)lr < (unsigned)TH && (unsigned)lc < (unsigned)TW);
+                    if (valid)
+                        reinterpret_cast<uint8_t *>(X)[(lr + h) * SB + lc + 4] = (uint8_t)s;
+                }
+                __syncthreads();
+            }
+            if (acc_now)
+                for (int i = tid; i < TH * TW; i += kTlThreads) {
+                    const int lr = (int)__umulhi((unsigned int)i, J.tg.inv_tw), lc = i - lr * TW;
+                    cnt[i] += reinterpret_cast<const uint8_t *>(X)[(lr + h) * SB + lc + 4];
+                }
+        }
+        // (a single Gibbs sweep, written back in place, still waits for the
+        // neighbours: they have then read their halo of the initial labels)
+        if (k + 1 == nsweeps && !(GIBBS && nsweeps == 1))
+            break;
+        // publish the border words of this sweep
+        const uint32_t tag = t + 1u;
+        unsigned long long *buf = J.xch + (size_t)(tag & 1u) * H * Wq;
+        if ((int)blockIdx.x != a.stall_tile - 1)
+            for (int i = tid; i < TH * TWq; i += kTlThreads) {
+                const int lr = i / TWq, lq = i - lr * TWq;
+                const bool border = lr < h || lr >= TH - h || lq == 0 || lq == TWq - 1;
+                if (border && r0 + lr < H && q0 + lq < Wq)
+                    st_word(buf + (size_t)(r0 + lr) * Wq + q0 + lq,
+                            ((unsigned long long)tag << 32) | X[(lr + h) * SW + lq + 1]);
+            }
+        uniforms(t + 1u);
+        // poll the halo: h rows above and below (with the corners where they
+        // are read), one word left and right of each row
+        const int nrow = 2 * h * SW, nh = nrow + 2 * TH;
+        for (int i = tid; i < nh && ok; i += kTlThreads) {
+            int sr, sq;
+            if (i < nrow) {
+                sr = i / SW;
+                sq = i - sr * SW;
+                if (NB == 4 && !GIBBS && (sq == 0 || sq == SW - 1))
+                    continue;   // no diagonal neighbours
+                sr = sr < h ? sr : sr + TH;
+            } else {
+                sr = h + ((i - nrow) >> 1);
+                sq = (i & 1) ? SW - 1 : 0;   // nrow is even
+            }
+            const int r = r0 - h + sr, q = q0 - 1 + sq;
+            if (r < 0 || r >= H || q < 0 || q >= Wq)
+                continue;
+            uint32_t w;
+            ok = poll_word(buf + (size_t)r * Wq + q, tag, w, err, limit);
+            if (ok)
+                X[sr * SW + sq] = w;
+        }
+    }
+    if (__syncthreads_or(!ok)) {
+        if (tid == 0)
+            atomicExch(err, 1);
+        return;
+    }
+    pol.finish(a);
+    // labels and counts back (any label of this plane that a neighbour read at
+    // the start was read before it published its first sweep, which this tile
+    // awaited, or the planes differ)
+    for (int i = tid; i < TH * TWq; i += kTlThreads) {
+        const int lr = i / TWq, lq = i - lr * TWq;
+        const int r = r0 + lr, c = c0 + 4 * lq;
+        if (r >= H || c >= W)
+            continue;
+        const uint32_t w = X[(lr + h) * SW + lq + 1];
+        float *pa = a.acc + (size_t)r * W + c;
+        const uint32_t *n4 = cnt + lr * TW + 4 * lq;
+        const int nv = min(4, W - c);
+        if (nv == 4)
+            *reinterpret_cast<uint32_t *>(xg_out + (size_t)r * a.pitch + c) = w;
+        for (int b = 0; b < nv; ++b) {
+            if (nv < 4)
+                xg_out[(size_t)r * a.pitch + c + b] = (uint8_t)(w >> (8 * b));
+            if (n4[b])
+                pa[b] += (float)n4[b];
+        }
+    }
+}
+
+// The tile grid of an image: at most `ctas` tiles of at least h rows, the
+// fewest rounds of kTlThreads sites per tile, then the smallest border.
+bool tile_geometry(int H, int W, int ctas, int h, TileGeom &best)
+{
+    const int Wq = (W + 3) / 4;
+    long best_cost = -1;
+    for (int nx = 1; nx <= ctas && nx <= Wq; ++nx) {
+        const int twq = (Wq + nx - 1) / nx;
+        const int tx = (Wq + twq - 1) / twq;
+        int th = (H + ctas / tx - 1) / (ctas / tx);
+        th = th < h ? h : th;
+        const int ty = (H + th - 1) / th;
+        if ((long)th * twq * 4 > kTlMaxSites || tx * ty > ctas)
+            continue;
+        const long rounds = ((long)th * twq * 4 + kTlThreads - 1) / kTlThreads;
+        // (rounds dominate; a border word costs far less than a round of draws)
+        const long cost = rounds * 1000 + 2 * (th + twq);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best.th = th;
+            best.twq = twq;
+            best.tiles_x = tx;
+            best.tiles_y = ty;
+            best.inv_tw = 0xFFFFFFFFu / (unsigned int)(4 * twq) + 1u;
+        }
+    }
+    return best_cost >= 0;
+}
+
+// The tiles of one image alone on the device: one CTA per SM while a round of
+// its threads covers the tile, two beyond.
+template <class P, bool GIBBS>
+bool plan_t(int H, int W, int ctas, bool two, TileGeom &tg, size_t &smem)
+{
+    if (ctas <= 0 || !tile_geometry(H, W, ctas, tile_halo(P::NB, GIBBS), tg))
+        return false;
+    smem = tile_smem<P, GIBBS>(tg.th, tg.twq);
+    return smem <= (size_t)(two ? kTlMaxSmem2 : kTlMaxSmem);
+}
+
+template <class P, bool GIBBS, int JOBS>
+cudaError_t launch_t(const TileLaunchT<JOBS> &L, int ctas, size_t smem, cudaStream_t st)
+{
+    static bool attr_set[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess)
+        return e;
+    if (dev >= 64)
+        return cudaErrorInvalidDevice;
+    auto kern = tile_kernel<P, GIBBS, JOBS>;
+    if (!attr_set[dev]) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTlMaxSmem);
+        if (e != cudaSuccess)
+            return e;
+        attr_set[dev] = true;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(kTlThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeCooperative;   // the CTAs wait on one another
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, L);
+}
+
+// f(policy, GIBBS) for the kind's instance.
+template <class F>
+auto with_policy(const TileKind &k, F f)
+{
+    const auto g = [&](auto pol) {
+        return k.gibbs ? f(pol, std::true_type{}) : f(pol, std::false_type{});
+    };
+    if (k.draw == TileKind::kBinary)
+        return k.nbhd == 8 ? g(static_cast<BinPol<8> *>(nullptr))
+                           : g(static_cast<BinPol<4> *>(nullptr));
+    if (k.draw == TileKind::kSegment)
+        return g(static_cast<SegPol *>(nullptr));
+    if (k.nbhd == 8)
+        return k.lmax == 8 ? (k.mask ? g(static_cast<SmallPol<8, 8, true> *>(nullptr))
+                                     : g(static_cast<SmallPol<8, 8, false> *>(nullptr)))
+                           : (k.mask ? g(static_cast<SmallPol<16, 8, true> *>(nullptr))
+                                     : g(static_cast<SmallPol<16, 8, false> *>(nullptr)));
+    return k.lmax == 8 ? (k.mask ? g(static_cast<SmallPol<8, 4, true> *>(nullptr))
+                                 : g(static_cast<SmallPol<8, 4, false> *>(nullptr)))
+                       : (k.mask ? g(static_cast<SmallPol<16, 4, true> *>(nullptr))
+                                 : g(static_cast<SmallPol<16, 4, false> *>(nullptr)));
+}
+
+}  // namespace
+
+bool tile_kind(const DevModel &m, bool gibbs, TileKind &k)
+{
+    k = TileKind{};
+    k.nbhd = m.nbhd;
+    k.gibbs = gibbs;
+    if (m.norm != 0 || (m.nbhd != 4 && m.nbhd != 8))
+        return false;
+    if (m.L == 2) {
+        k.draw = TileKind::kBinary;
+        return true;
+    }
+    if (m.L >= kSmallMinLabels && m.L <= kSmallMaxLabels && m.gam <= 0.0f && m.alpha <= 0.0f) {
+        k.draw = TileKind::kSmall;
+        k.lmax = m.L <= 8 ? 8 : 16;
+        k.mask = m.L != k.lmax;
+        return true;
+    }
+    k.draw = TileKind::kSegment;
+    return seg_eligible(m);
+}
+
+bool tile_plan(const TileKind &k, int H, int W, int sms, TileGeom &tg, size_t &smem)
+{
+    const bool two = (long long)H * W > (long long)sms * kTlThreads;
+    return tile_plan_ctas(k, H, W, two ? 2 * sms : sms, two, tg, smem);
+}
+
+bool tile_plan_ctas(const TileKind &k, int H, int W, int ctas, bool two, TileGeom &tg,
+                    size_t &smem)
+{
+    return with_policy(k, [&](auto pol, auto gibbs) {
+        using P = std::remove_pointer_t<decltype(pol)>;
+        return plan_t<P, decltype(gibbs)::value>(H, W, ctas, two, tg, smem);
+    });
+}
+
+size_t tile_xch_bytes(int H, int W)
+{
+    return (size_t)2 * H * ((W + 3) / 4) * sizeof(unsigned long long);
+}
+
+int tile_rounds(const TileGeom &tg)
+{
+    return (tg.th * tg.twq * 4 + kTlThreads - 1) / kTlThreads;
+}
+
+namespace {
+
+template <int JOBS>
+cudaError_t launch_checked(const TileKind &k, const TileLaunchT<JOBS> &L, int ctas, size_t smem,
+                           cudaStream_t st)
+{
+    if (L.njobs < 1 || L.njobs > JOBS || ctas < 1)
+        return cudaErrorInvalidValue;
+    if (L.nsweeps <= 0)
+        return cudaSuccess;
+    for (int i = 0; i < L.njobs; ++i) {
+        const TileJob &J = L.job[i];
+        TileKind kk;
+        if (!tile_kind(J.a.m, k.gibbs, kk) || !(kk == k) || J.xch == nullptr)
+            return cudaErrorInvalidValue;
+        if ((k.draw == TileKind::kSmall && !J.a.m.ptab) ||
+            (k.draw == TileKind::kBinary && !J.a.m.btab) ||
+            (k.draw == TileKind::kSegment && !J.a.m.stab))
+            return cudaErrorInvalidValue;
+        // word loads and stores of the planes
+        if ((J.a.pitch & 3) != 0 ||
+            ((reinterpret_cast<uintptr_t>(J.x0) | reinterpret_cast<uintptr_t>(J.x1) |
+              reinterpret_cast<uintptr_t>(J.a.g)) & 3u) != 0)
+            return cudaErrorMisalignedAddress;
+    }
+    return with_policy(k, [&](auto pol, auto gibbs) {
+        using P = std::remove_pointer_t<decltype(pol)>;
+        if constexpr (JOBS > 1 && decltype(gibbs)::value)
+            return cudaErrorInvalidValue;   // batches and the server run the PCA sampler
+        else
+            return launch_t<P, decltype(gibbs)::value, JOBS>(L, ctas, smem, st);
+    });
+}
+
+}  // namespace
+
+cudaError_t launch_tile(const TileKind &k, const TileLaunch &L, int ctas, size_t smem,
+                        cudaStream_t st)
+{
+    return launch_checked(k, L, ctas, smem, st);
+}
+
+cudaError_t launch_tile(const TileKind &k, const TilePack &L, int ctas, size_t smem,
+                        cudaStream_t st)
+{
+    return launch_checked(k, L, ctas, smem, st);
+}
+
+}  // namespace pcad

@@ -711,8 +711,8 @@ cudaError_t launch_gibbs_winw(const SweepArgs &a, const float *ftab, uint8_t *x,
         return cudaErrorInvalidValue;
     if (a.H <= 0 || a.W <= 0 || nsweeps == 0)
         return cudaSuccess;
-    if (seg_eligible(a.m))
-        return launch_gibbs_segw(a, ftab + kTabF, x, nsweeps, done, grab, err, st);
+    if (seg_eligible(a.m) && a.m.stab)
+        return launch_gibbs_segw(a, x, nsweeps, done, grab, err, st);
     const bool lmask = (a.m.L % kChunk) != 0;
     if (a.m.nbhd == 8)
         return lmask ? launch_gibbs_winw_t<8, true>(a, ftab, x, nsweeps, done, grab, err, st)
@@ -729,8 +729,8 @@ cudaError_t launch_pca_winw(const SweepArgs &a, const float *ftab, uint8_t *x0, 
         return cudaErrorInvalidValue;
     if (a.H <= 0 || a.W <= 0 || nsweeps == 0)
         return cudaSuccess;
-    if (seg_eligible(a.m))
-        return launch_pca_segw(a, ftab + kTabF, x0, x1, nsweeps, done, grab, err, par_from_t,
+    if (seg_eligible(a.m) && a.m.stab)
+        return launch_pca_segw(a, x0, x1, nsweeps, done, grab, err, par_from_t,
                                budget, st);
     const bool lmask = (a.m.L % kChunk) != 0;
     const int par = par_from_t ? 1 : 0;
@@ -751,8 +751,8 @@ cudaError_t launch_gibbs_win(const SweepArgs &a, int q, const float *ftab, cudaS
         return cudaErrorInvalidValue;
     if (a.H <= 0 || a.W <= 0)
         return cudaSuccess;
-    if (seg_eligible(a.m))
-        return launch_gibbs_seg(a, q, ftab + kTabF, st);
+    if (seg_eligible(a.m) && a.m.stab)
+        return launch_gibbs_seg(a, q, st);
     const bool lmask = (a.m.L % kChunk) != 0;
     if (a.m.nbhd == 8)
         return lmask ? launch_gibbs_win_t<8, true>(a, q, ftab, st)
@@ -774,8 +774,8 @@ cudaError_t launch_pca_win(const SweepArgs &a, const float *ftab, cudaStream_t s
         return cudaErrorInvalidValue;
     if (a.H <= 0 || a.W <= 0)
         return cudaSuccess;
-    if (seg_eligible(a.m))
-        return launch_pca_seg(a, ftab + kTabF, x0, x1, budget, st);
+    if (seg_eligible(a.m) && a.m.stab)
+        return launch_pca_seg(a, x0, x1, budget, st);
     const bool lmask = (a.m.L % kChunk) != 0;
     if (a.m.nbhd == 8)
         return lmask ? launch_win_t<8, true>(a, ftab, x0, x1, budget, st)
