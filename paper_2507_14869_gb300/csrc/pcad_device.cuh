@@ -577,8 +577,8 @@ __device__ __forceinline__ double weight64(const DevModel &m, int g, int xi, con
 }
 
 // Warp-cooperative FP64 evaluation of the draws of the lanes with `need`
-// set: for each such lane in turn, the 32 lanes compute 8 labels' FP64
-// weights each, an FP64 warp scan gives the CDF, and the lane holding u*Z
+// set: for each such lane in turn, the 32 lanes compute ceil(L / 32) labels'
+// FP64 weights each, an FP64 warp scan gives the CDF, and the lane holding u*Z
 // finds the label.  All 32 lanes of the warp must call this together.
 // Draws of lanes with `count` set are added to *counter.
 template <int NB, int NORM = 0>
@@ -594,6 +594,7 @@ __device__ __forceinline__ int warp_redraw_fp64(const DevModel &m, bool need, co
     const unsigned counted = todo & __ballot_sync(kFull, count);
     if (lane == 0 && counted)
         atomicAdd(counter, (unsigned long long)__popc(counted));
+    const int per = (m.L + 31) >> 5;   // labels per lane, in label order
     while (todo) {
         const int leader = __ffs((int)todo) - 1;
         todo &= todo - 1u;
@@ -608,9 +609,11 @@ __device__ __forceinline__ int warp_redraw_fp64(const DevModel &m, bool need, co
         double part = 0.0;
 #pragma unroll
         for (int k = 0; k < kChunk; ++k) {
-            const int sl = lane * kChunk + k;
+            if (k >= per)   // uniform
+                break;
+            const int sl = lane * per + k;
             w[k] = sl < m.L ? weight64<NB, NORM>(m, lg, lxi, lx, sl) : 0.0;
-            part = __dadd_rn(part, w[k]);
+            part = k == 0 ? w[0] : __dadd_rn(part, w[k]);
         }
         double incl = part;
 #pragma unroll
@@ -619,27 +622,39 @@ __device__ __forceinline__ int warp_redraw_fp64(const DevModel &m, bool need, co
             if (lane >= o)
                 incl = __dadd_rn(incl, v);
         }
+        // t = u Z (2^-24 by the exponent: exact)
         const double Z = __shfl_sync(kFull, incl, 31);
-        const double t = __dmul_rn((double)lub * (1.0 / 16777216.0), Z);
+        const double t = __dmul_rn((double)lub, __hiloint2double(__double2hiint(Z) - (24 << 20),
+                                                                 __double2loint(Z)));
         double excl = __shfl_up_sync(kFull, incl, 1);
         if (lane == 0)
             excl = 0.0;
-        const unsigned hit = __ballot_sync(kFull, t < incl);
+        // comparisons of non-negative doubles as integers: an FP64 instruction
+        // of one warp holds its scheduler's pipe for 64 cycles on GB300
+        const long long ti = __double_as_longlong(t);
+        const unsigned hit = __ballot_sync(kFull, ti < __double_as_longlong(incl));
         const int hl = hit ? __ffs((int)hit) - 1 : 31;
-        int res = 0;
-        if (lane == hl) {
-            double C = excl;
-            res = min(lane * kChunk + kChunk - 1, m.L - 1);
+        // the lane's labels, one per lane: their prefix sums in log2 steps
+        double C = 0.0;
 #pragma unroll
-            for (int k = 0; k < kChunk; ++k) {
-                C = __dadd_rn(C, w[k]);
-                if (t < C && lane * kChunk + k < m.L) {
-                    res = lane * kChunk + k;
-                    break;
-                }
-            }
+        for (int k = 0; k < kChunk; ++k) {
+            if (k >= per)
+                break;
+            const double v = __shfl_sync(kFull, w[k], hl);
+            C = lane == k ? v : C;
         }
-        res = __shfl_sync(kFull, res, hl);
+#pragma unroll
+        for (int o = 1; o < kChunk; o <<= 1) {
+            if (o >= per)
+                break;
+            const double v = __shfl_up_sync(kFull, C, o);
+            if (lane >= o)
+                C = __dadd_rn(C, v);
+        }
+        C = __dadd_rn(__shfl_sync(kFull, excl, hl), C);
+        const unsigned in = __ballot_sync(kFull, lane < per && hl * per + lane < m.L &&
+                                                     ti < __double_as_longlong(C));
+        const int res = in ? hl * per + __ffs((int)in) - 1 : min(hl * per + per - 1, m.L - 1);
         if (lane == leader)
             s = res;
     }
