@@ -1,10 +1,10 @@
-// Whole chains of small two-label images in one CTA
-// (lazy PCA, Section 5.2; checkerboard Gibbs, Section 5.1).
+// Whole chains of small two-label images in one launch, in shared memory
+// (lazy PCA, Section 5.2; checkerboard Gibbs, Section 5.1), and sweeps of
+// larger two-label images.
 //
 // A 64 x 64 binary chain does 4096 site-updates per sweep: one launch per
 // sweep costs more than the sweep.  Here one CTA of 1024 threads holds the
-// whole state in shared memory and runs every sweep of a run in one launch,
-// with one block barrier per sweep (PCA) or colour phase (Gibbs).
+// whole state in shared memory and runs every sweep of a run in one launch, with one block barrier per sweep (PCA) or colour phase (Gibbs).
 //
 // The draw.  With two labels the conditional law of site i depends on the
 // site only through its configuration (x_i, g_i, n1, nm): n1 neighbours at
@@ -114,11 +114,13 @@ inline int res_plane_bytes(int H, int W)
     return (H + 2) * (((W + 3) & ~3) + 8);
 }
 
+constexpr int kThrBytes = 6656;   // a ThrTab of either neighbourhood
+
 // Shared memory of a launch: table, one (Gibbs) or two (PCA) planes, base bytes.
 inline int res_smem_bytes(int nb, bool gibbs, int H, int W)
 {
-    const int ne = 4 * (nb + 1) * (nb + 1);
-    return ne * 16 + (gibbs ? 1 : 2) * res_plane_bytes(H, W) + H * ((W + 3) & ~3);
+    (void)nb;
+    return kThrBytes + (gibbs ? 1 : 2) * res_plane_bytes(H, W) + H * ((W + 3) & ~3);
 }
 
 // Label-1 neighbour counts of the 4 sites of the word at index o (one per
@@ -135,35 +137,78 @@ __device__ __forceinline__ uint32_t quad_counts(const uint32_t *X, int o, int pw
     return S;
 }
 
-// New labels of the bytes of `act` (a byte mask) of one quad: S holds base +
-// count per byte, M the current labels, u the uniforms.  Returns the labels
-// as bytes (other bytes 0); adds the draws the FP64 re-draw decides to nre.
-__device__ __forceinline__ uint32_t quad_draw(const uint4 *tab, uint32_t S, uint32_t M,
+// Thresholds of every configuration in shared memory: thr[] (one 32-bit read
+// and a compare per draw), the full entries for the rare draws near a
+// threshold, and the largest uncertain band.
+template <int NB>
+struct ThrTab {
+    int thr[NB == 4 ? btab_entries<4>() : 2 * 168];   // NB 4: [2 b + x]; 8: [168 x + b]
+    uint4 full[btab_entries<NB>()];
+    uint32_t band;
+};
+
+static_assert(sizeof(ThrTab<4>) <= kThrBytes && sizeof(ThrTab<8>) <= kThrBytes, "table space");
+
+template <int NB>
+__device__ __forceinline__ int thr_index(int e)
+{
+    return NB == 4 ? e : (e >> 1) + 168 * (e & 1);
+}
+
+// (ends with a block barrier)
+template <int NB>
+__device__ __forceinline__ void load_thresholds(ThrTab<NB> &tab, const uint4 *src, int tid, int n)
+{
+    if (tid == 0)
+        tab.band = 0u;
+    __syncthreads();
+    for (int i = tid; i < btab_entries<NB>(); i += n) {
+        const uint4 e = src[i];
+        tab.full[i] = e;
+        tab.thr[thr_index<NB>(i)] = (int)e.x;
+        atomicMax(&tab.band, e.z);
+    }
+    __syncthreads();
+}
+
+// New labels of one quad from its Philox words u: S holds base + count per
+// byte, M the current labels (0 or 1 per byte).  Returns the labels as bytes;
+// adds the draws of the bytes of `act` that the FP64 re-draw decides to nre:
+// those with u in [A, B), a band around the threshold, looked at only when
+// some draw of the quad lies within the largest band of its threshold.
+template <int NB>
+__device__ __forceinline__ uint32_t quad_draw(const ThrTab<NB> &tab, uint32_t S, uint32_t M,
                                               const uint32_t (&u)[4], uint32_t act, uint32_t &nre)
 {
+    const uint32_t K = NB == 4 ? 2u * S + M : S;   // NB 4: at most 99 per byte, no carry
     uint32_t out = 0u;
+    int near = 0x7FFFFFFF;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        if ((act >> (8 * j)) & 1u) {
-            const uint32_t key = ((S >> (8 * j)) & 0xFFu) * 2u + ((M >> (8 * j)) & 1u);
-            const uint4 e = tab[key];
-            out |= (u[j] >= e.x ? 1u : 0u) << (8 * j);
-            nre += (u[j] - e.y) < e.z ? 1u : 0u;
-        }
+        int i = (int)((K >> (8 * j)) & 0xFFu);
+        if (NB == 8)
+            i += 168 * (int)((M >> (8 * j)) & 1u);
+        const int d = (int)(u[j] >> 8) - tab.thr[i];
+        out |= d >= 0 ? 1u << (8 * j) : 0u;
+        near = min(near, abs(d));
+    }
+    if ((uint32_t)near <= tab.band) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if ((act >> (8 * j)) & 1u) {
+                const uint4 e = tab.full[((S >> (8 * j)) & 0xFFu) * 2u + ((M >> (8 * j)) & 1u)];
+                nre += ((u[j] >> 8) - e.y) < e.z ? 1u : 0u;
+            }
     }
     return out;
 }
 
-__device__ __forceinline__ void quad_uniforms(const SweepArgs &a, uint32_t tag, uint32_t t,
-                                              int r, int c4, uint32_t (&u)[4])
+__device__ __forceinline__ void quad_words(const SweepArgs &a, uint32_t tag, uint32_t t, int r,
+                                           int c4, uint32_t (&u)[4])
 {
-    uint32_t o0, o1, o2, o3;
     philox4x32_10((uint32_t)c4, (uint32_t)(r + a.row_off), t, (tag << 24) | (a.chain & 0xFFFFFFu),
-                  (uint32_t)(a.seed & 0xFFFFFFFFull), (uint32_t)(a.seed >> 32), o0, o1, o2, o3);
-    u[0] = o0 >> 8;
-    u[1] = o1 >> 8;
-    u[2] = o2 >> 8;
-    u[3] = o3 >> 8;
+                  (uint32_t)(a.seed & 0xFFFFFFFFull), (uint32_t)(a.seed >> 32), u[0], u[1], u[2],
+                  u[3]);
 }
 
 // Gibbs colour phase ph of a quad in row r: the bytes whose site has colour
@@ -188,14 +233,13 @@ __device__ __forceinline__ void resident_run(const SweepArgs &a, const uint4 *bt
                                              const uint8_t *xg_in, uint8_t *xg_out, int nsweeps)
 {
     extern __shared__ __align__(16) uint8_t sm[];
-    constexpr int NE = btab_entries<NB>();
     const int tid = (int)threadIdx.x;
     const int H = a.H, W = a.W;
     const int Wq = (W + 3) & ~3, P = Wq + 8, pw = P >> 2;
     const int plane = (H + 2) * P;
     const int nplanes = GIBBS ? 1 : 2;
-    uint4 *tab = reinterpret_cast<uint4 *>(sm);
-    uint8_t *const pl0 = sm + NE * 16;
+    ThrTab<NB> &tab = *reinterpret_cast<ThrTab<NB> *>(sm);
+    uint8_t *const pl0 = sm + kThrBytes;
     uint8_t *const pl1 = pl0 + (GIBBS ? 0 : plane);
     uint8_t *const bs = pl0 + nplanes * plane;
     {
@@ -203,10 +247,8 @@ __device__ __forceinline__ void resident_run(const SweepArgs &a, const uint4 *bt
         const int nz = (nplanes * plane + H * Wq) >> 2;
         for (int i = tid; i < nz; i += kResThreads)
             z[i] = 0u;   // borders, row padding and the base bytes of padding sites stay 0
-        for (int i = tid; i < NE; i += kResThreads)
-            tab[i] = btab[i];
     }
-    __syncthreads();
+    load_thresholds<NB>(tab, btab, tid, kResThreads);
     for (int i = tid; i < H * W; i += kResThreads) {
         const int r = i / W, c = i - (i / W) * W;
         const int gv = a.g[(size_t)r * a.pitch + c];
@@ -268,10 +310,10 @@ __device__ __forceinline__ void resident_run(const SweepArgs &a, const uint4 *bt
                 if (qo[i] < 0)
                     continue;
                 uint32_t u[4];
-                quad_uniforms(a, tag, t, qr[i], qc[i], u);
+                quad_words(a, tag, t, qr[i], qc[i], u);
                 uint32_t M;
                 const uint32_t S = quad_counts<NB>(X, qo[i], pw, M) + qb[i];
-                const uint32_t nw = quad_draw(tab, S, M, u, qm[i], nre);
+                const uint32_t nw = quad_draw<NB>(tab, S, M, u, qm[i], nre) & qm[i];
                 Y[qo[i]] = nw;
                 if (acc_now) {
                     clo[i] += nw & 0x00FF00FFu;
@@ -286,7 +328,7 @@ __device__ __forceinline__ void resident_run(const SweepArgs &a, const uint4 *bt
 #pragma unroll
             for (int i = 0; i < QPT; ++i)
                 if (qo[i] >= 0)
-                    quad_uniforms(a, tag, t, qr[i], qc[i], u[i]);
+                    quad_words(a, tag, t, qr[i], qc[i], u[i]);
 #pragma unroll 1
             for (int ph = 0; ph < kColours; ++ph) {
 #pragma unroll
@@ -296,8 +338,8 @@ __device__ __forceinline__ void resident_run(const SweepArgs &a, const uint4 *bt
                         continue;
                     uint32_t M;
                     const uint32_t S = quad_counts<NB>(X, qo[i], pw, M) + qb[i];
-                    const uint32_t nw = quad_draw(tab, S, M, u[i], act, nre);
-                    X[qo[i]] = (M & ~act) | nw;
+                    const uint32_t nw = quad_draw<NB>(tab, S, M, u[i], act, nre);
+                    X[qo[i]] = (M & ~act) | (nw & act);
                 }
                 __syncthreads();
             }
@@ -395,158 +437,166 @@ cudaError_t launch_res_q(const SweepArgs &a, const uint8_t *x_in, uint8_t *x_out
 }
 
 // ------------------------------------------------------- large images
-// Two labels on images too large for one CTA: one launch per sweep, the
-// same threshold table (a table read and a compare per site), persistent
-// blocks of 256 threads over tiles of 16 rows x 128 columns.  A block stages
-// its tile's label words with a one-word halo in shared memory (words
-// outside the image and bytes beyond W read as zero: a missing neighbour
-// counts as no label-1 neighbour, and its absence enters through nm), and
-// each thread takes two quads: neighbour counts by byte-wise adds, the base
-// (g (NB + 1) + nm) (NB + 1) from the observation word (g < 2, checked at
-// chain creation), one Philox call, four table reads, one 32-bit label
-// store and one float4 accumulator update.  The next tile's label words are
-// loaded into registers during the draws, and a tile's observation words
-// and accumulator sums before them.
+// Two labels on images too large for one CTA: one launch per sweep with the
+// same thresholds.  A warp owns a strip of 32 quads (128 columns) and walks
+// down its rows, a lane per quad: the label words above, at and below the row
+// stay in registers, the words left and right come from the neighbouring
+// lanes (lanes 0 and 31 load the strip's outer words), so labels need one
+// load per quad and no shared memory.  Neighbour counts by byte-wise adds, one
+// Philox call, four threshold reads and compares, one 32-bit label store.
+// Sums: a float4 per lane where rows of the accumulator are aligned, else the
+// warp's 128 sums as four coalesced words per lane (the labels by shuffles).
+// The next row's words are loaded before a row's draws.
+//
+// Bound by instruction issue (about 58 per site) at 0.55 of the memory rate:
+// 8192^2 151 us per sweep (4.44e11 site-updates/s) against 203 us for the
+// form that staged tiles of labels in shared memory and read a 16-byte entry
+// per draw; 2043 x 3001 17.9 us against 22.7.  256 threads at 75 registers (3
+// blocks per SM): held to 5 blocks 157 us and 21.6.
 constexpr int kBinThreads = 256;
-constexpr int kBinRows = 16;
-constexpr int kBinQW = 32;                 // quads (4-site words) per tile row
-constexpr int kBinPW = kBinQW + 2;         // staged words per row
-constexpr int kBinWords = (kBinRows + 2) * kBinPW;
+constexpr int kBinMaxRows = 16;            // rows per strip, at most
+constexpr int kBinQW = 32;                 // quads per strip
 
 // Planes: a.xin -> a.xout, or (x0 != nullptr) x0 / x1 holding the states of
 // even / odd sweep indices; budget (optional): a sweep with index >= *budget
 // is skipped (a chain of a batch or of the server).
 template <int NB>
 __global__ void __launch_bounds__(kBinThreads)
-    pca_binary_kernel(const SweepArgs a, int tiles_x, int ntiles, int acc_vec, uint8_t *x0,
+    pca_binary_kernel(const SweepArgs a, int strips_x, int nstrips, int rows, int acc_vec, uint8_t *x0,
                       uint8_t *x1, const uint32_t *budget)
 {
-    constexpr int NE = btab_entries<NB>();
-    __shared__ uint4 tab[NE];
-    __shared__ uint32_t X[kBinWords];
-    const int tid = (int)threadIdx.x;
+    __shared__ ThrTab<NB> tab;
     const uint32_t t = sweep_index(a);
     if (budget && t >= *budget)
         return;   // the whole launch, before any barrier
     const uint8_t *xin = x0 ? ((t & 1u) ? x1 : x0) : a.xin;
     uint8_t *xout = x0 ? ((t & 1u) ? x0 : x1) : a.xout;
-    for (int i = tid; i < NE; i += kBinThreads)
-        tab[i] = a.m.btab[i];
+    load_thresholds<NB>(tab, a.m.btab, (int)threadIdx.x, kBinThreads);
     const bool acc_on = accumulate_after(a, t);
     const int H = a.H, W = a.W, pitch = a.pitch;
     const int Wq = (W + 3) >> 2;
+    const int lane = (int)threadIdx.x & 31;
     uint32_t nre = 0u;
-    constexpr int kSlots = (kBinWords + kBinThreads - 1) / kBinThreads;
-    // the label words of a tile into registers (issued early, stored later)
-    auto stage_load = [&](int tile, uint32_t (&pw)[kSlots]) {
-        const int ty = tile / tiles_x, tx = tile - ty * tiles_x;
-        const int r0 = ty * kBinRows, q0 = tx * kBinQW;
-#pragma unroll
-        for (int sl = 0; sl < kSlots; ++sl) {
-            const int i = tid + sl * kBinThreads;
-            pw[sl] = 0u;
-            if (i < kBinWords) {
-                const int lr = i / kBinPW, lw = i - lr * kBinPW;
-                const int gr = r0 - 1 + lr, gq = q0 - 1 + lw;
-                if (gr >= 0 && gr < H && gq >= 0 && gq < Wq) {
-                    uint32_t w = *reinterpret_cast<const uint32_t *>(xin + (size_t)gr * pitch + 4 * gq);
-                    const int nv = W - 4 * gq;
-                    if (nv < 4)
-                        w &= (1u << (8 * nv)) - 1u;
-                    pw[sl] = w;
+    for (int strip = (int)(blockIdx.x * (kBinThreads / 32) + (threadIdx.x >> 5)); strip < nstrips;
+         strip += (int)gridDim.x * (kBinThreads / 32)) {
+        const int sy = strip / strips_x, sx = strip - sy * strips_x;
+        const int r0 = sy * rows, q = sx * kBinQW + lane;
+        const int r1 = min(r0 + rows, H);
+        const int nv = min(4, W - 4 * q);                 // sites of the quad inside
+        const uint32_t act = nv >= 4 ? 0xFFFFFFFFu : (nv > 0 ? (1u << (8 * nv)) - 1u : 0u);
+        // lanes 0 and 31 also read the word outside the strip.  Loads are
+        // unconditional, at clamped rows and quads, and masked.
+        const int qe = lane == 0 ? q - 1 : (lane == 31 ? q + 1 : q);
+        const uint32_t acte = qe >= 0 && qe < Wq
+                                  ? (W - 4 * qe >= 4 ? 0xFFFFFFFFu : (1u << (8 * (W - 4 * qe))) - 1u)
+                                  : 0u;
+        const int qc = min(q, Wq - 1), qec = min(max(qe, 0), Wq - 1);
+        const auto row_at = [&](int r) -> const uint8_t * {
+            return xin + (size_t)min(max(r, 0), H - 1) * pitch;
+        };
+        const auto ld = [](const uint8_t *p, int qq) -> uint32_t {
+            return *reinterpret_cast<const uint32_t *>(p + 4 * qq);
+        };
+        // the sums left + right of the 4 sites of word w (outer word e)
+        const auto sides = [&](uint32_t w, uint32_t e) -> uint32_t {
+            uint32_t l = __shfl_up_sync(0xFFFFFFFFu, w, 1), rr = __shfl_down_sync(0xFFFFFFFFu, w, 1);
+            l = lane == 0 ? e : l;
+            rr = lane == 31 ? e : rr;
+            return __funnelshift_l(l, w, 8) + __funnelshift_r(w, rr, 8);
+        };
+        const bool side = nv > 0 && (q == 0 || 4 * q + 4 >= W);   // a column has a missing side
+        const uint8_t *pu = row_at(r0 - 1), *p0 = row_at(r0), *p1 = row_at(r0 + 1);
+        uint32_t up = r0 > 0 ? ld(pu, qc) & act : 0u, M = ld(p0, qc) & act;
+        uint32_t dn = r0 + 1 < H ? ld(p1, qc) & act : 0u, dne = r0 + 1 < H ? ld(p1, qec) & acte : 0u;
+        uint32_t upS = 0u, Ms = sides(M, ld(p0, qec) & acte);
+        if (NB == 8)
+            upS = sides(up, r0 > 0 ? ld(pu, qec) & acte : 0u);
+        const uint8_t *pg = a.g + (size_t)r0 * pitch;
+        const uint8_t *p2 = row_at(r0 + 2);
+        uint8_t *po = xout + (size_t)r0 * pitch + 4 * q;
+        float *pa = a.acc + (size_t)r0 * W + 4 * kBinQW * sx;
+        const int left = W - 4 * kBinQW * sx;             // columns of the strip inside
+        uint32_t gw = ld(pg, qc);
+        for (int r = r0; r < r1; ++r) {
+            // in flight during the draws: the row after next, the next
+            // observations, this row's sums
+            const uint32_t m2 = r + 2 < H ? 0xFFFFFFFFu : 0u;
+            const uint32_t dn2 = ld(p2, qc) & act & m2, dne2 = ld(p2, qec) & acte & m2;
+            p2 += r + 3 < H ? pitch : 0;
+            pg += r + 1 < H ? pitch : 0;
+            const uint32_t gw2 = ld(pg, qc);
+            float4 A4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (acc_on) {
+                if (acc_vec) {
+                    if (nv >= 4)
+                        A4 = *reinterpret_cast<const float4 *>(pa + 4 * lane);
+                } else {
+                    A4.x = lane < left ? pa[lane] : 0.0f;
+                    A4.y = 32 + lane < left ? pa[32 + lane] : 0.0f;
+                    A4.z = 64 + lane < left ? pa[64 + lane] : 0.0f;
+                    A4.w = 96 + lane < left ? pa[96 + lane] : 0.0f;
                 }
             }
-        }
-    };
-    uint32_t pw[kSlots];
-    int tile = (int)blockIdx.x;
-    if (tile < ntiles)
-        stage_load(tile, pw);
-    for (; tile < ntiles; tile += (int)gridDim.x) {
-        const int ty = tile / tiles_x, tx = tile - ty * tiles_x;
-        const int r0 = ty * kBinRows, q0 = tx * kBinQW;
-        __syncthreads();   // the table is in place; the last tile's words are read
-#pragma unroll
-        for (int sl = 0; sl < kSlots; ++sl) {
-            const int i = tid + sl * kBinThreads;
-            if (i < kBinWords)
-                X[i] = pw[sl];
-        }
-        __syncthreads();
-        if (tile + (int)gridDim.x < ntiles)
-            stage_load(tile + (int)gridDim.x, pw);   // in flight during the draws
-        constexpr int kQ = kBinRows * kBinQW / kBinThreads;
-        uint32_t Gw[kQ];
-        float4 A4[kQ];
-#pragma unroll
-        for (int qi = 0; qi < kQ; ++qi) {   // the quads' observations and sums, issued first
-            const int k = tid + qi * kBinThreads;
-            const int lr = k / kBinQW, lq = k - lr * kBinQW;
-            const int gr = r0 + lr, gq = q0 + lq;
-            Gw[qi] = 0u;
-            A4[qi] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            if (gr < H && gq < Wq) {
-                Gw[qi] = *reinterpret_cast<const uint32_t *>(a.g + (size_t)gr * pitch + 4 * gq);
-                if (acc_on && acc_vec && 4 * gq + 4 <= W)
-                    A4[qi] = *reinterpret_cast<const float4 *>(a.acc + (size_t)gr * W + 4 * gq);
-            }
-        }
-#pragma unroll
-        for (int qi = 0; qi < kQ; ++qi) {
-            const int k = tid + qi * kBinThreads;
-            const int lr = k / kBinQW, lq = k - lr * kBinQW;
-            const int gr = r0 + lr, gq = q0 + lq;
-            if (gr >= H || gq >= Wq)
-                continue;
-            const int nv = min(4, W - 4 * gq);
-            const uint32_t act = nv >= 4 ? 0xFFFFFFFFu : (1u << (8 * nv)) - 1u;
-            uint32_t M;
-            uint32_t S = quad_counts<NB>(X, (lr + 1) * kBinPW + 1 + lq, kBinPW, M);
-            S += (Gw[qi] & act & 0x01010101u) * (uint32_t)((NB + 1) * (NB + 1));
-            if (gr == 0 || gr == H - 1 || gq == 0 || 4 * gq + 4 >= W) {
+            const uint32_t dnS = sides(dn, dne);
+            uint32_t S = up + dn + Ms;
+            if (NB == 8)
+                S += upS + dnS;
+            S += (gw & act & 0x01010101u) * (uint32_t)((NB + 1) * (NB + 1));
+            if (r == 0 || r == H - 1 || side) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int c = 4 * gq + j;
-                    int nm = (gr == 0) + (gr == H - 1) + (c == 0) + (c == W - 1);
+                    const int c = 4 * q + j;
+                    int nm = (r == 0) + (r == H - 1) + (c == 0) + (c == W - 1);
                     if (NB == 8)
-                        nm += (gr == 0 || c == 0) + (gr == 0 || c == W - 1) +
-                              (gr == H - 1 || c == 0) + (gr == H - 1 || c == W - 1);
+                        nm += (r == 0 || c == 0) + (r == 0 || c == W - 1) +
+                              (r == H - 1 || c == 0) + (r == H - 1 || c == W - 1);
                     S += (uint32_t)(nm * (NB + 1)) << (8 * j);
                 }
             }
             uint32_t u[4];
-            quad_uniforms(a, kTagPCA, t, gr, gq, u);
-            const uint32_t nw = quad_draw(tab, S, M, u, act, nre);
-            uint8_t *out = xout + (size_t)gr * pitch + 4 * gq;
-            float *acc = a.acc + (size_t)gr * W + 4 * gq;
+            quad_words(a, kTagPCA, t, r, q, u);
+            const uint32_t nw = quad_draw<NB>(tab, S, M, u, act, nre) & act;
             if (nv >= 4) {
-                *reinterpret_cast<uint32_t *>(out) = nw;
-                if (acc_on) {
-                    const float l0 = (float)(nw & 0xFFu), l1 = (float)((nw >> 8) & 0xFFu),
-                                l2 = (float)((nw >> 16) & 0xFFu), l3 = (float)(nw >> 24);
-                    if (acc_vec) {
-                        const float4 v = A4[qi];
-                        *reinterpret_cast<float4 *>(acc) =
-                            make_float4(v.x + l0, v.y + l1, v.z + l2, v.w + l3);
-                    } else {
-                        acc[0] += l0;
-                        acc[1] += l1;
-                        acc[2] += l2;
-                        acc[3] += l3;
+                *reinterpret_cast<uint32_t *>(po) = nw;
+            } else {
+                for (int j = 0; j < nv; ++j)
+                    po[j] = (uint8_t)(nw >> (8 * j));
+            }
+            po += pitch;
+            if (acc_on) {
+                // a byte to a float: in the mantissa of 2^23, less 2^23
+                const auto fl = [](uint32_t w, uint32_t sel) {
+                    return __fadd_rn(__uint_as_float(__byte_perm(w, 0x4B000000u, sel)), -8388608.0f);
+                };
+                if (acc_vec) {
+                    if (nv >= 4)
+                        *reinterpret_cast<float4 *>(pa + 4 * lane) =
+                            make_float4(A4.x + fl(nw, 0x7440u), A4.y + fl(nw, 0x7441u),
+                                        A4.z + fl(nw, 0x7442u), A4.w + fl(nw, 0x7443u));
+                } else {
+                    const float old[4] = {A4.x, A4.y, A4.z, A4.w};
+                    const uint32_t sel = 0x7440u + (uint32_t)(lane & 3);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int c = 32 * j + lane;
+                        const uint32_t w = __shfl_sync(0xFFFFFFFFu, nw, 8 * j + (lane >> 2));
+                        if (c < left)
+                            pa[c] = old[j] + fl(w, sel);
                     }
                 }
-            } else {
-                for (int j = 0; j < nv; ++j) {
-                    const uint32_t sl = (nw >> (8 * j)) & 0xFFu;
-                    out[j] = (uint8_t)sl;
-                    if (acc_on)
-                        acc[j] += (float)sl;
-                }
             }
+            pa += W;
+            up = M;
+            upS = Ms;
+            M = dn;
+            Ms = dnS;
+            dn = dn2;
+            dne = dne2;
+            gw = gw2;
         }
     }
     const uint32_t warp_re = __reduce_add_sync(0xFFFFFFFFu, nre);
-    if ((tid & 31) == 0 && warp_re != 0u)
+    if (lane == 0 && warp_re != 0u)
         atomicAdd(a.fp64_draws, (unsigned long long)warp_re);
 }
 
@@ -574,17 +624,24 @@ cudaError_t launch_binary_t(const SweepArgs &a, uint8_t *x0, uint8_t *x1, const 
     if (e != cudaSuccess)
         return e;
     const int Wq = (a.W + 3) >> 2;
-    const int tiles_x = (Wq + kBinQW - 1) / kBinQW;
-    const long long ntiles = (long long)tiles_x * ((a.H + kBinRows - 1) / kBinRows);
-    if (ntiles <= 0)
+    const int strips_x = (Wq + kBinQW - 1) / kBinQW;
+    if (a.H <= 0 || strips_x <= 0)
         return cudaSuccess;
-    if (ntiles >= (1ll << 31))
-        return cudaErrorInvalidValue;
+    constexpr int per = kBinThreads / 32;
     const long long cap = (long long)per_sm[dev] * sms;
-    const int grid = (int)(ntiles < cap ? ntiles : cap);
+    // rows per strip: whole waves of the resident warps (8 rows at 2043 x 3001
+    // left a quarter of a second wave)
+    const long long all = (long long)a.H * strips_x, warps = cap * per;
+    const long long waves = (all + warps * kBinMaxRows - 1) / (warps * kBinMaxRows);
+    const int rows = (int)((all + warps * waves - 1) / (warps * waves));
+    const long long nstrips = (long long)strips_x * ((a.H + rows - 1) / rows);
+    if (nstrips >= (1ll << 30))
+        return cudaErrorInvalidValue;
+    const long long need = (nstrips + per - 1) / per;
+    const int grid = (int)(need < cap ? need : cap);
     const int acc_vec = (a.W % 4 == 0 && (reinterpret_cast<uintptr_t>(a.acc) & 15u) == 0) ? 1 : 0;
-    pca_binary_kernel<NB><<<grid, kBinThreads, 0, st>>>(a, tiles_x, (int)ntiles, acc_vec, x0, x1,
-                                                        budget);
+    pca_binary_kernel<NB><<<grid, kBinThreads, 0, st>>>(a, strips_x, (int)nstrips, rows, acc_vec,
+                                                        x0, x1, budget);
     return cudaGetLastError();
 }
 
