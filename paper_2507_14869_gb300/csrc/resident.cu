@@ -3,8 +3,10 @@
 // larger two-label images.
 //
 // A 64 x 64 binary chain does 4096 site-updates per sweep: one launch per
-// sweep costs more than the sweep.  Here one CTA of 1024 threads holds the
-// whole state in shared memory and runs every sweep of a run in one launch, with one block barrier per sweep (PCA) or colour phase (Gibbs).
+// sweep costs more than the sweep.  Here one CTA of 1024 threads (a chain of
+// a batch, the smallest images) or a cluster of 8 (resident_cluster_kernel)
+// holds the whole state in shared memory and runs every sweep of a run in one
+// launch, with one block barrier per sweep (PCA) or colour phase (Gibbs).
 //
 // The draw.  With two labels the conditional law of site i depends on the
 // site only through its configuration (x_i, g_i, n1, nm): n1 neighbours at
@@ -377,6 +379,235 @@ __global__ void __launch_bounds__(kResThreads, 1)
     resident_run<NB, GIBBS, QPT>(a, a.m.btab, xg_in, xg_out, nsweeps);
 }
 
+// ------------------------------------------------------- one chain, 8 CTAs
+// One chain alone leaves 151 SMs idle, and its sweep is bound by the issue
+// slots of the one it has: 0.87 us for 64 x 64 (Gibbs 1.31), against 0.52
+// (0.90) here, bound by the latency of a pass and of the exchange.  A cluster of 8 CTAs takes the
+// chain in bands of rows with a halo of h rows: h sweeps (Gibbs: h colour
+// phases) run on shrinking extensions of the band, then each CTA pushes its
+// border rows into its neighbours' receive buffers through distributed shared
+// memory and the cluster's barrier makes them visible (two buffers in turn: a
+// buffer is written again only after the barrier that follows its reading).
+// Draws are keyed by (sweep, site), so both owners of an extended row draw the
+// same labels.  A thread keeps its quads, their base bytes, their counts and
+// the next sweep's uniforms in registers.
+constexpr int kClCtas = 8;
+constexpr int kClHalo = 4;                // rows: 4 PCA sweeps, 2 (1) Gibbs sweeps
+constexpr int kClThreads = 768;           // at most
+
+inline int cl_smem_bytes(bool gibbs, int band, int W)
+{
+    const int Wq4 = (W + 3) & ~3;
+    return kThrBytes + (gibbs ? 1 : 2) * (band + 2 * kClHalo) * (Wq4 + 8) + 4 * kClHalo * Wq4;
+}
+
+__device__ __forceinline__ uint32_t cluster_rank()
+{
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+__device__ __forceinline__ void cluster_sync()
+{
+    asm volatile("barrier.cluster.arrive.release;\n\t"
+                 "barrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Store v at the shared-memory word `local` of CTA `rank` of the cluster.
+__device__ __forceinline__ void st_cluster(const uint32_t *local, uint32_t rank, uint32_t v)
+{
+    uint32_t addr;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(addr)
+                 : "r"((uint32_t)__cvta_generic_to_shared(local)), "r"(rank));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+template <int NB, bool GIBBS, int QPT>
+__global__ void __cluster_dims__(kClCtas, 1, 1) __launch_bounds__(kClThreads, 1)
+    resident_cluster_kernel(const SweepArgs a, const uint8_t *xg_in, uint8_t *xg_out, int nsweeps,
+                            int band)
+{
+    extern __shared__ __align__(16) uint8_t sm[];
+    constexpr int h = kClHalo;
+    constexpr int kCol = !GIBBS ? 1 : (NB == 4 ? 2 : 4);
+    constexpr int K = h / kCol;                    // sweeps per exchange
+    const int tid = (int)threadIdx.x, nt = (int)blockDim.x;
+    const int rank = (int)cluster_rank();
+    const int H = a.H, W = a.W;
+    const int qrow = (W + 3) >> 2, pw = qrow + 2;  // quads, words per staged row
+    const int rows = band + 2 * h;                 // staged rows
+    const int r0 = rank * band;                    // the band's first image row
+    const int own = max(0, min(band, H - r0));     // its rows inside the image
+    ThrTab<NB> &tab = *reinterpret_cast<ThrTab<NB> *>(sm);
+    uint32_t *const pl0 = reinterpret_cast<uint32_t *>(sm + kThrBytes);
+    uint32_t *const pl1 = GIBBS ? pl0 : pl0 + rows * pw;
+    uint32_t *const recv = pl1 + rows * pw;        // [2 turns][above, below][h][qrow]
+    load_thresholds<NB>(tab, a.m.btab, tid, nt);
+    for (int i = tid; i < (GIBBS ? 1 : 2) * rows * pw; i += nt)
+        pl0[i] = 0u;   // outside the image, and the padding of rows
+    __syncthreads();
+    for (int i = tid; i < rows * qrow; i += nt) {
+        const int sr = i / qrow, q = i - sr * qrow, r = r0 - h + sr;
+        if (r < 0 || r >= H)
+            continue;
+        uint32_t w = *reinterpret_cast<const uint32_t *>(xg_in + (size_t)r * a.pitch + 4 * q);
+        const int nv = W - 4 * q;
+        if (nv < 4)
+            w &= (1u << (8 * nv)) - 1u;
+        pl0[sr * pw + 1 + q] = w;
+    }
+    // this thread's quads: rows -(h - 1) .. band + h - 2 of the band
+    int lr[QPT], qo[QPT], qc[QPT];
+    uint32_t qb[QPT], qm[QPT], clo[QPT], chi[QPT], un[QPT][4];
+    const int n = (band + 2 * h - 2) * qrow;
+#pragma unroll
+    for (int i = 0; i < QPT; ++i) {
+        const int q = tid + i * nt;
+        qb[i] = qm[i] = clo[i] = chi[i] = 0u;
+        lr[i] = q < n ? q / qrow - (h - 1) : 1 << 20;
+        qc[i] = q < n ? q % qrow : 0;
+        qo[i] = (lr[i] + h) * pw + 1 + qc[i];
+        const int r = r0 + lr[i];
+        if (q >= n || r < 0 || r >= H) {
+            lr[i] = 1 << 20;   // never active
+            continue;
+        }
+        const uint32_t gw = *reinterpret_cast<const uint32_t *>(a.g + (size_t)r * a.pitch + 4 * qc[i]);
+        const int nv = min(4, W - 4 * qc[i]);
+        qm[i] = nv >= 4 ? 0xFFFFFFFFu : (1u << (8 * nv)) - 1u;
+        for (int j = 0; j < nv; ++j) {
+            const int c = 4 * qc[i] + j;
+            int nm = (r == 0) + (r == H - 1) + (c == 0) + (c == W - 1);
+            if (NB == 8)
+                nm += (r == 0 || c == 0) + (r == 0 || c == W - 1) + (r == H - 1 || c == 0) +
+                      (r == H - 1 || c == W - 1);
+            qb[i] |= (uint32_t)(((int)((gw >> (8 * j)) & 1u) * (NB + 1) + nm) * (NB + 1)) << (8 * j);
+        }
+    }
+    const uint32_t t0 = sweep_index(a);
+    const uint32_t tag = GIBBS ? kTagGibbs : kTagPCA;
+    const auto uniforms = [&](uint32_t t) {
+#pragma unroll
+        for (int i = 0; i < QPT; ++i)
+            if (lr[i] < (1 << 20))
+                quad_words(a, tag, t, r0 + lr[i], qc[i], un[i]);
+    };
+    uniforms(t0);
+    cluster_sync();   // every CTA has read its rows: the last one may write them back
+    uint32_t nre = 0u;
+    int cur = 0, nacc = 0;
+    // add the counts of the 16-bit lanes to the accumulator and clear them
+    const auto flush = [&]() {
+#pragma unroll
+        for (int i = 0; i < QPT; ++i) {
+            if ((unsigned)lr[i] >= (unsigned)own)
+                continue;
+            const uint32_t cnt[4] = {clo[i] & 0xFFFFu, chi[i] & 0xFFFFu, clo[i] >> 16,
+                                     chi[i] >> 16};
+            float *accq = a.acc + (size_t)(r0 + lr[i]) * W + 4 * qc[i];
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (((qm[i] >> (8 * j)) & 1u) && cnt[j] != 0u)
+                    accq[j] += (float)cnt[j];
+            clo[i] = chi[i] = 0u;
+        }
+    };
+    int done = 0;
+    for (unsigned int x = 0;; ++x) {               // exchanges
+        const int ns = min(K, nsweeps - done);
+        for (int s = 0; s < ns; ++s) {
+            const uint32_t t = t0 + (uint32_t)(done + s);
+            const bool acc_now = accumulate_after(a, t);
+            uint32_t u[QPT][4];
+#pragma unroll
+            for (int i = 0; i < QPT; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    u[i][j] = un[i][j];
+            uint32_t *const X = cur ? pl1 : pl0;
+            uint32_t *const Y = GIBBS ? X : (cur ? pl0 : pl1);
+#pragma unroll 1
+            for (int ph = 0; ph < kCol; ++ph) {
+                const int e = (ns - s) * kCol - 1 - ph;   // rows beyond the band, each side
+#pragma unroll
+                for (int i = 0; i < QPT; ++i) {
+                    if ((unsigned)(lr[i] + e) >= (unsigned)(band + 2 * e))
+                        continue;
+                    const bool mine = (unsigned)lr[i] < (unsigned)own;
+                    uint32_t act = qm[i];
+                    if (GIBBS)
+                        act &= phase_mask<NB>(r0 + lr[i], ph);
+                    if (act == 0u)
+                        continue;
+                    uint32_t M;
+                    const uint32_t S = quad_counts<NB>(X, qo[i], pw, M) + qb[i];
+                    const uint32_t nw = quad_draw<NB>(tab, S, M, u[i], mine ? act : 0u, nre) & act;
+                    Y[qo[i]] = GIBBS ? (M & ~act) | nw : nw;
+                    if (acc_now && mine) {
+                        clo[i] += nw & 0x00FF00FFu;
+                        chi[i] += (nw >> 8) & 0x00FF00FFu;
+                    }
+                }
+                if (ph == kCol - 1)
+                    uniforms(t + 1u);   // independent of the labels: fills the pass
+                __syncthreads();
+            }
+            if (!GIBBS)
+                cur ^= 1;
+            if (acc_now && ++nacc == 0xFFFF) {   // a 16-bit lane is full
+                flush();
+                nacc = 0;
+            }
+        }
+        done += ns;
+        if (done == nsweeps)
+            break;
+        uint32_t *const X = cur ? pl1 : pl0;
+        uint32_t *const rv = recv + (x & 1u) * 2 * h * qrow;
+        // the band's first rows go below the upper neighbour's band, its last
+        // ones above the lower neighbour's (full there: only the last band of
+        // the image is short)
+        for (int i = tid; i < 2 * h * qrow; i += nt) {
+            const int up = i < h * qrow;
+            const int k = up ? i : i - h * qrow;
+            const int j = k / qrow, q = k - j * qrow;
+            const int row = up ? j : band - h + j;
+            if (row >= own || (up ? rank == 0 : rank + 1 == kClCtas))
+                continue;
+            st_cluster(rv + ((up ? h : 0) + j) * qrow + q, (uint32_t)(up ? rank - 1 : rank + 1),
+                       X[(row + h) * pw + 1 + q]);
+        }
+        cluster_sync();
+        for (int i = tid; i < 2 * h * qrow; i += nt) {
+            const int up = i < h * qrow;
+            const int k = up ? i : i - h * qrow;
+            const int j = k / qrow, q = k - j * qrow;
+            const int row = up ? j - h : band + j;
+            if (r0 + row >= 0 && r0 + row < H)
+                X[(row + h) * pw + 1 + q] = rv[((up ? 0 : h) + j) * qrow + q];
+        }
+        __syncthreads();
+    }
+    flush();
+    const uint32_t *fin = cur ? pl1 : pl0;
+    for (int i = tid; i < own * qrow; i += nt) {
+        const int r = i / qrow, q = i - r * qrow;
+        const uint32_t w = fin[(r + h) * pw + 1 + q];
+        uint8_t *out = xg_out + (size_t)(r0 + r) * a.pitch + 4 * q;
+        const int nv = min(4, W - 4 * q);
+        if (nv == 4)
+            *reinterpret_cast<uint32_t *>(out) = w;
+        else
+            for (int j = 0; j < nv; ++j)
+                out[j] = (uint8_t)(w >> (8 * j));
+    }
+    const uint32_t warp_re = __reduce_add_sync(0xFFFFFFFFu, nre);
+    if ((tid & 31) == 0 && warp_re != 0u)
+        atomicAdd(a.fp64_draws, (unsigned long long)warp_re);
+}
+
 // Batched chains: CTA b runs chain idx[b] (a PCA slot) with the table
 // tabs + b * kBtabStride, for the sweeps t0 .. t0 + n - 1 below the slot's
 // budget (t0 its device sweep counter); the planes follow the counter.
@@ -424,11 +655,41 @@ cudaError_t launch_res_t(const SweepArgs &a, const uint8_t *x_in, uint8_t *x_out
     return cudaGetLastError();
 }
 
+// Rows per CTA of the cluster form; 0 when the bands would be thinner than
+// the halo, or few quads leave nothing to share.
+inline int cluster_band(int H, int W)
+{
+    const int band = (H + kClCtas - 1) / kClCtas, qrow = (W + 3) >> 2;
+    if (band < kClHalo || H * qrow < 512)
+        return 0;
+    return (band + 2 * kClHalo - 2) * qrow <= 2 * kClThreads ? band : 0;
+}
+
+template <int NB, bool GIBBS, int QPT>
+cudaError_t launch_cl_t(const SweepArgs &a, const uint8_t *x_in, uint8_t *x_out, int n, int band,
+                        cudaStream_t st)
+{
+    const int qrow = (a.W + 3) >> 2;
+    const int quads = (band + 2 * kClHalo - 2) * qrow;
+    const int threads = ((quads + QPT - 1) / QPT + 31) & ~31;
+    const int smem = cl_smem_bytes(GIBBS, band, a.W);
+    if (threads > kClThreads || smem > 48 * 1024)
+        return cudaErrorInvalidValue;
+    resident_cluster_kernel<NB, GIBBS, QPT><<<kClCtas, threads, smem, st>>>(a, x_in, x_out, n, band);
+    return cudaGetLastError();
+}
+
 template <int NB, bool GIBBS>
 cudaError_t launch_res_q(const SweepArgs &a, const uint8_t *x_in, uint8_t *x_out, int n,
                          cudaStream_t st)
 {
     const int nq = a.H * (((a.W + 3) & ~3) >> 2);
+    const int band = cluster_band(a.H, a.W);
+    if (band > 0) {
+        const bool one = (band + 2 * kClHalo - 2) * ((a.W + 3) >> 2) <= kClThreads;
+        return one ? launch_cl_t<NB, GIBBS, 1>(a, x_in, x_out, n, band, st)
+                   : launch_cl_t<NB, GIBBS, 2>(a, x_in, x_out, n, band, st);
+    }
     if (nq <= kResThreads)
         return launch_res_t<NB, GIBBS, 1>(a, x_in, x_out, n, st);
     if (nq <= 2 * kResThreads)
