@@ -259,7 +259,7 @@ struct pcad_chain {
     long long wait_ns = 0;        // limit of each bounded device wait (0: the default, 1 s)
     int row_off = 0;              // global row of local row 0 (a band of a larger image)
     int stall_tile = 0;           // test aid: wavefront tile stall_tile - 1 never publishes
-    unsigned long long *esums = nullptr;   // energy reduction sums (device, 2 x u64)
+    unsigned long long *esums = nullptr;   // energy reduction sums (device, 3 x u64)
     EnergyCoef ecoef{};
     EnergyTrack track{};          // minimum-energy tracking (trace == nullptr: off)
     unsigned int *wave = nullptr; // wavefront kernel: per-tile counters + work counter
@@ -905,7 +905,7 @@ pcad_status reset_track(pcad_chain *ch)
 {
     const double inf = HUGE_VAL;
     CUDA_TRY(cudaMemsetAsync(ch->track.n, 0, sizeof(unsigned int), ch->stream));
-    CUDA_TRY(cudaMemsetAsync(ch->track.flag, 0, sizeof(int), ch->stream));
+    CUDA_TRY(cudaMemsetAsync(ch->track.which, 0, sizeof(int), ch->stream));
     CUDA_TRY(cudaMemsetAsync(ch->track.best_sweep, 0, sizeof(unsigned long long), ch->stream));
     CUDA_TRY(cudaMemcpyAsync(ch->track.best, &inf, sizeof(double), cudaMemcpyHostToDevice,
                              ch->stream));
@@ -1096,11 +1096,11 @@ pcad_status pcad_chain_track_energy(pcad_chain *ch, int capacity)
     ch->track = EnergyTrack{};
     if (capacity == 0)
         return PCAD_OK;
-    const size_t head = 64;   // best, best_sweep, n, flag
+    const size_t head = 256;   // best, best_sweep, n, which
     const size_t trace = align_up((size_t)capacity * sizeof(double), 256);
-    const size_t plane = (size_t)ch->pitch * ch->H;
+    const size_t plane = align_up((size_t)ch->pitch * ch->H, 256);
     void *blk = nullptr;
-    cudaError_t e = cudaMallocAsync(&blk, head + trace + plane, ch->stream);
+    cudaError_t e = cudaMallocAsync(&blk, head + trace + 2 * plane, ch->stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return fail(e == cudaErrorMemoryAllocation ? PCAD_ENOMEM : PCAD_ECUDA,
@@ -1111,10 +1111,11 @@ pcad_status pcad_chain_track_energy(pcad_chain *ch, int capacity)
     ch->track.best = (double *)p;
     ch->track.best_sweep = (unsigned long long *)(p + 8);
     ch->track.n = (unsigned int *)(p + 16);
-    ch->track.flag = (int *)(p + 20);
+    ch->track.which = (int *)(p + 20);
     ch->track.trace = (double *)(p + head);
     ch->track.cap = capacity;
-    ch->track.xb = (uint8_t *)(p + head + trace);
+    ch->track.xb[0] = (uint8_t *)(p + head + trace);
+    ch->track.xb[1] = ch->track.xb[0] + plane;
     return reset_track(ch);
 }
 
@@ -1151,7 +1152,9 @@ pcad_status pcad_chain_read_min_state(pcad_chain *ch, uint8_t *host_out, int out
     CUDA_TRY(cudaMemcpy(&bs, ch->track.best_sweep, sizeof(bs), cudaMemcpyDeviceToHost));
     if (bs == 0)
         return fail(PCAD_ESTATE, "no sweep has been tracked yet");
-    CUDA_TRY(read_labels(host_out, out_pitch, ch->track.xb, ch->pitch, ch->H, ch->W, ch->fplane,
+    int which = 0;
+    CUDA_TRY(cudaMemcpy(&which, ch->track.which, sizeof(which), cudaMemcpyDeviceToHost));
+    CUDA_TRY(read_labels(host_out, out_pitch, ch->track.xb[which & 1], ch->pitch, ch->H, ch->W, ch->fplane,
                          ch->stream));
     CUDA_TRY(cudaStreamSynchronize(ch->stream));
     if (energy)

@@ -236,11 +236,11 @@ struct EnergyTrack {
     unsigned int *n;                // entries recorded
     double *best;                   // lowest H so far (+inf initially)
     unsigned long long *best_sweep; // completed sweeps when it was reached
-    int *flag;                      // this sweep set a new minimum
-    uint8_t *xb;                    // the lowest-energy state (same pitch as x)
+    int *which;                     // the plane of xb that holds the lowest-energy state
+    uint8_t *xb[2];                 // it and a spare (same pitch as x)
 };
 
-// sums (2 x u64, zero on entry, zero again on return) <- integer sums of
+// sums (3 x u64, zero on entry, zero again on return) <- integer sums of
 // labelling x; out[0..2] <- H, pair sum, data sum (when out != nullptr); with
 // tracking, record H as the energy after sweep *tdev + sweep_off.
 cudaError_t launch_energy(const uint8_t *x, const uint8_t *g, int H, int W, int pitch,
