@@ -651,7 +651,6 @@ struct TileSet {
         TileKind kind;
         TilePack pack;
         int ctas = 0;
-        size_t smem = 0;
     };
     std::vector<Launch> launches;
     std::vector<int> slots;
@@ -662,34 +661,24 @@ struct TileSet {
     size_t bcap = 0;
 };
 
-// CTAs for the jobs of a launch: the fewest rounds of draws per sweep that
-// all jobs reach together on `cap` CTAs.
-bool tile_assign(const TileKind &k, std::vector<TileJob> &jobs, int cap, bool two, int &ctas,
-                 size_t &smem)
+// CTAs for the jobs of a launch: the smallest tiles that all jobs get together
+// on `cap` CTAs.
+bool tile_assign(const TileKind &k, std::vector<TileJob> &jobs, int cap, bool two, int &ctas)
 {
     long long total = 0;
     for (const TileJob &J : jobs)
         total += (long long)J.a.H * J.a.W;
-    for (int R = (int)std::max(1ll, total / ((long long)cap * 512)); R <= 16; ++R) {
+    // sites per CTA: the even share, then a step more until the grids fit
+    for (double per = (double)total / cap; per < 1e5; per *= 1.1) {
         ctas = 0;
-        smem = 0;
-        bool ok = true;
         for (TileJob &J : jobs) {
-            const int c0 = (int)(((long long)J.a.H * J.a.W + 512ll * R - 1) / (512ll * R));
-            bool got = false;
-            // (a tile grid may not use the CTAs it is offered evenly: a few more)
-            for (int c = c0; c <= c0 + c0 / 2 + 1 && c <= cap && !got; ++c) {
-                size_t b = 0;
-                if (tile_plan_ctas(k, J.a.H, J.a.W, c, two, J.tg, b) && tile_rounds(J.tg) <= R) {
-                    J.cta0 = ctas;
-                    ctas += J.tg.tiles_x * J.tg.tiles_y;
-                    smem = std::max(smem, b);
-                    got = true;
-                }
-            }
-            ok = ok && got;
+            const int c = (int)std::max(1.0, (double)J.a.H * J.a.W / per);
+            if (!tile_plan_ctas(k, J.a.H, J.a.W, std::min(c, cap), two, J.tg))
+                return false;   // larger tiles do not fit either
+            J.cta0 = ctas;
+            ctas += J.tg.tiles_x * J.tg.tiles_y;
         }
-        if (ok && ctas <= cap)
+        if (ctas <= cap)
             return true;
     }
     return false;
@@ -793,8 +782,8 @@ pcad_status tile_set_build(TileSet &ts, const std::vector<SlotDesc> &d,
                 total = 0;
                 for (const TileJob &J : jobs)
                     total += (long long)J.a.H * J.a.W;
-                const bool two = total > 512ll * sms;
-                fits = tile_assign(k, jobs, two ? 2 * sms : sms, two, L.ctas, L.smem);
+                const bool two = total > 1024ll * sms;
+                fits = tile_assign(k, jobs, two ? 2 * sms : sms, two, L.ctas);
                 if (!fits) {   // one chain less
                     jobs.pop_back();
                     --at;
@@ -832,11 +821,11 @@ pcad_status tile_set_issue(const TileSet &ts, int n, cudaStream_t st)
             one.njobs = 1;
             one.err = L.pack.err;
             one.job[0] = L.pack.job[0];
-            B_TRY(launch_tile(L.kind, one, L.ctas, L.smem, st));
+            B_TRY(launch_tile(L.kind, one, L.ctas, st));
         } else {
             TilePack p = L.pack;
             p.nsweeps = n;
-            B_TRY(launch_tile(L.kind, p, L.ctas, L.smem, st));
+            B_TRY(launch_tile(L.kind, p, L.ctas, st));
         }
     }
     return PCAD_OK;

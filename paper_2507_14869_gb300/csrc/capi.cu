@@ -267,8 +267,7 @@ struct pcad_chain {
     int sms = 0;                  // multiprocessors of the chain's device
     unsigned long long *xch = nullptr;   // tile-resident sweeps: border exchange (nullptr: not taken)
     TileKind tkind;
-    TileGeom tgeom{};
-    size_t tsmem = 0;
+    TilePlan tplan{};
     void *track_block = nullptr;
 };
 
@@ -371,13 +370,13 @@ bool uses_wave(const pcad_chain *ch);
 // AUTO (or SMALL) would run the small-label, wavefront, two-label, general or
 // windowed kernels; energy tracking needs every sweep's state.  Measured on
 // GB300, us per sweep (tile-resident / the kernel it replaces):
-//   small labels, to kTileMaxSites sites: 256^2 L = 9, 8 neighbours 2.8 / 6.7,
-//   L = 5 Gibbs 4.3 / 12.3 (four launches); L = 16 300^2 2.7 / 7.0, 512^2
-//   4.8 / 7.0, 1024^2 13.2 / 15.6 (2048^2, on TMA tiles: 45);
-//   two labels: 300^2 1.6 / 3.8, 600^2 2.7 / 4.5, 1000^2 5.1 / 5.8;
-//   segment draw: 256^2 L = 24 3.9 / 6.2, L = 64 4.4 / 8.5; at 512^2 L = 256
-//   the wavefront's 4 x 32-site items pack better (10.5 / 9.5; Gibbs, whose
-//   phases need no exchange here, 13.3 / 14.4; at 720^2 20.5 / 19.6): from 8
+//   small labels, to kTileMaxSites sites: 256^2 L = 9, 8 neighbours 2.2 / 6.7,
+//   L = 5 1.8 / 6.3, L = 5 Gibbs 3.9 / 12.3 (four launches); L = 16 300^2 2.6 /
+//   7.0, 512^2 4.7 / 7.0, 1024^2 13.6 / 15.6 (2048^2, not taken: 40);
+//   two labels: 300^2 1.3 / 3.8, 600^2 2.7 / 4.5, 1000^2 5.4 / 5.8;
+//   segment draw: 256^2 L = 24 3.7 / 6.2, L = 64 3.9 / 8.5; at 512^2 L = 256
+//   the wavefront's 4 x 32-site items pack better (11.7 / 9.5; Gibbs, whose
+//   phases need no exchange here, 13.3 / 14.4; at 720^2 20.4 / 19.6): from 8
 //   blocks of 4 x 32 sites per multiprocessor on, PCA stays with it, from
 //   kTileSegGibbsSites sites on Gibbs too.
 constexpr long long kTileSegGibbsSites = 300000;
@@ -522,8 +521,8 @@ pcad_status issue_sweeps(pcad_chain *ch, int off0, int n, int &cur, cudaStream_t
         L.job[0].x0 = ch->x[cur];
         L.job[0].x1 = ch->x[out];
         L.job[0].xch = ch->xch;
-        L.job[0].tg = ch->tgeom;
-        CUDA_TRY(launch_tile(ch->tkind, L, ch->tgeom.tiles_x * ch->tgeom.tiles_y, ch->tsmem, st));
+        L.job[0].tg = ch->tplan.tg;
+        CUDA_TRY(launch_tile(ch->tkind, L, ch->tplan.ctas, st));
         cur = out;
         return PCAD_OK;
     }
@@ -708,10 +707,9 @@ pcad_status create_common(const uint8_t *g_src, bool g_on_device, int H, int W, 
     // images AUTO gives the tensor-core sweep
     const bool gibbs = m->sampler != PCAD_SAMPLER_PCA;
     TileKind tkind;
-    TileGeom tgeom{};
-    size_t tsmem = 0;
+    TilePlan tplan{};
     const bool tile = (long long)H * W <= kTileMaxSites && tile_kind(tabs.dm, gibbs, tkind) &&
-                      tile_plan(tkind, H, W, sms, tgeom, tsmem);
+                      tile_plan(tkind, H, W, sms, tplan);
     const size_t xbytes = tile ? align_up(tile_xch_bytes(H, W), 256) : 0;
     const size_t sbytes =
         seg_structure(tabs.dm) ? align_up(seg_table_floats() * sizeof(float), 256) : 0;
@@ -747,8 +745,7 @@ pcad_status create_common(const uint8_t *g_src, bool g_on_device, int H, int W, 
         ch->xch = (unsigned long long *)p;
         p += xbytes;
         ch->tkind = tkind;
-        ch->tgeom = tgeom;
-        ch->tsmem = tsmem;
+        ch->tplan = tplan;
     }
     ch->sms = sms;
     ch->tdev = (uint32_t *)p;

@@ -10,19 +10,23 @@
 // all sweeps of a run: labels, observation, accumulator and tables stay in
 // shared memory, and only tile borders travel.
 //
-//   * Exchange.  After a sweep the tile's border words (4 labels) go to an
+//   * Exchange.  Every k sweeps the tile's border words (4 labels) go to an
 //     exchange buffer in global memory as 64-bit stores of (labels, tag = the
-//     sweep's number), and the neighbours' threads poll exactly the words of
-//     their halo until the tag is the sweep's: data and flag are one relaxed
-//     64-bit access, so a sweep waits for one store-to-load trip through L2
-//     and needs no fence.  Two buffers by sweep parity suffice: a tile writes
-//     sweep k + 2 only after its neighbours' words of k + 1 arrived, which
-//     they published after reading this tile's words of k.
-//   * Gibbs.  A sweep's 2 (4) colour phases run without exchange: the halo is
-//     2 (4) sites wide and phase q also updates the sites up to 1 - q (3 - q)
-//     beyond the tile.  Draws are keyed by (sweep, site), so both owners of
-//     such a site draw the same label.
-//   * The next sweep's uniforms are computed while the border words travel.
+//     number of sweeps done), and the neighbours' threads poll exactly the
+//     words of their halo until the tag is the awaited one: data and flag are
+//     one relaxed 64-bit access, so an exchange is one store-to-load trip
+//     through L2 and needs no fence.  Two buffers, used in turn, suffice: a
+//     tile writes exchange e + 2 only after its neighbours' words of e + 1
+//     arrived, which they published after reading this tile's words of e.
+//     Tags only grow between two resets of a chain; the buffers are cleared at
+//     creation and at a reset.
+//   * k sweeps per exchange.  The halo is h = k sites wide (Gibbs: k times the
+//     2 or 4 colour phases of a sweep); a sweep (phase) with e more to come
+//     before the next exchange also updates the sites up to e beyond the tile.
+//     Draws are keyed by (sweep, site), so every owner of such a site draws
+//     the same label.  k trades draws for exchanges (tile_geometry).
+//   * The uniforms of the next k sweeps are computed while the border words
+//     travel.
 //   * A launch holds one chain, or (batches, the server) several small ones,
 //     each on CTAs of its own.
 //
@@ -30,6 +34,7 @@
 // the two-label threshold table.  The CTAs wait on one another, so the launch is cooperative (all resident);
 // every poll is bounded (elapsed time, or another wait's error flag).
 // Measured times stand at uses_tile in capi.cu.
+#include <algorithm>
 #include <type_traits>
 
 #include "async_ptx.cuh"
@@ -43,8 +48,10 @@ namespace {
 
 using namespace sld;
 
-constexpr int kTlThreads = 512;
+constexpr int kTlThreads = 512;        // two CTAs per SM
+constexpr int kTlThreads1 = 1024;      // one: at most
 constexpr int kTlMaxSites = 8192;      // sites per tile
+constexpr int kTlMaxSweeps = 4;        // sweeps per exchange
 constexpr int kTlMaxSmem = 224 * 1024;    // one CTA per SM
 constexpr int kTlMaxSmem2 = 112 * 1024;   // two
 
@@ -77,9 +84,8 @@ __device__ __forceinline__ bool poll_word(const unsigned long long *p, uint32_t 
     return true;
 }
 
-// Halo width: a PCA sweep reads one site around the tile, a Gibbs sweep as
-// many as it has phases.
-__host__ __device__ constexpr int tile_halo(int nb, bool gibbs)
+// Colour phases of a sweep.
+__host__ __device__ constexpr int tile_phases(int nb, bool gibbs)
 {
     return !gibbs ? 1 : (nb == 4 ? 2 : 4);
 }
@@ -97,17 +103,18 @@ struct SmallPol {
     static constexpr uint32_t kFill = 0x10101010u;   // code 16: missing
     static constexpr int kTabBytes = kPtabWords * 4 + 16 * kAqStride * 4;
     static constexpr int kRowBytes = kPrefixStride * 4;
+    static constexpr double kNsSite = NB == 8 ? 1.6 : 1.4;   // one SM's time per draw (ns)
     uint32_t *pt;
     float *aq, *pre;
 
-    __device__ __forceinline__ void load(const DevModel &m, uint8_t *tab, uint8_t *row, int tid)
+    __device__ __forceinline__ void load(const DevModel &m, uint8_t *tab, uint8_t *row, int tid, int nt)
     {
         pt = reinterpret_cast<uint32_t *>(tab);
         aq = reinterpret_cast<float *>(tab + kPtabWords * 4);
         pre = reinterpret_cast<float *>(row);
-        for (int i = tid; i < kPtabWords / 4; i += kTlThreads)
+        for (int i = tid; i < kPtabWords / 4; i += nt)
             reinterpret_cast<uint4 *>(pt)[i] = __ldg(reinterpret_cast<const uint4 *>(m.ptab) + i);
-        fill_aq(m, aq, tid, kTlThreads);
+        fill_aq(m, aq, tid, nt);
     }
 
     __device__ __forceinline__ int draw(const SweepArgs &a, const uint8_t *me, int SB, int g,
@@ -149,12 +156,13 @@ struct SegPol {
     static constexpr uint32_t kFill = 0u;
     static constexpr int kTabBytes = seg::kSegFloats * 4;
     static constexpr int kRowBytes = 0;
+    static constexpr double kNsSite = 4.5;
     float *tab;
 
-    __device__ __forceinline__ void load(const DevModel &m, uint8_t *t, uint8_t *, int tid)
+    __device__ __forceinline__ void load(const DevModel &m, uint8_t *t, uint8_t *, int tid, int nt)
     {
         tab = reinterpret_cast<float *>(t);
-        for (int i = tid; i < seg::kSegFloats / 4; i += kTlThreads)
+        for (int i = tid; i < seg::kSegFloats / 4; i += nt)
             reinterpret_cast<float4 *>(tab)[i] =
                 __ldg(reinterpret_cast<const float4 *>(m.stab) + i);
     }
@@ -187,12 +195,13 @@ struct BinPol {
     static constexpr int kEntries = 4 * (NB + 1) * (NB + 1);
     static constexpr int kTabBytes = kEntries * 16;
     static constexpr int kRowBytes = 0;
+    static constexpr double kNsSite = 0.5;
     const uint4 *tab;
     uint32_t nre;
 
-    __device__ __forceinline__ void load(const DevModel &m, uint8_t *t, uint8_t *, int tid)
+    __device__ __forceinline__ void load(const DevModel &m, uint8_t *t, uint8_t *, int tid, int nt)
     {
-        for (int i = tid; i < kEntries; i += kTlThreads)
+        for (int i = tid; i < kEntries; i += nt)
             reinterpret_cast<uint4 *>(t)[i] = m.btab[i];
         tab = reinterpret_cast<const uint4 *>(t);
         nre = 0u;
@@ -223,25 +232,24 @@ struct BinPol {
 };
 
 // Shared memory of a tile (bytes), in the order of the kernel's pointers:
-// tables, thread scratch, uniforms, label planes, observation, counts.
+// tables, thread scratch, uniforms of k sweeps, label planes, observation,
+// counts.
 template <class P, bool GIBBS>
-size_t tile_smem(int th, int twq)
+size_t tile_smem(const TileGeom &tg, int nt)
 {
-    const int h = tile_halo(P::NB, GIBBS);
-    const size_t words = (size_t)(th + 2 * h) * (twq + 2);
-    return (size_t)P::kTabBytes + (size_t)kTlThreads * P::kRowBytes + words * 16 +
-           words * 4 * (GIBBS ? 1 : 2) + words * 4 + (size_t)th * twq * 16;
+    const size_t words = (size_t)(tg.th + 2 * tg.h) * (tg.twq + 2 * tg.hq);
+    return (size_t)P::kTabBytes + (size_t)nt * P::kRowBytes + words * 16 * tg.k +
+           words * 4 * (GIBBS ? 1 : 2) + words * 4 + (size_t)tg.th * tg.twq * 16;
 }
 
 template <class P, bool GIBBS, int JOBS>
-__global__ void __launch_bounds__(kTlThreads, 2)
+__global__ void __launch_bounds__(kTlThreads1, 1)
     tile_kernel(const __grid_constant__ TileLaunchT<JOBS> L)
 {
     constexpr bool MULTI = JOBS > 1;
     extern __shared__ __align__(16) uint8_t sm[];
     constexpr int NB = P::NB;
-    constexpr int h = tile_halo(NB, GIBBS);
-    constexpr int kCol = NB == 4 ? 2 : 4;
+    constexpr int kCol = tile_phases(NB, GIBBS);
     int j = 0;
     if (MULTI)
         while (j + 1 < L.njobs && (int)blockIdx.x >= L.job[j + 1].cta0)
@@ -250,9 +258,10 @@ __global__ void __launch_bounds__(kTlThreads, 2)
     const SweepArgs &a = J.a;
     int *const err = L.err;
     const int cta = (int)blockIdx.x - (MULTI ? J.cta0 : 0);
-    const int tid = (int)threadIdx.x;
+    const int tid = (int)threadIdx.x, nt = (int)blockDim.x;
     const int TH = J.tg.th, TWq = J.tg.twq, TW = 4 * TWq;
-    const int SW = TWq + 2, SB = 4 * SW;            // words and bytes per staged row
+    const int h = J.tg.h, hq = J.tg.hq, hb = 4 * hq;  // halo: rows, words, columns
+    const int SW = TWq + 2 * hq, SB = 4 * SW;         // words and bytes per staged row
     const int words = (TH + 2 * h) * SW;
     const int H = a.H, W = a.W, Wq = (W + 3) >> 2;
     const int ty = cta / J.tg.tiles_x, tx = cta - ty * J.tg.tiles_x;
@@ -269,19 +278,18 @@ __global__ void __launch_bounds__(kTlThreads, 2)
     const uint8_t *xg_in = J.par_from_t && (t0 & 1u) ? J.x1 : J.x0;
     uint8_t *xg_out = J.par_from_t ? (((t0 + (uint32_t)nsweeps) & 1u) ? J.x1 : J.x0) : J.x1;
 
-    uint8_t *const tab = sm;
     uint8_t *const row = sm + P::kTabBytes + tid * P::kRowBytes;
-    uint32_t *U = reinterpret_cast<uint32_t *>(sm + P::kTabBytes + kTlThreads * P::kRowBytes);
-    uint32_t *pl0 = U + 4 * words;
+    uint32_t *U = reinterpret_cast<uint32_t *>(sm + P::kTabBytes + nt * P::kRowBytes);
+    uint32_t *pl0 = U + 4 * words * J.tg.k;
     uint32_t *pl1 = GIBBS ? pl0 : pl0 + words;
     uint32_t *gw = pl1 + words;
     uint32_t *cnt = gw + words;                     // [TH][TW] label sums of this launch
     P pol;
-    pol.load(a.m, tab, row, tid);
+    pol.load(a.m, sm, row, tid, nt);
     // labels and observation with the halo
-    for (int i = tid; i < words; i += kTlThreads) {
+    for (int i = tid; i < words; i += nt) {
         const int sr = i / SW, sq = i - sr * SW;
-        const int r = r0 - h + sr, q = q0 - 1 + sq;
+        const int r = r0 - h + sr, q = q0 - hq + sq;
         uint32_t x = P::kFill, g = 0u;
         if (r >= 0 && r < H && q >= 0 && q < Wq) {
             x = *reinterpret_cast<const uint32_t *>(xg_in + (size_t)r * a.pitch + 4 * q);
@@ -298,75 +306,59 @@ __global__ void __launch_bounds__(kTlThreads, 2)
             pl1[i] = P::kFill;
         gw[i] = g;
     }
-    for (int i = tid; i < TH * TW; i += kTlThreads)
+    for (int i = tid; i < TH * TW; i += nt)
         cnt[i] = 0u;
 
     const long long limit = wait_limit(a.wait_ns);
     const uint32_t key0 = (uint32_t)(a.seed & 0xFFFFFFFFull), key1 = (uint32_t)(a.seed >> 32);
     const uint32_t ctr3 = ((GIBBS ? kTagGibbs : kTagPCA) << 24) | (a.chain & 0xFFFFFFu);
-    // the uniforms of a sweep: the tile's quads (Gibbs: with the halo's), at
-    // their staged word
-    const auto uniforms = [&](uint32_t t) {
-        const int nw = GIBBS ? words : TH * TWq;
-        for (int i = tid; i < nw; i += kTlThreads) {
-            int sr, sq;
-            if (GIBBS) {
-                sr = i / SW;
-                sq = i - sr * SW;
-            } else {
-                sr = i / TWq;
-                sq = i - sr * TWq + 1;
-                sr += h;
+    // the uniforms of `ns` sweeps from t on, at their staged words: sweep s
+    // updates up to (ns - s) kCol - 1 sites beyond the tile
+    const auto uniforms = [&](uint32_t t, int ns) {
+        for (int s = 0; s < ns; ++s) {
+            const int e = (ns - s) * kCol - 1, eq = (e + 3) >> 2;
+            const int per = TWq + 2 * eq, n = (TH + 2 * e) * per;
+            const unsigned int inv = 0xFFFFFFFFu / (unsigned int)per + 1u;
+            for (int i = tid; i < n; i += nt) {
+                // (per == 1: the reciprocal does not fit 32 bits)
+                const int ir = per == 1 ? i : (int)__umulhi((unsigned int)i, inv);
+                const int lr = ir - e, lq = i - ir * per - eq;
+                uint32_t o0, o1, o2, o3;
+                philox4x32_10((uint32_t)(q0 + lq), (uint32_t)(r0 + lr + a.row_off),
+                              t + (uint32_t)s, ctr3, key0, key1, o0, o1, o2, o3);
+                reinterpret_cast<uint4 *>(U)[s * words + (lr + h) * SW + lq + hq] =
+                    make_uint4(o0 >> 8, o1 >> 8, o2 >> 8, o3 >> 8);
             }
-            uint32_t o0, o1, o2, o3;
-            philox4x32_10((uint32_t)(q0 - 1 + sq), (uint32_t)(r0 - h + sr + a.row_off), t, ctr3,
-                          key0, key1, o0, o1, o2, o3);
-            reinterpret_cast<uint4 *>(U)[sr * SW + sq] =
-                make_uint4(o0 >> 8, o1 >> 8, o2 >> 8, o3 >> 8);
         }
     };
-    // the draw of the site at local (lr, lc) from plane X
-    const auto draw = [&](const uint32_t *X, int lr, int lc, bool valid, bool own) -> int {
-        const int o = (lr + h) * SB + lc + 4;
-        const int g = valid ? (int)reinterpret_cast<const uint8_t *>(gw)[o] : 0;
-        const uint32_t ub = valid ? U[o] : 0u;
-        return pol.draw(a, reinterpret_cast<const uint8_t *>(X) + o, SB, g, ub, r0 + lr, c0 + lc,
-                        valid, own);
-    };
-    uniforms(t0);
+    uniforms(t0, min(J.tg.k, nsweeps));
     bool ok = true;
     uint32_t *X = pl0;
-    for (int k = 0; k < nsweeps; ++k) {
-        const uint32_t t = t0 + (uint32_t)k;
-        const bool acc_now = accumulate_after(a, t);
+    int done = 0;
+    for (unsigned int x = 1;; ++x) {                // exchanges
+        const int ns = min(J.tg.k, nsweeps - done);
         // halo words and uniforms in place; leave together when a wait gave up
         if (__syncthreads_or(!ok)) {
             if (tid == 0)
                 atomicExch(err, 1);
             return;
         }
-        if constexpr (!GIBBS) {
-            uint32_t *Y = X == pl0 ? pl1 : pl0;
-            for (int b = 0; b < TH * TW; b += kTlThreads) {
-                const int i = b + tid;
-                const int lr = (int)__umulhi((unsigned int)i, J.tg.inv_tw), lc = i - lr * TW;
-                const bool valid = i < TH * TW && r0 + lr < H && c0 + lc < W;
-                const int s = draw(X, lr, lc, valid, true);
-                if (valid) {
-                    reinterpret_cast<uint8_t *>(Y)[(lr + h) * SB + lc + 4] = (uint8_t)s;
-                    if (acc_now)
-                        cnt[i] += (uint32_t)s;
-                }
-            }
-            X = Y;
-            __syncthreads();
-        } else {
+        for (int s = 0; s < ns; ++s) {
+            const uint32_t t = t0 + (uint32_t)(done + s);
+            const bool acc_now = accumulate_after(a, t);
+            const uint32_t *Us = U + 4 * s * words;
+            uint32_t *Y = GIBBS ? X : (X == pl0 ? pl1 : pl0);
 #pragma unroll 1
             for (int q = 0; q < kCol; ++q) {
-                // colour q of rows [-e, TH + e), columns [-e, TW + e)
-                const int e = kCol - 1 - q;
+                // sites of colour q of rows [-e, TH + e), columns [-e, TW + e)
+                const int e = (ns - s) * kCol - 1 - q;
                 int nr, per, sr0, sc0;   // rows, sites per row, first row and column
-                if (NB == 4) {
+                if (!GIBBS) {
+                    nr = TH + 2 * e;
+                    per = TW + 2 * e;
+                    sr0 = -e;
+                    sc0 = -e;
+                } else if (NB == 4) {
                     nr = TH + 2 * e;
                     per = (TW + 2 * e + 1) >> 1;
                     sr0 = -e;
@@ -377,61 +369,70 @@ __global__ void __launch_bounds__(kTlThreads, 2)
                     nr = (TH + e - sr0 + 1) >> 1;
                     per = (TW + e - sc0 + 1) >> 1;
                 }
-                const unsigned int inv = 0xFFFFFFFFu / (unsigned int)per + 1u;
-                for (int b = 0; b < nr * per; b += kTlThreads) {
+                const unsigned int inv = 0xFFFFFFFFu / (unsigned int)per + 1u;   // per >= 2
+                for (int b = 0; b < nr * per; b += nt) {
                     const int i = b + tid;
                     const int ir = (int)__umulhi((unsigned int)i, inv), ic = i - ir * per;
-                    const int lr = NB == 4 ? sr0 + ir : sr0 + 2 * ir;
-                    int lc = sc0 + 2 * ic;
-                    if (NB == 4)
+                    const int lr = GIBBS && NB == 8 ? sr0 + 2 * ir : sr0 + ir;
+                    int lc = GIBBS ? sc0 + 2 * ic : sc0 + ic;
+                    if (GIBBS && NB == 4)
                         lc += (r0 + lr + c0 + lc + q) & 1;
-                    const bool valid = ir < nr && lc < TW + e && (unsigned)(r0 + lr) < (unsigned)H &&
+                    const bool valid = ir < nr && lc < TW + e &&
+                                       (unsigned)(r0 + lr) < (unsigned)H &&
                                        (unsigned)(c0 + lc) < (unsigned)W;
-                    const int s = draw(X, lr, lc, valid,
-                                       (unsigned)lr < (unsigned)TH && (unsigned)lc < (unsigned)TW);
-                    if (valid)
-                        reinterpret_cast<uint8_t *>(X)[(lr + h) * SB + lc + 4] = (uint8_t)s;
+                    const bool own = (unsigned)lr < (unsigned)TH && (unsigned)lc < (unsigned)TW;
+                    const int o = (lr + h) * SB + lc + hb;
+                    const int g = valid ? (int)reinterpret_cast<const uint8_t *>(gw)[o] : 0;
+                    const uint32_t ub = valid ? Us[o] : 0u;
+                    const int v = pol.draw(a, reinterpret_cast<const uint8_t *>(X) + o, SB, g, ub,
+                                           r0 + lr, c0 + lc, valid, own);
+                    if (valid) {
+                        reinterpret_cast<uint8_t *>(Y)[o] = (uint8_t)v;
+                        if (own && acc_now)
+                            cnt[lr * TW + lc] += (uint32_t)v;
+                    }
                 }
                 __syncthreads();
             }
-            if (acc_now)
-                for (int i = tid; i < TH * TW; i += kTlThreads) {
-                    const int lr = (int)__umulhi((unsigned int)i, J.tg.inv_tw), lc = i - lr * TW;
-                    cnt[i] += reinterpret_cast<const uint8_t *>(X)[(lr + h) * SB + lc + 4];
-                }
+            X = Y;
         }
-        // (a single Gibbs sweep, written back in place, still waits for the
-        // neighbours: they have then read their halo of the initial labels)
-        if (k + 1 == nsweeps && !(GIBBS && nsweeps == 1))
+        done += ns;
+        // (a run of one exchange's sweeps, written back in place, still waits
+        // for the neighbours: they have then read their halo of the initial
+        // labels)
+        if (done == nsweeps && !(x == 1 && xg_in == xg_out))
             break;
-        // publish the border words of this sweep
-        const uint32_t tag = t + 1u;
-        unsigned long long *buf = J.xch + (size_t)(tag & 1u) * H * Wq;
+        // publish the border words
+        const uint32_t tag = t0 + (uint32_t)done;
+        unsigned long long *buf = J.xch + (size_t)(x & 1u) * H * Wq;
         if ((int)blockIdx.x != a.stall_tile - 1)
-            for (int i = tid; i < TH * TWq; i += kTlThreads) {
+            for (int i = tid; i < TH * TWq; i += nt) {
                 const int lr = i / TWq, lq = i - lr * TWq;
-                const bool border = lr < h || lr >= TH - h || lq == 0 || lq == TWq - 1;
+                const bool border = lr < h || lr >= TH - h || lq < hq || lq >= TWq - hq;
                 if (border && r0 + lr < H && q0 + lq < Wq)
                     st_word(buf + (size_t)(r0 + lr) * Wq + q0 + lq,
-                            ((unsigned long long)tag << 32) | X[(lr + h) * SW + lq + 1]);
+                            ((unsigned long long)tag << 32) | X[(lr + h) * SW + lq + hq]);
             }
-        uniforms(t + 1u);
+        uniforms(t0 + (uint32_t)done, min(J.tg.k, nsweeps - done));
         // poll the halo: h rows above and below (with the corners where they
-        // are read), one word left and right of each row
-        const int nrow = 2 * h * SW, nh = nrow + 2 * TH;
-        for (int i = tid; i < nh && ok; i += kTlThreads) {
+        // are read), hq words left and right of each row
+        const bool corners = NB == 8 || GIBBS || h > 1;
+        const int nrow = 2 * h * SW, nh = nrow + 2 * hq * TH;
+        for (int i = tid; i < nh && ok; i += nt) {
             int sr, sq;
             if (i < nrow) {
                 sr = i / SW;
                 sq = i - sr * SW;
-                if (NB == 4 && !GIBBS && (sq == 0 || sq == SW - 1))
+                if (!corners && (sq < hq || sq >= SW - hq))
                     continue;   // no diagonal neighbours
                 sr = sr < h ? sr : sr + TH;
             } else {
-                sr = h + ((i - nrow) >> 1);
-                sq = (i & 1) ? SW - 1 : 0;   // nrow is even
+                sr = (i - nrow) / (2 * hq);
+                sq = (i - nrow) - sr * 2 * hq;
+                sr += h;
+                sq = sq < hq ? sq : sq + TWq;
             }
-            const int r = r0 - h + sr, q = q0 - 1 + sq;
+            const int r = r0 - h + sr, q = q0 - hq + sq;
             if (r < 0 || r >= H || q < 0 || q >= Wq)
                 continue;
             uint32_t w;
@@ -439,6 +440,8 @@ __global__ void __launch_bounds__(kTlThreads, 2)
             if (ok)
                 X[sr * SW + sq] = w;
         }
+        if (done == nsweeps)
+            break;
     }
     if (__syncthreads_or(!ok)) {
         if (tid == 0)
@@ -446,15 +449,15 @@ __global__ void __launch_bounds__(kTlThreads, 2)
         return;
     }
     pol.finish(a);
-    // labels and counts back (any label of this plane that a neighbour read at
-    // the start was read before it published its first sweep, which this tile
-    // awaited, or the planes differ)
-    for (int i = tid; i < TH * TWq; i += kTlThreads) {
+    // labels and counts back (a label of this plane that a neighbour read at
+    // the start was read before it published its first exchange, which this
+    // tile awaited, or the planes differ)
+    for (int i = tid; i < TH * TWq; i += nt) {
         const int lr = i / TWq, lq = i - lr * TWq;
         const int r = r0 + lr, c = c0 + 4 * lq;
         if (r >= H || c >= W)
             continue;
-        const uint32_t w = X[(lr + h) * SW + lq + 1];
+        const uint32_t w = X[(lr + h) * SW + lq + hq];
         float *pa = a.acc + (size_t)r * W + c;
         const uint32_t *n4 = cnt + lr * TW + 4 * lq;
         const int nv = min(4, W - c);
@@ -469,48 +472,69 @@ __global__ void __launch_bounds__(kTlThreads, 2)
     }
 }
 
-// The tile grid of an image: at most `ctas` tiles of at least h rows, the
-// fewest rounds of kTlThreads sites per tile, then the smallest border.
-bool tile_geometry(int H, int W, int ctas, int h, TileGeom &best)
+// Time model of a sweep of a tile (ns; k sweeps per exchange), for the choice
+// of the grid and of k only: kNsPass per pass over the sites (block barrier
+// and the latency of one draw), `site` per site an SM draws, kNsExchange per
+// exchange.
+constexpr double kNsPass = 350.0, kNsExchange = 1300.0;
+
+double tile_cost(int th, int tw, int k, int phases, int per_sm, double site)
 {
-    const int Wq = (W + 3) / 4;
-    long best_cost = -1;
-    for (int nx = 1; nx <= ctas && nx <= Wq; ++nx) {
-        const int twq = (Wq + nx - 1) / nx;
-        const int tx = (Wq + twq - 1) / twq;
-        int th = (H + ctas / tx - 1) / (ctas / tx);
-        th = th < h ? h : th;
-        const int ty = (H + th - 1) / th;
-        if ((long)th * twq * 4 > kTlMaxSites || tx * ty > ctas)
-            continue;
-        const long rounds = ((long)th * twq * 4 + kTlThreads - 1) / kTlThreads;
-        // (rounds dominate; a border word costs far less than a round of draws)
-        const long cost = rounds * 1000 + 2 * (th + twq);
-        if (best_cost < 0 || cost < best_cost) {
-            best_cost = cost;
-            best.th = th;
-            best.twq = twq;
-            best.tiles_x = tx;
-            best.tiles_y = ty;
-            best.inv_tw = 0xFFFFFFFFu / (unsigned int)(4 * twq) + 1u;
+    double ns = kNsExchange;
+    for (int s = 0; s < k; ++s)
+        for (int q = 0; q < phases; ++q) {
+            const int e = (k - s) * phases - 1 - q;
+            ns += kNsPass + site * per_sm * (th + 2 * e) * (tw + 2 * e) / phases;
         }
-    }
-    return best_cost >= 0;
+    return ns / k;
 }
 
-// The tiles of one image alone on the device: one CTA per SM while a round of
-// its threads covers the tile, two beyond.
+// The tile grid of an image: at most `ctas` tiles of at least h rows and
+// columns, k sweeps per exchange.
 template <class P, bool GIBBS>
-bool plan_t(int H, int W, int ctas, bool two, TileGeom &tg, size_t &smem)
+bool tile_geometry(int H, int W, int ctas, int per_sm, TileGeom &best)
 {
-    if (ctas <= 0 || !tile_geometry(H, W, ctas, tile_halo(P::NB, GIBBS), tg))
-        return false;
-    smem = tile_smem<P, GIBBS>(tg.th, tg.twq);
-    return smem <= (size_t)(two ? kTlMaxSmem2 : kTlMaxSmem);
+    constexpr int phases = tile_phases(P::NB, GIBBS);
+    const size_t most = per_sm == 2 ? kTlMaxSmem2 : kTlMaxSmem;
+    const int Wq = (W + 3) / 4;
+    double best_cost = -1.0;
+    for (int k = 1; k <= (GIBBS ? 2 : kTlMaxSweeps); ++k)
+        for (int nx = 1; nx <= ctas && nx <= Wq; ++nx) {
+            TileGeom g{};
+            g.k = k;
+            g.h = k * phases;
+            g.hq = (g.h + 3) / 4;
+            g.twq = (Wq + nx - 1) / nx;
+            if (g.twq < g.hq)
+                g.twq = g.hq;
+            g.tiles_x = (Wq + g.twq - 1) / g.twq;
+            const int rows = ctas / g.tiles_x;
+            g.th = (H + rows - 1) / rows;
+            if (g.th < g.h)
+                g.th = g.h;
+            g.tiles_y = (H + g.th - 1) / g.th;
+            if ((long)g.th * g.twq * 4 > kTlMaxSites || g.tiles_x * g.tiles_y > ctas)
+                continue;
+            // one CTA per SM: a thread per site of the widest pass, if they are
+            // few (idle warps still take every barrier)
+            const long wide = (long)(g.th + 2 * g.h - 2) * (4 * g.twq + 2 * g.h - 2) / phases;
+            g.threads = per_sm == 2 ? kTlThreads
+                                    : (int)std::min<long>(kTlThreads1,
+                                                          std::max<long>(256, (wide + 127) / 128 * 128));
+            // (the scratch of the widest launch: a pack has its widest job's threads)
+            if (tile_smem<P, GIBBS>(g, per_sm == 2 ? kTlThreads : kTlThreads1) > most)
+                continue;
+            const double cost = tile_cost(g.th, 4 * g.twq, k, phases, per_sm, P::kNsSite);
+            if (best_cost < 0.0 || cost < best_cost) {
+                best_cost = cost;
+                best = g;
+            }
+        }
+    return best_cost >= 0.0;
 }
 
 template <class P, bool GIBBS, int JOBS>
-cudaError_t launch_t(const TileLaunchT<JOBS> &L, int ctas, size_t smem, cudaStream_t st)
+cudaError_t launch_t(const TileLaunchT<JOBS> &L, int ctas, cudaStream_t st)
 {
     static bool attr_set[64] = {};
     int dev = 0;
@@ -528,7 +552,15 @@ cudaError_t launch_t(const TileLaunchT<JOBS> &L, int ctas, size_t smem, cudaStre
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(ctas);
-    cfg.blockDim = dim3(kTlThreads);
+    int threads = 0;   // the widest job's; shared memory for every job with them
+    size_t smem = 0;
+    for (int i = 0; i < L.njobs; ++i)
+        threads = std::max(threads, L.job[i].tg.threads);
+    for (int i = 0; i < L.njobs; ++i)
+        smem = std::max(smem, tile_smem<P, GIBBS>(L.job[i].tg, threads));
+    if (threads < 1 || smem > (size_t)kTlMaxSmem)
+        return cudaErrorInvalidValue;
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
@@ -585,18 +617,22 @@ bool tile_kind(const DevModel &m, bool gibbs, TileKind &k)
     return seg_eligible(m);
 }
 
-bool tile_plan(const TileKind &k, int H, int W, int sms, TileGeom &tg, size_t &smem)
+bool tile_plan(const TileKind &k, int H, int W, int sms, TilePlan &p)
 {
-    const bool two = (long long)H * W > (long long)sms * kTlThreads;
-    return tile_plan_ctas(k, H, W, two ? 2 * sms : sms, two, tg, smem);
+    const bool two = (long long)H * W > (long long)sms * kTlThreads1;
+    if (!tile_plan_ctas(k, H, W, two ? 2 * sms : sms, two, p.tg))
+        return false;
+    p.ctas = p.tg.tiles_x * p.tg.tiles_y;
+    return true;
 }
 
-bool tile_plan_ctas(const TileKind &k, int H, int W, int ctas, bool two, TileGeom &tg,
-                    size_t &smem)
+bool tile_plan_ctas(const TileKind &k, int H, int W, int ctas, bool two, TileGeom &tg)
 {
+    if (ctas <= 0)
+        return false;
     return with_policy(k, [&](auto pol, auto gibbs) {
         using P = std::remove_pointer_t<decltype(pol)>;
-        return plan_t<P, decltype(gibbs)::value>(H, W, ctas, two, tg, smem);
+        return tile_geometry<P, decltype(gibbs)::value>(H, W, ctas, two ? 2 : 1, tg);
     });
 }
 
@@ -605,15 +641,10 @@ size_t tile_xch_bytes(int H, int W)
     return (size_t)2 * H * ((W + 3) / 4) * sizeof(unsigned long long);
 }
 
-int tile_rounds(const TileGeom &tg)
-{
-    return (tg.th * tg.twq * 4 + kTlThreads - 1) / kTlThreads;
-}
-
 namespace {
 
 template <int JOBS>
-cudaError_t launch_checked(const TileKind &k, const TileLaunchT<JOBS> &L, int ctas, size_t smem,
+cudaError_t launch_checked(const TileKind &k, const TileLaunchT<JOBS> &L, int ctas,
                            cudaStream_t st)
 {
     if (L.njobs < 1 || L.njobs > JOBS || ctas < 1)
@@ -640,22 +671,20 @@ cudaError_t launch_checked(const TileKind &k, const TileLaunchT<JOBS> &L, int ct
         if constexpr (JOBS > 1 && decltype(gibbs)::value)
             return cudaErrorInvalidValue;   // batches and the server run the PCA sampler
         else
-            return launch_t<P, decltype(gibbs)::value, JOBS>(L, ctas, smem, st);
+            return launch_t<P, decltype(gibbs)::value, JOBS>(L, ctas, st);
     });
 }
 
 }  // namespace
 
-cudaError_t launch_tile(const TileKind &k, const TileLaunch &L, int ctas, size_t smem,
-                        cudaStream_t st)
+cudaError_t launch_tile(const TileKind &k, const TileLaunch &L, int ctas, cudaStream_t st)
 {
-    return launch_checked(k, L, ctas, smem, st);
+    return launch_checked(k, L, ctas, st);
 }
 
-cudaError_t launch_tile(const TileKind &k, const TilePack &L, int ctas, size_t smem,
-                        cudaStream_t st)
+cudaError_t launch_tile(const TileKind &k, const TilePack &L, int ctas, cudaStream_t st)
 {
-    return launch_checked(k, L, ctas, smem, st);
+    return launch_checked(k, L, ctas, st);
 }
 
 }  // namespace pcad

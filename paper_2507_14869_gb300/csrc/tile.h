@@ -23,7 +23,14 @@ struct TileKind {
 struct TileGeom {
     int th, twq;          // rows and quads (4-site words) per tile
     int tiles_x, tiles_y;
-    unsigned int inv_tw;  // ceil(2^32 / (4 twq)): s / (4 twq) = umulhi(s, inv_tw), s < 2^16
+    int k;                // sweeps per exchange
+    int h, hq;            // halo: rows (and columns), words
+    int threads;          // per CTA
+};
+
+struct TilePlan {
+    TileGeom tg;
+    int ctas;
 };
 
 // One chain of a launch.  Its sweeps are those at *a.sweep_base + a.sweep_off
@@ -57,18 +64,12 @@ static_assert(sizeof(TilePack) <= 32000, "kernel parameter space");
 bool tile_kind(const DevModel &m, bool gibbs, TileKind &k);
 // Tiles of an image alone on the device, or on at most `ctas` CTAs with two
 // or one per SM; false when they do not fit.
-bool tile_plan(const TileKind &k, int H, int W, int sms, TileGeom &tg, size_t &smem);
-bool tile_plan_ctas(const TileKind &k, int H, int W, int ctas, bool two, TileGeom &tg,
-                    size_t &smem);
+bool tile_plan(const TileKind &k, int H, int W, int sms, TilePlan &p);
+bool tile_plan_ctas(const TileKind &k, int H, int W, int ctas, bool two, TileGeom &tg);
 size_t tile_xch_bytes(int H, int W);
-// Whole rounds of a CTA's threads over the sites of a tile.
-int tile_rounds(const TileGeom &tg);
-// One cooperative launch of `ctas` CTAs (all the jobs' tiles) with smem bytes
-// (the largest job's).
-cudaError_t launch_tile(const TileKind &k, const TileLaunch &L, int ctas, size_t smem,
-                        cudaStream_t s);
-cudaError_t launch_tile(const TileKind &k, const TilePack &L, int ctas, size_t smem,
-                        cudaStream_t s);
+// One cooperative launch of `ctas` CTAs (all the jobs' tiles).
+cudaError_t launch_tile(const TileKind &k, const TileLaunch &L, int ctas, cudaStream_t s);
+cudaError_t launch_tile(const TileKind &k, const TilePack &L, int ctas, cudaStream_t s);
 // Chains, batches and the server take tile-resident launches for images of at
 // most this many sites.
 constexpr long long kTileMaxSites = 1ll << 20;
