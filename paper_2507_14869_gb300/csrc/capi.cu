@@ -595,8 +595,7 @@ pcad_status issue_sweeps(pcad_chain *ch, int off0, int n, int &cur, cudaStream_t
             if (small_tma(ch))
                 CUDA_TRY(launch_pca_small_tma(ch->xmap[cur], ch->gmap, a, ch->err, st));
             else if (uses_small(ch))
-                // chains check g < L at creation: the data term from a table
-                CUDA_TRY(launch_pca_small(a, st, nullptr, nullptr, nullptr, true));
+                CUDA_TRY(launch_pca_small(a, st));
             else if (uses_binary(ch))
                 CUDA_TRY(launch_pca_binary(a, st));
             else if (uses_win(ch))

@@ -382,12 +382,10 @@ bool pca_small_eligible(const DevModel &m);
 cudaError_t launch_pca_small_tma(const CUtensorMap &xmap, const CUtensorMap &gmap,
                                  const SweepArgs &a, int *err, cudaStream_t s);
 // x0 / x1 (optional): the planes of even / odd sweep indices, used in place of
-// a.xin / a.xout; budget (optional): sweeps with index >= *budget are skipped;
-// aq: the data term from a table of the observations g < 16 (observations
-// checked against L: chains use it).
+// a.xin / a.xout; budget (optional): sweeps with index >= *budget are skipped.
+// Observations below 16 (checked against L by chains, batches and the server).
 cudaError_t launch_pca_small(const SweepArgs &a, cudaStream_t s, uint8_t *x0 = nullptr,
-                             uint8_t *x1 = nullptr, const uint32_t *budget = nullptr,
-                             bool aq = false);
+                             uint8_t *x1 = nullptr, const uint32_t *budget = nullptr);
 
 // Whole chains of small two-label images in one CTA (state in shared
 // memory): L = 2, 4 or 8 neighbours, the thresholds table m.btab built, at

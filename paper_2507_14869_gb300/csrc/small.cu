@@ -14,25 +14,22 @@
 //     memory read per pair and four integer adds give the exact P(s) of all
 //     16 labels, four per 32-bit word (every byte <= 120, no carries).
 //   * Weights by the formula of the general kernel, w(s) =
-//     2^fl(alpha q + fl(gam P)), q = (g - s)^2 and P exact integers, two
+//     2^fl(gam P + fl(alpha q)), q = (g - s)^2 and P exact integers, two
 //     labels per packed FP32x2 instruction (every lane rounds as the scalar
 //     operation).  A byte of P becomes an exact float by placing it in the
-//     mantissa of 2^23 and subtracting 2^23.  Chains (whose observations are
-//     checked against L at creation) take fl(alpha q) from a 16 x 16 table in
-//     shared memory instead: one FFMA per label, fl(gam P + fl(alpha q)),
-//     within the same 3u |v| exponent bound; batches and the server keep the
-//     arithmetic form.  (Products of two table
+//     mantissa of 2^23 and subtracting 2^23; fl(alpha q) comes from a 16 x 16
+//     table in shared memory (observations are checked against L), within the
+//     same 3u |v| exponent bound.  (Products of two table
 //     factors per label measured slower: the per-lane table reads conflict
 //     in shared memory, while the exponential unit has room.)
-//   * Inverse CDF over chunks of 4 labels: in-chunk prefix sums (3
-//     roundings), chunk prefix (3 more), the inertia correction delta =
-//     w(x_i)(e^lambda - 1) (w(x_i) read back from the weights in shared
-//     memory) joined once to the chunk prefix, one join per probed label:
-//     every C_k within 8u and Z within 7u of exact, inside the 22u summation
-//     budget of the per-site certified margin (valid because gam <= 0 and
-//     alpha <= 0 keep both exponent terms non-positive).  The chunk, then the
-//     label in it, are found by comparisons; draws within the margin of a CDF
-//     boundary are re-drawn by the warp in FP64.
+//   * Inverse CDF over chunks of 4 labels (small_draw.cuh): packed chunk sums,
+//     the inertia atom delta = w(x_i)(e^lambda - 1) joined once to w(x_i) in
+//     the thread's row of weights in shared memory and to the chunk prefixes
+//     from x_i's chunk on, so that the search has no further case for x_i; the
+//     chunk, then the label in it, by comparisons.  Draws within the certified
+//     margin of a CDF boundary are re-drawn by the warp in FP64.  (The chosen
+//     chunk's weights by selects from registers instead of the row measured 11 %
+//     slower.)
 //
 // Persistent blocks of 128 threads take tiles of 16 x 32 sites in a
 // grid-stride loop; a thread updates the 4 sites of its column in rows
@@ -82,7 +79,7 @@ __global__ void ptab_kernel(int T, uint32_t *out)
 // planes: a.xin -> a.xout, or (par_from_t) x0 / x1 holding the states of
 // even / odd sweep indices; budget (optional): sweeps with index >= *budget
 // are skipped (a chain of a batch or of the server).
-template <int LMAX, int NB, bool MASK, bool AQ>
+template <int LMAX, int NB, bool MASK>
 __global__ void __launch_bounds__(kThreads) pca_small_kernel(const SweepArgs a, int tiles_x,
                                                              int ntiles, uint8_t *x0, uint8_t *x1,
                                                              int par_from_t,
@@ -92,13 +89,12 @@ __global__ void __launch_bounds__(kThreads) pca_small_kernel(const SweepArgs a, 
     __shared__ __align__(16) uint32_t U_s[kWarps * kSPT * kBX];
     __shared__ __align__(16) uint32_t codes[kCodeWords];
     __shared__ __align__(16) float pre_s[kThreads * kPrefixStride];
-    __shared__ __align__(16) float aq_s[AQ ? 16 * kAqStride : 4];
+    __shared__ __align__(16) float aq_s[16 * kAqStride];
     const int lane = (int)threadIdx.x, wp = (int)threadIdx.y;
     const int tid = wp * kBX + lane;
     for (int i = tid; i < kPtabWords / 4; i += kThreads)
         reinterpret_cast<uint4 *>(pt)[i] = __ldg(reinterpret_cast<const uint4 *>(a.m.ptab) + i);
-    if (AQ)   // ordered before use by the tile loop's first barrier
-        fill_aq(a.m, aq_s, tid, kThreads);
+    fill_aq(a.m, aq_s, tid, kThreads);   // ordered before use by the tile loop's first barrier
     const uint32_t t = sweep_index(a);
     if (budget && t >= *budget)
         return;   // the whole launch: before any barrier
@@ -176,7 +172,7 @@ __global__ void __launch_bounds__(kThreads) pca_small_kernel(const SweepArgs a, 
             int s = 0;
             bool certain = true;
             if (valid)
-                s = draw_small<LMAX, NB, MASK, AQ>(a.m, pt, nc, g[i], xi, ub, pre, certain, aq_s);
+                s = draw_small<LMAX, NB, MASK>(a.m, pt, nc, g[i], xi, ub, pre, certain, aq_s);
             const bool need = valid && !certain;
             if (__any_sync(0xFFFFFFFFu, need)) {
                 SiteIn<NB> in{};
@@ -214,8 +210,12 @@ __global__ void __launch_bounds__(kThreads) pca_small_kernel(const SweepArgs a, 
 // sites of a row (one Philox call each): neighbour codes from the box (no
 // bounds tests for tiles whose halo lies inside the image), the 4 labels
 // stored as one 32-bit word and the accumulator read-modify-written as one
-// float4, loaded before the draws.  The data term comes from the table
-// (chains: g < L checked).
+// float4, loaded before the draws; the tile's labels are read as words of 4
+// sites.  Bound by instruction issue and shared memory (about 217 instructions
+// and 65 shared-memory wavefronts per 32 sites).  8192^2, L = 16: 572 us per
+// sweep (1.17e11 site-updates/s) with 3 blocks per SM (71 registers) against
+// 637 us for the form that read bytes and joined the atom label by label; 608
+// with 2 blocks per SM, 584 with 4.
 constexpr int kTmThreads = 256;
 constexpr int kTmBoxW = 96, kTmBoxH = 48;   // the box of encode_plane_map
 constexpr int kTmOutW = 64, kTmOutH = kTmBoxH - 2;
@@ -257,26 +257,47 @@ __device__ __forceinline__ void small_tma_tile(const SweepArgs &a, const uint8_t
         if (rowv && gc0 < W)
             philox4x32_10((uint32_t)gc0 >> 2, (uint32_t)(gr + a.row_off), t, ctr3, key0, key1, w0,
                           w1, w2, w3);
+        // the 4 sites' labels, neighbours and observations as words
+        const uint8_t *me = xb + lr * kTmBoxW + lc0;
+        const uint32_t M = *reinterpret_cast<const uint32_t *>(me);
+        const uint32_t Up = *reinterpret_cast<const uint32_t *>(me - kTmBoxW);
+        const uint32_t Dn = *reinterpret_cast<const uint32_t *>(me + kTmBoxW);
+        const uint32_t Gw = *reinterpret_cast<const uint32_t *>(gb + lr * kTmBoxW + lc0);
+        const uint32_t Le = __byte_perm(M, me[-1], 0x2104), Ri = __byte_perm(M, me[4], 0x4321);
+        uint32_t UL = 0u, UR = 0u, DL = 0u, DR = 0u;
+        if constexpr (NB == 8) {
+            UL = __byte_perm(Up, me[-kTmBoxW - 1], 0x2104);
+            UR = __byte_perm(Up, me[-kTmBoxW + 4], 0x4321);
+            DL = __byte_perm(Dn, me[kTmBoxW - 1], 0x2104);
+            DR = __byte_perm(Dn, me[kTmBoxW + 4], 0x4321);
+        }
         uint32_t packed = 0u;
-#pragma unroll 1
+#pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const int lc = lc0 + q, gc = gc0 + q;
+            const int gc = gc0 + q;
             const bool valid = rowv && (INTERIOR || gc < W);
             const uint32_t ub = (q == 0 ? w0 : (q == 1 ? w1 : (q == 2 ? w2 : w3))) >> 8;
-            const uint8_t *me = xb + lr * kTmBoxW + lc;
-            int nc[NB];
-#pragma unroll
-            for (int j = 0; j < NB; ++j) {
+            const auto at = [&](uint32_t w, int j) -> int {   // byte q, or missing
                 const bool inside = INTERIOR || ((unsigned)(gr + dr[j]) < (unsigned)H &&
                                                  (unsigned)(gc + dc[j]) < (unsigned)W);
-                nc[j] = inside ? (int)me[dr[j] * kTmBoxW + dc[j]] : 16;
+                return inside ? (int)((w >> (8 * q)) & 0xFFu) : 16;
+            };
+            int nc[NB];
+            nc[0] = at(Up, 0);
+            nc[1] = at(Dn, 1);
+            nc[2] = at(Le, 2);
+            nc[3] = at(Ri, 3);
+            if constexpr (NB == 8) {
+                nc[4] = at(UL, 4);
+                nc[5] = at(UR, 5);
+                nc[6] = at(DL, 6);
+                nc[7] = at(DR, 7);
             }
-            const int xi = me[0];
-            const int gv = gb[lr * kTmBoxW + lc];
+            const int xi = (int)((M >> (8 * q)) & 0xFFu), gv = (int)((Gw >> (8 * q)) & 0xFFu);
             int sl = 0;
             bool certain = true;
             if (valid)
-                sl = draw_small<LMAX, NB, MASK, true>(a.m, pt, nc, gv, xi, ub, pre, certain, aq);
+                sl = draw_small<LMAX, NB, MASK>(a.m, pt, nc, gv, xi, ub, pre, certain, aq);
             const bool need = valid && !certain;
             if (__any_sync(kFull, need)) {
                 SiteIn<NB> in{};
@@ -317,7 +338,7 @@ __device__ __forceinline__ void small_tma_tile(const SweepArgs &a, const uint8_t
 }
 
 template <int LMAX, int NB, bool MASK>
-__global__ void __launch_bounds__(kTmThreads)
+__global__ void __launch_bounds__(kTmThreads, 3)
     pca_small_tma_kernel(const __grid_constant__ CUtensorMap xmap,
                          const __grid_constant__ CUtensorMap gmap, const SweepArgs a, int tiles_x,
                          int ntiles, int acc_vec, int *err)
@@ -426,7 +447,7 @@ cudaError_t launch_small_tma_t(const CUtensorMap &xmap, const CUtensorMap &gmap,
     return cudaGetLastError();
 }
 
-template <int LMAX, int NB, bool MASK, bool AQ>
+template <int LMAX, int NB, bool MASK>
 cudaError_t launch_small_t(const SweepArgs &a, uint8_t *x0, uint8_t *x1, int par_from_t,
                            const uint32_t *budget, cudaStream_t st)
 {
@@ -439,7 +460,7 @@ cudaError_t launch_small_t(const SweepArgs &a, uint8_t *x0, uint8_t *x1, int par
         return cudaErrorInvalidDevice;
     if (per_sm[dev] == 0) {
         int n = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pca_small_kernel<LMAX, NB, MASK, AQ>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, pca_small_kernel<LMAX, NB, MASK>,
                                                           kThreads, 0);
         if (e != cudaSuccess)
             return e;
@@ -457,20 +478,20 @@ cudaError_t launch_small_t(const SweepArgs &a, uint8_t *x0, uint8_t *x1, int par
         return cudaErrorInvalidValue;
     const long long cap = (long long)per_sm[dev] * sms;
     const int grid = (int)(ntiles < cap ? ntiles : cap);
-    pca_small_kernel<LMAX, NB, MASK, AQ><<<grid, dim3(kBX, kWarps), 0, st>>>(
+    pca_small_kernel<LMAX, NB, MASK><<<grid, dim3(kBX, kWarps), 0, st>>>(
         a, tiles_x, (int)ntiles, x0, x1, par_from_t, budget);
     return cudaGetLastError();
 }
 
-template <int NB, bool AQ>
+template <int NB>
 cudaError_t dispatch_small(const SweepArgs &a, uint8_t *x0, uint8_t *x1, int par_from_t,
                            const uint32_t *budget, cudaStream_t st)
 {
     if (a.m.L <= 8)
-        return a.m.L == 8 ? launch_small_t<8, NB, false, AQ>(a, x0, x1, par_from_t, budget, st)
-                          : launch_small_t<8, NB, true, AQ>(a, x0, x1, par_from_t, budget, st);
-    return a.m.L == 16 ? launch_small_t<16, NB, false, AQ>(a, x0, x1, par_from_t, budget, st)
-                       : launch_small_t<16, NB, true, AQ>(a, x0, x1, par_from_t, budget, st);
+        return a.m.L == 8 ? launch_small_t<8, NB, false>(a, x0, x1, par_from_t, budget, st)
+                          : launch_small_t<8, NB, true>(a, x0, x1, par_from_t, budget, st);
+    return a.m.L == 16 ? launch_small_t<16, NB, false>(a, x0, x1, par_from_t, budget, st)
+                       : launch_small_t<16, NB, true>(a, x0, x1, par_from_t, budget, st);
 }
 
 }  // namespace
@@ -515,7 +536,7 @@ bool pca_small_eligible(const DevModel &m)
 }
 
 cudaError_t launch_pca_small(const SweepArgs &a, cudaStream_t st, uint8_t *x0, uint8_t *x1,
-                             const uint32_t *budget, bool aq)
+                             const uint32_t *budget)
 {
     if (!pca_small_eligible(a.m))
         return cudaErrorInvalidValue;
@@ -525,11 +546,8 @@ cudaError_t launch_pca_small(const SweepArgs &a, cudaStream_t st, uint8_t *x0, u
                                 : reinterpret_cast<uintptr_t>(a.xin);
     if ((a.pitch & 3) != 0 || (align & 3u) != 0)
         return cudaErrorMisalignedAddress;
-    if (aq)
-        return a.m.nbhd == 8 ? dispatch_small<8, true>(a, x0, x1, par, budget, st)
-                             : dispatch_small<4, true>(a, x0, x1, par, budget, st);
-    return a.m.nbhd == 8 ? dispatch_small<8, false>(a, x0, x1, par, budget, st)
-                         : dispatch_small<4, false>(a, x0, x1, par, budget, st);
+    return a.m.nbhd == 8 ? dispatch_small<8>(a, x0, x1, par, budget, st)
+                         : dispatch_small<4>(a, x0, x1, par, budget, st);
 }
 
 }  // namespace pcad

@@ -25,19 +25,26 @@ __device__ __forceinline__ void fill_aq(const DevModel &m, float *aq, int tid, i
     }
 }
 
-// The draw of one site from its neighbour codes nc[] and observation g.
-// Returns the label; `certain` is false when the uniform lies within the
-// certified margin of the chosen label's CDF interval (the caller re-draws
-// it in FP64).  pt: the pair table in shared memory; pre: this thread's row
-// of shared memory (kPrefixStride floats), which receives the weights.  AQ:
-// the data term from the table aq (fill_aq; g < 16), the exponent
-// fl(gam P + fl(alpha q)) in one FFMA per label; otherwise
-// fl(alpha q + fl(gam P)).  Both terms are non-positive, so either form is
-// within 3u |v| of the exact exponent, the per-site margin's bound.
-template <int LMAX, int NB, bool MASK, bool AQ = false>
+// The draw of one site from its neighbour codes nc[] and observation g (below
+// 16).  Returns the label; `certain` is false when the uniform lies within the
+// certified margin of an end of the chosen label's CDF interval, or of 0 or Z
+// (the caller re-draws it in FP64).  pt: the pair table in shared memory; pre:
+// this thread's row of shared memory (kPrefixStride floats), which receives
+// the weights; aq: the data-term table (fill_aq): the exponent is
+// fl(gam P + fl(alpha q)), both terms non-positive, so within 3u |v| of the
+// exact one, the per-site margin's bound.
+//
+// The inertia atom delta is added to w(x_i) in the thread's row and to the
+// chunk prefixes at and above x_i's chunk, so neither the chunk nor the label
+// search looks at x_i again.  Roundings: chunk sums 2, chunk prefix 3, delta's
+// join 1, the label prefix 4 and w(x_i) + delta 1: every C_k within 11u, Z
+// within 6u, t 1u, inside the 22u of summation in the margin.  A chunk chosen
+// off by one through these roundings leaves t within a few u Z of the tested
+// interval's end, inside the margin.
+template <int LMAX, int NB, bool MASK>
 __device__ __forceinline__ int draw_small(const DevModel &m, const uint32_t *pt, const int (&nc)[NB],
                                           int g, int xi, uint32_t ub, float *pre, bool &certain,
-                                          const float *aq = nullptr)
+                                          const float *aq)
 {
     constexpr int NW = LMAX / 4;      // table words used per pair = chunks of 4 labels
     uint32_t P[NW];
@@ -78,86 +85,71 @@ __device__ __forceinline__ int draw_small(const DevModel &m, const uint32_t *pt,
             P[1] = a.y;
         }
     }
-    const float gf = (float)g;
-    const float2 a2 = make_float2(m.alpha, m.alpha), g2 = make_float2(m.gam, m.gam);
+    const float2 g2 = make_float2(m.gam, m.gam);
     const float2 off2 = make_float2(-8388608.0f, -8388608.0f);
-    const float2 gg = make_float2(gf, gf);
-    float w[LMAX];
-    float4 aq4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-#pragma unroll
-    for (int s = 0; s < LMAX; s += 2) {
-        const uint32_t p = P[s >> 2];
-        const float2 pm = make_float2(
-            __uint_as_float(__byte_perm(p, 0x4B000000u, 0x7440u | (uint32_t)(s & 3))),
-            __uint_as_float(__byte_perm(p, 0x4B000000u, 0x7440u | (uint32_t)((s + 1) & 3))));
-        const float2 Pf = __fadd2_rn(pm, off2);
-        float2 v;
-        if constexpr (AQ) {
-            if ((s & 3) == 0)
-                aq4 = *reinterpret_cast<const float4 *>(aq + g * kAqStride + s);
-            v = __ffma2_rn(g2, Pf, (s & 3) == 0 ? make_float2(aq4.x, aq4.y)
-                                                : make_float2(aq4.z, aq4.w));
-        } else {
-            const float2 dg = __fadd2_rn(gg, make_float2(-(float)s, -(float)(s + 1)));
-            v = __ffma2_rn(a2, __fmul2_rn(dg, dg), __fmul2_rn(g2, Pf));
-        }
-        w[s] = ex2_ftz(v.x);
-        w[s + 1] = ex2_ftz(v.y);
-        if (MASK) {
-            w[s] = s < m.L ? w[s] : 0.0f;
-            w[s + 1] = s + 1 < m.L ? w[s + 1] : 0.0f;
-        }
-    }
-    // the weights (to shared memory) and the chunk prefix G over the in-chunk
-    // sums ((w0 + w1) + w2) + w3
-    float G[NW];
+    const float4 *aqr = reinterpret_cast<const float4 *>(aq + g * kAqStride);
+    float S[NW];
 #pragma unroll
     for (int c = 0; c < NW; ++c) {
-        const float p3 = __fadd_rn(__fadd_rn(__fadd_rn(w[4 * c], w[4 * c + 1]), w[4 * c + 2]),
-                                   w[4 * c + 3]);
-        reinterpret_cast<float4 *>(pre)[c] =
-            make_float4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
-        G[c] = c == 0 ? p3 : __fadd_rn(G[c - 1], p3);
+        const uint32_t p = P[c];
+        const float4 q = aqr[c];
+        // bytes to floats: the byte in the mantissa of 2^23, less 2^23
+        const float2 p0 = __fadd2_rn(
+            make_float2(__uint_as_float(__byte_perm(p, 0x4B000000u, 0x7440u)),
+                        __uint_as_float(__byte_perm(p, 0x4B000000u, 0x7441u))), off2);
+        const float2 p1 = __fadd2_rn(
+            make_float2(__uint_as_float(__byte_perm(p, 0x4B000000u, 0x7442u)),
+                        __uint_as_float(__byte_perm(p, 0x4B000000u, 0x7443u))), off2);
+        const float2 v0 = __ffma2_rn(g2, p0, make_float2(q.x, q.y));
+        const float2 v1 = __ffma2_rn(g2, p1, make_float2(q.z, q.w));
+        float2 w0 = make_float2(ex2_ftz(v0.x), ex2_ftz(v0.y));
+        float2 w1 = make_float2(ex2_ftz(v1.x), ex2_ftz(v1.y));
+        if (MASK) {
+            w0.x = 4 * c < m.L ? w0.x : 0.0f;
+            w0.y = 4 * c + 1 < m.L ? w0.y : 0.0f;
+            w1.x = 4 * c + 2 < m.L ? w1.x : 0.0f;
+            w1.y = 4 * c + 3 < m.L ? w1.y : 0.0f;
+        }
+        reinterpret_cast<float4 *>(pre)[c] = make_float4(w0.x, w0.y, w1.x, w1.y);
+        const float2 h = __fadd2_rn(w0, w1);
+        S[c] = __fadd_rn(h.x, h.y);
     }
-    // inertia correction from w(x_i) as evaluated above
-    const float delta = m.em1 != 0.0f ? __fmul_rn(pre[xi], m.em1) : 0.0f;
-    const float G0 = G[NW - 1];
-    const float Z = __fadd_rn(G0, delta);
-    const float t = __fmul_rn((float)ub * (1.0f / 16777216.0f), Z);
-    const float margin = __fmul_rn(site_margin(m, G0, delta), Z);
-    // chunk: the number of chunk ends <= t, compared with t - delta where
-    // delta is added (at and above x_i); Gp: the chunk prefix before it.  Any
-    // rounding here only selects which label's interval is certified below:
-    // a chunk chosen off by one leaves t within a few u Z of that interval's
-    // end, inside the margin, and goes to FP64.
-    const float tmd = __fsub_rn(t, delta);
+    // the inertia atom joins w(x_i) in the row and the prefixes from its chunk on
+    float delta = 0.0f;
+    if (m.em1 != 0.0f) {
+        const float wx = pre[xi];
+        delta = __fmul_rn(wx, m.em1);
+        pre[xi] = __fadd_rn(wx, delta);
+    }
+    float G[NW];
+    G[0] = S[0];
+#pragma unroll
+    for (int c = 1; c < NW; ++c)
+        G[c] = __fadd_rn(G[c - 1], S[c]);
+#pragma unroll
+    for (int c = 0; c < NW; ++c)
+        G[c] = 4 * c + 3 >= xi ? __fadd_rn(G[c], delta) : G[c];   // (always for the last)
+    const float Z = G[NW - 1];
+    const float t = __fmul_rn((float)ub, __fmul_rn(Z, 1.0f / 16777216.0f));
+    // site_margin times Z
+    const float margin =
+        __fmaf_rn(__fmaf_rn(m.kb1, __fsub_rn(m.hb, lg2_ftz(Z)), m.kb0), Z, m.kbr * delta);
     int cs = 0;
     float Gp = 0.0f;
 #pragma unroll
     for (int c = 0; c + 1 < NW; ++c) {
-        const bool below = G[c] <= ((4 * c + 3 >= xi) ? tmd : t);
+        const bool below = G[c] <= t;
         cs += below ? 1 : 0;
         Gp = below ? G[c] : Gp;
     }
-    // the chosen chunk's in-chunk prefix sums, as summed for G; C_k joins
-    // them to Gp or to Gp + delta (two roundings either way)
     const float4 wc = reinterpret_cast<const float4 *>(pre)[cs];
-    const float p1 = __fadd_rn(wc.x, wc.y), p2 = __fadd_rn(p1, wc.z), p3 = __fadd_rn(p2, wc.w);
-    const int base = 4 * cs;
-    const float Gpd = __fadd_rn(Gp, delta);
-    const float C0 = __fadd_rn((base >= xi) ? Gpd : Gp, wc.x);
-    const float C1 = __fadd_rn((base + 1 >= xi) ? Gpd : Gp, p1);
-    const float C2 = __fadd_rn((base + 2 >= xi) ? Gpd : Gp, p2);
-    const float C3 = __fadd_rn((base + 3 >= xi) ? Gpd : Gp, p3);
+    const float C0 = __fadd_rn(Gp, wc.x), C1 = __fadd_rn(C0, wc.y), C2 = __fadd_rn(C1, wc.z),
+                C3 = __fadd_rn(C2, wc.w);
     const bool b0 = C0 <= t, b1 = C1 <= t, b2 = C2 <= t;
-    const int k = (int)b0 + (int)b1 + (int)b2;
     const float hiC = b2 ? C3 : (b1 ? C2 : (b0 ? C1 : C0));
-    const float Cm = (base - 1 >= xi) ? Gpd : Gp;   // before the chunk
-    const float loC = b2 ? C2 : (b1 ? C1 : (b0 ? C0 : Cm));
-    const int s = base + k;
-    certain = (t < hiC) & (s < m.L) & ((s == m.L - 1) | (__fsub_rn(hiC, t) > margin)) &
-              ((s == 0) | (__fsub_rn(t, loC) > margin));
-    return min(s, m.L - 1);
+    const float loC = b2 ? C2 : (b1 ? C1 : (b0 ? C0 : Gp));
+    certain = fminf(__fsub_rn(hiC, t), __fsub_rn(t, loC)) > margin;
+    return 4 * cs + (int)b0 + (int)b1 + (int)b2;
 }
 
 }  // namespace sld

@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kTbThreads)
                         codes_from_box<NB>(xp, lr, lc, gr, gc, a.H, a.W, nc);
                         xi = xp[lr * kBoxW + lc];
                         gv = gs[lr * kBoxW + lc];
-                        s = sld::draw_small<SL, NB, MASK, true>(
+                        s = sld::draw_small<SL, NB, MASK>(
                             a.m, pt, nc, gv, xi, w >> 8, pre_s + tid * sld::kPrefixStride,
                             certain, aq_s);
                     }

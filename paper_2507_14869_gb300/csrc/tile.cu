@@ -134,7 +134,7 @@ struct SmallPol {
                 nc[7] = me[SB + 1];
             }
             xi = me[0];
-            s = draw_small<LMAX, NB, MASK, true>(a.m, pt, nc, g, xi, ub, pre, certain, aq);
+            s = draw_small<LMAX, NB, MASK>(a.m, pt, nc, g, xi, ub, pre, certain, aq);
         }
         if (__any_sync(0xFFFFFFFFu, valid && !certain)) {
             SiteIn<NB> in{};
