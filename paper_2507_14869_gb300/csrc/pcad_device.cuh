@@ -605,15 +605,14 @@ __device__ __forceinline__ int warp_redraw_fp64(const DevModel &m, bool need, co
         for (int j = 0; j < NB; ++j)
             lx[j] = __shfl_sync(kFull, in.xni[j], leader);
         const uint32_t lub = __shfl_sync(kFull, in.ub, leader);
-        double w[kChunk];
         double part = 0.0;
 #pragma unroll
         for (int k = 0; k < kChunk; ++k) {
             if (k >= per)   // uniform
                 break;
             const int sl = lane * per + k;
-            w[k] = sl < m.L ? weight64<NB, NORM>(m, lg, lxi, lx, sl) : 0.0;
-            part = k == 0 ? w[0] : __dadd_rn(part, w[k]);
+            const double w = sl < m.L ? weight64<NB, NORM>(m, lg, lxi, lx, sl) : 0.0;
+            part = k == 0 ? w : __dadd_rn(part, w);
         }
         double incl = part;
 #pragma unroll
@@ -634,15 +633,10 @@ __device__ __forceinline__ int warp_redraw_fp64(const DevModel &m, bool need, co
         const long long ti = __double_as_longlong(t);
         const unsigned hit = __ballot_sync(kFull, ti < __double_as_longlong(incl));
         const int hl = hit ? __ffs((int)hit) - 1 : 31;
-        // the lane's labels, one per lane: their prefix sums in log2 steps
-        double C = 0.0;
-#pragma unroll
-        for (int k = 0; k < kChunk; ++k) {
-            if (k >= per)
-                break;
-            const double v = __shfl_sync(kFull, w[k], hl);
-            C = lane == k ? v : C;
-        }
+        // the lane's labels, one per lane: their prefix sums in log2 steps (the
+        // weights again: kept, they cost the callers' draws spilled registers)
+        const int sk = hl * per + lane;
+        double C = lane < per && sk < m.L ? weight64<NB, NORM>(m, lg, lxi, lx, sk) : 0.0;
 #pragma unroll
         for (int o = 1; o < kChunk; o <<= 1) {
             if (o >= per)
@@ -652,7 +646,7 @@ __device__ __forceinline__ int warp_redraw_fp64(const DevModel &m, bool need, co
                 C = __dadd_rn(C, v);
         }
         C = __dadd_rn(__shfl_sync(kFull, excl, hl), C);
-        const unsigned in = __ballot_sync(kFull, lane < per && hl * per + lane < m.L &&
+        const unsigned in = __ballot_sync(kFull, lane < per && sk < m.L &&
                                                      ti < __double_as_longlong(C));
         const int res = in ? hl * per + __ffs((int)in) - 1 : min(hl * per + per - 1, m.L - 1);
         if (lane == leader)
