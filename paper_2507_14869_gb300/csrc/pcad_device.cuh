@@ -519,6 +519,20 @@ __device__ __forceinline__ float chunk_weights_n(const DevModel &m, const __half
     return S;
 }
 
+// Per-site margin of the Lp draw (gam, alpha <= 0).  With c = csite >= 0, common
+// to all labels, and W = |alpha q| + |gam P| + |kappa R| >= 0 the exponent is
+// c - W; its three rounded coefficients and three roundings give |dv| <=
+// u (W + (c + k) + (c + b + k) + (c + W)) <= u (4 W + 3 c), and E_p W = c +
+// H(p) - log2 Z <= c + log2 L - log2 Z.  So the weights move a CDF value by at
+// most u ln2 (4 (log2 L - log2 Z) + 7 c) + e_ex2; the 22u of summation and the
+// slack as in site_margin.  (The model-wide bound eta re-drew 2.0e-4 of the
+// sites of a 33-label image.)
+__device__ __forceinline__ float site_margin_norm(const DevModel &m, float Z, float c)
+{
+    const float w = __fmaf_rn(2.3333335f, c, 1.3333334f * __fsub_rn(m.hb, lg2_ftz(Z)));
+    return __fmaf_rn(m.kb1, w, m.kb0);
+}
+
 // FP32 inverse-CDF draw with the Lp price (no single-label correction: the
 // price is part of every weight); as draw_fp32.
 template <int NC, int NB, int NORM>
@@ -550,7 +564,8 @@ __device__ __forceinline__ int draw_fp32_norm(const DevModel &m, float *Gcol, in
         G = tt;
         Gcol[c * gstride] = G;
     }
-    return cdf_select(m, m.eta, [&](int cc) { return Gcol[cc * gstride]; }, NC, G, 0.0f, in.xi,
+    const float eta = m.gam <= 0.0f && m.alpha <= 0.0f ? site_margin_norm(m, G, csite) : m.eta;
+    return cdf_select(m, eta, [&](int cc) { return Gcol[cc * gstride]; }, NC, G, 0.0f, in.xi,
                       in.ub, certain, [&](int cs, float (&pp)[kChunk]) {
                           chunk_weights_n<NB, true, true, NORM>(m, xh, T2, gf, xif, csite, cs, pp);
                       });
