@@ -82,6 +82,19 @@ __device__ __forceinline__ unsigned long long globaltimer_ns()
 }
 
 // The error flag, read past L1 (another SM may have set it).
+// Wait until the grids this launch depends on have finished (their writes
+// visible); let the next launch of the stream start once every block of this
+// one has (launch_dependent).
+__device__ __forceinline__ void grid_dep_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+__device__ __forceinline__ void grid_dep_launch()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ int ld_flag(const int *p)
 {
     int v;

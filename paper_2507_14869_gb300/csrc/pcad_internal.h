@@ -4,6 +4,7 @@
 #include <cmath>
 #include <cstddef>
 #include <cstdint>
+#include <utility>
 #include <vector>
 
 #include <cuda.h>
@@ -228,6 +229,24 @@ struct EnergyCoef {
     unsigned long long n_sites;
 };
 EnergyCoef energy_coef(const pcad_model &m, long n_sites);
+
+// Launch a kernel that may start while its predecessor in the stream drains
+// (programmatic dependent launch): it calls grid_dep_wait() before it touches
+// global memory, and grid_dep_launch() to let its own successor start likewise.
+template <class... KA, class... A>
+cudaError_t launch_dependent(void (*kernel)(KA...), dim3 grid, dim3 block, cudaStream_t st, A &&...args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
+}
 
 // Minimum-energy tracking state (device pointers; trace == nullptr: off).
 struct EnergyTrack {

@@ -727,6 +727,8 @@ __global__ void __launch_bounds__(kBinThreads)
                       uint8_t *x1, const uint32_t *budget)
 {
     __shared__ ThrTab<NB> tab;
+    grid_dep_launch();
+    grid_dep_wait();
     const uint32_t t = sweep_index(a);
     if (budget && t >= *budget)
         return;   // the whole launch, before any barrier
@@ -901,9 +903,8 @@ cudaError_t launch_binary_t(const SweepArgs &a, uint8_t *x0, uint8_t *x1, const 
     const long long need = (nstrips + per - 1) / per;
     const int grid = (int)(need < cap ? need : cap);
     const int acc_vec = (a.W % 4 == 0 && (reinterpret_cast<uintptr_t>(a.acc) & 15u) == 0) ? 1 : 0;
-    pca_binary_kernel<NB><<<grid, kBinThreads, 0, st>>>(a, strips_x, (int)nstrips, rows, acc_vec,
-                                                        x0, x1, budget);
-    return cudaGetLastError();
+    return launch_dependent(pca_binary_kernel<NB>, grid, kBinThreads, st, a, strips_x, (int)nstrips,
+                            rows, acc_vec, x0, x1, budget);
 }
 
 }  // namespace
