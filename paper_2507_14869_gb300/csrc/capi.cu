@@ -451,11 +451,9 @@ bool uses_small(const pcad_chain *ch)
 // The small-label kernel's launch form for large images: persistent blocks
 // over TMA-loaded 64 x 46 tiles, the next tile's box in flight during the
 // draw (launch_pca_small_tma), from kSmallTmaMinSites sites.  Measured on
-// GB300 at L = 16 (site-updates/s, TMA tiles / persistent 16 x 32 tiles):
-// 8192^2 1.049e11 / 0.954e11, 4096^2 1.015e11 / 0.953e11, 3072^2
-// 0.997e11 / 0.959e11, 2048^2 0.931e11 / 0.926e11, 1024^2 0.588e11 /
-// 0.691e11; 8 neighbours at 4096^2: L = 5 10.9e10 / 10.4e10, L = 16
-// 9.5e10 / 9.1e10.
+// GB300 at L = 16: 2048^2 39.4 us per sweep against 40.4 with the persistent
+// 16 x 32 tiles; at 1024^2, below the line (and tile-resident with AUTO), 0.59e11
+// against 0.69e11 site-updates/s, its 391 tiles leaving a last wave half empty.
 bool small_tma(const pcad_chain *ch)
 {
     return ch->maps_ready && (long long)ch->H * ch->W >= kSmallTmaMinSites && uses_small(ch);

@@ -390,7 +390,7 @@ constexpr int kSmallMinLabels = 3;
 constexpr int kSmallMaxLabels = 16;
 // From this many sites a small-label chain sweeps on TMA-loaded tiles
 // (launch_pca_small_tma) instead of 16 x 32 staged tiles.
-constexpr long long kSmallTmaMinSites = 1ll << 23;
+constexpr long long kSmallTmaMinSites = 1ll << 21;
 int ptab_words();
 cudaError_t launch_ptab(int T, uint32_t *out, cudaStream_t s);
 bool pca_small_eligible(const DevModel &m);

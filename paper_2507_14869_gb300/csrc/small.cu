@@ -37,7 +37,7 @@
 // pair table (4.6 KB) into shared memory once.  Per tile, the block stages
 // the tile's labels with a one-site halo as table codes (aligned 32-bit
 // loads, one barrier), and each warp computes the uniforms of its own 4 rows
-// (one Philox call per 4 sites, one per lane).  Images of 2^23 sites and
+// (one Philox call per 4 sites, one per lane).  Images of 2^21 sites and
 // more take the same draw on TMA-loaded tiles instead (pca_small_tma_kernel
 // below: no per-thread staging, the next tile's copy in flight).
 #include "async_ptx.cuh"
