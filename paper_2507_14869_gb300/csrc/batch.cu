@@ -515,10 +515,11 @@ pcad_status tc_set_issue(const TcSet &ts, const std::vector<SlotDesc> &desc,
 // launch skips sweeps at or past the chain's budget, so a captured slice
 // stays valid for any start.  One pair table per distinct truncation T.
 constexpr long kSmallBigTiles = 1216;
-// Two-label chains of at least kBinBigSites sites (one wave of the
-// two-label sweep's 16 x 128-site tiles at 8 blocks per SM) run the
-// two-label sweep the same way, each with its own threshold table.
-constexpr long kBinBigSites = 1216L * 16 * 128;
+// Two-label chains of at least kBinBigSites sites (those above the tile-resident
+// limit, mostly) run the two-label sweep the same way, each with its own
+// threshold table: 1413 x 1016 took 15 us per sweep in the batched CUDA-core
+// kernel, 5.5 us on its own launches.
+constexpr long kBinBigSites = 1l << 18;
 
 struct SmallSet {
     std::vector<int> big;          // slots launched one at a time
@@ -642,8 +643,7 @@ pcad_status small_set_retable(const SmallSet &ss, const SlotDesc &d, int i, cuda
 // sites, up to kTilePackSites sites together (more rounds of draws per launch
 // than its exchange costs); planes by the device sweep counter, budget-aware.
 // Segment-draw chains from kWinWaveBlocks blocks per SM on stay with the
-// wavefront (as in capi.cu).  Measured on GB300 against the batched kernels:
-// the design doc's batch and serve rows.
+// wavefront (as in capi.cu, which has the measured times of both).
 constexpr long long kTilePackSites = 1ll << 20;
 
 struct TileSet {
