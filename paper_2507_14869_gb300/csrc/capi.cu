@@ -370,10 +370,10 @@ bool uses_wave(const pcad_chain *ch);
 // AUTO (or SMALL) would run the small-label, wavefront, two-label, general or
 // windowed kernels; energy tracking needs every sweep's state.  Measured on
 // GB300, us per sweep (tile-resident / the kernel it replaces):
-//   small labels, to kTileMaxSites sites: 256^2 L = 9, 8 neighbours 2.2 / 6.7,
-//   L = 5 1.8 / 6.3, L = 5 Gibbs 3.9 / 12.3 (four launches); L = 16 300^2 2.6 /
-//   7.0, 512^2 4.7 / 7.0, 1024^2 13.6 / 15.6 (2048^2, not taken: 40);
-//   two labels: 300^2 1.3 / 3.8, 600^2 2.7 / 4.5, 1000^2 5.4 / 5.8;
+//   small labels, to kTileMaxSites sites: 256^2 L = 9, 8 neighbours 2.1 / 6.7,
+//   L = 5 1.8 / 6.3, L = 5 Gibbs 3.8 / 12.3 (four launches); L = 16 300^2 2.5 /
+//   7.0, 512^2 4.3 / 7.0, 1024^2 11.5 / 15.6 (2048^2, not taken: 39);
+//   two labels: 300^2 1.1 / 3.3, 600^2 2.1 / 3.4, 1000^2 3.7 / 5.4;
 //   segment draw: 256^2 L = 24 3.7 / 6.2, L = 64 3.9 / 8.5; at 512^2 L = 256
 //   the wavefront's 4 x 32-site items pack better (11.7 / 9.5; Gibbs, whose
 //   phases need no exchange here, 13.3 / 14.4; at 720^2 20.4 / 19.6): from 8

@@ -27,6 +27,10 @@
 //     the same label.  k trades draws for exchanges (tile_geometry).
 //   * The uniforms of the next k sweeps are computed while the border words
 //     travel.
+//   * Lazy PCA on larger tiles draws whole words: a thread takes the 4 sites of
+//     a word (words of labels, observations and uniforms; four draws in
+//     flight) instead of one site.  Small tiles keep one site per thread: the
+//     latency of a pass counts there, not its instructions.
 //   * A launch holds one chain, or (batches, the server) several small ones,
 //     each on CTAs of its own.
 //
@@ -50,6 +54,8 @@ using namespace sld;
 
 constexpr int kTlThreads = 512;        // two CTAs per SM
 constexpr int kTlThreads1 = 1024;      // one: at most
+constexpr int kTlThreadsW = 384;       // the same for draws of words (80 registers)
+constexpr int kTlThreadsW1 = 768;
 constexpr int kTlMaxSites = 8192;      // sites per tile
 constexpr int kTlMaxSweeps = 4;        // sweeps per exchange
 constexpr int kTlMaxSmem = 224 * 1024;    // one CTA per SM
@@ -104,6 +110,11 @@ struct SmallPol {
     static constexpr int kTabBytes = kPtabWords * 4 + 16 * kAqStride * 4;
     static constexpr int kRowBytes = kPrefixStride * 4;
     static constexpr double kNsSite = NB == 8 ? 1.6 : 1.4;   // one SM's time per draw (ns)
+    static constexpr bool kWords = true;                     // draw4()
+    // words per tile from which it is used: 512^2 on 216-word tiles 4.3 us per
+    // sweep against 4.6, 300^2 on 150 2.6 against 2.45
+    static constexpr int kWordsMin = 192;
+    static constexpr double kNsSiteWords = NB == 8 ? 1.5 : 1.3;
     uint32_t *pt;
     float *aq, *pre;
 
@@ -148,6 +159,58 @@ struct SmallPol {
         }
         return s;
     }
+    // The new labels of word o (4 sites in a row) of the staged plane X: those
+    // of the bytes of `act`, fill elsewhere.
+    __device__ __forceinline__ uint32_t draw4(const SweepArgs &a, const uint32_t *X, int o, int SW,
+                                              uint32_t G, const uint4 &u, uint32_t act, int, int,
+                                              bool own)
+    {
+        const uint8_t *me = reinterpret_cast<const uint8_t *>(X + o);
+        const int SB = 4 * SW;
+        const uint32_t M = X[o], Up = X[o - SW], Dn = X[o + SW];
+        const uint32_t Le = __byte_perm(M, me[-1], 0x2104), Ri = __byte_perm(M, me[4], 0x4321);
+        uint32_t UL = 0u, UR = 0u, DL = 0u, DR = 0u;
+        if constexpr (NB == 8) {
+            UL = __byte_perm(Up, me[-SB - 1], 0x2104);
+            UR = __byte_perm(Up, me[-SB + 4], 0x4321);
+            DL = __byte_perm(Dn, me[SB - 1], 0x2104);
+            DR = __byte_perm(Dn, me[SB + 4], 0x4321);
+        }
+        uint32_t packed = kFill;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const auto at = [&](uint32_t w) { return (int)((w >> (8 * q)) & 0xFFu); };
+            int nc[NB];
+            nc[0] = at(Up);
+            nc[1] = at(Dn);
+            nc[2] = at(Le);
+            nc[3] = at(Ri);
+            if constexpr (NB == 8) {
+                nc[4] = at(UL);
+                nc[5] = at(UR);
+                nc[6] = at(DL);
+                nc[7] = at(DR);
+            }
+            const bool valid = ((act >> (8 * q)) & 1u) != 0u;
+            const uint32_t ub = q == 0 ? u.x : (q == 1 ? u.y : (q == 2 ? u.z : u.w));
+            int s = 16;
+            bool certain = true;
+            if (valid)
+                s = draw_small<LMAX, NB, MASK>(a.m, pt, nc, at(G), at(M), ub, pre, certain, aq);
+            if (__any_sync(0xFFFFFFFFu, !certain)) {
+                SiteIn<NB> in{};
+                in.g = at(G);
+                in.xi = at(M);
+                in.ub = ub;
+#pragma unroll
+                for (int j = 0; j < NB; ++j)
+                    in.xni[j] = nc[j] != 16 ? nc[j] : kMissingLabelI;
+                s = warp_redraw_fp64<NB>(a.m, !certain, in, s, a.fp64_draws, own);
+            }
+            packed ^= (uint32_t)(s ^ 16) << (8 * q);
+        }
+        return packed;
+    }
     __device__ __forceinline__ void finish(const SweepArgs &) {}
 };
 
@@ -156,7 +219,8 @@ struct SegPol {
     static constexpr uint32_t kFill = 0u;
     static constexpr int kTabBytes = seg::kSegFloats * 4;
     static constexpr int kRowBytes = 0;
-    static constexpr double kNsSite = 4.5;
+    static constexpr double kNsSite = 4.5, kNsSiteWords = 4.5;
+    static constexpr bool kWords = false;
     float *tab;
 
     __device__ __forceinline__ void load(const DevModel &m, uint8_t *t, uint8_t *, int tid, int nt)
@@ -196,6 +260,9 @@ struct BinPol {
     static constexpr int kTabBytes = kEntries * 16;
     static constexpr int kRowBytes = 0;
     static constexpr double kNsSite = 0.5;
+    static constexpr bool kWords = true;
+    static constexpr int kWordsMin = 32;   // 300^2 1.0 us against 1.3, 1000^2 3.7 against 5.6
+    static constexpr double kNsSiteWords = 0.25;
     const uint4 *tab;
     uint32_t nre;
 
@@ -223,6 +290,38 @@ struct BinPol {
         nre += own && ub - e.y < e.z ? 1u : 0u;
         return ub >= e.x ? 1 : 0;
     }
+    __device__ __forceinline__ uint32_t draw4(const SweepArgs &a, const uint32_t *X, int o, int SW,
+                                              uint32_t G, const uint4 &u, uint32_t act, int r, int c,
+                                              bool own)
+    {
+        const uint32_t M = X[o], U = X[o - SW], D = X[o + SW];
+        uint32_t S = U + D + __funnelshift_l(X[o - 1], M, 8) + __funnelshift_r(M, X[o + 1], 8);
+        if constexpr (NB == 8)
+            S += __funnelshift_l(X[o - SW - 1], U, 8) + __funnelshift_r(U, X[o - SW + 1], 8) +
+                 __funnelshift_l(X[o + SW - 1], D, 8) + __funnelshift_r(D, X[o + SW + 1], 8);
+        S += G * (uint32_t)((NB + 1) * (NB + 1));
+        const bool top = r == 0, bot = r + 1 == a.H;
+        if (top || bot || c == 0 || c + 4 >= a.W) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int le = c + q == 0, ri = c + q + 1 == a.W;
+                int nm = top + bot + le + ri;
+                if constexpr (NB == 8)
+                    nm += (top | le) + (top | ri) + (bot | le) + (bot | ri);
+                S += (uint32_t)(nm * (NB + 1)) << (8 * q);
+            }
+        }
+        uint32_t out = 0u;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t ub = q == 0 ? u.x : (q == 1 ? u.y : (q == 2 ? u.z : u.w));
+            const uint4 e = tab[((S >> (8 * q)) & 0xFFu) * 2 + ((M >> (8 * q)) & 1u)];
+            const bool on = ((act >> (8 * q)) & 1u) != 0u;
+            nre += own && on && ub - e.y < e.z ? 1u : 0u;
+            out |= ub >= e.x ? 1u << (8 * q) : 0u;
+        }
+        return out & act;
+    }
     __device__ __forceinline__ void finish(const SweepArgs &a)
     {
         const uint32_t n = __reduce_add_sync(0xFFFFFFFFu, nre);
@@ -238,12 +337,15 @@ template <class P, bool GIBBS>
 size_t tile_smem(const TileGeom &tg, int nt)
 {
     const size_t words = (size_t)(tg.th + 2 * tg.h) * (tg.twq + 2 * tg.hq);
+    const size_t plane = ((words + 3) & ~(size_t)3) * 4;   // what follows is 16-byte aligned
     return (size_t)P::kTabBytes + (size_t)nt * P::kRowBytes + words * 16 * tg.k +
-           words * 4 * (GIBBS ? 1 : 2) + words * 4 + (size_t)tg.th * tg.twq * 16;
+           plane * (GIBBS ? 1 : 2) + plane + (size_t)tg.th * tg.twq * 16;
 }
 
-template <class P, bool GIBBS, int JOBS>
-__global__ void __launch_bounds__(kTlThreads1, 1)
+// WORDS (lazy PCA): a thread draws the 4 sites of a word (large tiles), else
+// one site.
+template <class P, bool GIBBS, int JOBS, bool WORDS>
+__global__ void __launch_bounds__(WORDS ? kTlThreadsW1 : kTlThreads1, 1)
     tile_kernel(const __grid_constant__ TileLaunchT<JOBS> L)
 {
     constexpr bool MULTI = JOBS > 1;
@@ -281,9 +383,10 @@ __global__ void __launch_bounds__(kTlThreads1, 1)
     uint8_t *const row = sm + P::kTabBytes + tid * P::kRowBytes;
     uint32_t *U = reinterpret_cast<uint32_t *>(sm + P::kTabBytes + nt * P::kRowBytes);
     uint32_t *pl0 = U + 4 * words * J.tg.k;
-    uint32_t *pl1 = GIBBS ? pl0 : pl0 + words;
-    uint32_t *gw = pl1 + words;
-    uint32_t *cnt = gw + words;                     // [TH][TW] label sums of this launch
+    const int plane = (words + 3) & ~3;
+    uint32_t *pl1 = GIBBS ? pl0 : pl0 + plane;
+    uint32_t *gw = pl1 + plane;
+    uint32_t *cnt = gw + plane;                     // [TH][TW] label sums of this launch
     P pol;
     pol.load(a.m, sm, row, tid, nt);
     // labels and observation with the halo
@@ -352,6 +455,42 @@ __global__ void __launch_bounds__(kTlThreads1, 1)
             for (int q = 0; q < kCol; ++q) {
                 // sites of colour q of rows [-e, TH + e), columns [-e, TW + e)
                 const int e = (ns - s) * kCol - 1 - q;
+                if constexpr (WORDS) {
+                    // the words that hold them; labels of other sites in
+                    // those words stay undefined
+                    const int eq = (e + 3) >> 2, per = TWq + 2 * eq, n = (TH + 2 * e) * per;
+                    const unsigned int inv = 0xFFFFFFFFu / (unsigned int)per + 1u;
+                    for (int b = 0; b < n; b += nt) {
+                        const int i = b + tid;
+                        const int ir = per == 1 ? i : (int)__umulhi((unsigned int)i, inv);
+                        const int lr = ir - e, lq = i - ir * per - eq, lc = 4 * lq;
+                        const int lo = max(-e - lc, 0), hi = min(min(TW + e, W - c0) - lc, 4);
+                        const bool valid = i < n && (unsigned)(r0 + lr) < (unsigned)H &&
+                                           c0 + lc >= 0 && lo < hi;
+                        const uint32_t act = valid ? (0xFFFFFFFFu << (8 * lo)) &
+                                                         (0xFFFFFFFFu >> (8 * (4 - hi)))
+                                                   : 0u;
+                        const bool own = (unsigned)lr < (unsigned)TH && (unsigned)lq < (unsigned)TWq;
+                        const int o = valid ? (lr + h) * SW + lq + hq : SW + 1;
+                        const uint4 u = reinterpret_cast<const uint4 *>(Us)[o];
+                        const uint32_t v = pol.draw4(a, X, o, SW, gw[o], u, act, r0 + lr, c0 + lc, own);
+                        if (valid) {
+                            Y[o] = v;
+                            if (own && acc_now) {
+                                uint4 *pc = reinterpret_cast<uint4 *>(cnt + lr * TW + lc);
+                                const uint32_t w = v & act;
+                                uint4 n4 = *pc;
+                                n4.x += w & 0xFFu;
+                                n4.y += (w >> 8) & 0xFFu;
+                                n4.z += (w >> 16) & 0xFFu;
+                                n4.w += w >> 24;
+                                *pc = n4;
+                            }
+                        }
+                    }
+                    __syncthreads();
+                    continue;
+                }
                 int nr, per, sr0, sc0;   // rows, sites per row, first row and column
                 if (!GIBBS) {
                     nr = TH + 2 * e;
@@ -474,19 +613,29 @@ __global__ void __launch_bounds__(kTlThreads1, 1)
 
 // Time model of a sweep of a tile (ns; k sweeps per exchange), for the choice
 // of the grid and of k only: kNsPass per pass over the sites (block barrier
-// and the latency of one draw), `site` per site an SM draws, kNsExchange per
-// exchange.
-constexpr double kNsPass = 350.0, kNsExchange = 1300.0;
+// and the latency of one draw; kNsPassWords, of four), `site` per site an SM
+// draws, kNsExchange per exchange.
+constexpr double kNsPass = 350.0, kNsPassWords = 550.0, kNsExchange = 1300.0;
 
-double tile_cost(int th, int tw, int k, int phases, int per_sm, double site)
+double tile_cost(const TileGeom &g, int phases, int per_sm, double site, bool words)
 {
     double ns = kNsExchange;
-    for (int s = 0; s < k; ++s)
+    for (int s = 0; s < g.k; ++s)
         for (int q = 0; q < phases; ++q) {
-            const int e = (k - s) * phases - 1 - q;
-            ns += kNsPass + site * per_sm * (th + 2 * e) * (tw + 2 * e) / phases;
+            const int e = (g.k - s) * phases - 1 - q;
+            const double row = words ? 4.0 * (g.twq + 2 * ((e + 3) / 4)) : 4.0 * g.twq + 2 * e;
+            ns += (words ? kNsPassWords : kNsPass) + site * per_sm * (g.th + 2 * e) * row / phases;
         }
-    return ns / k;
+    return ns / g.k;
+}
+
+// Tiles of which a lazy-PCA sweep draws whole words.
+template <class P, bool GIBBS>
+bool draws_words(const TileGeom &g)
+{
+    if constexpr (P::kWords && !GIBBS)
+        return g.th * g.twq >= P::kWordsMin;
+    return false;
 }
 
 // The tile grid of an image: at most `ctas` tiles of at least h rows and
@@ -524,7 +673,9 @@ bool tile_geometry(int H, int W, int ctas, int per_sm, TileGeom &best)
             // (the scratch of the widest launch: a pack has its widest job's threads)
             if (tile_smem<P, GIBBS>(g, per_sm == 2 ? kTlThreads : kTlThreads1) > most)
                 continue;
-            const double cost = tile_cost(g.th, 4 * g.twq, k, phases, per_sm, P::kNsSite);
+            const bool words = draws_words<P, GIBBS>(g);
+            const double cost =
+                tile_cost(g, phases, per_sm, words ? P::kNsSiteWords : P::kNsSite, words);
             if (best_cost < 0.0 || cost < best_cost) {
                 best_cost = cost;
                 best = g;
@@ -533,8 +684,18 @@ bool tile_geometry(int H, int W, int ctas, int per_sm, TileGeom &best)
     return best_cost >= 0.0;
 }
 
-template <class P, bool GIBBS, int JOBS>
-cudaError_t launch_t(const TileLaunchT<JOBS> &L, int ctas, cudaStream_t st)
+// Threads of a launch that draws words: one per word of the widest pass, as
+// far as they go.
+inline int word_threads(const TileGeom &g)
+{
+    if (g.threads == kTlThreads)   // two CTAs per SM
+        return kTlThreadsW;
+    const int wide = (g.th + 2 * g.h - 2) * (g.twq + 2 * ((g.h + 2) / 4));
+    return std::min(kTlThreadsW1, std::max(256, (wide + 127) / 128 * 128));
+}
+
+template <class P, bool GIBBS, int JOBS, bool WORDS>
+cudaError_t launch_w(const TileLaunchT<JOBS> &L, int ctas, cudaStream_t st)
 {
     static bool attr_set[64] = {};
     int dev = 0;
@@ -543,7 +704,7 @@ cudaError_t launch_t(const TileLaunchT<JOBS> &L, int ctas, cudaStream_t st)
         return e;
     if (dev >= 64)
         return cudaErrorInvalidDevice;
-    auto kern = tile_kernel<P, GIBBS, JOBS>;
+    auto kern = tile_kernel<P, GIBBS, JOBS, WORDS>;
     if (!attr_set[dev]) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kTlMaxSmem);
         if (e != cudaSuccess)
@@ -555,7 +716,7 @@ cudaError_t launch_t(const TileLaunchT<JOBS> &L, int ctas, cudaStream_t st)
     int threads = 0;   // the widest job's; shared memory for every job with them
     size_t smem = 0;
     for (int i = 0; i < L.njobs; ++i)
-        threads = std::max(threads, L.job[i].tg.threads);
+        threads = std::max(threads, WORDS ? word_threads(L.job[i].tg) : L.job[i].tg.threads);
     for (int i = 0; i < L.njobs; ++i)
         smem = std::max(smem, tile_smem<P, GIBBS>(L.job[i].tg, threads));
     if (threads < 1 || smem > (size_t)kTlMaxSmem)
@@ -569,6 +730,21 @@ cudaError_t launch_t(const TileLaunchT<JOBS> &L, int ctas, cudaStream_t st)
     cfg.attrs = at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, L);
+}
+
+// Draws of words where the tiles of every chain of the launch hold enough of
+// them; results do not depend on the choice.
+template <class P, bool GIBBS, int JOBS>
+cudaError_t launch_t(const TileLaunchT<JOBS> &L, int ctas, cudaStream_t st)
+{
+    if constexpr (P::kWords && !GIBBS) {
+        bool words = true;
+        for (int i = 0; i < L.njobs; ++i)
+            words = words && draws_words<P, GIBBS>(L.job[i].tg);
+        if (words)
+            return launch_w<P, GIBBS, JOBS, true>(L, ctas, st);
+    }
+    return launch_w<P, GIBBS, JOBS, false>(L, ctas, st);
 }
 
 // f(policy, GIBBS) for the kind's instance.

@@ -50,7 +50,7 @@ def plain(g, nb, gibbs, sweeps):
     return x[1:-1, 1:-1]
 
 
-def tiled(g, nb, gibbs, sweeps, th, twq, k):
+def tiled(g, nb, gibbs, sweeps, th, twq, k, words=False):
     H, W = g.shape
     Wq = (W + 3) // 4
     ncol = (2 if nb == 4 else 4) if gibbs else 1
@@ -104,7 +104,28 @@ def tiled(g, nb, gibbs, sweeps, th, twq, k):
                         sc0 = -e + ((-e + q) & 1)
                         nr, per = (TH + e - sr0 + 1) >> 1, (TW + e - sc0 + 1) >> 1
                     seen, inv = set(), 0xFFFFFFFF // per + 1
-                    for i in range(nr * per):
+                    if words:   # 4 sites of a word at a time; its other sites undefined
+                        perw, eqw = TWq + 2 * ((e + 3) >> 2), (e + 3) >> 2
+                        for i in range((TH + 2 * e) * perw):
+                            ir = i if perw == 1 else (i * (0xFFFFFFFF // perw + 1)) >> 32
+                            lr, lq = ir - e, i - ir * perw - eqw
+                            lo = max(-e - 4 * lq, 0)
+                            hi = min(TW + e - 4 * lq, W - c0 - 4 * lq, 4)
+                            if not (0 <= r0 + lr < H and c0 + 4 * lq >= 0 and lo < hi):
+                                continue
+                            assert (lr, lq) in U
+                            o = (lr + h) * SW + lq + hq   # words read around it
+                            assert SW <= o and o + SW + 1 <= SR * SW
+                            for b in range(4):
+                                lc, sr, sb = 4 * lq + b, lr + h, 4 * (lq + hq) + b
+                                if not lo <= b < hi:
+                                    Y[sr, sb] = 99 if inside[sr, sb] else 16
+                                    continue
+                                seen.add((lr, lc))
+                                n = [X[sr + a, sb + c] for a, c in offsets(nb)]
+                                assert 0 < sb < 4 * SW - 1 and 99 not in n
+                                Y[sr, sb] = toy(n, X[sr, sb], G[sr, sb], done + s, r0 + lr, c0 + lc)
+                    for i in range(0 if words else nr * per):
                         ir = (i * inv) >> 32
                         ic = i - ir * per
                         assert (ir, ic) == divmod(i, per)
@@ -176,7 +197,10 @@ def test_tiles_equal_the_plain_sweep(H, W, th, twq, nb, gibbs, k):
     h = k * ((2 if nb == 4 else 4) if gibbs else 1)
     th, twq = max(th, h), max(twq, (h + 3) // 4)
     g = np.random.default_rng(H * 100 + W).integers(0, 15, (H, W))
-    assert (tiled(g, nb, gibbs, 4, th, twq, k) == plain(g, nb, gibbs, 4)).all()
+    want = plain(g, nb, gibbs, 4)
+    assert (tiled(g, nb, gibbs, 4, th, twq, k) == want).all()
+    if not gibbs:
+        assert (tiled(g, nb, gibbs, 4, th, twq, k, words=True) == want).all()
 
 
 def test_grids_cover_the_image():
