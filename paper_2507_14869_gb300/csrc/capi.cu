@@ -371,12 +371,12 @@ bool uses_wave(const pcad_chain *ch);
 // windowed kernels; energy tracking needs every sweep's state.  Measured on
 // GB300, us per sweep (tile-resident / the kernel it replaces):
 //   small labels, to kTileMaxSites sites: 256^2 L = 9, 8 neighbours 2.1 / 6.7,
-//   L = 5 1.8 / 6.3, L = 5 Gibbs 3.8 / 12.3 (four launches); L = 16 300^2 2.5 /
-//   7.0, 512^2 4.3 / 7.0, 1024^2 11.5 / 15.6 (2048^2, not taken: 39);
-//   two labels: 300^2 1.1 / 3.3, 600^2 2.1 / 3.4, 1000^2 3.7 / 5.4;
-//   segment draw: 256^2 L = 24 3.7 / 6.2, L = 64 3.9 / 8.5; at 512^2 L = 256
-//   the wavefront's 4 x 32-site items pack better (11.7 / 9.5; Gibbs, whose
-//   phases need no exchange here, 13.3 / 14.4; at 720^2 20.4 / 19.6): from 8
+//   L = 5 1.7 / 6.3, L = 5 Gibbs 3.7 / 12.3 (four launches); L = 16 300^2 2.2 /
+//   7.0, 512^2 4.2 / 7.0, 1024^2 11.4 / 15.6 (2048^2, not taken: 39);
+//   two labels: 300^2 1.0 / 3.3, 600^2 2.1 / 3.4, 1000^2 3.7 / 5.4;
+//   segment draw: 256^2 L = 24 3.3 / 6.2, L = 64 3.5 / 8.5; at 512^2 L = 256
+//   the wavefront's 4 x 32-site items pack better (10.4 / 9.4; Gibbs, whose
+//   phases need no exchange here, 13.0 / 14.4; at 720^2 21.1 / 19.6): from 8
 //   blocks of 4 x 32 sites per multiprocessor on, PCA stays with it, from
 //   kTileSegGibbsSites sites on Gibbs too.
 constexpr long long kTileSegGibbsSites = 300000;

@@ -52,10 +52,12 @@ namespace {
 
 using namespace sld;
 
-constexpr int kTlThreads = 512;        // two CTAs per SM
-constexpr int kTlThreads1 = 1024;      // one: at most
-constexpr int kTlThreadsW = 384;       // the same for draws of words (80 registers)
-constexpr int kTlThreadsW1 = 768;
+// Threads of a CTA, two or (at most) one per SM: 64 registers, or 80 for the
+// draws that need them (words, segments: spilled at 64; but a Gibbs phase of
+// segment draws gains more from one round of 1024 threads: 512^2 13.0 us
+// per sweep against 13.5).
+constexpr int kTlThreads = 512, kTlThreads1 = 1024;
+constexpr int kTlWideThreads = 384, kTlWideThreads1 = 768;
 constexpr int kTlMaxSites = 8192;      // sites per tile
 constexpr int kTlMaxSweeps = 4;        // sweeps per exchange
 constexpr int kTlMaxSmem = 224 * 1024;    // one CTA per SM
@@ -110,6 +112,7 @@ struct SmallPol {
     static constexpr int kTabBytes = kPtabWords * 4 + 16 * kAqStride * 4;
     static constexpr int kRowBytes = kPrefixStride * 4;
     static constexpr double kNsSite = NB == 8 ? 1.6 : 1.4;   // one SM's time per draw (ns)
+    static constexpr bool kWide = false;
     static constexpr bool kWords = true;                     // draw4()
     // words per tile from which it is used: 512^2 on 216-word tiles 4.3 us per
     // sweep against 4.6, 300^2 on 150 2.6 against 2.45
@@ -221,6 +224,7 @@ struct SegPol {
     static constexpr int kRowBytes = 0;
     static constexpr double kNsSite = 4.5, kNsSiteWords = 4.5;
     static constexpr bool kWords = false;
+    static constexpr bool kWide = true;   // 80 registers
     float *tab;
 
     __device__ __forceinline__ void load(const DevModel &m, uint8_t *t, uint8_t *, int tid, int nt)
@@ -260,6 +264,7 @@ struct BinPol {
     static constexpr int kTabBytes = kEntries * 16;
     static constexpr int kRowBytes = 0;
     static constexpr double kNsSite = 0.5;
+    static constexpr bool kWide = false;
     static constexpr bool kWords = true;
     static constexpr int kWordsMin = 32;   // 300^2 1.0 us against 1.3, 1000^2 3.7 against 5.6
     static constexpr double kNsSiteWords = 0.25;
@@ -330,6 +335,13 @@ struct BinPol {
     }
 };
 
+template <class P, bool GIBBS>
+__host__ __device__ constexpr int tile_threads(bool two)
+{
+    return P::kWide && !GIBBS ? (two ? kTlWideThreads : kTlWideThreads1)
+                              : (two ? kTlThreads : kTlThreads1);
+}
+
 // Shared memory of a tile (bytes), in the order of the kernel's pointers:
 // tables, thread scratch, uniforms of k sweeps, label planes, observation,
 // counts.
@@ -345,7 +357,7 @@ size_t tile_smem(const TileGeom &tg, int nt)
 // WORDS (lazy PCA): a thread draws the 4 sites of a word (large tiles), else
 // one site.
 template <class P, bool GIBBS, int JOBS, bool WORDS>
-__global__ void __launch_bounds__(WORDS ? kTlThreadsW1 : kTlThreads1, 1)
+__global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBBS>(false), 1)
     tile_kernel(const __grid_constant__ TileLaunchT<JOBS> L)
 {
     constexpr bool MULTI = JOBS > 1;
@@ -415,13 +427,28 @@ __global__ void __launch_bounds__(WORDS ? kTlThreadsW1 : kTlThreads1, 1)
     const long long limit = wait_limit(a.wait_ns);
     const uint32_t key0 = (uint32_t)(a.seed & 0xFFFFFFFFull), key1 = (uint32_t)(a.seed >> 32);
     const uint32_t ctr3 = ((GIBBS ? kTagGibbs : kTagPCA) << 24) | (a.chain & 0xFFFFFFu);
+    // 2^32 / divisor of a pass's and the uniforms' places, by e (an integer
+    // division per thread and pass costs a fifth of a small tile's pass)
+    constexpr int kMaxE = (GIBBS ? 2 : kTlMaxSweeps) * kCol;
+    __shared__ unsigned int inv_pass[kMaxE], inv_uni[kMaxE];
+    if (tid < kMaxE) {
+        const int e = tid, q = kCol - 1 - e % kCol;
+        const int words_row = TWq + 2 * ((e + 3) >> 2);
+        int per = words_row;
+        if (!WORDS)
+            per = !GIBBS ? TW + 2 * e
+                         : (NB == 4 ? (TW + 2 * e + 1) >> 1 : (TW + 2 * e - ((-e + q) & 1) + 1) >> 1);
+        inv_pass[e] = 0xFFFFFFFFu / (unsigned int)per + 1u;
+        inv_uni[e] = 0xFFFFFFFFu / (unsigned int)words_row + 1u;
+    }
+    __syncthreads();
     // the uniforms of `ns` sweeps from t on, at their staged words: sweep s
     // updates up to (ns - s) kCol - 1 sites beyond the tile
     const auto uniforms = [&](uint32_t t, int ns) {
         for (int s = 0; s < ns; ++s) {
             const int e = (ns - s) * kCol - 1, eq = (e + 3) >> 2;
             const int per = TWq + 2 * eq, n = (TH + 2 * e) * per;
-            const unsigned int inv = 0xFFFFFFFFu / (unsigned int)per + 1u;
+            const unsigned int inv = inv_uni[e];
             for (int i = tid; i < n; i += nt) {
                 // (per == 1: the reciprocal does not fit 32 bits)
                 const int ir = per == 1 ? i : (int)__umulhi((unsigned int)i, inv);
@@ -446,6 +473,16 @@ __global__ void __launch_bounds__(WORDS ? kTlThreadsW1 : kTlThreads1, 1)
                 atomicExch(err, 1);
             return;
         }
+        // A pass computes its first sites' places and reads their inputs before
+        // the barrier that ends the pass before it.
+        bool fresh = true;   // no pass since the last barrier
+        // (a run of one exchange's sweeps, written back in place, still waits
+        // for the neighbours: they have then read their halo of the initial
+        // labels)
+        const bool more = done + ns < nsweeps || (x == 1 && xg_in == xg_out);
+        const bool pub = more && (int)blockIdx.x != a.stall_tile - 1;
+        const uint32_t tag = t0 + (uint32_t)(done + ns);
+        unsigned long long *buf = J.xch + (size_t)(x & 1u) * H * Wq;
         for (int s = 0; s < ns; ++s) {
             const uint32_t t = t0 + (uint32_t)(done + s);
             const bool acc_now = accumulate_after(a, t);
@@ -459,7 +496,7 @@ __global__ void __launch_bounds__(WORDS ? kTlThreadsW1 : kTlThreads1, 1)
                     // the words that hold them; labels of other sites in
                     // those words stay undefined
                     const int eq = (e + 3) >> 2, per = TWq + 2 * eq, n = (TH + 2 * e) * per;
-                    const unsigned int inv = 0xFFFFFFFFu / (unsigned int)per + 1u;
+                    const unsigned int inv = inv_pass[e];
                     for (int b = 0; b < n; b += nt) {
                         const int i = b + tid;
                         const int ir = per == 1 ? i : (int)__umulhi((unsigned int)i, inv);
@@ -473,7 +510,11 @@ __global__ void __launch_bounds__(WORDS ? kTlThreadsW1 : kTlThreads1, 1)
                         const bool own = (unsigned)lr < (unsigned)TH && (unsigned)lq < (unsigned)TWq;
                         const int o = valid ? (lr + h) * SW + lq + hq : SW + 1;
                         const uint4 u = reinterpret_cast<const uint4 *>(Us)[o];
-                        const uint32_t v = pol.draw4(a, X, o, SW, gw[o], u, act, r0 + lr, c0 + lc, own);
+                        const uint32_t G = gw[o];
+                        if (b == 0 && !fresh)
+                            __syncthreads();
+                        fresh = false;
+                        const uint32_t v = pol.draw4(a, X, o, SW, G, u, act, r0 + lr, c0 + lc, own);
                         if (valid) {
                             Y[o] = v;
                             if (own && acc_now) {
@@ -488,7 +529,6 @@ __global__ void __launch_bounds__(WORDS ? kTlThreadsW1 : kTlThreads1, 1)
                             }
                         }
                     }
-                    __syncthreads();
                     continue;
                 }
                 int nr, per, sr0, sc0;   // rows, sites per row, first row and column
@@ -508,7 +548,7 @@ __global__ void __launch_bounds__(WORDS ? kTlThreadsW1 : kTlThreads1, 1)
                     nr = (TH + e - sr0 + 1) >> 1;
                     per = (TW + e - sc0 + 1) >> 1;
                 }
-                const unsigned int inv = 0xFFFFFFFFu / (unsigned int)per + 1u;   // per >= 2
+                const unsigned int inv = inv_pass[e];   // per >= 2
                 for (int b = 0; b < nr * per; b += nt) {
                     const int i = b + tid;
                     const int ir = (int)__umulhi((unsigned int)i, inv), ic = i - ir * per;
@@ -523,6 +563,9 @@ __global__ void __launch_bounds__(WORDS ? kTlThreadsW1 : kTlThreads1, 1)
                     const int o = (lr + h) * SB + lc + hb;
                     const int g = valid ? (int)reinterpret_cast<const uint8_t *>(gw)[o] : 0;
                     const uint32_t ub = valid ? Us[o] : 0u;
+                    if (b == 0 && !fresh)
+                        __syncthreads();
+                    fresh = false;
                     const int v = pol.draw(a, reinterpret_cast<const uint8_t *>(X) + o, SB, g, ub,
                                            r0 + lr, c0 + lc, valid, own);
                     if (valid) {
@@ -531,20 +574,14 @@ __global__ void __launch_bounds__(WORDS ? kTlThreadsW1 : kTlThreads1, 1)
                             cnt[lr * TW + lc] += (uint32_t)v;
                     }
                 }
-                __syncthreads();
             }
             X = Y;
         }
+        __syncthreads();
         done += ns;
-        // (a run of one exchange's sweeps, written back in place, still waits
-        // for the neighbours: they have then read their halo of the initial
-        // labels)
-        if (done == nsweeps && !(x == 1 && xg_in == xg_out))
+        if (!more)
             break;
-        // publish the border words
-        const uint32_t tag = t0 + (uint32_t)done;
-        unsigned long long *buf = J.xch + (size_t)(x & 1u) * H * Wq;
-        if ((int)blockIdx.x != a.stall_tile - 1)
+        if (pub)   // publish the border words
             for (int i = tid; i < TH * TWq; i += nt) {
                 const int lr = i / TWq, lq = i - lr * TWq;
                 const bool border = lr < h || lr >= TH - h || lq < hq || lq >= TWq - hq;
@@ -614,12 +651,12 @@ __global__ void __launch_bounds__(WORDS ? kTlThreadsW1 : kTlThreads1, 1)
 // Time model of a sweep of a tile (ns; k sweeps per exchange), for the choice
 // of the grid and of k only: kNsPass per pass over the sites (block barrier
 // and the latency of one draw; kNsPassWords, of four), `site` per site an SM
-// draws, kNsExchange per exchange.
-constexpr double kNsPass = 350.0, kNsPassWords = 550.0, kNsExchange = 1300.0;
+// draws, kNsExchange per exchange and kNsHaloWord per word of its halo.
+constexpr double kNsPass = 350.0, kNsPassWords = 550.0, kNsExchange = 1300.0, kNsHaloWord = 0.5;
 
 double tile_cost(const TileGeom &g, int phases, int per_sm, double site, bool words)
 {
-    double ns = kNsExchange;
+    double ns = kNsExchange + kNsHaloWord * per_sm * (2 * g.h * (g.twq + 2 * g.hq) + 2 * g.hq * g.th);
     for (int s = 0; s < g.k; ++s)
         for (int q = 0; q < phases; ++q) {
             const int e = (g.k - s) * phases - 1 - q;
@@ -651,6 +688,7 @@ bool tile_geometry(int H, int W, int ctas, int per_sm, TileGeom &best)
         for (int nx = 1; nx <= ctas && nx <= Wq; ++nx) {
             TileGeom g{};
             g.k = k;
+            g.two = per_sm == 2;
             g.h = k * phases;
             g.hq = (g.h + 3) / 4;
             g.twq = (Wq + nx - 1) / nx;
@@ -667,11 +705,11 @@ bool tile_geometry(int H, int W, int ctas, int per_sm, TileGeom &best)
             // one CTA per SM: a thread per site of the widest pass, if they are
             // few (idle warps still take every barrier)
             const long wide = (long)(g.th + 2 * g.h - 2) * (4 * g.twq + 2 * g.h - 2) / phases;
-            g.threads = per_sm == 2 ? kTlThreads
-                                    : (int)std::min<long>(kTlThreads1,
+            g.threads = per_sm == 2 ? tile_threads<P, GIBBS>(true)
+                                    : (int)std::min<long>(tile_threads<P, GIBBS>(false),
                                                           std::max<long>(256, (wide + 127) / 128 * 128));
             // (the scratch of the widest launch: a pack has its widest job's threads)
-            if (tile_smem<P, GIBBS>(g, per_sm == 2 ? kTlThreads : kTlThreads1) > most)
+            if (tile_smem<P, GIBBS>(g, tile_threads<P, GIBBS>(per_sm == 2)) > most)
                 continue;
             const bool words = draws_words<P, GIBBS>(g);
             const double cost =
@@ -688,10 +726,10 @@ bool tile_geometry(int H, int W, int ctas, int per_sm, TileGeom &best)
 // far as they go.
 inline int word_threads(const TileGeom &g)
 {
-    if (g.threads == kTlThreads)   // two CTAs per SM
-        return kTlThreadsW;
+    if (g.two)
+        return kTlWideThreads;
     const int wide = (g.th + 2 * g.h - 2) * (g.twq + 2 * ((g.h + 2) / 4));
-    return std::min(kTlThreadsW1, std::max(256, (wide + 127) / 128 * 128));
+    return std::min(kTlWideThreads1, std::max(256, (wide + 127) / 128 * 128));
 }
 
 template <class P, bool GIBBS, int JOBS, bool WORDS>

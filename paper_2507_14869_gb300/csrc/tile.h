@@ -26,6 +26,7 @@ struct TileGeom {
     int k;                // sweeps per exchange
     int h, hq;            // halo: rows (and columns), words
     int threads;          // per CTA
+    bool two;             // two CTAs per SM
 };
 
 struct TilePlan {
