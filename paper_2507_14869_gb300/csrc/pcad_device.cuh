@@ -225,6 +225,17 @@ __device__ __forceinline__ float2 prior_pair(const __half2 (&xr)[NB], __half2 k2
     return __half22float2(P2);
 }
 
+// The same for T = 1 (the Potts prior): the neighbours that differ, counted.
+template <int NB>
+__device__ __forceinline__ float2 prior_pair_eq(const __half2 (&xr)[NB], __half2 k2)
+{
+    __half2 P2 = __hsub2(__float2half2_rn((float)NB), __heq2(xr[0], k2));
+#pragma unroll
+    for (int j = 1; j < NB; ++j)
+        P2 = __hsub2(P2, __heq2(xr[j], k2));
+    return __half22float2(P2);
+}
+
 // Weights of labels [8c, 8c + 8); returns their sequential sum and, when
 // PREFIX, the inclusive running sums p[k].  Labels >= L weigh 0 when MASK.
 template <int NB, bool MASK, bool PREFIX>
@@ -487,15 +498,9 @@ __device__ __forceinline__ int draw_fp32(const DevModel &m, float *Gcol, int gst
 // ------------------------------------------------- Lp inertia price (p = 1, 2)
 // Exponent v' = alpha (g - s)^2 + gam P(s) + kappa R(s) + c with R = |s - x_i|^p
 // (exact integers) and the per-site shift c = |kappa| |g - x_i|^p, evaluated
-// as one FFMA chain: kappa R + c, + gam P, + alpha Q.
-
-__device__ __forceinline__ float label_wn(const DevModel &m, float P, float dg, float R, float c)
-{
-    const float q = __fmul_rn(dg, dg);
-    const float t1 = __fmaf_rn(m.kappa, R, c);
-    const float t2 = __fmaf_rn(m.gam, P, t1);
-    return ex2_ftz(__fmaf_rn(m.alpha, q, t2));
-}
+// as one FFMA chain: kappa R + c, + gam P, + alpha Q, two labels per packed FP32x2
+// instruction.  (301 x 453, 33 labels, 8 neighbours, L1: 10.3 -> 9.8 us per
+// sweep, with the equality counts of prior_pair_eq.)
 
 // Weights of labels [8c, 8c + 8) with the Lp price; as chunk_weights.
 template <int NB, bool MASK, bool PREFIX, int NORM>
@@ -511,15 +516,20 @@ __device__ __forceinline__ float chunk_weights_n(const DevModel &m, const __half
         xr[j] = __hsub2(xh[j], sb2);
     const float dgb = gf - sbf;
     const float dxb = sbf - xif;
+    const float2 dg2 = make_float2(dgb, dgb), dx2 = make_float2(dxb, dxb);
+    const float2 ka2 = make_float2(m.kappa, m.kappa), ga2 = make_float2(m.gam, m.gam),
+                 al2 = make_float2(m.alpha, m.alpha), cs2 = make_float2(csite, csite);
     float S = 0.0f;
 #pragma unroll
     for (int kk = 0; kk < kChunk; kk += 2) {
-        const float2 P = prior_pair<NB>(xr, __floats2half2_rn((float)kk, (float)(kk + 1)), T2);
-        const float d0 = dxb + (float)kk, d1 = dxb + (float)(kk + 1);
-        const float R0 = NORM == 1 ? fabsf(d0) : __fmul_rn(d0, d0);
-        const float R1 = NORM == 1 ? fabsf(d1) : __fmul_rn(d1, d1);
-        float e0 = label_wn(m, P.x, dgb - (float)kk, R0, csite);
-        float e1 = label_wn(m, P.y, dgb - (float)(kk + 1), R1, csite);
+        const __half2 k2 = __floats2half2_rn((float)kk, (float)(kk + 1));
+        const float2 P = m.T == 1 ? prior_pair_eq<NB>(xr, k2) : prior_pair<NB>(xr, k2, T2);
+        const float2 d = __fadd2_rn(dx2, make_float2((float)kk, (float)(kk + 1)));
+        const float2 R = NORM == 1 ? make_float2(fabsf(d.x), fabsf(d.y)) : __fmul2_rn(d, d);
+        const float2 dg = __fadd2_rn(dg2, make_float2(-(float)kk, -(float)(kk + 1)));
+        const float2 v = __ffma2_rn(al2, __fmul2_rn(dg, dg),
+                                    __ffma2_rn(ga2, P, __ffma2_rn(ka2, R, cs2)));
+        float e0 = ex2_ftz(v.x), e1 = ex2_ftz(v.y);
         if (MASK) {
             if (c * kChunk + kk >= m.L) e0 = 0.0f;
             if (c * kChunk + kk + 1 >= m.L) e1 = 0.0f;
