@@ -342,6 +342,14 @@ __host__ __device__ constexpr int tile_threads(bool two)
                               : (two ? kTlThreads : kTlThreads1);
 }
 
+// Words of a staged plane: what follows is 16-byte aligned, and a zero word lies
+// before and behind each (draws of whole words read the words around theirs; a
+// byte-wise sum must not carry from an undefined one).
+__host__ __device__ constexpr int tile_plane(int words)
+{
+    return (words + 4) & ~3;
+}
+
 // Shared memory of a tile (bytes), in the order of the kernel's pointers:
 // tables, thread scratch, uniforms of k sweeps, label planes, observation,
 // counts.
@@ -349,9 +357,9 @@ template <class P, bool GIBBS>
 size_t tile_smem(const TileGeom &tg, int nt)
 {
     const size_t words = (size_t)(tg.th + 2 * tg.h) * (tg.twq + 2 * tg.hq);
-    const size_t plane = ((words + 3) & ~(size_t)3) * 4;   // what follows is 16-byte aligned
+    const size_t plane = tile_plane((int)words) * 4;
     return (size_t)P::kTabBytes + (size_t)nt * P::kRowBytes + words * 16 * tg.k +
-           plane * (GIBBS ? 1 : 2) + plane + (size_t)tg.th * tg.twq * 16;
+           16 + plane * (GIBBS ? 1 : 2) + plane + (size_t)tg.th * tg.twq * 16;
 }
 
 // WORDS (lazy PCA): a thread draws the 4 sites of a word (large tiles), else
@@ -394,8 +402,8 @@ __global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBB
 
     uint8_t *const row = sm + P::kTabBytes + tid * P::kRowBytes;
     uint32_t *U = reinterpret_cast<uint32_t *>(sm + P::kTabBytes + nt * P::kRowBytes);
-    uint32_t *pl0 = U + 4 * words * J.tg.k;
-    const int plane = (words + 3) & ~3;
+    uint32_t *pl0 = U + 4 * words * J.tg.k + 4;
+    const int plane = tile_plane(words);
     uint32_t *pl1 = GIBBS ? pl0 : pl0 + plane;
     uint32_t *gw = pl1 + plane;
     uint32_t *cnt = gw + plane;                     // [TH][TW] label sums of this launch
@@ -423,6 +431,11 @@ __global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBB
     }
     for (int i = tid; i < TH * TW; i += nt)
         cnt[i] = 0u;
+    if (tid < plane - words) {
+        pl0[words + tid] = 0u;
+        pl1[words + tid] = 0u;
+        pl0[-1] = 0u;
+    }
 
     const long long limit = wait_limit(a.wait_ns);
     const uint32_t key0 = (uint32_t)(a.seed & 0xFFFFFFFFull), key1 = (uint32_t)(a.seed >> 32);
