@@ -598,8 +598,18 @@ pcad_status issue_sweeps(pcad_chain *ch, int off0, int n, int &cur, cudaStream_t
                 CUDA_TRY(launch_pca_binary(a, st));
             else if (uses_win(ch))
                 CUDA_TRY(launch_pca_win(a, ch->ftab, st));
-            else
-                CUDA_TRY(launch_pca_sweep(a, st));
+            else {
+                // the launch reduces the energy of the state it reads, so only
+                // the last state of the run needs one of its own
+                EnergyJob ej{};
+                if (ch->track.trace && k > done)
+                    ej = EnergyJob{ch->ecoef, ch->track, ch->esums};
+                CUDA_TRY(launch_pca_sweep(a, st, ej));
+                if (ch->track.trace && k + 1 < n) {
+                    cur ^= 1;
+                    continue;
+                }
+            }
             cur ^= 1;
             if (ch->track.trace)
                 CUDA_TRY(launch_energy(ch->x[cur], ch->g, ch->H, ch->W, ch->pitch, ch->ecoef,

@@ -14,7 +14,7 @@
 // The sums are reduced exactly in integers; H is combined from them in FP64 by
 // one thread.  Pairs are counted once: right and down neighbours
 // (and the two lower diagonals for the 8-neighbourhood), free boundary.
-#include "pcad_internal.h"
+#include "energy_dev.cuh"
 
 namespace pcad {
 
@@ -48,17 +48,9 @@ __global__ void __launch_bounds__(kEThreads)
     const long n = (long)H * Wq;
     const uint32_t T4 = (uint32_t)min(k.T, 255) * 0x01010101u;
     uint8_t *const spare = tr.trace ? (*tr.which ? tr.xb[0] : tr.xb[1]) : nullptr;
-    // the last block's inputs, early: nothing writes them before it does
-    unsigned int trn = 0;
-    int trw = 0;
-    double best = 0.0;
-    unsigned long long done = 0;
-    if (tr.trace && threadIdx.x == 0) {
-        trn = *tr.n;
-        trw = *tr.which;
-        best = *tr.best;
-        done = (unsigned long long)(*tdev + sweep_off) + 1ull;
-    }
+    EnergyLast last{};   // early: nothing writes it before the last block does
+    if (tr.trace && threadIdx.x == 0)
+        last = energy_last(tr, tdev, sweep_off);
     // 64 bits: a thread may see any share of a large image
     unsigned long long pair = 0, data = 0;
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -115,33 +107,7 @@ __global__ void __launch_bounds__(kEThreads)
     __threadfence();
     if (atomicAdd(&sums[2], 1ull) != (unsigned long long)gridDim.x - 1ull)
         return;
-    // the last block: every block's sums are in (and every block has read
-    // tr.which); zero them for the next reduction
-    __threadfence();
-    const double fp = (double)atomicExch(&sums[0], 0ull), fd = (double)atomicExch(&sums[1], 0ull);
-    sums[2] = 0;
-    double e = __dmul_rn(k.pair_c, fp);
-    if (k.gauss)
-        e = __dadd_rn(e, __ddiv_rn(fd, k.two_s2));
-    else if (!k.none)
-        e = __dadd_rn(e, __dadd_rn(__dmul_rn(k.lf_same, __dsub_rn((double)k.n_sites, fd)),
-                                   __dmul_rn(k.lf_diff, fd)));
-    if (out) {   // H and the two sums (exact in FP64: both are < 2^53)
-        out[0] = e;
-        out[1] = fp;
-        out[2] = fd;
-    }
-    if (tr.trace) {
-        if (trn < (unsigned int)tr.cap) {
-            tr.trace[trn] = e;
-            *tr.n = trn + 1;
-        }
-        if (e < best) {
-            *tr.best = e;
-            *tr.best_sweep = done;
-            *tr.which = trw ^ 1;
-        }
-    }
+    energy_finish(k, sums, out, tr, last);
 }
 
 int reduce_grid(long n)

@@ -94,8 +94,6 @@ cudaError_t launch_advance(uint32_t *counter, uint32_t n, cudaStream_t s);
 // Number of 8-label chunks rounded up to an instantiated size.
 int chunk_class(int L);
 
-// Launch one PCA sweep (xin -> xout) on `stream`.
-cudaError_t launch_pca_sweep(const SweepArgs &a, cudaStream_t stream);
 
 // Launch Gibbs colour phase q (0..ncolours-1) in place on a.xin.  When
 // a.accumulate is set, the phase must be the last of the sweep.
@@ -258,6 +256,18 @@ struct EnergyTrack {
     int *which;                     // the plane of xb that holds the lowest-energy state
     uint8_t *xb[2];                 // it and a spare (same pitch as x)
 };
+
+// The energy of the state a sweep reads, reduced by the sweep's launch (tr.trace
+// set): sums as launch_energy's; recorded as the energy after the sweep before.
+struct EnergyJob {
+    EnergyCoef k;
+    EnergyTrack tr;
+    unsigned long long *sums;
+};
+
+// Launch one PCA sweep (xin -> xout) on `stream`; ej: track a.xin's energy too.
+cudaError_t launch_pca_sweep(const SweepArgs &a, cudaStream_t stream,
+                             const EnergyJob &ej = EnergyJob{});
 
 // sums (3 x u64, zero on entry, zero again on return) <- integer sums of
 // labelling x; out[0..2] <- H, pair sum, data sum (when out != nullptr); with

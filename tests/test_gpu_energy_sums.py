@@ -12,7 +12,10 @@ pytestmark = pytest.mark.gpu
 
 MODELS = [Model(L=16, pair=1, pair_coef=0.6, pair_T=3, sigma=1.2, inertia=1.0),
           Model(L=16, nbhd=8, pair=1, pair_coef=0.15, pair_T=30, sigma=1.2, inertia=1.0),
-          Model(L=2, nbhd=8, pair=0, pair_coef=0.5, noise=1, flip_p=0.2, inertia=0.5)]
+          Model(L=2, nbhd=8, pair=0, pair_coef=0.5, noise=1, flip_p=0.2, inertia=0.5),
+          # sweeps that reduce the energy of the state they read
+          Model(L=16, nbhd=8, pair=0, pair_coef=0.5, sigma=1.2, inertia=1.0, inertia_norm=1),
+          Model(L=20, pair=1, pair_coef=0.2, pair_T=9, sigma=2.0, inertia=1.0, inertia_norm=2)]
 
 
 @pytest.mark.parametrize("H,W", [(1, 1), (1, 5), (5, 1), (3, 4), (4, 7), (33, 66), (1100, 1031)])
@@ -27,6 +30,12 @@ def test_sums_and_minimum(H, W, k):
         trace, x = ch.energies(), ch.sample()
         xmin, emin, smin = ch.min_state()
         e, pair, data = ch.energy()
+        ch.reset()
+        steps = []
+        for _ in range(12):      # one sweep per call: each state's energy on its own
+            ch.run(1)
+            steps.append(ch.energy()[0])
+    assert np.array_equal(trace, steps)
     assert (pair, data) == oen.energy_terms(m, g, x)
     assert trace[-1] == e
     assert smin == int(np.argmin(trace)) + 1 and emin == trace.min()
