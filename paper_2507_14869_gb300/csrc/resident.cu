@@ -31,23 +31,18 @@
 // (g_i, nm) in the table's index.  One Philox call gives the quad's four
 // uniforms of the sweep.  Posterior-mean counts accumulate in packed 16-bit
 // registers and reach global memory at the end of the launch.
-#include "pcad_internal.h"
+#include "binary_draw.cuh"
 
 namespace pcad {
 
 namespace {
 
+using namespace bind;
+
 constexpr int kResThreads = 1024;
 constexpr int kResMaxQuadsPerThread = 4;
 constexpr int kResMaxSmem = 200 * 1024;
 
-// Table entries: configuration index e = 2 (b + n1) + x_i with the base
-// b = (g (NB + 1) + nm) (NB + 1).
-template <int NB>
-constexpr int btab_entries()
-{
-    return 4 * (NB + 1) * (NB + 1);
-}
 constexpr int kBtabStride = 4 * 9 * 9;   // entries per table in a batch's table array
 
 __device__ unsigned long long g_btab_redraws;   // re-draw counter of the bisection (unused)
@@ -116,8 +111,6 @@ inline int res_plane_bytes(int H, int W)
     return (H + 2) * (((W + 3) & ~3) + 8);
 }
 
-constexpr int kThrBytes = 6656;   // a ThrTab of either neighbourhood
-
 // Shared memory of a launch: table, one (Gibbs) or two (PCA) planes, base bytes.
 inline int res_smem_bytes(int nb, bool gibbs, int H, int W)
 {
@@ -137,72 +130,6 @@ __device__ __forceinline__ uint32_t quad_counts(const uint32_t *X, int o, int pw
         S += ((U << 8) | (X[o - pw - 1] >> 24)) + ((U >> 8) | (X[o - pw + 1] << 24)) +
              ((D << 8) | (X[o + pw - 1] >> 24)) + ((D >> 8) | (X[o + pw + 1] << 24));
     return S;
-}
-
-// Thresholds of every configuration in shared memory: thr[] (one 32-bit read
-// and a compare per draw), the full entries for the rare draws near a
-// threshold, and the largest uncertain band.
-template <int NB>
-struct ThrTab {
-    int thr[NB == 4 ? btab_entries<4>() : 2 * 168];   // NB 4: [2 b + x]; 8: [168 x + b]
-    uint4 full[btab_entries<NB>()];
-    uint32_t band;
-};
-
-static_assert(sizeof(ThrTab<4>) <= kThrBytes && sizeof(ThrTab<8>) <= kThrBytes, "table space");
-
-template <int NB>
-__device__ __forceinline__ int thr_index(int e)
-{
-    return NB == 4 ? e : (e >> 1) + 168 * (e & 1);
-}
-
-// (ends with a block barrier)
-template <int NB>
-__device__ __forceinline__ void load_thresholds(ThrTab<NB> &tab, const uint4 *src, int tid, int n)
-{
-    if (tid == 0)
-        tab.band = 0u;
-    __syncthreads();
-    for (int i = tid; i < btab_entries<NB>(); i += n) {
-        const uint4 e = src[i];
-        tab.full[i] = e;
-        tab.thr[thr_index<NB>(i)] = (int)e.x;
-        atomicMax(&tab.band, e.z);
-    }
-    __syncthreads();
-}
-
-// New labels of one quad from its Philox words u: S holds base + count per
-// byte, M the current labels (0 or 1 per byte).  Returns the labels as bytes;
-// adds the draws of the bytes of `act` that the FP64 re-draw decides to nre:
-// those with u in [A, B), a band around the threshold, looked at only when
-// some draw of the quad lies within the largest band of its threshold.
-template <int NB>
-__device__ __forceinline__ uint32_t quad_draw(const ThrTab<NB> &tab, uint32_t S, uint32_t M,
-                                              const uint32_t (&u)[4], uint32_t act, uint32_t &nre)
-{
-    const uint32_t K = NB == 4 ? 2u * S + M : S;   // NB 4: at most 99 per byte, no carry
-    uint32_t out = 0u;
-    int near = 0x7FFFFFFF;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        int i = (int)((K >> (8 * j)) & 0xFFu);
-        if (NB == 8)
-            i += 168 * (int)((M >> (8 * j)) & 1u);
-        const int d = (int)(u[j] >> 8) - tab.thr[i];
-        out |= d >= 0 ? 1u << (8 * j) : 0u;
-        near = min(near, abs(d));
-    }
-    if ((uint32_t)near <= tab.band) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if ((act >> (8 * j)) & 1u) {
-                const uint4 e = tab.full[((S >> (8 * j)) & 0xFFu) * 2u + ((M >> (8 * j)) & 1u)];
-                nre += ((u[j] >> 8) - e.y) < e.z ? 1u : 0u;
-            }
-    }
-    return out;
 }
 
 __device__ __forceinline__ void quad_words(const SweepArgs &a, uint32_t tag, uint32_t t, int r,
@@ -381,8 +308,8 @@ __global__ void __launch_bounds__(kResThreads, 1)
 
 // ------------------------------------------------------- one chain, 8 CTAs
 // One chain alone leaves 151 SMs idle, and its sweep is bound by the issue
-// slots of the one it has: 0.87 us for 64 x 64 (Gibbs 1.31), against 0.52
-// (0.90) here, bound by the latency of a pass and of the exchange.  A cluster of 8 CTAs takes the
+// slots of the one it has: 0.87 us for 64 x 64 (Gibbs 1.31), against 0.50
+// (0.85) here, bound by the latency of a pass and of the exchange.  A cluster of 8 CTAs takes the
 // chain in bands of rows with a halo of h rows: h sweeps (Gibbs: h colour
 // phases) run on shrinking extensions of the band, then each CTA pushes its
 // border rows into its neighbours' receive buffers through distributed shared
@@ -392,13 +319,13 @@ __global__ void __launch_bounds__(kResThreads, 1)
 // same labels.  A thread keeps its quads, their base bytes, their counts and
 // the next sweep's uniforms in registers.
 constexpr int kClCtas = 8;
-constexpr int kClHalo = 4;                // rows: 4 PCA sweeps, 2 (1) Gibbs sweeps
+constexpr int kClHalo = 8;                // rows, at most: 8 PCA sweeps, 4 (2) Gibbs sweeps
 constexpr int kClThreads = 768;           // at most
 
-inline int cl_smem_bytes(bool gibbs, int band, int W)
+inline int cl_smem_bytes(bool gibbs, int band, int h, int W)
 {
     const int Wq4 = (W + 3) & ~3;
-    return kThrBytes + (gibbs ? 1 : 2) * (band + 2 * kClHalo) * (Wq4 + 8) + 4 * kClHalo * Wq4;
+    return kThrBytes + (gibbs ? 1 : 2) * (band + 2 * h) * (Wq4 + 8) + 4 * h * Wq4;
 }
 
 __device__ __forceinline__ uint32_t cluster_rank()
@@ -424,15 +351,15 @@ __device__ __forceinline__ void st_cluster(const uint32_t *local, uint32_t rank,
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
-template <int NB, bool GIBBS, int QPT>
+template <int NB, bool GIBBS, int QPT, int h>
 __global__ void __cluster_dims__(kClCtas, 1, 1) __launch_bounds__(kClThreads, 1)
     resident_cluster_kernel(const SweepArgs a, const uint8_t *xg_in, uint8_t *xg_out, int nsweeps,
                             int band)
 {
     extern __shared__ __align__(16) uint8_t sm[];
-    constexpr int h = kClHalo;
     constexpr int kCol = !GIBBS ? 1 : (NB == 4 ? 2 : 4);
     constexpr int K = h / kCol;                    // sweeps per exchange
+    static_assert(K >= 1, "halo");
     const int tid = (int)threadIdx.x, nt = (int)blockDim.x;
     const int rank = (int)cluster_rank();
     const int H = a.H, W = a.W;
@@ -655,27 +582,33 @@ cudaError_t launch_res_t(const SweepArgs &a, const uint8_t *x_in, uint8_t *x_out
     return cudaGetLastError();
 }
 
-// Rows per CTA of the cluster form; 0 when the bands would be thinner than
-// the halo, or few quads leave nothing to share.
-inline int cluster_band(int H, int W)
+// Quads of a CTA of the cluster form with bands of `band` rows and a halo of h.
+inline int cluster_quads(int band, int h, int W)
 {
-    const int band = (H + kClCtas - 1) / kClCtas, qrow = (W + 3) >> 2;
-    if (band < kClHalo || H * qrow < 512)
-        return 0;
-    return (band + 2 * kClHalo - 2) * qrow <= 2 * kClThreads ? band : 0;
+    return (band + 2 * h - 2) * ((W + 3) >> 2);
 }
 
-template <int NB, bool GIBBS, int QPT>
+// Halo of the cluster form: 8 rows (64 x 64: 0.50 us per sweep, Gibbs 0.85,
+// against 0.52 and 0.90 with 4, 0.67 and 1.15 with 2), 4 where the bands are
+// thinner or a thread would hold more than a quad; 0: not taken (bands thinner
+// than that, or few quads, which leave nothing to share).
+inline int cluster_halo(int band, int H, int W)
+{
+    if (band < 4 || H * ((W + 3) >> 2) < 512 || cluster_quads(band, 4, W) > 2 * kClThreads)
+        return 0;
+    return band >= kClHalo && cluster_quads(band, kClHalo, W) <= kClThreads ? kClHalo : 4;
+}
+
+template <int NB, bool GIBBS, int QPT, int h>
 cudaError_t launch_cl_t(const SweepArgs &a, const uint8_t *x_in, uint8_t *x_out, int n, int band,
                         cudaStream_t st)
 {
-    const int qrow = (a.W + 3) >> 2;
-    const int quads = (band + 2 * kClHalo - 2) * qrow;
-    const int threads = ((quads + QPT - 1) / QPT + 31) & ~31;
-    const int smem = cl_smem_bytes(GIBBS, band, a.W);
+    const int threads = ((cluster_quads(band, h, a.W) + QPT - 1) / QPT + 31) & ~31;
+    const int smem = cl_smem_bytes(GIBBS, band, h, a.W);
     if (threads > kClThreads || smem > 48 * 1024)
         return cudaErrorInvalidValue;
-    resident_cluster_kernel<NB, GIBBS, QPT><<<kClCtas, threads, smem, st>>>(a, x_in, x_out, n, band);
+    resident_cluster_kernel<NB, GIBBS, QPT, h>
+        <<<kClCtas, threads, smem, st>>>(a, x_in, x_out, n, band);
     return cudaGetLastError();
 }
 
@@ -684,12 +617,13 @@ cudaError_t launch_res_q(const SweepArgs &a, const uint8_t *x_in, uint8_t *x_out
                          cudaStream_t st)
 {
     const int nq = a.H * (((a.W + 3) & ~3) >> 2);
-    const int band = cluster_band(a.H, a.W);
-    if (band > 0) {
-        const bool one = (band + 2 * kClHalo - 2) * ((a.W + 3) >> 2) <= kClThreads;
-        return one ? launch_cl_t<NB, GIBBS, 1>(a, x_in, x_out, n, band, st)
-                   : launch_cl_t<NB, GIBBS, 2>(a, x_in, x_out, n, band, st);
-    }
+    const int band = (a.H + kClCtas - 1) / kClCtas, h = cluster_halo(band, a.H, a.W);
+    if (h == kClHalo)
+        return launch_cl_t<NB, GIBBS, 1, kClHalo>(a, x_in, x_out, n, band, st);
+    if (h > 0)
+        return cluster_quads(band, 4, a.W) <= kClThreads
+                   ? launch_cl_t<NB, GIBBS, 1, 4>(a, x_in, x_out, n, band, st)
+                   : launch_cl_t<NB, GIBBS, 2, 4>(a, x_in, x_out, n, band, st);
     if (nq <= kResThreads)
         return launch_res_t<NB, GIBBS, 1>(a, x_in, x_out, n, st);
     if (nq <= 2 * kResThreads)
