@@ -373,7 +373,8 @@ bool uses_wave(const pcad_chain *ch);
 //   small labels, to kTileMaxSites sites: 256^2 L = 9, 8 neighbours 2.1 / 6.7,
 //   L = 5 1.7 / 6.3, L = 5 Gibbs 3.7 / 12.3 (four launches); L = 16 300^2 2.2 /
 //   7.0, 512^2 4.2 / 7.0, 1024^2 11.4 / 15.6 (2048^2, not taken: 39);
-//   two labels: 300^2 1.0 / 3.3, 600^2 2.1 / 3.4, 1000^2 3.7 / 5.4;
+//   two labels: 300^2 1.1 / 3.3, 600^2 2.1 / 3.4, 1000^2 3.6 / 5.4, 1500^2 6.3 /
+//   8.9, 2000^2 9.3 / 14.4, 2043 x 3001 13.1 / 17.7 (to kTileMaxBinarySites);
 //   segment draw: 256^2 L = 24 3.3 / 6.2, L = 64 3.5 / 8.5; at 512^2 L = 256
 //   the wavefront's 4 x 32-site items pack better (10.4 / 9.4; Gibbs, whose
 //   phases need no exchange here, 13.0 / 14.4; at 720^2 21.1 / 19.6): from 8
@@ -399,6 +400,21 @@ bool uses_tile(const pcad_chain *ch)
         return false;   // AUTO's tensor-core images
     const long long sites = (long long)ch->H * ch->W;
     return sites < (gibbs ? kTileSegGibbsSites : 8LL * 128 * ch->sms);
+}
+
+// Runs of fewer sweeps keep the per-sweep kernels: a tile-resident launch reads
+// the planes, waits for all its blocks and writes the sums back.  us per sweep
+// (tile-resident / per-sweep) of calls of 1, 2 and 4 sweeps: two labels 600^2
+// 13.8 / 9.3, 8.7 / 7.7, 5.4 / 6.9; L = 16 1024^2 24.8 / 20.8, 18.4 / 19.3; L = 24
+// 256^2 13.6 / 11.3, 8.5 / 9.8; Gibbs (several launches per sweep) L = 5 256^2
+// 13.5 / 24.3, L = 256 512^2 26 / 45.
+int tile_min_sweeps(const pcad_chain *ch)
+{
+    if (ch->model.sampler != PCAD_SAMPLER_PCA)
+        return 1;
+    if (ch->tplan.tg.compact)
+        return kTileCompactSweeps;
+    return ch->tkind.draw == TileKind::kBinary ? 4 : 2;
 }
 
 // Unblocked sweeps (PCA or Gibbs) on the CUDA-core windowed kernels: on
@@ -507,7 +523,7 @@ pcad_status issue_sweeps(pcad_chain *ch, int off0, int n, int &cur, cudaStream_t
         cur = out;
         return PCAD_OK;
     }
-    if (uses_tile(ch) && n > 0) {
+    if (uses_tile(ch) && n >= tile_min_sweeps(ch)) {
         a.sweep_off = (uint32_t)off0;
         const bool gibbs = ch->model.sampler != PCAD_SAMPLER_PCA;
         const int out = gibbs ? cur : cur ^ (n & 1);
@@ -715,7 +731,9 @@ pcad_status create_common(const uint8_t *g_src, bool g_on_device, int H, int W, 
     const bool gibbs = m->sampler != PCAD_SAMPLER_PCA;
     TileKind tkind;
     TilePlan tplan{};
-    const bool tile = (long long)H * W <= kTileMaxSites && tile_kind(tabs.dm, gibbs, tkind) &&
+    const bool tile = tile_kind(tabs.dm, gibbs, tkind) &&
+                      (long long)H * W <= (tkind.draw == TileKind::kBinary && !gibbs
+                                               ? kTileMaxBinarySites : kTileMaxSites) &&
                       tile_plan(tkind, H, W, sms, tplan);
     const size_t xbytes = tile ? align_up(tile_xch_bytes(H, W), 256) : 0;
     const size_t sbytes =

@@ -31,6 +31,11 @@
 //     a word (words of labels, observations and uniforms; four draws in
 //     flight) instead of one site.  Small tiles keep one site per thread: the
 //     latency of a pass counts there, not its instructions.
+//   * Two-label tiles above 8192 sites are compact: uniforms drawn in the pass
+//     instead of staged, sums as bytes (written back every 255 sweeps), so that
+//     an image of 8 megapixels fits the SMs' shared memory.  2043 x 3001: 13.1 us
+//     per sweep (4.7e11 site-updates/s, bound by instruction issue) against
+//     17.7 with a launch per sweep.
 //   * A launch holds one chain, or (batches, the server) several small ones,
 //     each on CTAs of its own.
 //
@@ -42,6 +47,7 @@
 #include <type_traits>
 
 #include "async_ptx.cuh"
+#include "binary_draw.cuh"
 #include "seg_draw.cuh"
 #include "small_draw.cuh"
 #include "tile.h"
@@ -51,6 +57,7 @@ namespace pcad {
 namespace {
 
 using namespace sld;
+using namespace bind;
 
 // Threads of a CTA, two or (at most) one per SM: 64 registers, or 80 for the
 // draws that need them (words, segments: spilled at 64; but a Gibbs phase of
@@ -58,7 +65,7 @@ using namespace sld;
 // per sweep against 13.5).
 constexpr int kTlThreads = 512, kTlThreads1 = 1024;
 constexpr int kTlWideThreads = 384, kTlWideThreads1 = 768;
-constexpr int kTlMaxSites = 8192;      // sites per tile
+constexpr int kTlMaxSites = 8192;      // sites per tile, if it is not compact
 constexpr int kTlMaxSweeps = 4;        // sweeps per exchange
 constexpr int kTlMaxSmem = 224 * 1024;    // one CTA per SM
 constexpr int kTlMaxSmem2 = 112 * 1024;   // two
@@ -117,6 +124,7 @@ struct SmallPol {
     // words per tile from which it is used: 512^2 on 216-word tiles 4.3 us per
     // sweep against 4.6, 300^2 on 150 2.6 against 2.45
     static constexpr int kWordsMin = 192;
+    static constexpr bool kCompact = false;
     static constexpr double kNsSiteWords = NB == 8 ? 1.5 : 1.3;
     uint32_t *pt;
     float *aq, *pre;
@@ -163,7 +171,7 @@ struct SmallPol {
         return s;
     }
     // The new labels of word o (4 sites in a row) of the staged plane X: those
-    // of the bytes of `act`, fill elsewhere.
+    // of the bytes of `act`, fill elsewhere; u: the word's Philox words.
     __device__ __forceinline__ uint32_t draw4(const SweepArgs &a, const uint32_t *X, int o, int SW,
                                               uint32_t G, const uint4 &u, uint32_t act, int, int,
                                               bool own)
@@ -195,7 +203,7 @@ struct SmallPol {
                 nc[7] = at(DR);
             }
             const bool valid = ((act >> (8 * q)) & 1u) != 0u;
-            const uint32_t ub = q == 0 ? u.x : (q == 1 ? u.y : (q == 2 ? u.z : u.w));
+            const uint32_t ub = (q == 0 ? u.x : (q == 1 ? u.y : (q == 2 ? u.z : u.w))) >> 8;
             int s = 16;
             bool certain = true;
             if (valid)
@@ -223,7 +231,7 @@ struct SegPol {
     static constexpr int kTabBytes = seg::kSegFloats * 4;
     static constexpr int kRowBytes = 0;
     static constexpr double kNsSite = 4.5, kNsSiteWords = 4.5;
-    static constexpr bool kWords = false;
+    static constexpr bool kWords = false, kCompact = false;
     static constexpr bool kWide = true;   // 80 registers
     float *tab;
 
@@ -260,22 +268,21 @@ template <int NB_>
 struct BinPol {
     static constexpr int NB = NB_;
     static constexpr uint32_t kFill = 0u;   // a missing neighbour is no label-1 neighbour
-    static constexpr int kEntries = 4 * (NB + 1) * (NB + 1);
-    static constexpr int kTabBytes = kEntries * 16;
+    static constexpr int kTabBytes = kThrBytes;
     static constexpr int kRowBytes = 0;
     static constexpr double kNsSite = 0.5;
     static constexpr bool kWide = false;
     static constexpr bool kWords = true;
     static constexpr int kWordsMin = 32;   // 300^2 1.0 us against 1.3, 1000^2 3.7 against 5.6
     static constexpr double kNsSiteWords = 0.25;
-    const uint4 *tab;
+    static constexpr bool kCompact = true;
+    ThrTab<NB> *tab;
     uint32_t nre;
 
     __device__ __forceinline__ void load(const DevModel &m, uint8_t *t, uint8_t *, int tid, int nt)
     {
-        for (int i = tid; i < kEntries; i += nt)
-            reinterpret_cast<uint4 *>(t)[i] = m.btab[i];
-        tab = reinterpret_cast<const uint4 *>(t);
+        tab = reinterpret_cast<ThrTab<NB> *>(t);
+        load_thresholds<NB>(*tab, m.btab, tid, nt);
         nre = 0u;
     }
 
@@ -291,7 +298,7 @@ struct BinPol {
             n1 += me[-SB - 1] + me[-SB + 1] + me[SB - 1] + me[SB + 1];
             nm += (top | le) + (top | ri) + (bot | le) + (bot | ri);
         }
-        const uint4 e = tab[((g * (NB + 1) + nm) * (NB + 1) + n1) * 2 + me[0]];
+        const uint4 e = tab->full[((g * (NB + 1) + nm) * (NB + 1) + n1) * 2 + me[0]];
         nre += own && ub - e.y < e.z ? 1u : 0u;
         return ub >= e.x ? 1 : 0;
     }
@@ -316,16 +323,8 @@ struct BinPol {
                 S += (uint32_t)(nm * (NB + 1)) << (8 * q);
             }
         }
-        uint32_t out = 0u;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t ub = q == 0 ? u.x : (q == 1 ? u.y : (q == 2 ? u.z : u.w));
-            const uint4 e = tab[((S >> (8 * q)) & 0xFFu) * 2 + ((M >> (8 * q)) & 1u)];
-            const bool on = ((act >> (8 * q)) & 1u) != 0u;
-            nre += own && on && ub - e.y < e.z ? 1u : 0u;
-            out |= ub >= e.x ? 1u << (8 * q) : 0u;
-        }
-        return out & act;
+        const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+        return quad_draw<NB>(*tab, S, M, w, own ? act : 0u, nre) & act;
     }
     __device__ __forceinline__ void finish(const SweepArgs &a)
     {
@@ -358,8 +357,9 @@ size_t tile_smem(const TileGeom &tg, int nt)
 {
     const size_t words = (size_t)(tg.th + 2 * tg.h) * (tg.twq + 2 * tg.hq);
     const size_t plane = tile_plane((int)words) * 4;
-    return (size_t)P::kTabBytes + (size_t)nt * P::kRowBytes + words * 16 * tg.k +
-           16 + plane * (GIBBS ? 1 : 2) + plane + (size_t)tg.th * tg.twq * 16;
+    return (size_t)P::kTabBytes + (size_t)nt * P::kRowBytes +
+           (tg.compact ? 0 : words * 16 * tg.k) + 16 + plane * (GIBBS ? 1 : 2) + plane +
+           (size_t)tg.th * tg.twq * (tg.compact ? 4 : 16);
 }
 
 // WORDS (lazy PCA): a thread draws the 4 sites of a word (large tiles), else
@@ -402,11 +402,12 @@ __global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBB
 
     uint8_t *const row = sm + P::kTabBytes + tid * P::kRowBytes;
     uint32_t *U = reinterpret_cast<uint32_t *>(sm + P::kTabBytes + nt * P::kRowBytes);
-    uint32_t *pl0 = U + 4 * words * J.tg.k + 4;
+    const bool compact = WORDS && P::kCompact && J.tg.compact;
+    uint32_t *pl0 = U + (compact ? 0 : 4 * words * J.tg.k) + 4;
     const int plane = tile_plane(words);
     uint32_t *pl1 = GIBBS ? pl0 : pl0 + plane;
     uint32_t *gw = pl1 + plane;
-    uint32_t *cnt = gw + plane;                     // [TH][TW] label sums of this launch
+    uint32_t *cnt = gw + plane;   // [TH][TW] label sums of this launch (compact: as bytes)
     P pol;
     pol.load(a.m, sm, row, tid, nt);
     // labels and observation with the halo
@@ -429,7 +430,7 @@ __global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBB
             pl1[i] = P::kFill;
         gw[i] = g;
     }
-    for (int i = tid; i < TH * TW; i += nt)
+    for (int i = tid; i < (compact ? TH * TWq : TH * TW); i += nt)
         cnt[i] = 0u;
     if (tid < plane - words) {
         pl0[words + tid] = 0u;
@@ -458,7 +459,7 @@ __global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBB
     // the uniforms of `ns` sweeps from t on, at their staged words: sweep s
     // updates up to (ns - s) kCol - 1 sites beyond the tile
     const auto uniforms = [&](uint32_t t, int ns) {
-        for (int s = 0; s < ns; ++s) {
+        for (int s = 0; s < (compact ? 0 : ns); ++s) {
             const int e = (ns - s) * kCol - 1, eq = (e + 3) >> 2;
             const int per = TWq + 2 * eq, n = (TH + 2 * e) * per;
             const unsigned int inv = inv_uni[e];
@@ -470,14 +471,34 @@ __global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBB
                 philox4x32_10((uint32_t)(q0 + lq), (uint32_t)(r0 + lr + a.row_off),
                               t + (uint32_t)s, ctr3, key0, key1, o0, o1, o2, o3);
                 reinterpret_cast<uint4 *>(U)[s * words + (lr + h) * SW + lq + hq] =
-                    make_uint4(o0 >> 8, o1 >> 8, o2 >> 8, o3 >> 8);
+                    WORDS ? make_uint4(o0, o1, o2, o3)
+                          : make_uint4(o0 >> 8, o1 >> 8, o2 >> 8, o3 >> 8);
             }
         }
     };
+    // the byte counts to the accumulator
+    const auto flush = [&]() {
+        for (int i = tid; i < TH * TWq; i += nt) {
+            const int lr = i / TWq, lq = i - lr * TWq;
+            const uint32_t n4 = cnt[i];
+            if (n4 == 0u)   // (always, outside the image)
+                continue;
+            cnt[i] = 0u;
+            float *pa = a.acc + (size_t)(r0 + lr) * W + c0 + 4 * lq;
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+                if ((n4 >> (8 * b)) & 0xFFu)
+                    pa[b] += (float)((n4 >> (8 * b)) & 0xFFu);
+        }
+    };
+    int nacc = 0;   // sweeps in the byte counts
     uniforms(t0, min(J.tg.k, nsweeps));
     bool ok = true;
     uint32_t *X = pl0;
     int done = 0;
+    const bool ring = TH > 2 * h && TWq > 2 * hq;   // some words are not border words
+    const int nrows = ring ? 2 * h * TWq : TH * TWq;
+    const int nborder = ring ? nrows + (TH - 2 * h) * 2 * hq : nrows;
     for (unsigned int x = 1;; ++x) {                // exchanges
         const int ns = min(J.tg.k, nsweeps - done);
         // halo words and uniforms in place; leave together when a wait gave up
@@ -522,7 +543,12 @@ __global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBB
                                                    : 0u;
                         const bool own = (unsigned)lr < (unsigned)TH && (unsigned)lq < (unsigned)TWq;
                         const int o = valid ? (lr + h) * SW + lq + hq : SW + 1;
-                        const uint4 u = reinterpret_cast<const uint4 *>(Us)[o];
+                        uint4 u;
+                        if (compact)
+                            philox4x32_10((uint32_t)(q0 + lq), (uint32_t)(r0 + lr + a.row_off), t, ctr3,
+                                          key0, key1, u.x, u.y, u.z, u.w);
+                        else
+                            u = reinterpret_cast<const uint4 *>(Us)[o];
                         const uint32_t G = gw[o];
                         if (b == 0 && !fresh)
                             __syncthreads();
@@ -530,7 +556,10 @@ __global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBB
                         const uint32_t v = pol.draw4(a, X, o, SW, G, u, act, r0 + lr, c0 + lc, own);
                         if (valid) {
                             Y[o] = v;
-                            if (own && acc_now) {
+                            if (compact) {
+                                if (own && acc_now)
+                                    cnt[lr * TWq + lq] += v & act;
+                            } else if (own && acc_now) {
                                 uint4 *pc = reinterpret_cast<uint4 *>(cnt + lr * TW + lc);
                                 const uint32_t w = v & act;
                                 uint4 n4 = *pc;
@@ -589,16 +618,30 @@ __global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBB
                 }
             }
             X = Y;
+            if (compact && acc_now && ++nacc == 255) {   // the counts are full
+                __syncthreads();
+                flush();
+                nacc = 0;   // (each count is its own thread's again after the next barrier)
+            }
         }
         __syncthreads();
         done += ns;
         if (!more)
             break;
-        if (pub)   // publish the border words
-            for (int i = tid; i < TH * TWq; i += nt) {
-                const int lr = i / TWq, lq = i - lr * TWq;
-                const bool border = lr < h || lr >= TH - h || lq < hq || lq >= TWq - hq;
-                if (border && r0 + lr < H && q0 + lq < Wq)
+        if (pub)   // publish the border words: whole rows, then the sides of the others
+            for (int i = tid; i < nborder; i += nt) {
+                int lr, lq;
+                if (i < nrows) {
+                    lr = i / TWq;
+                    lq = i - lr * TWq;
+                    lr += ring && lr >= h ? TH - 2 * h : 0;
+                } else {
+                    lr = (i - nrows) / (2 * hq);
+                    lq = i - nrows - lr * 2 * hq;
+                    lr += h;
+                    lq += lq < hq ? 0 : TWq - 2 * hq;
+                }
+                if (r0 + lr < H && q0 + lq < Wq)
                     st_word(buf + (size_t)(r0 + lr) * Wq + q0 + lq,
                             ((unsigned long long)tag << 32) | X[(lr + h) * SW + lq + hq]);
             }
@@ -641,6 +684,8 @@ __global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBB
     // labels and counts back (a label of this plane that a neighbour read at
     // the start was read before it published its first exchange, which this
     // tile awaited, or the planes differ)
+    if (compact)
+        flush();
     for (int i = tid; i < TH * TWq; i += nt) {
         const int lr = i / TWq, lq = i - lr * TWq;
         const int r = r0 + lr, c = c0 + 4 * lq;
@@ -655,7 +700,7 @@ __global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBB
         for (int b = 0; b < nv; ++b) {
             if (nv < 4)
                 xg_out[(size_t)r * a.pitch + c + b] = (uint8_t)(w >> (8 * b));
-            if (n4[b])
+            if (!compact && n4[b])
                 pa[b] += (float)n4[b];
         }
     }
@@ -691,7 +736,7 @@ bool draws_words(const TileGeom &g)
 // The tile grid of an image: at most `ctas` tiles of at least h rows and
 // columns, k sweeps per exchange.
 template <class P, bool GIBBS>
-bool tile_geometry(int H, int W, int ctas, int per_sm, TileGeom &best)
+bool tile_geometry(int H, int W, int ctas, int per_sm, bool compact, TileGeom &best)
 {
     constexpr int phases = tile_phases(P::NB, GIBBS);
     const size_t most = per_sm == 2 ? kTlMaxSmem2 : kTlMaxSmem;
@@ -713,7 +758,8 @@ bool tile_geometry(int H, int W, int ctas, int per_sm, TileGeom &best)
             if (g.th < g.h)
                 g.th = g.h;
             g.tiles_y = (H + g.th - 1) / g.th;
-            if ((long)g.th * g.twq * 4 > kTlMaxSites || g.tiles_x * g.tiles_y > ctas)
+            g.compact = compact && P::kCompact && !GIBBS && g.th * g.twq * 4 > kTlMaxSites;
+            if ((!g.compact && (long)g.th * g.twq * 4 > kTlMaxSites) || g.tiles_x * g.tiles_y > ctas)
                 continue;
             // one CTA per SM: a thread per site of the widest pass, if they are
             // few (idle warps still take every barrier)
@@ -844,10 +890,25 @@ bool tile_kind(const DevModel &m, bool gibbs, TileKind &k)
     return seg_eligible(m);
 }
 
+namespace {
+
+bool plan_geometry(const TileKind &k, int H, int W, int ctas, bool two, bool compact, TileGeom &tg)
+{
+    if (ctas <= 0)
+        return false;
+    return with_policy(k, [&](auto pol, auto gibbs) {
+        using P = std::remove_pointer_t<decltype(pol)>;
+        return tile_geometry<P, decltype(gibbs)::value>(H, W, ctas, two ? 2 : 1, compact, tg);
+    });
+}
+
+}  // namespace
+
 bool tile_plan(const TileKind &k, int H, int W, int sms, TilePlan &p)
 {
     const bool two = (long long)H * W > (long long)sms * kTlThreads1;
-    if (!tile_plan_ctas(k, H, W, two ? 2 * sms : sms, two, p.tg))
+    if (!(two && plan_geometry(k, H, W, 2 * sms, true, false, p.tg)) &&
+        !plan_geometry(k, H, W, sms, false, true, p.tg))
         return false;
     p.ctas = p.tg.tiles_x * p.tg.tiles_y;
     return true;
@@ -855,12 +916,7 @@ bool tile_plan(const TileKind &k, int H, int W, int sms, TilePlan &p)
 
 bool tile_plan_ctas(const TileKind &k, int H, int W, int ctas, bool two, TileGeom &tg)
 {
-    if (ctas <= 0)
-        return false;
-    return with_policy(k, [&](auto pol, auto gibbs) {
-        using P = std::remove_pointer_t<decltype(pol)>;
-        return tile_geometry<P, decltype(gibbs)::value>(H, W, ctas, two ? 2 : 1, tg);
-    });
+    return plan_geometry(k, H, W, ctas, two, false, tg);
 }
 
 size_t tile_xch_bytes(int H, int W)

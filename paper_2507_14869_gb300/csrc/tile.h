@@ -27,6 +27,7 @@ struct TileGeom {
     int h, hq;            // halo: rows (and columns), words
     int threads;          // per CTA
     bool two;             // two CTAs per SM
+    bool compact;         // two labels: no staged uniforms, byte counts
 };
 
 struct TilePlan {
@@ -74,5 +75,9 @@ cudaError_t launch_tile(const TileKind &k, const TilePack &L, int ctas, cudaStre
 // Chains, batches and the server take tile-resident launches for images of at
 // most this many sites.
 constexpr long long kTileMaxSites = 1ll << 20;
+// Two-label PCA chains: as long as their tiles fit (about 50000 sites per SM;
+// tiles above 8192 sites are compact, for runs of at least kTileCompactSweeps).
+constexpr long long kTileMaxBinarySites = 8ll << 20;
+constexpr int kTileCompactSweeps = 16;
 
 }  // namespace pcad
