@@ -65,7 +65,8 @@ NCU_DIRECT_BYTES_PER_SITE = None
 NCU_DIRECT_NOTE = "ncu dram__bytes_read+write of one pca_direct_kernel launch at 8192^2 L=16"
 NCU_WIN_BYTES_PER_SITE = (402903040 + 286483712) / (8192 * 8192)
 NCU_WIN_NOTE = ("ncu dram__bytes_read+write of one accumulating pca_win_kernel launch at "
-                "8192^2 L=256 (profiles/pca_win_l256_8192sq.md)")
+                "8192^2 L=256 (profiles/pca_win_l256_8192sq.md); pca_seg_kernel moves the same "
+                "planes")
 NCU_SMALL_BYTES_PER_SITE = (408240384 + 280811264) / (8192 * 8192)
 NCU_SMALL_NOTE = ("ncu dram__bytes_read+write of one accumulating pca_small_tma_kernel launch "
                   "at 8192^2 L=16 (profiles/pca_small_tma_l16_6144sq.md)")
@@ -77,13 +78,18 @@ KERNEL_NAMES = {
     2: "pca_tcw_kernel<4,0,0,0> (tcgen05 windowed tent sums, CUDA-core CDF, wavefront, "
        "one launch per 32 sweeps)",
     3: "pca_wave_kernel (CUDA cores, wavefront, one launch per 32 sweeps)",
-    4: "small-label draw (CUDA cores, prior sums from a pair table, one launch per sweep; "
-       "pca_small_tma_kernel on TMA-loaded tiles from 2^23 sites, else pca_small_kernel)",
-    5: "resident_kernel (two labels, whole run in one single-CTA launch, state in shared "
+    4: "small-label draw (CUDA cores, prior sums from a pair table; pca_small_tma_kernel on "
+       "TMA-loaded tiles from 2^21 sites, tile_kernel (a run per launch) to 2^20, else "
+       "pca_small_kernel)",
+    5: "resident_cluster_kernel (two labels, whole run in one launch of a cluster of 8 CTAs; "
+       "resident_kernel, one CTA, for the smallest images; state in shared "
        "memory, exact per-configuration thresholds)",
-    6: "pca_win_kernel (CUDA cores, hull chunks from a tent-byte table, one launch per sweep)",
-    7: "pca_winw_kernel (the windowed draw as a wavefront, one launch per 32 sweeps)",
-    8: "pca_binary_kernel (two labels, threshold table, one launch per sweep)",
+    6: "pca_seg_kernel (CUDA cores, segment sums from prefix tables between the kinks of the "
+       "prior, one launch per sweep; pca_win_kernel for models it does not take)",
+    7: "pca_segw_kernel (the segment draw as a wavefront, one launch per 32 sweeps; "
+       "pca_winw_kernel for models it does not take)",
+    8: "pca_binary_kernel (two labels, threshold table, one launch per sweep; tile_kernel, a run "
+       "per launch, to about 8e6 sites)",
 }
 
 
@@ -540,7 +546,7 @@ def _gibbs_8192(pc, stream, timed, noisy, m, clean, cid, steps=2):
     sites = noisy.size
     name = {2: "pca_tcw_kernel<4,0,0,0,1> (checkerboard Gibbs on the tensor-core wavefront, 2 "
                "colour phases per sweep)",
-            6: "gibbs_win_kernel (CUDA cores, windowed draw, one launch per colour phase, 2 "
+            6: "gibbs_seg_kernel (CUDA cores, segment draw, one launch per colour phase, 2 "
                "phases per sweep)"}.get(kind, "gibbs_cb_kernel (2 colour phases)")
     return {"value": sites / (ms_sweep * 1e-3), "unit": "site-updates/s",
             "ms_per_step": sum(ms) / steps, "ms_per_sweep": ms_sweep, "steps": steps,
@@ -578,7 +584,7 @@ BATCH_SWEEPS, BATCH_BURN = 200, 50
 def _binary64(pc, torch, stream, n_batch=512, reps=5):
     """The two-label image workload (64 x 64, Ising c_P = 1.2, flip p = 0.1,
     lambda = 1, 500 sweeps, burn-in 100): one chain on the default kernel
-    (the resident one: the whole run in one single-CTA launch) against
+    (the resident one: the whole run in one launch of a cluster) against
     per-sweep launches in CUDA graphs, lazy PCA and checkerboard Gibbs,
     device-timed; the wall clock of create (host image) + run + read mean;
     then n_batch such chains (distinct images) as one batch against the same

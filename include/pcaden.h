@@ -169,14 +169,16 @@ pcad_status pcad_chain_set_blocking(pcad_chain *ch, int k);
  * PCAD_EINVAL otherwise) runs one launch per sweep that takes the prior sums
  * of all labels of a site from a table of neighbour pairs (16 bytes per pair
  * of labels, in shared memory) and draws from chunk prefix sums in
- * registers; same labels as the other kernels.  Images of at least 2^23
+ * registers; same labels as the other kernels.  Images of at least 2^21
  * sites sweep on TMA-loaded 64 x 46 tiles in persistent blocks (the next
- * tile's copy in flight during the draw), smaller ones on persistent
+ * tile's copy in flight during the draw), images of up to 2^20 sites run
+ * tile-resident (below), others on persistent
  * 16 x 32 tiles staged by the threads.  AUTO takes it for every model it
  * accepts.  PCAD_KERNEL_RESIDENT (L = 2, 4- or 8-neighbourhood,
  * either sampler, H * ceil(W / 4) <= 4096, e.g. up to 128 x 128, and at most
  * 200 KB of shared memory; PCAD_EINVAL otherwise) runs all the sweeps of a
- * run in one launch of one 1024-thread CTA that keeps the state in shared
+ * run in one launch of a cluster of 8 CTAs (the smallest images: one CTA)
+ * that keeps the state in shared
  * memory and draws each site from a table of exact thresholds on its
  * uniform, one per site configuration (x_i, g_i, label-1 neighbours,
  * neighbours outside the image), computed at set-up from the FP32 draw and
@@ -191,16 +193,28 @@ pcad_status pcad_chain_set_blocking(pcad_chain *ch, int k);
  * its neighbours' tents reach, their tent sums read from a table of 8 tents
  * per 8-byte shared-memory entry, the other chunks' sums from a table of the
  * observation, the sites of a block sorted by the number of such chunks so
- * that a warp's lanes do similar work; same labels.  PCAD_KERNEL_WINDOW_WAVE
- * (the same models, either sampler) runs the windowed draw as one
+ * that a warp's lanes do similar work; same labels.  Models with 4
+ * neighbours and pair_coef >= 0 whose tables fit FP32's range take the segment
+ * draw in its place: the prior is linear between its 12 kinks, so a draw sums 13
+ * segments from prefix tables of the data term; same labels.  PCAD_KERNEL_WINDOW_WAVE
+ * (the same models, either sampler) runs these draws as one
  * persistent wavefront launch per block of sweeps (of Gibbs colour phases),
  * as PCAD_KERNEL_WAVE does the CUDA-core draw (energy tracking: one launch
  * per sweep); same labels.  PCAD_KERNEL_BINARY (L = 2, 4- or 8-neighbourhood,
  * PCA sampler; PCAD_EINVAL otherwise) runs one launch per sweep that draws
  * each site by one read of the resident kernel's threshold table and a
- * compare (persistent blocks over tiles of 16 x 128 sites staged in shared
- * memory); same labels and the same FP64 re-draw count.  AUTO takes it for
- * two-label images of at least 2^18 sites. */
+ * compare (warps walk down strips of 128 columns with the labels in
+ * registers); same labels and the same FP64 re-draw count.  AUTO takes it for
+ * two-label images of at least 2^18 sites.
+ *
+ * Tile-resident runs.  With AUTO (or SMALL) a run of sweeps of a mid-size
+ * image is one cooperative launch in which every CTA keeps a tile in shared
+ * memory and exchanges its border with its neighbours: small labels and two
+ * labels to 2^20 sites (two-label PCA to about 8e6), the segment draw's models
+ * below the wavefront's images; not with energy tracking, temporal blocking or
+ * runs of very few sweeps.  Same draws and labels; the kernel in use is reported
+ * as the kind that it stands in for.  Its waits are bounded
+ * (pcad_chain_set_wait_limit). */
 typedef enum {
     PCAD_KERNEL_AUTO = 0,
     PCAD_KERNEL_CUDA_CORE = 1,
