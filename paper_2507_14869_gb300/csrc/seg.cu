@@ -4,19 +4,19 @@
 // the windowed draw (win.cu) for the models seg_eligible accepts, in the same
 // two launch forms:
 //
-//   * one launch per sweep (per colour phase): persistent blocks of 256
-//     threads, each warp taking tiles of 4 x 32 sites (64 columns x 4 rows of
-//     cells for Gibbs) on its own.  A block copies the model's prefix tables
-//     (18 KB) into shared memory once per launch; there is no other block
-//     barrier.  A lane owns a column of the tile and walks its 4 rows with
-//     the labels above, at and below it in registers; one Philox call per
-//     lane and tile serves the tile's 128 sites.
-//     Bound by instruction issue: about 800 thread instructions per
-//     site-update (700 in the draw) at 70 % issue, ALU pipe 55 %, DRAM 2 %.
-//     L = 256, T = 30, sigma = 25, 8192^2: 1.84 ms per sweep (3.66e10
-//     site-updates/s) against 4.04 ms for the windowed draw; 3 blocks per SM
-//     (80 registers) against 1.88 ms with 2 and 1.95 ms with 4.  Gibbs at
-//     4096^2: 492 us per sweep (3.4e10).
+//   * one launch per sweep (per colour phase): one persistent block per SM (24
+//     warps, 80 registers; colour phases 32 warps, 64), its warps taking tiles
+//     of 4 x 32 sites (64 columns x 4 rows of cells for Gibbs) as they come
+//     free.  A block copies the model's prefix tables (18 KB) into shared
+//     memory once per launch; there is no other block barrier.  A lane owns a
+//     column of the tile and walks its 4 rows with the labels above, at and
+//     below it in registers; one Philox call per lane and tile serves the tile's
+//     128 sites.
+//     Bound by instruction issue: 831 thread instructions per site-update (700
+//     in the draw) at 75 to 80 % issue, ALU pipe 55 %, DRAM 2 %.
+//     L = 256, T = 30, sigma = 25, 8192^2: 1.60 ms per sweep (4.19e10
+//     site-updates/s) against 4.05 ms for the windowed draw.  Gibbs at 4096^2:
+//     434 us per sweep (3.9e10; 479 with a fixed share per warp).
 //   * the wavefront for images of few tiles: the sweeps of a block in one
 //     persistent launch, items and waits as in win.cu's wavefront, one site
 //     per thread.  512^2: 9.4 us per sweep against 17.9 us (Gibbs 14.4 against
@@ -31,8 +31,10 @@ using namespace seg;
 
 constexpr int kSX = 32;
 constexpr int kSY = 4;
-constexpr int kSegWarps = 8;                 // per-sweep blocks
+constexpr int kSegWarps = 24;                // per-sweep blocks: one per SM (80 registers)
 constexpr int kSegThreads = 32 * kSegWarps;
+constexpr int kSegGibbsWarps = 32;           // per colour phase (64 registers)
+constexpr int kSegGibbsThreads = 32 * kSegGibbsWarps;
 constexpr int kSegwThreads = kSX * kSY;      // wavefront blocks
 constexpr double kBias = 3.9443045261050590e-31;   // 2^-101
 
@@ -69,14 +71,31 @@ __device__ __forceinline__ void load_tab(float *tab, const float *src, int tid, 
         reinterpret_cast<float4 *>(tab)[i] = __ldg(reinterpret_cast<const float4 *>(src) + i);
 }
 
+// A warp's next tile: groups of WARPS tiles go to the blocks in turn, and a
+// block's warps take its tiles as they come free.  With a fixed share per warp
+// and three blocks of 8 warps per SM the scheduler ran the oldest warps ahead,
+// and the last part of a sweep had few left (30 % of warps active on average
+// against 37.5 % resident): one block per SM whose warps share its tiles, 8192^2,
+// L = 256 1773 -> 1603 us per sweep (three such blocks per SM: 1786).
+template <int WARPS>
+__device__ __forceinline__ int next_tile(int *taken, int lane)
+{
+    int n = 0;
+    if (lane == 0)
+        n = atomicAdd(taken, 1);
+    n = __shfl_sync(0xFFFFFFFFu, n, 0);
+    return ((n / WARPS) * (int)gridDim.x + (int)blockIdx.x) * WARPS + n % WARPS;
+}
+
 // One lazy-PCA sweep: a.xin -> a.xout (or the planes x0 / x1 by the parity of
 // the sweep index), skipped at or past *budget.
-__global__ void __launch_bounds__(kSegThreads, 3)
+__global__ void __launch_bounds__(kSegThreads, 1)
     pca_seg_kernel(const SweepArgs a, int tiles_x, int ntiles, uint8_t *x0,
                    uint8_t *x1, const uint32_t *budget)
 {
     __shared__ __align__(16) float tab[kSegFloats];
     __shared__ __align__(16) uint32_t U_s[kSegWarps][kSY * kSX];
+    __shared__ int s_taken;
     const uint32_t t = sweep_index(a);
     if (budget && t >= *budget)
         return;   // the whole launch, before any barrier
@@ -84,12 +103,13 @@ __global__ void __launch_bounds__(kSegThreads, 3)
     uint8_t *xout = x0 ? ((t & 1u) ? x0 : x1) : a.xout;
     const int lane = (int)threadIdx.x & 31, wp = (int)threadIdx.x >> 5;
     load_tab(tab, a.m.stab, (int)threadIdx.x, kSegThreads);
+    if (threadIdx.x == 0)
+        s_taken = 0;
     __syncthreads();
     const bool acc_on = accumulate_after(a, t);
     const int H = a.H, W = a.W;
     uint32_t *U = U_s[wp];
-    for (int tile = (int)blockIdx.x * kSegWarps + wp; tile < ntiles;
-         tile += (int)gridDim.x * kSegWarps) {
+    for (int tile; (tile = next_tile<kSegWarps>(&s_taken, lane)) < ntiles;) {
         const int ty = tile / tiles_x, tx = tile - ty * tiles_x;
         const int r0 = ty * kSY, c = tx * kSX + lane;
         block_uniforms(a, r0, tx * kSX, t, U);
@@ -263,20 +283,22 @@ __device__ __forceinline__ void gibbs_uniforms(const SweepArgs &a, int row0, int
 // the column pair 2 l; after the last phase (a.last_phase) the pairs are
 // accumulated.  A phase writes one colour and reads the other, but for the
 // site's own label, which only the accumulation reads, after its own write.
-__global__ void __launch_bounds__(kSegThreads, 4)
+__global__ void __launch_bounds__(kSegGibbsThreads, 1)
     gibbs_seg_kernel(const SweepArgs a, int q, int tiles_x, int ntiles)
 {
     __shared__ __align__(16) float tab[kSegFloats];
-    __shared__ __align__(16) uint32_t U_s[kSegWarps][kSY * 2 * kSX];
+    __shared__ __align__(16) uint32_t U_s[kSegGibbsWarps][kSY * 2 * kSX];
+    __shared__ int s_taken;
     uint8_t *x = const_cast<uint8_t *>(a.xin);
     const uint32_t t = sweep_index(a);
     const int lane = (int)threadIdx.x & 31, wp = (int)threadIdx.x >> 5;
-    load_tab(tab, a.m.stab, (int)threadIdx.x, kSegThreads);
+    load_tab(tab, a.m.stab, (int)threadIdx.x, kSegGibbsThreads);
+    if (threadIdx.x == 0)
+        s_taken = 0;
     __syncthreads();
     const bool acc_on = a.last_phase && accumulate_after(a, t);
     uint32_t *U = U_s[wp];
-    for (int tile = (int)blockIdx.x * kSegWarps + wp; tile < ntiles;
-         tile += (int)gridDim.x * kSegWarps) {
+    for (int tile; (tile = next_tile<kSegGibbsWarps>(&s_taken, lane)) < ntiles;) {
         const int ty = tile / tiles_x, tx = tile - ty * tiles_x;
         const int r0 = ty * kSY, c0 = 2 * (tx * kSX + lane);
         gibbs_uniforms(a, r0, tx, t, lane, U);
@@ -489,15 +511,15 @@ cudaError_t launch_gibbs_seg(const SweepArgs &a, int q, cudaStream_t st)
 {
     static int per_sm[64] = {};
     int cap = 0;
-    cudaError_t e = resident(gibbs_seg_kernel, kSegThreads, per_sm, cap);
+    cudaError_t e = resident(gibbs_seg_kernel, kSegGibbsThreads, per_sm, cap);
     if (e != cudaSuccess)
         return e;
     const int tiles_x = (a.W + 2 * kSX - 1) / (2 * kSX);
     const long long ntiles = (long long)tiles_x * ((a.H + kSY - 1) / kSY);
     if (ntiles >= (1ll << 30))
         return cudaErrorInvalidValue;
-    const long long need = (ntiles + kSegWarps - 1) / kSegWarps;
-    gibbs_seg_kernel<<<(int)(need < cap ? need : cap), kSegThreads, 0, st>>>(a, q, tiles_x,
+    const long long need = (ntiles + kSegGibbsWarps - 1) / kSegGibbsWarps;
+    gibbs_seg_kernel<<<(int)(need < cap ? need : cap), kSegGibbsThreads, 0, st>>>(a, q, tiles_x,
                                                                              (int)ntiles);
     return cudaGetLastError();
 }
