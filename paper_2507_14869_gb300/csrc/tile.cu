@@ -743,13 +743,16 @@ bool tile_geometry(int H, int W, int ctas, int per_sm, bool compact, TileGeom &b
     const int Wq = (W + 3) / 4;
     double best_cost = -1.0;
     for (int k = 1; k <= (GIBBS ? 2 : kTlMaxSweeps); ++k)
-        for (int nx = 1; nx <= ctas && nx <= Wq; ++nx) {
+        for (int nx = 1, wide = 0; nx <= ctas && nx <= Wq; ++nx) {
+            if ((Wq + nx - 1) / nx == wide)
+                continue;   // the same tiles as with fewer columns of them
+            wide = (Wq + nx - 1) / nx;
             TileGeom g{};
             g.k = k;
             g.two = per_sm == 2;
             g.h = k * phases;
             g.hq = (g.h + 3) / 4;
-            g.twq = (Wq + nx - 1) / nx;
+            g.twq = wide;
             if (g.twq < g.hq)
                 g.twq = g.hq;
             g.tiles_x = (Wq + g.twq - 1) / g.twq;
@@ -763,10 +766,10 @@ bool tile_geometry(int H, int W, int ctas, int per_sm, bool compact, TileGeom &b
                 continue;
             // one CTA per SM: a thread per site of the widest pass, if they are
             // few (idle warps still take every barrier)
-            const long wide = (long)(g.th + 2 * g.h - 2) * (4 * g.twq + 2 * g.h - 2) / phases;
+            const long most_sites = (long)(g.th + 2 * g.h - 2) * (4 * g.twq + 2 * g.h - 2) / phases;
             g.threads = per_sm == 2 ? tile_threads<P, GIBBS>(true)
                                     : (int)std::min<long>(tile_threads<P, GIBBS>(false),
-                                                          std::max<long>(256, (wide + 127) / 128 * 128));
+                                                          std::max<long>(256, (most_sites + 127) / 128 * 128));
             // (the scratch of the widest launch: a pack has its widest job's threads)
             if (tile_smem<P, GIBBS>(g, tile_threads<P, GIBBS>(per_sm == 2)) > most)
                 continue;
