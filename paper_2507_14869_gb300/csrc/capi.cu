@@ -372,8 +372,8 @@ bool uses_wave(const pcad_chain *ch);
 // windowed kernels; energy tracking needs every sweep's state.  Measured on
 // GB300, us per sweep (tile-resident / the kernel it replaces):
 //   small labels, to kTileMaxSites sites: 256^2 L = 9, 8 neighbours 2.1 / 6.7,
-//   L = 5 1.7 / 6.3, L = 5 Gibbs 3.7 / 12.3 (four launches); L = 16 300^2 2.2 /
-//   7.0, 512^2 4.2 / 7.0, 1024^2 11.4 / 15.6 (2048^2, not taken: 39);
+//   L = 5 1.7 / 6.3, L = 5 Gibbs 3.7 / 12.3 (four launches); L = 16 300^2 2.1 /
+//   7.0, 512^2 4.1 / 7.0, 1024^2 10.9 / 15.6 (2048^2, not taken: 39);
 //   two labels: 300^2 1.1 / 3.3, 600^2 2.1 / 3.4, 1000^2 3.6 / 5.4, 1500^2 6.3 /
 //   8.9, 2000^2 9.3 / 14.4, 2043 x 3001 13.1 / 17.7 (to kTileMaxBinarySites);
 //   segment draw: 256^2 L = 24 3.3 / 6.2, L = 64 3.5 / 8.5; at 512^2 L = 256
@@ -468,7 +468,7 @@ bool uses_small(const pcad_chain *ch)
 // The small-label kernel's launch form for large images: persistent blocks
 // over TMA-loaded 64 x 46 tiles, the next tile's box in flight during the
 // draw (launch_pca_small_tma), from kSmallTmaMinSites sites.  Measured on
-// GB300 at L = 16: 2048^2 39.4 us per sweep against 40.4 with the persistent
+// GB300 at L = 16: 2048^2 39.4 us per sweep (38.6 now) against 40.4 with the persistent
 // 16 x 32 tiles; at 1024^2, below the line (and tile-resident with AUTO), 0.59e11
 // against 0.69e11 site-updates/s, its 391 tiles leaving a last wave half empty.
 bool small_tma(const pcad_chain *ch)

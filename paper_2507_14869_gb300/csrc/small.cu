@@ -18,8 +18,9 @@
 //     labels per packed FP32x2 instruction (every lane rounds as the scalar
 //     operation).  A byte of P becomes an exact float by placing it in the
 //     mantissa of 2^23 and subtracting 2^23; fl(alpha q) comes from a 16 x 16
-//     table in shared memory (observations are checked against L), within the
-//     same 3u |v| exponent bound.  (Products of two table
+//     table in shared memory (observations are checked against L) for half the
+//     labels and is computed for the others, within the same 3u |v| exponent
+//     bound.  (Products of two table
 //     factors per label measured slower: the per-lane table reads conflict
 //     in shared memory, while the exponential unit has room.)
 //   * Inverse CDF over chunks of 4 labels (small_draw.cuh): packed chunk sums,
@@ -212,10 +213,10 @@ __global__ void __launch_bounds__(kThreads) pca_small_kernel(const SweepArgs a, 
 // stored as one 32-bit word and the accumulator read-modify-written as one
 // float4, loaded before the draws; the tile's labels are read as words of 4
 // sites.  Bound by instruction issue and shared memory (about 217 instructions
-// and 65 shared-memory wavefronts per 32 sites).  8192^2, L = 16: 572 us per
-// sweep (1.17e11 site-updates/s) with 3 blocks per SM (71 registers) against
-// 637 us for the form that read bytes and joined the atom label by label; 608
-// with 2 blocks per SM, 584 with 4.
+// and 65 shared-memory wavefronts per 32 sites).  8192^2, L = 16: 538 us per
+// sweep (1.25e11 site-updates/s) with 3 blocks per SM (72 registers) against
+// 637 us for the form that read bytes and joined the atom label by label
+// (2 blocks per SM were 6 % slower, 4 2 %).
 constexpr int kTmThreads = 256;
 constexpr int kTmBoxW = 96, kTmBoxH = 48;   // the box of encode_plane_map
 constexpr int kTmOutW = 64, kTmOutH = kTmBoxH - 2;
