@@ -298,24 +298,27 @@ pcad_status pcad_chain_read_min_state(pcad_chain *ch, uint8_t *host_out, int out
                                       double *energy, uint64_t *sweep);
 
 /* Failure detection (no counterpart in the paper: the sweep of Section 5.2
- * needs no waits, but the wavefront, tensor-core and TMA-tiled kernels
- * that run it wait on one another's tiles, on MMA completion and on tile
- * loads).  Every such device-side wait is bounded by elapsed time: after
+ * needs no waits, but the wavefront, tensor-core, TMA-tiled and tile-resident
+ * kernels that run it wait on one another's tiles, on MMA completion and on
+ * tile loads).  Every such device-side wait is bounded by elapsed time: after
  * `seconds` (default 1.0; accepted range [1e-4, 60], PCAD_EINVAL outside)
  * it gives up and sets the chain's error flag, every other wait and work
- * item of the launch stops as soon as it sees the flag, the kernel returns
- * and pcad_chain_sync reports PCAD_ETIMEOUT.  The sample and accumulator
- * are then undefined; pcad_chain_reset clears the flag and restarts the
- * chain.  Applies to sweeps queued after the call. */
+ * item of the launch stops as soon as it sees the flag, and the kernel
+ * returns.  The state and accumulator are then undefined: pcad_chain_sync and
+ * every synchronous read of them (sample, mean, metrics, energy, energies,
+ * lowest-energy state, export) report PCAD_ETIMEOUT until pcad_chain_reset
+ * clears the flag and restarts the chain.  Applies to sweeps queued after
+ * the call. */
 pcad_status pcad_chain_set_wait_limit(pcad_chain *ch, double seconds);
 
 /* Test aid for the failure path above: with tile >= 0, tile `tile` of the
  * wavefront CUDA-core kernel's and the tensor-core kernel's grid (4 x 32
- * sites, row-major; Gibbs: 8 x 32) never reports a finished sweep, so the
- * tiles around it wait for a dependency that never arrives until their
- * bounded wait runs out.  tile = -1 (the default) turns it off; PCAD_EINVAL
- * for tile outside [-1, tiles).  Applies to sweeps queued after the call;
- * no other kernel is affected. */
+ * sites, row-major; Gibbs: 8 x 32) never reports a finished sweep, and CTA
+ * `tile` of a tile-resident launch (where it has as many) never publishes its
+ * border, so the tiles around it wait for a dependency that never arrives
+ * until their bounded wait runs out.  tile = -1 (the default) turns it off;
+ * PCAD_EINVAL for tile outside [-1, tiles), tiles of the wavefront's grid.
+ * Applies to sweeps queued after the call; no other kernel is affected. */
 pcad_status pcad_chain_inject_stall(pcad_chain *ch, int tile);
 
 /* Row offset of a chain that holds a band of rows of a larger image: its
@@ -337,7 +340,8 @@ pcad_status pcad_chain_set_row_offset(pcad_chain *ch, int row_off);
 pcad_status pcad_chain_write_rows_dev(pcad_chain *ch, int row0, int nrows, const uint8_t *src_dev,
                                       int src_pitch);
 
-/* Block until the chain's queued work is done. */
+/* Block until the chain's queued work is done (PCAD_ETIMEOUT: a bounded wait
+ * gave up). */
 pcad_status pcad_chain_sync(pcad_chain *ch);
 
 /* Copy the current sample (the paper's retrieved image is the last sample,

@@ -268,7 +268,7 @@ struct pcad_chain {
     unsigned long long *xch = nullptr;   // tile-resident sweeps: border exchange (nullptr: not taken)
     TileKind tkind;
     TilePlan tplan{};
-    bool tile_ran = false;               // a tile-resident launch was issued: sync reads err
+    bool waits = false;                  // a launch with bounded waits was issued: err may be set
     void *track_block = nullptr;
 };
 
@@ -537,8 +537,8 @@ pcad_status issue_sweeps(pcad_chain *ch, int off0, int n, int &cur, cudaStream_t
         L.job[0].x1 = ch->x[out];
         L.job[0].xch = ch->xch;
         L.job[0].tg = ch->tplan.tg;
+        ch->waits = true;
         CUDA_TRY(launch_tile(ch->tkind, L, ch->tplan.ctas, st));
-        ch->tile_ran = true;
         cur = out;
         return PCAD_OK;
     }
@@ -546,6 +546,7 @@ pcad_status issue_sweeps(pcad_chain *ch, int off0, int n, int &cur, cudaStream_t
         // tensor-core wavefront: all n sweeps in one launch, or one launch
         // per sweep when every sweep's state is needed (energy tracking)
         const int per = ch->track.trace ? 1 : n;
+        ch->waits = true;
         for (int k = 0; k < n; k += per) {
             a.sweep_off = (uint32_t)(off0 + k);
             CUDA_TRY(cudaMemsetAsync(ch->wave, 0,
@@ -566,6 +567,7 @@ pcad_status issue_sweeps(pcad_chain *ch, int off0, int n, int &cur, cudaStream_t
         return PCAD_OK;
     }
     if (uses_winw(ch) && n > 0) {
+        ch->waits = true;
         a.sweep_off = (uint32_t)off0;
         CUDA_TRY(cudaMemsetAsync(ch->wave, 0, (size_t)(ch->wave_tiles + 1) * sizeof(unsigned int),
                                  st));
@@ -582,6 +584,7 @@ pcad_status issue_sweeps(pcad_chain *ch, int off0, int n, int &cur, cudaStream_t
     }
     if (uses_wave(ch) && n > 0) {
         // one persistent launch for all n sweeps: counters zeroed first
+        ch->waits = true;
         a.sweep_off = (uint32_t)off0;
         CUDA_TRY(cudaMemsetAsync(ch->wave, 0, (size_t)(ch->wave_tiles + 1) * sizeof(unsigned int),
                                  st));
@@ -595,6 +598,7 @@ pcad_status issue_sweeps(pcad_chain *ch, int off0, int n, int &cur, cudaStream_t
     int done = 0;
     if (ch->model.sampler == PCAD_SAMPLER_PCA && ch->tb_k > 0) {
         // temporally blocked: tb_k sweeps per launch, always into the other plane
+        ch->waits = true;
         for (; done + ch->tb_k <= n; done += ch->tb_k) {
             a.sweep_off = (uint32_t)(off0 + done);
             a.xin = ch->x[cur];
@@ -608,9 +612,10 @@ pcad_status issue_sweeps(pcad_chain *ch, int off0, int n, int &cur, cudaStream_t
         if (ch->model.sampler == PCAD_SAMPLER_PCA) {
             a.xin = ch->x[cur];
             a.xout = ch->x[cur ^ 1];
-            if (small_tma(ch))
+            if (small_tma(ch)) {
+                ch->waits = true;
                 CUDA_TRY(launch_pca_small_tma(ch->xmap[cur], ch->gmap, a, ch->err, st));
-            else if (uses_small(ch))
+            } else if (uses_small(ch))
                 CUDA_TRY(launch_pca_small(a, st));
             else if (uses_binary(ch))
                 CUDA_TRY(launch_pca_binary(a, st));
@@ -960,15 +965,16 @@ pcad_status pcad_chain_reset(pcad_chain *ch)
     return PCAD_OK;
 }
 
-pcad_status pcad_chain_sync(pcad_chain *ch)
+namespace {
+
+// Wait for the stream's work and report a wait of its kernels that gave up: the
+// planes, sums and energies are then undefined, so every call that hands them
+// back ends here.  The error flag comes behind the work in the stream (one round
+// trip: a copy after the synchronisation cost another 7 us).
+pcad_status wait_work(pcad_chain *ch)
 {
-    if (!ch)
-        return fail(PCAD_EINVAL, "chain is NULL");
-    // the error flag of the kernels that wait, behind their work in the stream
-    // (one round trip: a copy after the synchronisation cost another 7 us)
     int e = 0;
-    if (ch->tb_k > 0 || uses_tc(ch) || uses_wave(ch) || uses_winw(ch) || small_tma(ch) ||
-        ch->tile_ran)
+    if (ch->waits)
         CUDA_TRY(cudaMemcpyAsync(&e, ch->err, sizeof(int), cudaMemcpyDeviceToHost, ch->stream));
     CUDA_TRY(cudaStreamSynchronize(ch->stream));
     if (e == 2)
@@ -977,6 +983,15 @@ pcad_status pcad_chain_sync(pcad_chain *ch)
         return fail(PCAD_ETIMEOUT, "a bounded wait of the sweep kernel (tile load, MMA "
                                    "completion or wavefront dependency) gave up");
     return PCAD_OK;
+}
+
+}  // namespace
+
+pcad_status pcad_chain_sync(pcad_chain *ch)
+{
+    if (!ch)
+        return fail(PCAD_EINVAL, "chain is NULL");
+    return wait_work(ch);
 }
 
 namespace {
@@ -1092,7 +1107,9 @@ pcad_status pcad_chain_energy(pcad_chain *ch, double *energy, uint64_t *pair_sum
                            ch->mscratch, EnergyTrack{}, ch->tdev, 0, ch->stream));
     CUDA_TRY(cudaMemcpyAsync(res, ch->mscratch, sizeof(res), cudaMemcpyDeviceToHost,
                              ch->stream));
-    CUDA_TRY(cudaStreamSynchronize(ch->stream));
+    const pcad_status st = wait_work(ch);
+    if (st != PCAD_OK)
+        return st;
     *energy = res[0];
     if (pair_sum)
         *pair_sum = (uint64_t)res[1];
@@ -1153,7 +1170,9 @@ pcad_status pcad_chain_read_energies(pcad_chain *ch, double *host, int max, int 
         return fail(PCAD_ESTATE, "energy tracking is off");
     }
     unsigned int cnt = 0;
-    CUDA_TRY(cudaStreamSynchronize(ch->stream));
+    const pcad_status st = wait_work(ch);
+    if (st != PCAD_OK)
+        return st;
     CUDA_TRY(cudaMemcpy(&cnt, ch->track.n, sizeof(cnt), cudaMemcpyDeviceToHost));
     const int k = (int)cnt < max ? (int)cnt : max;
     if (k > 0)
@@ -1172,7 +1191,9 @@ pcad_status pcad_chain_read_min_state(pcad_chain *ch, uint8_t *host_out, int out
         return fail(PCAD_ESTATE, "energy tracking is off");
     double best = 0.0;
     unsigned long long bs = 0;
-    CUDA_TRY(cudaStreamSynchronize(ch->stream));
+    const pcad_status st = wait_work(ch);
+    if (st != PCAD_OK)
+        return st;
     CUDA_TRY(cudaMemcpy(&best, ch->track.best, sizeof(best), cudaMemcpyDeviceToHost));
     CUDA_TRY(cudaMemcpy(&bs, ch->track.best_sweep, sizeof(bs), cudaMemcpyDeviceToHost));
     if (bs == 0)
@@ -1334,8 +1355,7 @@ pcad_status pcad_chain_read_sample(pcad_chain *ch, uint8_t *host_out, int out_pi
         return fail(PCAD_EINVAL, "out_pitch < W");
     CUDA_TRY(read_labels(host_out, out_pitch, ch->x[ch->cur], ch->pitch, ch->H, ch->W, ch->fplane,
                          ch->stream));
-    CUDA_TRY(cudaStreamSynchronize(ch->stream));
-    return PCAD_OK;
+    return wait_work(ch);
 }
 
 pcad_status pcad_chain_read_sample_dev(pcad_chain *ch, uint8_t *dev_out, int out_pitch)
@@ -1359,8 +1379,7 @@ pcad_status pcad_chain_read_mean(pcad_chain *ch, float *host_out)
     CUDA_TRY(launch_mean(ch->acc, (float)ch->n_acc, ch->fplane, n, ch->stream));
     CUDA_TRY(cudaMemcpyAsync(host_out, ch->fplane, n * sizeof(float), cudaMemcpyDeviceToHost,
                              ch->stream));
-    CUDA_TRY(cudaStreamSynchronize(ch->stream));
-    return PCAD_OK;
+    return wait_work(ch);
 }
 
 pcad_status pcad_chain_write_sample(pcad_chain *ch, const uint8_t *host_in, int in_pitch)
@@ -1428,7 +1447,9 @@ pcad_status pcad_chain_metrics(pcad_chain *ch, const uint8_t *clean_host, int cl
     double res[2];
     CUDA_TRY(cudaMemcpyAsync(res, ch->mscratch + 8, sizeof(res), cudaMemcpyDeviceToHost,
                              ch->stream));
-    CUDA_TRY(cudaStreamSynchronize(ch->stream));
+    const pcad_status st = wait_work(ch);
+    if (st != PCAD_OK)
+        return st;
     if (psnr_db)
         *psnr_db = res[0];
     if (ssim)
@@ -1518,7 +1539,9 @@ pcad_status pcad_chain_export(pcad_chain *ch, void *host_blob, size_t *bytes)
     CUDA_TRY(read_labels(hx + n, ch->W, ch->g, ch->pitch, ch->H, ch->W, ch->fplane, ch->stream));
     CUDA_TRY(cudaMemcpyAsync(b + sizeof(h) + 2 * n, ch->acc, n * sizeof(float),
                              cudaMemcpyDeviceToHost, ch->stream));
-    CUDA_TRY(cudaStreamSynchronize(ch->stream));
+    st = wait_work(ch);
+    if (st != PCAD_OK)
+        return st;
     *bytes = need;
     return PCAD_OK;
 }
