@@ -457,13 +457,16 @@ void pcad_batch_destroy(pcad_batch *b);
 /* -------------------------------------------------------------- server
  * Continuous batching of denoising requests (no counterpart in the paper:
  * a serving loop around the sweep of Section 5.2).  Submitted requests are
- * admitted into slots as slots free up and their device memory fits the HBM
- * budget; every pcad_server_step chooses the requests to run, advances them
- * by one slice of sweeps in shared launches, and retires the requests whose
- * sweep budget is spent (their sample and posterior mean are copied to host
- * memory held by the server until polled).  State and sweep counters stay
- * on the device between slices; a request's results do not depend on what
- * else was running, nor on the policy below. */
+ * admitted into slots as slots free up and their planes, sums and model tables
+ * fit the HBM budget; memory that only makes a slot's sweeps faster (border
+ * exchange, prefix tables) is taken from what is left of it and given back for
+ * the next request, so all of a slot's memory lies within the budget.  Every
+ * pcad_server_step chooses the requests to run, advances them by one slice of
+ * sweeps in shared launches, and retires the requests whose sweep budget is
+ * spent (their sample and posterior mean are copied to host memory held by the
+ * server until polled).  State and sweep counters stay on the device between
+ * slices; a request's results do not depend on what else was running, nor on
+ * the policy below. */
 typedef struct pcad_server pcad_server;
 
 /* Scheduling policy.  PCAD_SERVE_FIFO: admit first come first served and
@@ -504,6 +507,8 @@ pcad_status pcad_server_step(pcad_server *sv, int slice_sweeps, int *n_active, i
  * forgets the request. */
 pcad_status pcad_server_poll(pcad_server *sv, uint64_t id, int *state, uint8_t *sample_out,
                              float *mean_out);
+/* *hbm_used: device memory of the admitted requests' slots (at most the
+ * budget), slices run so far, FP64 re-draws of the slots. */
 pcad_status pcad_server_info(pcad_server *sv, size_t *hbm_used, uint64_t *slices,
                              uint64_t *fp64_draws);
 void pcad_server_destroy(pcad_server *sv);

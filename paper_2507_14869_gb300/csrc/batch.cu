@@ -135,31 +135,57 @@ size_t slot_bytes(const pcad_job &j)
 }
 
 // Device memory of a slot beside its block: the segment draw's prefix tables
-// and the border exchange of its tile-resident sweeps (null: not its models,
-// or too many sites).  Not part of the HBM accounting: at most 18 KB and 4
-// bytes a site of images up to kTileMaxSites.
+// (18 KB) and the border exchange of its tile-resident sweeps (4 bytes a site).
+// Optional: a slot without it runs the kernels that need neither, with the same
+// results.
 struct SlotSide {
     float *stab = nullptr;
     unsigned long long *xch = nullptr;
 };
 
-size_t side_bytes(const pcad_job &j, size_t &stab, size_t &xch)
+// Chains the windowed sweep takes run it as their own launches, as the
+// chain API does for such images: from kWinBigBlocks blocks of 4 x 32 sites
+// per multiprocessor one launch per sweep, from kWinWaveBlocks one
+// wavefront launch per slice (on GB300 1.3-1.5x the tensor-core sweep
+// there); planes by the device sweep counter, budget-aware.
+constexpr long kWinBigBlocks = 100;
+constexpr long kWinWaveBlocks = 8;
+
+int device_sms()
 {
-    const int T = j.model.pair == PCAD_PAIR_POTTS ? 1 : j.model.pair_T;
+    int sms = 0, dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess)
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
+// What a slot of this job can use: tables if its labels take the segment draw,
+// the exchange if tile_set_build may take it.  fixed: the coefficients stay
+// (the server); those of a batch's chains may change (c < 0 and back).
+size_t side_bytes(const pcad_job &j, bool fixed, size_t &stab, size_t &xch)
+{
     DevModel m{};
     m.L = j.model.L;
     m.nbhd = j.model.nbhd;
-    m.T = T;
-    stab = seg_structure(m) ? al((size_t)seg_table_floats() * sizeof(float)) : 0;
-    xch = (long long)j.H * j.W <= kTileMaxSites ? al(tile_xch_bytes(j.H, j.W)) : 0;
+    m.T = j.model.pair == PCAD_PAIR_POTTS ? 1 : j.model.pair_T;
+    stab = xch = 0;
+    if (fixed && m.L > 2 && j.model.pair_coef < 0.0f)
+        return 0;
+    const long long sites = (long long)j.H * j.W;
+    const bool segments = m.L > kSmallMaxLabels && seg_structure(m);
+    if (segments)
+        stab = al((size_t)seg_table_floats() * sizeof(float));
+    if (segments ? sites < kWinWaveBlocks * 128 * device_sms()
+                 : m.L <= kSmallMaxLabels && sites <= kTileMaxSites)
+        xch = al(tile_xch_bytes(j.H, j.W));
     return stab + xch;
 }
 
 // A slot's side memory at `mem` (side_bytes of it), exchange words cleared.
-pcad_status side_init(const pcad_job &j, void *mem, cudaStream_t s, SlotSide &sd)
+pcad_status side_init(const pcad_job &j, bool fixed, void *mem, cudaStream_t s, SlotSide &sd)
 {
     size_t stab = 0, xch = 0;
-    side_bytes(j, stab, xch);
+    side_bytes(j, fixed, stab, xch);
     sd.stab = stab ? (float *)mem : nullptr;
     sd.xch = xch ? (unsigned long long *)((char *)mem + stab) : nullptr;
     if (xch)
@@ -341,14 +367,6 @@ struct TcGroup {
     int nc_max = 0;
     WaveBuf wb;
 };
-
-// Chains the windowed sweep takes run it as their own launches, as the
-// chain API does for such images: from kWinBigBlocks blocks of 4 x 32 sites
-// per multiprocessor one launch per sweep, from kWinWaveBlocks one
-// wavefront launch per slice (on GB300 1.3-1.5x the tensor-core sweep
-// there); planes by the device sweep counter, budget-aware.
-constexpr long kWinBigBlocks = 100;
-constexpr long kWinWaveBlocks = 8;
 
 struct TcSet {
     std::vector<TcGroup> groups;
@@ -1314,14 +1332,11 @@ pcad_status pcad_batch_create(const pcad_job *jobs, int n, int autotune, void *c
     for (int i = 0; i < n; ++i) {
         size_t u = 0, v = 0;
         soff[i] = stotal;
-        stotal += side_bytes(jobs[i], u, v);
+        stotal += side_bytes(jobs[i], false, u, v);
     }
-    if (stotal > 0 &&
-        (e = cudaMallocAsync(&b->side_block, stotal, b->stream)) != cudaSuccess) {
-        b->side_block = nullptr;
+    if (stotal > 0 && cudaMallocAsync(&b->side_block, stotal, b->stream) != cudaSuccess) {
+        b->side_block = nullptr;   // the chains run without
         cudaGetLastError();
-        return bail(set_error(e == cudaErrorMemoryAllocation ? PCAD_ENOMEM : PCAD_ECUDA,
-                              cudaGetErrorString(e)));
     }
     e = cudaMemsetAsync(base + off_ctr, 0, al(n * 16), b->stream);
     if (e == cudaSuccess)
@@ -1330,8 +1345,9 @@ pcad_status pcad_batch_create(const pcad_job *jobs, int n, int autotune, void *c
         return bail(set_error(PCAD_ECUDA, cudaGetErrorString(e)));
     for (int i = 0; i < n; ++i) {
         const int pitch = (jobs[i].W + 15) / 16 * 16;
-        pcad_status st =
-            side_init(jobs[i], (char *)b->side_block + soff[i], b->stream, b->side[i]);
+        pcad_status st = PCAD_OK;
+        if (b->side_block)
+            st = side_init(jobs[i], false, (char *)b->side_block + soff[i], b->stream, b->side[i]);
         if (st == PCAD_OK)
             st = init_slot(jobs[i], base, mem[i], pitch, b->d_t + i, b->d_budget + i, fp64 + i,
                            b->side[i], b->stream, b->desc[i]);
@@ -1568,7 +1584,8 @@ struct Request {
     uint64_t t = 0;              // sweeps done (host mirror)
     size_t bytes = 0;
     void *mem = nullptr;
-    void *side = nullptr;        // its slot's side memory
+    void *side = nullptr;        // its slot's side memory, if it holds any
+    size_t side_bytes = 0;
     double t_submit = 0.0;       // seconds (steady clock)
     double unit_cost = 0.0;      // estimated seconds per site-update
     std::vector<uint8_t> sample;
@@ -1597,7 +1614,8 @@ double unit_cost(const pcad_model &m)
 
 struct pcad_server {
     int max_slots = 0;
-    size_t budget = 0, used = 0;
+    size_t budget = 0, used = 0;  // used: the slots' blocks
+    size_t side_used = 0;         // their side memory
     cudaStream_t stream = nullptr;
     void *ctl = nullptr;          // descriptors, counters, grab
     SlotDesc *d_slots = nullptr;
@@ -1639,23 +1657,70 @@ int free_slot(const pcad_server *sv)
     return -1;
 }
 
+// Take back the side memory of an admitted request (behind the sweeps that use
+// it, in stream order); its next slices run without.
+pcad_status drop_side(pcad_server *sv, Request &rq)
+{
+    SlotDesc &d = sv->desc[rq.slot];
+    d.m.stab = nullptr;
+    B_TRY(cudaMemcpyAsync(sv->d_slots + rq.slot, &d, sizeof(d), cudaMemcpyHostToDevice,
+                          sv->stream));
+    sv->side[rq.slot] = SlotSide{};
+    sv->items_dirty = true;   // launches hold its pointers
+    sv->side_used -= rq.side_bytes;
+    void *p = rq.side;
+    rq.side = nullptr;
+    rq.side_bytes = 0;
+    B_TRY(cudaFreeAsync(p, sv->stream));
+    return PCAD_OK;
+}
+
+// Take back side memory until the slots' memory leaves `bytes` of the budget.
+pcad_status make_room(pcad_server *sv, size_t bytes)
+{
+    for (int i = sv->max_slots - 1; i >= 0 && sv->side_used > 0; --i) {
+        if (sv->used + sv->side_used + bytes <= sv->budget)
+            break;
+        if (sv->slot_req[i] == 0 || !sv->reqs[sv->slot_req[i]].side)
+            continue;
+        pcad_status st = drop_side(sv, sv->reqs[sv->slot_req[i]]);
+        if (st != PCAD_OK)
+            return st;
+    }
+    return PCAD_OK;
+}
+
 // Give request rq (pending, taken off the queue by the caller) slot `slot`
-// and its device memory, copy its observation and initialise its state.
+// and its device memory, copy its observation and initialise its state.  The
+// block decides whether a request is admitted (the callers compare it with the
+// budget and the other blocks); side memory takes what the blocks leave.
 pcad_status admit_one(pcad_server *sv, Request &rq, int slot)
 {
+    pcad_status rs = make_room(sv, rq.bytes);
+    if (rs != PCAD_OK)
+        return rs;
     cudaError_t e = cudaMallocAsync(&rq.mem, rq.bytes, sv->stream);
+    if (e == cudaErrorMemoryAllocation && sv->side_used > 0) {
+        cudaGetLastError();
+        rs = make_room(sv, sv->budget);   // all of it
+        if (rs != PCAD_OK)
+            return rs;
+        B_TRY(cudaStreamSynchronize(sv->stream));
+        e = cudaMallocAsync(&rq.mem, rq.bytes, sv->stream);
+    }
     if (e != cudaSuccess) {
+        rq.mem = nullptr;
         cudaGetLastError();
         return set_error(PCAD_ENOMEM, cudaGetErrorString(e));
     }
     size_t u = 0, v = 0;
-    const size_t sbytes = side_bytes(rq.job, u, v);
-    if (sbytes > 0 && (e = cudaMallocAsync(&rq.side, sbytes, sv->stream)) != cudaSuccess) {
+    rq.side_bytes = side_bytes(rq.job, true, u, v);
+    if (rq.side_bytes > 0 &&
+        (sv->used + sv->side_used + rq.bytes + rq.side_bytes > sv->budget ||
+         cudaMallocAsync(&rq.side, rq.side_bytes, sv->stream) != cudaSuccess)) {
         rq.side = nullptr;
+        rq.side_bytes = 0;
         cudaGetLastError();
-        cudaFreeAsync(rq.mem, sv->stream);
-        rq.mem = nullptr;
-        return set_error(PCAD_ENOMEM, cudaGetErrorString(e));
     }
     const int pitch = (rq.job.W + 15) / 16 * 16;
     SlotMem sm = job_layout(rq.job, pitch, 0);
@@ -1663,7 +1728,10 @@ pcad_status admit_one(pcad_server *sv, Request &rq, int slot)
     j.g_host = rq.g.data();
     j.g_pitch = rq.job.W;
     SlotDesc d{};
-    pcad_status st = side_init(j, rq.side, sv->stream, sv->side[slot]);
+    pcad_status st = PCAD_OK;
+    sv->side[slot] = SlotSide{};
+    if (rq.side)
+        st = side_init(j, true, rq.side, sv->stream, sv->side[slot]);
     if (st == PCAD_OK)
         st = init_slot(j, (char *)rq.mem, sm, pitch, sv->d_t + slot, sv->d_budget + slot,
                        sv->d_fp64 + slot, sv->side[slot], sv->stream, d);
@@ -1679,6 +1747,7 @@ pcad_status admit_one(pcad_server *sv, Request &rq, int slot)
     sv->desc[slot] = d;
     sv->slot_req[slot] = rq.id;
     sv->used += rq.bytes;
+    sv->side_used += rq.side_bytes;
     sv->active_sites += (size_t)rq.job.H * rq.job.W;
     rq.slot = slot;
     rq.state = 1;
@@ -2019,6 +2088,7 @@ pcad_status pcad_server_step(pcad_server *sv, int slice_sweeps, int *n_active, i
             rq.side = nullptr;
             sv->side[i] = SlotSide{};
             sv->used -= rq.bytes;
+            sv->side_used -= rq.side_bytes;
             sv->active_sites -= (size_t)d.H * d.W;
             sv->slot_req[i] = 0;
             rq.state = 2;
@@ -2080,7 +2150,7 @@ pcad_status pcad_server_info(pcad_server *sv, size_t *hbm_used, uint64_t *slices
     if (!sv)
         return set_error(PCAD_EINVAL, "server is NULL");
     if (hbm_used)
-        *hbm_used = sv->used;
+        *hbm_used = sv->used + sv->side_used;
     if (slices)
         *slices = sv->slices;
     if (fp64_draws) {
