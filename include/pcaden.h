@@ -431,7 +431,7 @@ pcad_status pcad_batch_set_model(pcad_batch *b, int i, const pcad_model *m);
 /* Restart every chain from its observation (asynchronous). */
 pcad_status pcad_batch_reset(pcad_batch *b);
 /* Wait for the batch's queued work.  PCAD_ETIMEOUT: a bounded wait inside a
- * wavefront launch gave up (the batch's results are invalid). */
+ * launch gave up (the batch's results are invalid until pcad_batch_reset). */
 pcad_status pcad_batch_sync(pcad_batch *b);
 /* Choose the tiling: tile_rows a multiple of 4 in [4, 64], order 0 (image
  * order), 1 (costliest first) or 2 (wavefront, one launch per 16 sweeps).

@@ -1175,6 +1175,8 @@ pcad_status batch_reset_state(pcad_batch *b)
     }
     B_TRY(cudaMemsetAsync(b->d_t, 0, b->n * sizeof(uint32_t), b->stream));
     B_TRY(cudaMemsetAsync(b->d_fp64, 0, b->n * sizeof(unsigned long long), b->stream));
+    // a wait that gave up before the reset: its flag would end every later wait
+    B_TRY(cudaMemsetAsync(b->d_err, 0, sizeof(int), b->stream));
     b->t = 0;
     return PCAD_OK;
 }
@@ -1568,6 +1570,12 @@ void pcad_batch_destroy(pcad_batch *b)
 }
 
 }  // extern "C"
+
+// The device flag of a batch's bounded waits (tests set it: no public call makes
+// a batch's wait run out).
+namespace pcad {
+int *batch_error_flag(pcad_batch *b) { return b->d_err; }
+}  // namespace pcad
 
 // ------------------------------------------------------------------ server
 
