@@ -1045,7 +1045,7 @@ namespace {
 pcad_status batch_set_items(pcad_batch *b, int rows, int lpt, int slice)
 {
     std::vector<int> all(b->n), not_res, not_tile, others, active;
-    b->items_dirty = false;
+    b->items_dirty = true;   // until all of it is in place: a failure half way is built again
     for (int i = 0; i < b->n; ++i)
         all[i] = i;
     // small two-label chains run resident, mid-size chains tile-resident,
@@ -1087,6 +1087,7 @@ pcad_status batch_set_items(pcad_batch *b, int rows, int lpt, int slice)
         cudaGraphExecDestroy(b->graph);
         b->graph = nullptr;
     }
+    b->items_dirty = false;
     return PCAD_OK;
 }
 
