@@ -266,6 +266,7 @@ struct pcad_chain {
     int wave_tiles = 0;
     int sms = 0;                  // multiprocessors of the chain's device
     unsigned long long *xch = nullptr;   // tile-resident sweeps: border exchange (nullptr: not taken)
+    size_t clear_bytes = 0;              // the sums and, behind them, xch
     TileKind tkind;
     TilePlan tplan{};
     bool waits = false;                  // a launch with bounded waits was issued: err may be set
@@ -383,6 +384,21 @@ bool uses_wave(const pcad_chain *ch);
 //   kTileSegGibbsSites sites on Gibbs too.
 constexpr long long kTileSegGibbsSites = 300000;
 
+// The images of that rule: a chain holds an exchange buffer for these only.
+bool tile_sizes(const TileKind &k, const DevModel &m, int H, int W, int sms)
+{
+    const long long sites = (long long)H * W;
+    if (k.draw == TileKind::kBinary)   // (the smallest run resident)
+        return !resident_fits(m.L, m.nbhd, H, W) &&
+               sites <= (k.gibbs ? kTileMaxSites : kTileMaxBinarySites);
+    if (k.draw == TileKind::kSmall)
+        return sites <= kTileMaxSites;
+    const long long blocks = (long long)((W + 31) / 32) * ((H + 3) / 4);
+    if (pca_tc_auto(m) && blocks < 8LL * sms)
+        return false;   // AUTO's tensor-core images
+    return sites < (k.gibbs ? kTileSegGibbsSites : 8LL * 128 * sms);
+}
+
 bool uses_tile(const pcad_chain *ch)
 {
     if (!ch->xch || ch->tb_k > 0 || ch->track.trace || uses_resident(ch))
@@ -393,14 +409,7 @@ bool uses_tile(const pcad_chain *ch)
         return false;
     if (ch->kernel == PCAD_KERNEL_SMALL)
         return k.draw == TileKind::kSmall && !gibbs;
-    if (ch->kernel != PCAD_KERNEL_AUTO)
-        return false;
-    if (k.draw != TileKind::kSegment)
-        return true;
-    if (pca_tc_auto(ch->dm) && win_auto_mode(ch) == 0)
-        return false;   // AUTO's tensor-core images
-    const long long sites = (long long)ch->H * ch->W;
-    return sites < (gibbs ? kTileSegGibbsSites : 8LL * 128 * ch->sms);
+    return ch->kernel == PCAD_KERNEL_AUTO;
 }
 
 // Runs of fewer sweeps keep the per-sweep kernels: a tile-resident launch reads
@@ -733,32 +742,41 @@ pcad_status create_common(const uint8_t *g_src, bool g_on_device, int H, int W, 
     int sms = 0, dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess)
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // tile-resident sweeps: the models of tile_kind, but those whose small
-    // images AUTO gives the tensor-core sweep
     const bool gibbs = m->sampler != PCAD_SAMPLER_PCA;
     TileKind tkind;
     TilePlan tplan{};
-    const bool tile = tile_kind(tabs.dm, gibbs, tkind) &&
-                      (long long)H * W <= (tkind.draw == TileKind::kBinary && !gibbs
-                                               ? kTileMaxBinarySites : kTileMaxSites) &&
-                      tile_plan(tkind, H, W, sms, tplan);
-    const size_t xbytes = tile ? align_up(tile_xch_bytes(H, W), 256) : 0;
+    bool tile = tile_kind(tabs.dm, gibbs, tkind) && tile_sizes(tkind, tabs.dm, H, W, sms) &&
+                tile_plan(tkind, H, W, sms, tplan);
     const size_t sbytes =
         seg_structure(tabs.dm) ? align_up(seg_table_floats() * sizeof(float), 256) : 0;
-    const size_t total =
-        sbytes + xbytes + 3 * plane + 2 * fbytes + cbytes + tbytes + wbytes + pbytes + bbytes + obytes + misc;
-    cudaError_t e = cudaMallocAsync(&ch->block, total, ch->stream);
+    const size_t own = sbytes + 3 * plane + 2 * fbytes + cbytes + tbytes + wbytes + pbytes + bbytes +
+                       obytes + misc;
+    size_t xbytes = tile ? align_up(tile_xch_bytes(H, W), 256) : 0;
+    cudaError_t e = cudaMallocAsync(&ch->block, own + xbytes, ch->stream);
+    if (e == cudaErrorMemoryAllocation && tile) {   // the chain runs without
+        cudaGetLastError();
+        tile = false;
+        xbytes = 0;
+        e = cudaMallocAsync(&ch->block, own, ch->stream);
+    }
     if (e != cudaSuccess) {
         delete ch;
         cudaGetLastError();
         return fail(e == cudaErrorMemoryAllocation ? PCAD_ENOMEM : PCAD_ECUDA,
-                    "device allocation of %zu bytes: %s", total, cudaGetErrorString(e));
+                    "device allocation of %zu bytes: %s", own + xbytes, cudaGetErrorString(e));
     }
     char *p = (char *)ch->block;
     ch->x[0] = (uint8_t *)p; p += plane;
     ch->x[1] = (uint8_t *)p; p += plane;
     ch->g = (uint8_t *)p; p += plane;
     ch->acc = (float *)p; p += fbytes;
+    if (tile) {   // behind the sums: cleared with them
+        ch->xch = (unsigned long long *)p;
+        p += xbytes;
+        ch->tkind = tkind;
+        ch->tplan = tplan;
+    }
+    ch->clear_bytes = fbytes + xbytes;
     ch->fplane = (float *)p; p += fbytes;
     ch->clean = (uint8_t *)p; p += cbytes;
     ch->ta64 = (double *)p; p += align_up(kTable * sizeof(double), 256);
@@ -772,12 +790,6 @@ pcad_status create_common(const uint8_t *g_src, bool g_on_device, int H, int W, 
     if (sbytes) {
         ch->stab = (float *)p;
         p += sbytes;
-    }
-    if (tile) {
-        ch->xch = (unsigned long long *)p;
-        p += xbytes;
-        ch->tkind = tkind;
-        ch->tplan = tplan;
     }
     ch->sms = sms;
     ch->tdev = (uint32_t *)p;
@@ -799,7 +811,7 @@ pcad_status create_common(const uint8_t *g_src, bool g_on_device, int H, int W, 
         e = cudaMemcpy2DAsync(ch->x[0], ch->pitch, ch->g, ch->pitch, W, H,
                               cudaMemcpyDeviceToDevice, ch->stream);
     if (e == cudaSuccess)
-        e = cudaMemsetAsync(ch->acc, 0, fbytes, ch->stream);
+        e = cudaMemsetAsync(ch->acc, 0, ch->clear_bytes, ch->stream);   // (no tag is 0)
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(ch->ta64, tabs.ta64, sizeof(tabs.ta64), cudaMemcpyHostToDevice,
                             ch->stream);
@@ -811,8 +823,6 @@ pcad_status create_common(const uint8_t *g_src, bool g_on_device, int H, int W, 
                             cudaMemcpyHostToDevice, ch->stream);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(ch->tdev, 0, misc, ch->stream);
-    if (e == cudaSuccess && tile)
-        e = cudaMemsetAsync(ch->xch, 0, xbytes, ch->stream);   // no tag is 0
     if (e == cudaSuccess && m->L <= kSmallMaxLabels)
         e = launch_ptab(tabs.dm.T, ch->ptab, ch->stream);
     if (e == cudaSuccess && (pca_tc_eligible(tabs.dm) || pca_win_eligible(tabs.dm)))
@@ -949,14 +959,12 @@ pcad_status pcad_chain_reset(pcad_chain *ch)
 {
     if (!ch)
         return fail(PCAD_EINVAL, "chain is NULL");
-    const size_t n = (size_t)ch->H * ch->W;
     CUDA_TRY(cudaMemcpy2DAsync(ch->x[0], ch->pitch, ch->g, ch->pitch, ch->W, ch->H,
                                cudaMemcpyDeviceToDevice, ch->stream));
-    CUDA_TRY(cudaMemsetAsync(ch->acc, 0, n * sizeof(float), ch->stream));
+    // the sums, and the border words: the sweep index, hence their tags, starts again
+    CUDA_TRY(cudaMemsetAsync(ch->acc, 0, ch->clear_bytes, ch->stream));
     CUDA_TRY(cudaMemsetAsync(ch->tdev, 0, 16, ch->stream));
     CUDA_TRY(cudaMemsetAsync(ch->err, 0, sizeof(int), ch->stream));
-    if (ch->xch)   // the sweep index, hence the border words' tags, starts again
-        CUDA_TRY(cudaMemsetAsync(ch->xch, 0, tile_xch_bytes(ch->H, ch->W), ch->stream));
     ch->cur = 0;
     ch->t = 0;
     ch->n_acc = 0;
