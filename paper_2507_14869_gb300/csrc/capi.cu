@@ -413,18 +413,28 @@ bool uses_tile(const pcad_chain *ch)
 }
 
 // Runs of fewer sweeps keep the per-sweep kernels: a tile-resident launch reads
-// the planes, waits for all its blocks and writes the sums back.  us per sweep
-// (tile-resident / per-sweep) of calls of 1, 2 and 4 sweeps: two labels 600^2
-// 13.8 / 9.3, 8.7 / 7.7, 5.4 / 6.9; L = 16 1024^2 24.8 / 20.8, 18.4 / 19.3; L = 24
-// 256^2 13.6 / 11.3, 8.5 / 9.8; Gibbs (several launches per sweep) L = 5 256^2
-// 13.5 / 24.3, L = 256 512^2 26 / 45.
+// the planes, waits for all its blocks and writes the sums back.  us per call, run
+// and sync (tile-resident / per-sweep):
+//   two labels 300^2 3 sweeps 33 / 33, 4 34 / 36; 600^2 4 46 / 33, 6 47 / 40, 8
+//   47 / 48; 1000^2 4 49 / 41, 8 63 / 63; 2000^2 8 119 / 111, 16 193 / 202; 2043 x
+//   3001 4 108 / 92, 16 263 / 316;
+//   L = 9, 8 neighbours 256^2 2 35 / 29, 3 34 / 35; 700^2 4 61 / 57, 5 71 / 67, 6
+//   75 / 77; L = 16 1000^2 3 71 / 58, 5 88 / 87; L = 64 256^2 2 33 / 33, 3 37 / 42;
+//   where the per-sweep kernel is the wavefront: L = 16 512^2 2 35 / 48, 700^2 2
+//   46 / 53;
+//   Gibbs (several launches per sweep) 1 sweep: L = 5 256^2 14 / 24, L = 256 512^2
+//   26 / 45.
 int tile_min_sweeps(const pcad_chain *ch)
 {
     if (ch->model.sampler != PCAD_SAMPLER_PCA)
         return 1;
-    if (ch->tplan.tg.compact)
-        return kTileCompactSweeps;
-    return ch->tkind.draw == TileKind::kBinary ? 4 : 2;
+    const long long sites = (long long)ch->H * ch->W;
+    if (ch->tkind.draw == TileKind::kBinary)
+        return ch->tplan.tg.compact || sites >= (1 << 21) ? kTileCompactSweeps
+                                                          : (sites >= (1 << 17) ? 8 : 4);
+    if (uses_wave(ch))
+        return 2;
+    return sites >= (1 << 18) ? 5 : 3;
 }
 
 // Unblocked sweeps (PCA or Gibbs) on the CUDA-core windowed kernels: on
