@@ -181,11 +181,11 @@ size_t side_bytes(const pcad_job &j, bool fixed, size_t &stab, size_t &xch)
     return stab + xch;
 }
 
-// A slot's side memory at `mem` (side_bytes of it), exchange words cleared.
-pcad_status side_init(const pcad_job &j, bool fixed, void *mem, cudaStream_t s, SlotSide &sd)
+// A server slot's side memory at `mem` (side_bytes of it), exchange words cleared.
+pcad_status side_init(const pcad_job &j, void *mem, cudaStream_t s, SlotSide &sd)
 {
     size_t stab = 0, xch = 0;
-    side_bytes(j, fixed, stab, xch);
+    side_bytes(j, true, stab, xch);
     sd.stab = stab ? (float *)mem : nullptr;
     sd.xch = xch ? (unsigned long long *)((char *)mem + stab) : nullptr;
     if (xch)
@@ -1035,6 +1035,7 @@ struct pcad_batch {
     TileSet tile;                    // mid-size chains, tile-resident
     std::vector<SlotSide> side;
     void *side_block = nullptr;
+    size_t xch_bytes = 0;            // its border exchanges, at its start
     bool items_dirty = false;        // a model change may move a slot to another launch
     float tune_ms = 0.0f;
     cudaGraphExec_t graph = nullptr;
@@ -1171,9 +1172,9 @@ pcad_status batch_reset_state(pcad_batch *b)
         B_TRY(cudaMemcpy2DAsync(d.x[0], d.pitch, d.g, d.pitch, d.W, d.H, cudaMemcpyDeviceToDevice,
                                 b->stream));
         B_TRY(cudaMemsetAsync(d.acc, 0, (size_t)d.H * d.W * sizeof(float), b->stream));
-        if (b->side[i].xch)   // the sweep indices, hence the words' tags, start again
-            B_TRY(cudaMemsetAsync(b->side[i].xch, 0, tile_xch_bytes(d.H, d.W), b->stream));
     }
+    if (b->xch_bytes > 0)   // the sweep indices, hence the border words' tags, start again
+        B_TRY(cudaMemsetAsync(b->side_block, 0, b->xch_bytes, b->stream));
     B_TRY(cudaMemsetAsync(b->d_t, 0, b->n * sizeof(uint32_t), b->stream));
     B_TRY(cudaMemsetAsync(b->d_fp64, 0, b->n * sizeof(unsigned long long), b->stream));
     // a wait that gave up before the reset: its flag would end every later wait
@@ -1329,17 +1330,30 @@ pcad_status pcad_batch_create(const pcad_job *jobs, int n, int autotune, void *c
         delete b;
         return st;
     };
+    // the exchanges of all chains, then their prefix tables
     b->side.resize(n);
-    std::vector<size_t> soff(n);
+    std::vector<size_t> stabs(n), xchs(n);
     size_t stotal = 0;
     for (int i = 0; i < n; ++i) {
-        size_t u = 0, v = 0;
-        soff[i] = stotal;
-        stotal += side_bytes(jobs[i], false, u, v);
+        side_bytes(jobs[i], false, stabs[i], xchs[i]);
+        b->xch_bytes += xchs[i];
+        stotal += stabs[i] + xchs[i];
     }
     if (stotal > 0 && cudaMallocAsync(&b->side_block, stotal, b->stream) != cudaSuccess) {
         b->side_block = nullptr;   // the chains run without
         cudaGetLastError();
+        b->xch_bytes = 0;
+    }
+    if (b->side_block) {
+        char *x = (char *)b->side_block, *t = x + b->xch_bytes;
+        for (int i = 0; i < n; ++i) {
+            b->side[i].xch = xchs[i] ? (unsigned long long *)x : nullptr;
+            b->side[i].stab = stabs[i] ? (float *)t : nullptr;
+            x += xchs[i];
+            t += stabs[i];
+        }
+        if ((e = cudaMemsetAsync(b->side_block, 0, b->xch_bytes, b->stream)) != cudaSuccess)
+            return bail(set_error(PCAD_ECUDA, cudaGetErrorString(e)));
     }
     e = cudaMemsetAsync(base + off_ctr, 0, al(n * 16), b->stream);
     if (e == cudaSuccess)
@@ -1348,12 +1362,8 @@ pcad_status pcad_batch_create(const pcad_job *jobs, int n, int autotune, void *c
         return bail(set_error(PCAD_ECUDA, cudaGetErrorString(e)));
     for (int i = 0; i < n; ++i) {
         const int pitch = (jobs[i].W + 15) / 16 * 16;
-        pcad_status st = PCAD_OK;
-        if (b->side_block)
-            st = side_init(jobs[i], false, (char *)b->side_block + soff[i], b->stream, b->side[i]);
-        if (st == PCAD_OK)
-            st = init_slot(jobs[i], base, mem[i], pitch, b->d_t + i, b->d_budget + i, fp64 + i,
-                           b->side[i], b->stream, b->desc[i]);
+        pcad_status st = init_slot(jobs[i], base, mem[i], pitch, b->d_t + i, b->d_budget + i,
+                                   fp64 + i, b->side[i], b->stream, b->desc[i]);
         if (st != PCAD_OK)
             return bail(st);
         b->jobs.push_back(jobs[i]);
@@ -1740,7 +1750,7 @@ pcad_status admit_one(pcad_server *sv, Request &rq, int slot)
     pcad_status st = PCAD_OK;
     sv->side[slot] = SlotSide{};
     if (rq.side)
-        st = side_init(j, true, rq.side, sv->stream, sv->side[slot]);
+        st = side_init(j, rq.side, sv->stream, sv->side[slot]);
     if (st == PCAD_OK)
         st = init_slot(j, (char *)rq.mem, sm, pitch, sv->d_t + slot, sv->d_budget + slot,
                        sv->d_fp64 + slot, sv->side[slot], sv->stream, d);
