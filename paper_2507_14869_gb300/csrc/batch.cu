@@ -584,8 +584,10 @@ pcad_status small_set_build(SmallSet &ss, const std::vector<SlotDesc> &d,
         ss.bcap = std::max(ss.bin.size(), 2 * ss.bcap);
         B_TRY(cudaMallocAsync((void **)&ss.btabs, ss.bcap * bin_tab_entries() * sizeof(uint4), st));
     }
+    std::vector<BtabJob> bt;
     for (size_t p = 0; p < ss.bin.size(); ++p)
-        B_TRY(launch_btab(d[ss.bin[p]].m, ss.btabs + p * bin_tab_entries(), st));
+        bt.push_back(BtabJob{d[ss.bin[p]].m, ss.btabs + p * bin_tab_entries()});
+    B_TRY(launch_btabs(bt.data(), (int)bt.size(), st));
     if (ss.table_T.size() > ss.cap) {
         if (ss.tables)
             B_TRY(cudaFreeAsync(ss.tables, st));
@@ -752,7 +754,7 @@ pcad_status tile_set_build(TileSet &ts, const std::vector<SlotDesc> &d,
         ts.bcap = std::max(nbin, 2 * ts.bcap);
         B_TRY(cudaMallocAsync((void **)&ts.btabs, ts.bcap * bin_tab_entries() * sizeof(uint4), st));
     }
-    size_t bin = 0;
+    std::vector<BtabJob> bt;
     for (auto &gr : groups) {
         const TileKind k = gr.first;
         std::vector<int> &v = gr.second;
@@ -816,8 +818,8 @@ pcad_status tile_set_build(TileSet &ts, const std::vector<SlotDesc> &d,
             L.pack.err = err;
             for (size_t q = 0; q < jobs.size(); ++q) {
                 if (k.draw == TileKind::kBinary) {
-                    uint4 *t = ts.btabs + bin++ * bin_tab_entries();
-                    B_TRY(launch_btab(jobs[q].a.m, t, st));
+                    uint4 *t = ts.btabs + bt.size() * bin_tab_entries();
+                    bt.push_back(BtabJob{jobs[q].a.m, t});
                     jobs[q].a.m.btab = t;
                 }
                 L.pack.job[q] = jobs[q];
@@ -826,6 +828,7 @@ pcad_status tile_set_build(TileSet &ts, const std::vector<SlotDesc> &d,
             ts.launches.push_back(L);
         }
     }
+    B_TRY(launch_btabs(bt.data(), (int)bt.size(), st));
     return PCAD_OK;
 }
 
@@ -916,8 +919,10 @@ pcad_status res_set_build(ResSet &rs, const std::vector<SlotDesc> &d, const std:
         return PCAD_OK;
     B_TRY(cudaMemcpyAsync(rs.d_idx, idx.data(), idx.size() * sizeof(int), cudaMemcpyHostToDevice,
                           st));
+    std::vector<BtabJob> bt;
     for (size_t p = 0; p < idx.size(); ++p)
-        B_TRY(launch_btab(d[idx[p]].m, rs.tabs + p * res_tab_entries(), st));
+        bt.push_back(BtabJob{d[idx[p]].m, rs.tabs + p * res_tab_entries()});
+    B_TRY(launch_btabs(bt.data(), (int)bt.size(), st));
     return PCAD_OK;
 }
 

@@ -439,6 +439,12 @@ cudaError_t launch_resident(const SweepArgs &a, const uint8_t *x_in, uint8_t *x_
 // the model's FP32 draw and FP64 re-draw; btab_bytes() of device memory.
 int btab_bytes();
 cudaError_t launch_btab(const DevModel &m, uint4 *out, cudaStream_t s);
+// The tables of several models, in one launch for each 64 of a neighbourhood.
+struct BtabJob {
+    DevModel m;
+    uint4 *out;
+};
+cudaError_t launch_btabs(const BtabJob *jobs, int n, cudaStream_t s);
 // Batched form: whether a two-label chain of this size runs resident, its
 // shared memory, and one launch of `count` chains (slot indices idx[0..count),
 // all with nbhd neighbours, tables at tabs + b * btab_bytes()) for n sweeps
