@@ -193,10 +193,11 @@ pcad_status side_init(const pcad_job &j, void *mem, cudaStream_t s, SlotSide &sd
     return PCAD_OK;
 }
 
-// Build a slot: copy g, x0 <- g, acc <- 0, tables; fill the descriptor.
+// Build a slot: copy g, x0 <- g, acc <- 0, tables (the segment draw's: appended to
+// `seg`, launched by the caller); fill the descriptor.
 pcad_status init_slot(const pcad_job &j, char *base, const SlotMem &sm, int pitch,
                       uint32_t *tdev, const uint32_t *budget, unsigned long long *fp64,
-                      const SlotSide &sd, cudaStream_t s, SlotDesc &d)
+                      const SlotSide &sd, std::vector<SegTabJob> &seg, cudaStream_t s, SlotDesc &d)
 {
     double ta64[511];
     std::vector<double> pr64;
@@ -214,7 +215,7 @@ pcad_status init_slot(const pcad_job &j, char *base, const SlotMem &sm, int pitc
     dm.pr64 = (const double *)(base + sm.pr);
     dm.stab = seg_eligible(dm) ? sd.stab : nullptr;
     if (dm.stab)
-        B_TRY(launch_seg_table(dm, sd.stab, s));
+        seg.push_back(SegTabJob{dm, sd.stab});
     d = SlotDesc{};
     d.g = (const uint8_t *)(base + sm.g);
     d.x[0] = (uint8_t *)(base + sm.x0);
@@ -1365,17 +1366,20 @@ pcad_status pcad_batch_create(const pcad_job *jobs, int n, int autotune, void *c
         e = cudaMemsetAsync(b->d_err, 0, sizeof(int), b->stream);
     if (e != cudaSuccess)
         return bail(set_error(PCAD_ECUDA, cudaGetErrorString(e)));
+    std::vector<SegTabJob> seg;
     for (int i = 0; i < n; ++i) {
         const int pitch = (jobs[i].W + 15) / 16 * 16;
         pcad_status st = init_slot(jobs[i], base, mem[i], pitch, b->d_t + i, b->d_budget + i,
-                                   fp64 + i, b->side[i], b->stream, b->desc[i]);
+                                   fp64 + i, b->side[i], seg, b->stream, b->desc[i]);
         if (st != PCAD_OK)
             return bail(st);
         b->jobs.push_back(jobs[i]);
         b->jobs.back().g_host = nullptr;
     }
-    e = cudaMemcpyAsync(b->d_slots, b->desc.data(), n * sizeof(SlotDesc), cudaMemcpyHostToDevice,
-                        b->stream);
+    e = launch_seg_tables(seg.data(), (int)seg.size(), b->stream);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(b->d_slots, b->desc.data(), n * sizeof(SlotDesc),
+                            cudaMemcpyHostToDevice, b->stream);
     if (e != cudaSuccess)
         return bail(set_error(PCAD_ECUDA, cudaGetErrorString(e)));
     pcad_status st = autotune ? batch_autotune(b) : batch_set_items(b, 4, 1, kSlice);
@@ -1754,13 +1758,15 @@ pcad_status admit_one(pcad_server *sv, Request &rq, int slot)
     SlotDesc d{};
     pcad_status st = PCAD_OK;
     sv->side[slot] = SlotSide{};
+    std::vector<SegTabJob> seg;
     if (rq.side)
         st = side_init(j, rq.side, sv->stream, sv->side[slot]);
     if (st == PCAD_OK)
         st = init_slot(j, (char *)rq.mem, sm, pitch, sv->d_t + slot, sv->d_budget + slot,
-                       sv->d_fp64 + slot, sv->side[slot], sv->stream, d);
+                       sv->d_fp64 + slot, sv->side[slot], seg, sv->stream, d);
     if (st != PCAD_OK)
         return st;
+    B_TRY(launch_seg_tables(seg.data(), (int)seg.size(), sv->stream));
     const uint32_t zero = 0, bud = (uint32_t)rq.nsweeps;
     const unsigned long long z64 = 0;
     B_TRY(cudaMemcpyAsync(sv->d_t + slot, &zero, 4, cudaMemcpyHostToDevice, sv->stream));

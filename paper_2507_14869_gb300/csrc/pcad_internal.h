@@ -367,6 +367,12 @@ float seg_offset(const DevModel &m);   // DevModel::cbs of a model's coefficient
 bool seg_eligible(const DevModel &m);
 bool seg_structure(const DevModel &m);
 cudaError_t launch_seg_table(const DevModel &m, float *out, cudaStream_t s);
+// The tables of several models, in one launch for each 64.
+struct SegTabJob {
+    DevModel m;
+    float *out;
+};
+cudaError_t launch_seg_tables(const SegTabJob *jobs, int n, cudaStream_t s);
 cudaError_t launch_pca_seg(const SweepArgs &a, uint8_t *x0, uint8_t *x1,
                            const uint32_t *budget, cudaStream_t s);
 cudaError_t launch_gibbs_seg(const SweepArgs &a, int q, cudaStream_t s);

@@ -21,6 +21,8 @@
 //     persistent launch, items and waits as in win.cu's wavefront, one site
 //     per thread.  512^2: 9.4 us per sweep against 17.9 us (Gibbs 14.4 against
 //     26 us).
+#include <algorithm>
+
 #include "seg_draw.cuh"
 
 namespace pcad {
@@ -38,11 +40,20 @@ constexpr int kSegGibbsThreads = 32 * kSegGibbsWarps;
 constexpr int kSegwThreads = kSX * kSY;      // wavefront blocks
 constexpr double kBias = 3.9443045261050590e-31;   // 2^-101
 
-// Row blockIdx.x - 4 of the prefix tables, one thread per entry: FP64 terms
-// (the model's data factors times 2^(mu k d), mu the FP32 coefficient the
-// sweeps use), an FP64 scan, one rounding.
-__global__ void __launch_bounds__(kSegRow) seg_table_kernel(const DevModel m, float *out)
+// Row blockIdx.x - 4 of the prefix tables of job blockIdx.y, one thread per entry:
+// FP64 terms (the model's data factors times 2^(mu k d), mu the FP32 coefficient
+// the sweeps use), an FP64 scan, one rounding.
+template <int N>
+struct SegTabJobs {
+    SegTabJob job[N];
+};
+
+template <int N>
+__global__ void __launch_bounds__(kSegRow)
+    seg_table_kernel(const __grid_constant__ SegTabJobs<N> jobs)
 {
+    const DevModel &m = jobs.job[N > 1 ? blockIdx.y : 0].m;
+    float *const out = jobs.job[N > 1 ? blockIdx.y : 0].out;
     __shared__ double v[2][kSegRow];
     const int k = (int)blockIdx.x - 4, j = (int)threadIdx.x;
     const int d = j - 256;
@@ -483,9 +494,27 @@ bool seg_eligible(const DevModel &m)
 
 cudaError_t launch_seg_table(const DevModel &m, float *out, cudaStream_t st)
 {
-    if (!seg_eligible(m) || m.ta64 == nullptr)
-        return cudaErrorInvalidValue;
-    seg_table_kernel<<<kSegRows, kSegRow, 0, st>>>(m, out);
+    const SegTabJob j{m, out};
+    return launch_seg_tables(&j, 1, st);
+}
+
+cudaError_t launch_seg_tables(const SegTabJob *jobs, int n, cudaStream_t st)
+{
+    for (int i = 0; i < n; ++i)
+        if (!seg_eligible(jobs[i].m) || jobs[i].m.ta64 == nullptr)
+            return cudaErrorInvalidValue;
+    constexpr int kMost = 64;
+    for (int i = 0; i < n; i += kMost) {
+        const int k = n - i < kMost ? n - i : kMost;
+        if (k == 1) {
+            const SegTabJobs<1> one{{jobs[i]}};
+            seg_table_kernel<1><<<kSegRows, kSegRow, 0, st>>>(one);
+            continue;
+        }
+        SegTabJobs<kMost> many;
+        std::copy(jobs + i, jobs + i + k, many.job);
+        seg_table_kernel<kMost><<<dim3(kSegRows, k), kSegRow, 0, st>>>(many);
+    }
     return cudaGetLastError();
 }
 
