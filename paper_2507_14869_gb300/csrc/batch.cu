@@ -129,11 +129,6 @@ SlotMem job_layout(const pcad_job &j, int pitch, size_t base)
                        base);
 }
 
-size_t slot_bytes(const pcad_job &j)
-{
-    return job_layout(j, (int)((j.W + 15) / 16 * 16), 0).end;
-}
-
 // Device memory of a slot beside its block: the segment draw's prefix tables
 // (18 KB) and the border exchange of its tile-resident sweeps (4 bytes a site).
 // Optional: a slot without it runs the kernels that need neither, with the same
@@ -1610,6 +1605,7 @@ struct Request {
     bool running = false;        // admitted and in the current slice's run set
     int slot = -1;
     uint64_t t = 0;              // sweeps done (host mirror)
+    SlotMem sm{};                // its block's layout (from the model's tables: found once)
     size_t bytes = 0;
     void *mem = nullptr;
     void *side = nullptr;        // its slot's side memory, if it holds any
@@ -1751,7 +1747,6 @@ pcad_status admit_one(pcad_server *sv, Request &rq, int slot)
         cudaGetLastError();
     }
     const int pitch = (rq.job.W + 15) / 16 * 16;
-    SlotMem sm = job_layout(rq.job, pitch, 0);
     pcad_job j = rq.job;
     j.g_host = rq.g.data();
     j.g_pitch = rq.job.W;
@@ -1762,7 +1757,7 @@ pcad_status admit_one(pcad_server *sv, Request &rq, int slot)
     if (rq.side)
         st = side_init(j, rq.side, sv->stream, sv->side[slot]);
     if (st == PCAD_OK)
-        st = init_slot(j, (char *)rq.mem, sm, pitch, sv->d_t + slot, sv->d_budget + slot,
+        st = init_slot(j, (char *)rq.mem, rq.sm, pitch, sv->d_t + slot, sv->d_budget + slot,
                        sv->d_fp64 + slot, sv->side[slot], seg, sv->stream, d);
     if (st != PCAD_OK)
         return st;
@@ -2033,7 +2028,8 @@ pcad_status pcad_server_submit(pcad_server *sv, const pcad_job *job, int nsweeps
     rq.job = *job;
     rq.job.g_host = nullptr;
     rq.nsweeps = nsweeps;
-    rq.bytes = slot_bytes(*job);
+    rq.sm = job_layout(*job, (job->W + 15) / 16 * 16, 0);
+    rq.bytes = rq.sm.end;
     rq.t_submit = now_s();
     rq.unit_cost = unit_cost(job->model);
     if (rq.bytes > sv->budget)
