@@ -270,6 +270,8 @@ struct pcad_chain {
     TileKind tkind;
     TilePlan tplan{};
     bool waits = false;                  // a launch with bounded waits was issued: err may be set
+    int flag = 0, *flag_pin = nullptr;   // where a check copies err (flag_pin: pinned)
+    int checks = 0;
     void *track_block = nullptr;
 };
 
@@ -985,22 +987,45 @@ pcad_status pcad_chain_reset(pcad_chain *ch)
 
 namespace {
 
-// Wait for the stream's work and report a wait of its kernels that gave up: the
-// planes, sums and energies are then undefined, so every call that hands them
-// back ends here.  The error flag comes behind the work in the stream (one round
-// trip: a copy after the synchronisation cost another 7 us).
-pcad_status wait_work(pcad_chain *ch)
+// A call that hands back planes, sums or energies asks for the error flag of the
+// kernels that wait (post_check), enqueues its own copies, then waits for the
+// stream and reports a wait that gave up (end_check): what it read is then
+// undefined.  The flag's copy to pageable memory costs a call 8 us, to pinned
+// memory, ahead of the call's own copies, 1 us; a pinned word costs up to 254 us (the
+// first of a process, with its release), so a chain takes one when it has spent as
+// much on its checks.
+constexpr int kPinChecks = 32;
+
+pcad_status post_check(pcad_chain *ch)
 {
-    int e = 0;
-    if (ch->waits)
-        CUDA_TRY(cudaMemcpyAsync(&e, ch->err, sizeof(int), cudaMemcpyDeviceToHost, ch->stream));
+    if (!ch->waits)
+        return PCAD_OK;
+    if (!ch->flag_pin && ++ch->checks == kPinChecks &&
+        cudaMallocHost((void **)&ch->flag_pin, sizeof(int)) != cudaSuccess) {
+        ch->flag_pin = nullptr;
+        cudaGetLastError();
+    }
+    CUDA_TRY(cudaMemcpyAsync(ch->flag_pin ? ch->flag_pin : &ch->flag, ch->err, sizeof(int),
+                             cudaMemcpyDeviceToHost, ch->stream));
+    return PCAD_OK;
+}
+
+pcad_status end_check(pcad_chain *ch)
+{
     CUDA_TRY(cudaStreamSynchronize(ch->stream));
+    const int e = !ch->waits ? 0 : (ch->flag_pin ? *ch->flag_pin : ch->flag);
     if (e == 2)
         return fail(PCAD_ECUDA, "tensor-core sweep: shared memory not 1024-byte aligned");
     if (e)
         return fail(PCAD_ETIMEOUT, "a bounded wait of the sweep kernel (tile load, MMA "
                                    "completion or wavefront dependency) gave up");
     return PCAD_OK;
+}
+
+pcad_status wait_work(pcad_chain *ch)
+{
+    const pcad_status st = post_check(ch);
+    return st == PCAD_OK ? end_check(ch) : st;
 }
 
 }  // namespace
@@ -1121,11 +1146,14 @@ pcad_status pcad_chain_energy(pcad_chain *ch, double *energy, uint64_t *pair_sum
     if (!ch || !energy)
         return fail(PCAD_EINVAL, "chain or energy is NULL");
     double res[3] = {0.0, 0.0, 0.0};
+    pcad_status st = post_check(ch);
+    if (st != PCAD_OK)
+        return st;
     CUDA_TRY(launch_energy(ch->x[ch->cur], ch->g, ch->H, ch->W, ch->pitch, ch->ecoef, ch->esums,
                            ch->mscratch, EnergyTrack{}, ch->tdev, 0, ch->stream));
     CUDA_TRY(cudaMemcpyAsync(res, ch->mscratch, sizeof(res), cudaMemcpyDeviceToHost,
                              ch->stream));
-    const pcad_status st = wait_work(ch);
+    st = end_check(ch);
     if (st != PCAD_OK)
         return st;
     *energy = res[0];
@@ -1371,9 +1399,12 @@ pcad_status pcad_chain_read_sample(pcad_chain *ch, uint8_t *host_out, int out_pi
         return fail(PCAD_EINVAL, "NULL argument");
     if (out_pitch < ch->W)
         return fail(PCAD_EINVAL, "out_pitch < W");
+    pcad_status st = post_check(ch);
+    if (st != PCAD_OK)
+        return st;
     CUDA_TRY(read_labels(host_out, out_pitch, ch->x[ch->cur], ch->pitch, ch->H, ch->W, ch->fplane,
                          ch->stream));
-    return wait_work(ch);
+    return end_check(ch);
 }
 
 pcad_status pcad_chain_read_sample_dev(pcad_chain *ch, uint8_t *dev_out, int out_pitch)
@@ -1393,11 +1424,14 @@ pcad_status pcad_chain_read_mean(pcad_chain *ch, float *host_out)
         return fail(PCAD_EINVAL, "NULL argument");
     if (ch->n_acc == 0)
         return fail(PCAD_ESTATE, "no sweep accumulated yet");
+    pcad_status st = post_check(ch);
+    if (st != PCAD_OK)
+        return st;
     const long n = (long)ch->H * ch->W;
     CUDA_TRY(launch_mean(ch->acc, (float)ch->n_acc, ch->fplane, n, ch->stream));
     CUDA_TRY(cudaMemcpyAsync(host_out, ch->fplane, n * sizeof(float), cudaMemcpyDeviceToHost,
                              ch->stream));
-    return wait_work(ch);
+    return end_check(ch);
 }
 
 pcad_status pcad_chain_write_sample(pcad_chain *ch, const uint8_t *host_in, int in_pitch)
@@ -1450,9 +1484,12 @@ pcad_status pcad_chain_metrics(pcad_chain *ch, const uint8_t *clean_host, int cl
     if (clean_pitch < ch->W)
         return fail(PCAD_EINVAL, "clean_pitch < W");
     const long n = (long)ch->H * ch->W;
+    if (which == 0 && ch->n_acc == 0)
+        return fail(PCAD_ESTATE, "no sweep accumulated yet");
+    pcad_status st = post_check(ch);
+    if (st != PCAD_OK)
+        return st;
     if (which == 0) {
-        if (ch->n_acc == 0)
-            return fail(PCAD_ESTATE, "no sweep accumulated yet");
         CUDA_TRY(launch_mean(ch->acc, (float)ch->n_acc, ch->fplane, n, ch->stream));
     } else {
         CUDA_TRY(launch_labels_to_float(ch->x[ch->cur], ch->pitch, ch->H, ch->W, ch->fplane,
@@ -1465,7 +1502,7 @@ pcad_status pcad_chain_metrics(pcad_chain *ch, const uint8_t *clean_host, int cl
     double res[2];
     CUDA_TRY(cudaMemcpyAsync(res, ch->mscratch + 8, sizeof(res), cudaMemcpyDeviceToHost,
                              ch->stream));
-    const pcad_status st = wait_work(ch);
+    st = end_check(ch);
     if (st != PCAD_OK)
         return st;
     if (psnr_db)
@@ -1548,6 +1585,9 @@ pcad_status pcad_chain_export(pcad_chain *ch, void *host_blob, size_t *bytes)
     pcad_status st = pcad_chain_stats(ch, &h.fp64);
     if (st != PCAD_OK)
         return st;
+    st = post_check(ch);
+    if (st != PCAD_OK)
+        return st;
     char *b = (char *)host_blob;
     memcpy(b, &h, sizeof(h));
     // layout: header | current labels | observation | accumulator
@@ -1557,7 +1597,7 @@ pcad_status pcad_chain_export(pcad_chain *ch, void *host_blob, size_t *bytes)
     CUDA_TRY(read_labels(hx + n, ch->W, ch->g, ch->pitch, ch->H, ch->W, ch->fplane, ch->stream));
     CUDA_TRY(cudaMemcpyAsync(b + sizeof(h) + 2 * n, ch->acc, n * sizeof(float),
                              cudaMemcpyDeviceToHost, ch->stream));
-    st = wait_work(ch);
+    st = end_check(ch);
     if (st != PCAD_OK)
         return st;
     *bytes = need;
@@ -1625,6 +1665,8 @@ void pcad_chain_destroy(pcad_chain *ch)
         cudaFreeAsync(ch->track_block, ch->stream);
     cudaFreeAsync(ch->block, ch->stream);
     cudaStreamSynchronize(ch->stream);
+    if (ch->flag_pin)
+        cudaFreeHost(ch->flag_pin);
     delete ch;
 }
 
