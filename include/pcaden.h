@@ -473,7 +473,7 @@ typedef struct pcad_server pcad_server;
  * run every admitted request in every slice (the GPU is shared among all
  * of them).  PCAD_SERVE_SRPT (the default): shortest remaining work first
  * -- each step orders queued and admitted requests by estimated remaining
- * GPU time (sites x sweeps left x a per-label-count cost) minus `aging` x
+ * GPU time (sites x sweeps left x a cost by model and size) minus `aging` x
  * the seconds since submission, and runs the shortest ones until they hold
  * the fill target of sites (pcad_server_set_limits; by default two waves
  * of 4 x 32-site tiles); admitted requests outside that set keep their

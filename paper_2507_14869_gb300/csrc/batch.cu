@@ -1622,14 +1622,28 @@ double now_s()
         .count();
 }
 
-// Estimated GB300 seconds per site-update of a model, for the scheduling
-// order only (results never depend on it): the tensor-core sweep at
-// L >= 192 (1.07e10 site-updates/s), else the CUDA-core kernels, whose time
-// grows with L (measured 1.1e11 at L = 2, 4.9e10 at L = 16).
-double unit_cost(const pcad_model &m)
+// Estimated GB300 seconds per site-update of a request, for the scheduling order
+// and the length of a slice only (results never depend on it).  Measured in
+// batches of mid-size images (100 to 600 a side, tile-resident): two labels 4.3e-12,
+// L = 16 1.5e-11, L = 9 with 8 neighbours 1.5e-11, the segment draw 3.6e-11 at
+// L = 64 and 4.2e-11 at L = 256; images of 2^20 sites and more take 0.55 of that
+// (2.3e-12, 8.0e-12, 2.4e-11).  Other models: the tensor-core sweep at L >= 192
+// (1.07e10 site-updates/s), else the CUDA-core kernels, whose time grows with L.
+double unit_cost(const pcad_job &j)
 {
-    const int T = m.pair == PCAD_PAIR_POTTS ? 1 : m.pair_T;
-    if (m.L >= kTcAutoLabels && T <= kTcMaxT && m.inertia_norm == 0)
+    const pcad_model &m = j.model;
+    DevModel d{};
+    d.L = m.L;
+    d.nbhd = m.nbhd;
+    d.T = m.pair == PCAD_PAIR_POTTS ? 1 : m.pair_T;
+    const double large = (long long)j.H * j.W > kTileMaxSites ? 0.55 : 1.0;
+    if (m.L == 2)
+        return 4.3e-12 * large;
+    if (m.pair_coef >= 0.0f && m.L <= kSmallMaxLabels)
+        return 1.5e-11 * large;
+    if (m.pair_coef >= 0.0f && seg_structure(d))
+        return 4.0e-11 * large;
+    if (m.L >= kTcAutoLabels && d.T <= kTcMaxT && m.inertia_norm == 0)
         return 9.3e-11;
     return 7.4e-12 + 8.1e-13 * m.L;
 }
@@ -2031,7 +2045,7 @@ pcad_status pcad_server_submit(pcad_server *sv, const pcad_job *job, int nsweeps
     rq.sm = job_layout(*job, (job->W + 15) / 16 * 16, 0);
     rq.bytes = rq.sm.end;
     rq.t_submit = now_s();
-    rq.unit_cost = unit_cost(job->model);
+    rq.unit_cost = unit_cost(*job);
     if (rq.bytes > sv->budget)
         return set_error(PCAD_ENOMEM, "request larger than the whole HBM budget");
     rq.g.resize((size_t)job->H * job->W);
