@@ -214,7 +214,11 @@ pcad_status pcad_chain_set_blocking(pcad_chain *ch, int k);
  * below the wavefront's images; not with energy tracking, temporal blocking or
  * runs of very few sweeps.  Same draws and labels; the kernel in use is reported
  * as the kind that it stands in for.  Its waits are bounded
- * (pcad_chain_set_wait_limit). */
+ * (pcad_chain_set_wait_limit).  Such a launch takes every multiprocessor: chains
+ * on several streams mostly run one after the other, where launches per sweep
+ * overlapped (16 chains of 256^2, 9 labels: 2.0 us per sweep and chain instead of
+ * 1.0).  Many images at once belong in a batch (0.9), which shares the
+ * multiprocessors among them. */
 typedef enum {
     PCAD_KERNEL_AUTO = 0,
     PCAD_KERNEL_CUDA_CORE = 1,

@@ -358,8 +358,8 @@ bool uses_tc(const pcad_chain *ch)
            win_auto_mode(ch) == 0;
 }
 
-// Whole runs of sweeps of small two-label images in one single-CTA launch
-// (state in shared memory): on request, or with AUTO for every image it
+// Whole runs of sweeps of small two-label images in one launch of a cluster of 8
+// CTAs or, the smallest, of one (state in shared memory): on request, or with AUTO for every image it
 // accepts, without energy tracking or temporal blocking.
 bool uses_resident(const pcad_chain *ch)
 {
@@ -384,6 +384,14 @@ bool uses_wave(const pcad_chain *ch);
 //   phases need no exchange here, 13.0 / 14.4; at 720^2 21.1 / 19.6): from 8
 //   blocks of 4 x 32 sites per multiprocessor on, PCA stays with it, from
 //   kTileSegGibbsSites sites on Gibbs too.
+// These are the times of one chain at a time.  Of several chains on streams of
+// their own only those whose blocks fit an SM together run at once, so each takes
+// its time alone, where launches per sweep overlapped: us per sweep and chain, n
+// chains at once (tile-resident / per-sweep / in one batch): 256^2 L = 9, 8
+// neighbours n = 2 2.1 / 3.2 / 1.8, 4 2.0 / 1.8 / 1.3, 16 2.0 / 1.0 / 0.9; L = 16 n =
+// 4 1.8 / 1.9 / 1.1, 16 1.8 / 1.0 / 0.7; L = 64 n = 16 3.4 / 2.9 / 2.1; 1000^2 L = 16
+// n = 4 10.7 / 9.5 / 11.5, two labels 3.7 / 3.0 / 4.3; 300^2 two labels n = 16 0.6 /
+// 0.9 / 0.4, 128^2 L = 16 0.8 / 0.8 / 0.3.  A chain does not know what else runs.
 constexpr long long kTileSegGibbsSites = 300000;
 
 // The images of that rule: a chain holds an exchange buffer for these only.
@@ -475,10 +483,10 @@ bool ensure_maps(pcad_chain *ch)
 // Unblocked PCA sweeps on the small-label kernel: on request, or with AUTO
 // for the models it accepts (3 <= L <= 16, c >= 0, L0 price) unless the
 // wavefront kernel is chosen (L = 16 at 1/2 to 3 waves of 4 x 32 tiles,
-// where the small-label kernel's 16 x 32 tiles leave SMs idle).  Measured on
-// GB300 at L = 16: 1.05e11 site-updates/s at 8192^2 (TMA tiles) and 6.9e10
-// at 1024^2 against 4.9e10 and 4.1e10 for the general per-sweep kernel;
-// 3.2e10 at 512^2 against 3.7e10 for the wavefront kernel.
+// where the small-label kernel's 16 x 32 tiles leave SMs idle) or the run is
+// tile-resident (uses_tile).  Measured on GB300 at L = 16: 1.25e11
+// site-updates/s at 8192^2 (TMA tiles) against 4.9e10 for the general per-sweep
+// kernel; 1000^2, a launch per sweep, 7.0e10.
 bool uses_small(const pcad_chain *ch)
 {
     if (ch->model.sampler != PCAD_SAMPLER_PCA || ch->tb_k > 0 || !pca_small_eligible(ch->dm))
@@ -536,8 +544,8 @@ pcad_status issue_sweeps(pcad_chain *ch, int off0, int n, int &cur, cudaStream_t
 {
     SweepArgs a = make_args(ch);
     if (uses_resident(ch) && n > 0) {
-        // all n sweeps in one single-CTA launch; PCA ends in the other plane
-        // when n is odd, Gibbs in place
+        // all n sweeps in one launch; PCA ends in the other plane when n is odd,
+        // Gibbs in place
         a.sweep_off = (uint32_t)off0;
         const bool gibbs = ch->model.sampler != PCAD_SAMPLER_PCA;
         const int out = gibbs ? cur : cur ^ (n & 1);

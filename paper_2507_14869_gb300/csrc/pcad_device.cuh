@@ -81,7 +81,6 @@ __device__ __forceinline__ unsigned long long globaltimer_ns()
     return t;
 }
 
-// The error flag, read past L1 (another SM may have set it).
 // Wait until the grids this launch depends on have finished (their writes
 // visible); let the next launch of the stream start once every block of this
 // one has (launch_dependent).
@@ -95,6 +94,7 @@ __device__ __forceinline__ void grid_dep_launch()
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// The error flag, read past L1 (another SM may have set it).
 __device__ __forceinline__ int ld_flag(const int *p)
 {
     int v;
