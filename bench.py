@@ -50,6 +50,13 @@ G512_WORKLOAD = ("greyscale 512x512, L=256 (uint8), Gaussian sigma=20, truncated
 SFU_PEAK_T = 152 * 32 * 2.070e9 / 1e12
 SFU_PEAK_SOURCE = ("152 SMs x 32 ex2/clk/SM x 2070 MHz (unit count x max clock; an "
                    "ex2.approx.ftz loop measured 29.9/clk/SM)")
+# warp instructions: 4 per SM per clock x 152 SMs x 2070 MHz; a segment draw takes 14
+# exponentials whatever L, so its sweeps are set against the issue rate
+ISSUE_PEAK_T = 152 * 4 * 2.070e9 / 1e12
+ISSUE_PEAK_SOURCE = "152 SMs x 4 warp instructions/clk/SM x 2070 MHz (unit count x max clock)"
+# warp instructions per 32 site-updates (ncu smsp__inst_executed.sum,
+# profiles/seg_tile_small_binary.md); tile_kernel draws its halos' sites twice
+NCU_SEG_INST = {"pca_seg": 842.0, "gibbs_seg": 845.0, "pca_segw": 951.0, "tile_gibbs_512": 1129.0}
 HBM_PEAK_FALLBACK = 6800.0   # GB/s, used only if MEASURED_PEAKS.json is absent
 
 # DRAM bytes (read + write) per site-update of each kernel, from ncu captures
@@ -63,10 +70,9 @@ NCU_TC_NOTE = ("ncu dram__bytes_read+write of one accumulating 32-sweep pca_tcw_
                "at 4096^2 L=256 (profiles/pca_tc_l256_4096sq.md), scaled by sites to 8192^2")
 NCU_DIRECT_BYTES_PER_SITE = None
 NCU_DIRECT_NOTE = "ncu dram__bytes_read+write of one pca_direct_kernel launch at 8192^2 L=16"
-NCU_WIN_BYTES_PER_SITE = (402903040 + 286483712) / (8192 * 8192)
-NCU_WIN_NOTE = ("ncu dram__bytes_read+write of one accumulating pca_win_kernel launch at "
-                "8192^2 L=256 (profiles/pca_win_l256_8192sq.md); pca_seg_kernel moves the same "
-                "planes")
+NCU_SEG_BYTES_PER_SITE = (402863872 + 280239360) / (8192 * 8192)
+NCU_SEG_NOTE = ("ncu dram__bytes_read+write of one accumulating pca_seg_kernel launch at "
+                "8192^2 L=256 (profiles/seg_tile_small_binary.md)")
 NCU_SMALL_BYTES_PER_SITE = (408240384 + 280811264) / (8192 * 8192)
 NCU_SMALL_NOTE = ("ncu dram__bytes_read+write of one accumulating pca_small_tma_kernel launch "
                   "at 8192^2 L=16 (profiles/pca_small_tma_l16_6144sq.md)")
@@ -121,11 +127,12 @@ def _args():
     p.add_argument("--kernel", default="auto",
                    choices=list(KERNEL_KINDS),
                    help="kernel of the unblocked PCA sweep (headline chain and profile case): "
-                        "auto = for eligible models with L >= 32 the windowed CUDA-core sweep "
-                        "on large images and the tensor-core sweep on small ones (L >= 192), "
-                        "else the small-label, resident, two-label, per-sweep or wavefront "
-                        "CUDA-core kernel; tensor = prior sums by tcgen05.mma; window = the "
-                        "windowed sweep; binary = the two-label sweep")
+                        "auto = for eligible models with L >= 32 the segment (else windowed) "
+                        "sweep on large images and the tensor-core sweep on small ones (L >= "
+                        "192), else the small-label, resident, two-label, tile-resident, "
+                        "per-sweep or wavefront CUDA-core kernel; tensor = prior sums by "
+                        "tcgen05.mma; window = the segment or windowed sweep; binary = the "
+                        "two-label sweep")
     p.add_argument("--images", type=int, default=128, help="batch: number of images")
     p.add_argument("--requests", type=int, default=200, help="serve: requests per rate")
     p.add_argument("--rates", default="10,25,50,200",
@@ -227,6 +234,18 @@ def _sfu_roofline(sites, L, ms_per_sweep, kernel, traffic=None, traffic_note=Non
             "kernel": kernel, "peak_source": SFU_PEAK_SOURCE, "ms_per_sweep": ms_per_sweep,
             "work_per_unit": f"one label evaluation (one exponential on the SFU in a direct "
                              f"evaluation), L={L} per site-update"}
+
+
+def _issue_roofline(sites, inst, ms_per_sweep, kernel, traffic=None, traffic_note=None):
+    """The instruction-issue bound of a segment draw: inst warp instructions per
+    32 site-updates, counted by ncu."""
+    achieved = sites / 32 * inst / (ms_per_sweep * 1e-3) / 1e12
+    return {"bound": "issue", "achieved": achieved, "peak": ISSUE_PEAK_T,
+            "unit": "T warp instructions/s", "frac": achieved / ISSUE_PEAK_T,
+            "traffic": traffic, "traffic_source": traffic_note,
+            "traffic_unit": "DRAM bytes per launch (1 sweep)", "kernel": kernel,
+            "peak_source": ISSUE_PEAK_SOURCE, "ms_per_sweep": ms_per_sweep,
+            "work_per_unit": f"{inst:g} warp instructions per 32 site-updates (ncu)"}
 
 
 def _crop(a, side):
@@ -375,11 +394,14 @@ def run_ours(a):
     pca.close()
     spl = 32 if pca_kind in (2, 3, 7) else 1       # sweeps per launch
     per_site = {2: NCU_TC_BYTES_PER_SITE, 1: NCU_DIRECT_BYTES_PER_SITE,
-                6: NCU_WIN_BYTES_PER_SITE}.get(pca_kind)
+                6: NCU_SEG_BYTES_PER_SITE}.get(pca_kind)
     traffic = per_site * sites * spl if per_site else None
-    note = {2: NCU_TC_NOTE, 6: NCU_WIN_NOTE}.get(pca_kind, NCU_DIRECT_NOTE)
-    roof = _sfu_roofline(sites, LABELS, ms_sweep, KERNEL_NAMES.get(pca_kind, str(pca_kind)),
-                         traffic, note, spl)
+    note = {2: NCU_TC_NOTE, 6: NCU_SEG_NOTE}.get(pca_kind, NCU_DIRECT_NOTE)
+    name = KERNEL_NAMES.get(pca_kind, str(pca_kind))
+    if pca_kind == 6:
+        roof = _issue_roofline(sites, NCU_SEG_INST["pca_seg"], ms_sweep, name, traffic, note)
+    else:
+        roof = _sfu_roofline(sites, LABELS, ms_sweep, name, traffic, note, spl)
     roof["algorithmic_bytes_per_launch"] = 11 * sites * spl
     roof["hbm_frac"] = (_algo_bytes(sites, SWEEPS, BURN_IN) / (ms_sweep * SWEEPS * 1e-3) / 1e9
                         / hbm_peak)
@@ -552,7 +574,8 @@ def _gibbs_8192(pc, stream, timed, noisy, m, clean, cid, steps=2):
             "ms_per_step": sum(ms) / steps, "ms_per_sweep": ms_sweep, "steps": steps,
             "psnr_db": p, "ssim": s, "kernel": name,
             "launches_per_step": _launches_per_run(kind, SWEEPS, sampler=1),
-            "roofline": _sfu_roofline(sites, LABELS, ms_sweep, name)}
+            "roofline": (_issue_roofline(sites, NCU_SEG_INST["gibbs_seg"], ms_sweep, name)
+                         if kind == 6 else _sfu_roofline(sites, LABELS, ms_sweep, name))}
 
 
 def _greyscale512(pc, stream, timed, cid, no_gibbs, steps=5):
@@ -570,10 +593,13 @@ def _greyscale512(pc, stream, timed, cid, no_gibbs, steps=5):
         kind = ch.kernel_in_use()
         ch.close()
         ms_sweep = sum(ms) / (steps * G512_SWEEPS)
+        # kind 7: the segment wavefront; Gibbs of this size runs it tile-resident
+        inst = NCU_SEG_INST["tile_gibbs_512" if sampler else "pca_segw"]
+        roof = (_issue_roofline(noisy.size, inst, ms_sweep, str(kind)) if kind == 7 else
+                _sfu_roofline(noisy.size, 256, ms_sweep, str(kind)))
         out[name] = {"value": noisy.size / (ms_sweep * 1e-3), "unit": "site-updates/s",
                      "ms_per_step": sum(ms) / steps, "psnr_db": p, "ssim": s, "kernel": kind,
-                     "roofline": {k: v for k, v in _sfu_roofline(
-                         noisy.size, 256, ms_sweep, str(kind)).items()
+                     "roofline": {k: v for k, v in roof.items()
                          if k in ("bound", "achieved", "peak", "unit", "frac", "ms_per_sweep")}}
     return out
 

@@ -12,7 +12,7 @@
 //     column of the tile and walks its 4 rows with the labels above, at and
 //     below it in registers; one Philox call per lane and tile serves the tile's
 //     128 sites.
-//     Bound by instruction issue: 847 thread instructions per site-update (700
+//     Bound by instruction issue: 842 warp instructions per 32 site-updates (700
 //     in the draw) at 88 % issue, ALU pipe 65 %, DRAM 5 %.
 //     L = 256, T = 30, sigma = 25, 8192^2: 1.60 ms per sweep (4.19e10
 //     site-updates/s) against 4.05 ms for the windowed draw.  Gibbs at 4096^2:
