@@ -476,9 +476,9 @@ typedef struct pcad_server pcad_server;
 /* Scheduling policy.  PCAD_SERVE_FIFO: admit first come first served and
  * run every admitted request in every slice (the GPU is shared among all
  * of them).  PCAD_SERVE_SRPT (the default): shortest remaining work first
- * -- each step orders queued and admitted requests by estimated remaining
- * GPU time (sites x sweeps left x a cost by model and size) minus `aging` x
- * the seconds since submission, and runs the shortest ones until they hold
+ * -- each step orders queued and admitted requests by remaining cost (sites x
+ * sweeps left x a cost by model and size, 3.5 times the GPU time measured for
+ * such requests) minus `aging` x the seconds since submission, and runs the shortest ones until they hold
  * the fill target of sites (pcad_server_set_limits; by default two waves
  * of 4 x 32-site tiles); admitted requests outside that set keep their
  * device state and pause.  Default aging 0.2.  PCAD_EINVAL for an unknown

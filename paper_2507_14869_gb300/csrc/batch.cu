@@ -45,8 +45,18 @@ constexpr int kOrderWave = 2;     // batch work order: one wavefront launch per 
 // active set has at least 4 tiles of 4 rows per resident block (measured on
 // single requests of 300^2..1376^2 and on a 50 req/s mix).
 constexpr int kServeTallTiles = 4;
-// SRPT server: least estimated GPU time of a full slice of the run set.
-constexpr double kMinSliceSeconds = 1e-3;
+// SRPT server: a request's cost in the schedule's seconds is kCostScale times its
+// measured GPU time, the scale at which the default aging (0.2 schedule seconds per
+// second waited) serves best; the run set of a full slice costs at least
+// kMinSliceSeconds (0.57 ms of GPU time), so that the host's part of a slice stays
+// small.  200 requests of 128^2 to 2048^2, L = 16 and 256, at 25 / 50 / 100 / 200 a
+// second, p50 (p99) in seconds: these 0.036 (0.29), 0.11 (0.64), 0.18 (2.8), 0.25
+// (3.5); slices of 1e-3 0.032 (0.28), 0.083 (0.64), 0.18 (2.8), 0.23 (3.5), but a
+// backlog of ten 42.4 ms against 41.9; scale 1 and slices of 1e-3 0.039 (0.28), 0.16
+// (0.60), 0.76 (2.5), 1.1 (3.4); the replaced kernels' costs 0.036 (0.34), 0.10 (0.70),
+// 0.35 (3.0), 0.36 (3.7), 42.1 ms.
+constexpr double kCostScale = 3.5;
+constexpr double kMinSliceSeconds = 2e-3;
 constexpr size_t kAlign = 256;
 constexpr int kTableBytes = 4096;  // 511 doubles
 
@@ -1611,7 +1621,7 @@ struct Request {
     void *side = nullptr;        // its slot's side memory, if it holds any
     size_t side_bytes = 0;
     double t_submit = 0.0;       // seconds (steady clock)
-    double unit_cost = 0.0;      // estimated seconds per site-update
+    double unit_cost = 0.0;      // schedule seconds per site-update
     std::vector<uint8_t> sample;
     std::vector<float> mean;
 };
@@ -1820,8 +1830,8 @@ pcad_status server_admit_fifo(pcad_server *sv)
 }
 
 // Shortest remaining work first, with aging: every step orders the queued
-// and admitted requests by estimated remaining GPU time (sites x sweeps
-// left x unit cost) minus `aging` x time waited since submission, and runs
+// and admitted requests by estimated remaining cost (sites x sweeps left x
+// unit cost) minus `aging` x time waited since submission, and runs
 // the shortest ones until the run set holds the fill target of sites (at
 // least one request), admitting queued ones as slots and the HBM budget
 // allow.  Admitted requests outside the run set keep their state on the
@@ -1845,11 +1855,11 @@ pcad_status server_schedule_srpt(pcad_server *sv)
     const size_t fill = sv->max_active_sites
                             ? sv->max_active_sites
                             : (size_t)2 * (size_t)std::max(sv->grid, 1) * 128;
-    // without an explicit target, also at least kMinSliceSeconds of estimated
-    // work per slice, so the host's per-slice cost stays small against it
+    // without an explicit target, also at least kMinSliceSeconds of cost per
+    // slice, so the host's per-slice cost stays small against it
     const double min_time = sv->max_active_sites ? 0.0 : kMinSliceSeconds;
     size_t run_sites = 0;
-    double run_time = 0.0;    // estimated seconds per sweep of the run set
+    double run_time = 0.0;    // cost per sweep of the run set
     std::vector<uint64_t> run;
     for (const auto &pr : order) {
         if (!run.empty() && run_sites >= fill && run_time * kSlice >= min_time)
@@ -2045,7 +2055,7 @@ pcad_status pcad_server_submit(pcad_server *sv, const pcad_job *job, int nsweeps
     rq.sm = job_layout(*job, (job->W + 15) / 16 * 16, 0);
     rq.bytes = rq.sm.end;
     rq.t_submit = now_s();
-    rq.unit_cost = unit_cost(*job);
+    rq.unit_cost = kCostScale * unit_cost(*job);
     if (rq.bytes > sv->budget)
         return set_error(PCAD_ENOMEM, "request larger than the whole HBM budget");
     rq.g.resize((size_t)job->H * job->W);
