@@ -25,6 +25,13 @@ using namespace pcad;
 namespace {
 
 thread_local std::string g_err;
+
+// Waits of this process's chains that gave up, in managed memory: the kernels touch
+// it only then, so the host's look at it is a load.
+__managed__ int g_gave_up;
+
+int waits_given_up() { return *static_cast<volatile int *>(&g_gave_up); }
+
 constexpr int kGraphSweeps = 32;    // sweeps per captured block (even)
 constexpr int kTable = 511;
 
@@ -270,8 +277,7 @@ struct pcad_chain {
     TileKind tkind;
     TilePlan tplan{};
     bool waits = false;                  // a launch with bounded waits was issued: err may be set
-    int flag = 0, *flag_pin = nullptr;   // where a check copies err (flag_pin: pinned)
-    int checks = 0;
+    int gave_up = 0;                     // the count of waits at which err was last known to be 0
     void *track_block = nullptr;
 };
 
@@ -293,6 +299,7 @@ SweepArgs make_args(const pcad_chain *ch)
     a.wait_ns = ch->wait_ns;
     a.stall_tile = ch->stall_tile;
     a.row_off = ch->row_off;
+    a.gave_up = &g_gave_up;
     a.m = ch->dm;
     return a;
 }
@@ -812,6 +819,7 @@ pcad_status create_common(const uint8_t *g_src, bool g_on_device, int H, int W, 
         p += sbytes;
     }
     ch->sms = sms;
+    ch->gave_up = waits_given_up();
     ch->tdev = (uint32_t *)p;
     ch->fp64 = (unsigned long long *)(p + 8);
     ch->mscratch = (double *)(p + 16);
@@ -995,45 +1003,28 @@ pcad_status pcad_chain_reset(pcad_chain *ch)
 
 namespace {
 
-// A call that hands back planes, sums or energies asks for the error flag of the
-// kernels that wait (post_check), enqueues its own copies, then waits for the
-// stream and reports a wait that gave up (end_check): what it read is then
-// undefined.  The flag's copy to pageable memory costs a call 8 us, to pinned
-// memory, ahead of the call's own copies, 1 us; a pinned word costs up to 254 us (the
-// first of a process, with its release), so a chain takes one when it has spent as
-// much on its checks.
-constexpr int kPinChecks = 32;
-
-pcad_status post_check(pcad_chain *ch)
-{
-    if (!ch->waits)
-        return PCAD_OK;
-    if (!ch->flag_pin && ++ch->checks == kPinChecks &&
-        cudaMallocHost((void **)&ch->flag_pin, sizeof(int)) != cudaSuccess) {
-        ch->flag_pin = nullptr;
-        cudaGetLastError();
-    }
-    CUDA_TRY(cudaMemcpyAsync(ch->flag_pin ? ch->flag_pin : &ch->flag, ch->err, sizeof(int),
-                             cudaMemcpyDeviceToHost, ch->stream));
-    return PCAD_OK;
-}
-
-pcad_status end_check(pcad_chain *ch)
+// Wait for the stream's work and report a wait of its kernels that gave up: the
+// planes, sums and energies are then undefined, so every call that hands them
+// back ends here.  The flag is copied only if some wait of the process has given up
+// since it was last known to be clear: the copy costs 8 us (1 us to page-locked
+// memory, whose set-up costs more than a short-lived chain's reads), a look at the
+// count none.
+pcad_status wait_work(pcad_chain *ch)
 {
     CUDA_TRY(cudaStreamSynchronize(ch->stream));
-    const int e = !ch->waits ? 0 : (ch->flag_pin ? *ch->flag_pin : ch->flag);
+    const int n = waits_given_up();
+    if (!ch->waits || n == ch->gave_up)
+        return PCAD_OK;
+    int e = 0;
+    CUDA_TRY(cudaMemcpyAsync(&e, ch->err, sizeof(int), cudaMemcpyDeviceToHost, ch->stream));
+    CUDA_TRY(cudaStreamSynchronize(ch->stream));
     if (e == 2)
         return fail(PCAD_ECUDA, "tensor-core sweep: shared memory not 1024-byte aligned");
     if (e)
         return fail(PCAD_ETIMEOUT, "a bounded wait of the sweep kernel (tile load, MMA "
                                    "completion or wavefront dependency) gave up");
+    ch->gave_up = n;
     return PCAD_OK;
-}
-
-pcad_status wait_work(pcad_chain *ch)
-{
-    const pcad_status st = post_check(ch);
-    return st == PCAD_OK ? end_check(ch) : st;
 }
 
 }  // namespace
@@ -1154,14 +1145,11 @@ pcad_status pcad_chain_energy(pcad_chain *ch, double *energy, uint64_t *pair_sum
     if (!ch || !energy)
         return fail(PCAD_EINVAL, "chain or energy is NULL");
     double res[3] = {0.0, 0.0, 0.0};
-    pcad_status st = post_check(ch);
-    if (st != PCAD_OK)
-        return st;
     CUDA_TRY(launch_energy(ch->x[ch->cur], ch->g, ch->H, ch->W, ch->pitch, ch->ecoef, ch->esums,
                            ch->mscratch, EnergyTrack{}, ch->tdev, 0, ch->stream));
     CUDA_TRY(cudaMemcpyAsync(res, ch->mscratch, sizeof(res), cudaMemcpyDeviceToHost,
                              ch->stream));
-    st = end_check(ch);
+    const pcad_status st = wait_work(ch);
     if (st != PCAD_OK)
         return st;
     *energy = res[0];
@@ -1407,12 +1395,9 @@ pcad_status pcad_chain_read_sample(pcad_chain *ch, uint8_t *host_out, int out_pi
         return fail(PCAD_EINVAL, "NULL argument");
     if (out_pitch < ch->W)
         return fail(PCAD_EINVAL, "out_pitch < W");
-    pcad_status st = post_check(ch);
-    if (st != PCAD_OK)
-        return st;
     CUDA_TRY(read_labels(host_out, out_pitch, ch->x[ch->cur], ch->pitch, ch->H, ch->W, ch->fplane,
                          ch->stream));
-    return end_check(ch);
+    return wait_work(ch);
 }
 
 pcad_status pcad_chain_read_sample_dev(pcad_chain *ch, uint8_t *dev_out, int out_pitch)
@@ -1432,14 +1417,11 @@ pcad_status pcad_chain_read_mean(pcad_chain *ch, float *host_out)
         return fail(PCAD_EINVAL, "NULL argument");
     if (ch->n_acc == 0)
         return fail(PCAD_ESTATE, "no sweep accumulated yet");
-    pcad_status st = post_check(ch);
-    if (st != PCAD_OK)
-        return st;
     const long n = (long)ch->H * ch->W;
     CUDA_TRY(launch_mean(ch->acc, (float)ch->n_acc, ch->fplane, n, ch->stream));
     CUDA_TRY(cudaMemcpyAsync(host_out, ch->fplane, n * sizeof(float), cudaMemcpyDeviceToHost,
                              ch->stream));
-    return end_check(ch);
+    return wait_work(ch);
 }
 
 pcad_status pcad_chain_write_sample(pcad_chain *ch, const uint8_t *host_in, int in_pitch)
@@ -1494,9 +1476,6 @@ pcad_status pcad_chain_metrics(pcad_chain *ch, const uint8_t *clean_host, int cl
     const long n = (long)ch->H * ch->W;
     if (which == 0 && ch->n_acc == 0)
         return fail(PCAD_ESTATE, "no sweep accumulated yet");
-    pcad_status st = post_check(ch);
-    if (st != PCAD_OK)
-        return st;
     if (which == 0) {
         CUDA_TRY(launch_mean(ch->acc, (float)ch->n_acc, ch->fplane, n, ch->stream));
     } else {
@@ -1510,7 +1489,7 @@ pcad_status pcad_chain_metrics(pcad_chain *ch, const uint8_t *clean_host, int cl
     double res[2];
     CUDA_TRY(cudaMemcpyAsync(res, ch->mscratch + 8, sizeof(res), cudaMemcpyDeviceToHost,
                              ch->stream));
-    st = end_check(ch);
+    const pcad_status st = wait_work(ch);
     if (st != PCAD_OK)
         return st;
     if (psnr_db)
@@ -1593,9 +1572,6 @@ pcad_status pcad_chain_export(pcad_chain *ch, void *host_blob, size_t *bytes)
     pcad_status st = pcad_chain_stats(ch, &h.fp64);
     if (st != PCAD_OK)
         return st;
-    st = post_check(ch);
-    if (st != PCAD_OK)
-        return st;
     char *b = (char *)host_blob;
     memcpy(b, &h, sizeof(h));
     // layout: header | current labels | observation | accumulator
@@ -1605,7 +1581,7 @@ pcad_status pcad_chain_export(pcad_chain *ch, void *host_blob, size_t *bytes)
     CUDA_TRY(read_labels(hx + n, ch->W, ch->g, ch->pitch, ch->H, ch->W, ch->fplane, ch->stream));
     CUDA_TRY(cudaMemcpyAsync(b + sizeof(h) + 2 * n, ch->acc, n * sizeof(float),
                              cudaMemcpyDeviceToHost, ch->stream));
-    st = end_check(ch);
+    st = wait_work(ch);
     if (st != PCAD_OK)
         return st;
     *bytes = need;
@@ -1673,8 +1649,6 @@ void pcad_chain_destroy(pcad_chain *ch)
         cudaFreeAsync(ch->track_block, ch->stream);
     cudaFreeAsync(ch->block, ch->stream);
     cudaStreamSynchronize(ch->stream);
-    if (ch->flag_pin)
-        cudaFreeHost(ch->flag_pin);
     delete ch;
 }
 

@@ -94,6 +94,15 @@ __device__ __forceinline__ void grid_dep_launch()
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// A bounded wait gave up: the launch's error flag, then (unless null) the count that
+// the host looks at without a copy.
+__device__ __forceinline__ void report_wait(int *err, int *gave_up, int code = 1)
+{
+    atomicExch(err, code);
+    if (gave_up)
+        atomicAdd_system(gave_up, 1);
+}
+
 // The error flag, read past L1 (another SM may have set it).
 __device__ __forceinline__ int ld_flag(const int *p)
 {

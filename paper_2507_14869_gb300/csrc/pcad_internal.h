@@ -33,6 +33,7 @@ struct SweepArgs {
     long long wait_ns;        // limit of each bounded device wait (0: kWaitLimitNs)
     int stall_tile;           // test aid: wavefront tile stall_tile - 1 never publishes (0: off)
     DevModel m;
+    int *gave_up;             // counts waits that gave up where the host sees it (nullptr: not kept)
 };
 
 __device__ __forceinline__ uint32_t sweep_index(const SweepArgs &a)

@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kSegwThreads, 8)
                 }
             }
             if (!ok)
-                atomicExch(err, 1);
+                report_wait(err, a.gave_up);
             __syncwarp();
         } else if (wp == 1 && run) {
             block_uniforms(a, ty * kSY, tx * kSX, t, U_s);
@@ -384,7 +384,7 @@ __global__ void __launch_bounds__(kSegwThreads, 7)
                 }
             }
             if (!ok)
-                atomicExch(err, 1);
+                report_wait(err, a.gave_up);
             __syncwarp();
         } else if (wp == 1 || wp == 2) {
             gibbs_uniforms(a, ty * kSY, tx, t, (wp - 1) * 32 + lane, U_s);

@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kTmThreads, 3)
             // record, then wait (bounded) for the copies still in flight
             // before the block's shared memory is released
             if (tid == 0)
-                atomicExch(err, 1);
+                report_wait(err, a.gave_up);
             mbar_wait_timed(&bar[b], ph, limit);
             if (next < ntiles)
                 mbar_wait_timed(&bar[b ^ 1], b ? phase0 : phase1, limit);

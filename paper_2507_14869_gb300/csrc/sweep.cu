@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kThreads, PCAD_WAVE_MIN_BLOCKS) pca_wave_kerne
                 }
             }
             if (!ok)
-                atomicExch(err, 1);
+                report_wait(err, a.gave_up);
             __syncwarp();
         } else if (threadIdx.y == 1) {
             block_uniforms(a, ty * kBY, tx * kBX, t0 + (uint32_t)k, U_s);

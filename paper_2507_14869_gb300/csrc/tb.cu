@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(kTbThreads)
         // the copies may still land: wait for them (bounded again) before the
         // block's shared memory is released
         if (tid == 0)
-            atomicExch(err, 1);
+            report_wait(err, a.gave_up);
         mbar_wait_timed(&bar, 0u, limit);
         return;
     }

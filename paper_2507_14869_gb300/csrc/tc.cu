@@ -349,7 +349,7 @@ __device__ __forceinline__ void tc_wait_item(const TcParams &p, const TcItem &ii
         dep_counter(p.done + ii.base, ii.k, ii.tile, ii.tiles_x, ii.tiles_y, lane);
     const unsigned int seen = (d && d == pre_d) ? pre : (d ? ld_acquire_gpu(d) : 0u);
     if (!wait_counter(d, (unsigned int)ii.k, seen, p.err, wait_limit(p.wait_ns)))
-        atomicExch(p.err, 1);
+        report_wait(p.err, p.a.gave_up);
 }
 
 // Shared memory of one group's FP64 re-draws.
@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(kThr, 1) pca_tcw_kernel(const TcParams p)
     const int lane = tid & 31;
     if (smem_u32(smem) & 1023u) {      // the swizzled operands need 1024-byte alignment
         if (tid == 0)
-            atomicExch(p.err, 2);
+            report_wait(p.err, p.a.gave_up, 2);
         return;
     }
     const int ncm = p.nc_max;
@@ -722,7 +722,7 @@ __global__ void __launch_bounds__(kThr, 1) pca_tcw_kernel(const TcParams p)
 
             // window chunks from TMEM
             if (!mbar_wait_timed(&mbar[grp], (uint32_t)(uses & 1), limit)) {
-                atomicExch(p.err, 1);
+                report_wait(p.err, p.a.gave_up);
                 ok = false;
             }
             ++uses;
@@ -872,7 +872,7 @@ __global__ void __launch_bounds__(kThr, 1) pca_tcw_kernel(const TcParams p)
                 } else if (knext >= 0) {   // looked at during this item
                     if (!BUDGET || t0 + (uint32_t)knext < tlim)
                         if (!wait_counter(dnext, (unsigned int)knext, seen, p.err, limit))
-                            atomicExch(p.err, 1);
+                            report_wait(p.err, p.a.gave_up);
                 } else {
                     const TcItem in2 = tc_decode<BATCH>(p, nx);
                     if (!BUDGET || t0 + (uint32_t)in2.k < tlim)

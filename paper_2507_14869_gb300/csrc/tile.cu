@@ -504,7 +504,7 @@ __global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBB
         // halo words and uniforms in place; leave together when a wait gave up
         if (__syncthreads_or(!ok)) {
             if (tid == 0)
-                atomicExch(err, 1);
+                report_wait(err, a.gave_up);
             return;
         }
         // A pass computes its first sites' places and reads their inputs before
@@ -677,7 +677,7 @@ __global__ void __launch_bounds__(WORDS ? kTlWideThreads1 : tile_threads<P, GIBB
     }
     if (__syncthreads_or(!ok)) {
         if (tid == 0)
-            atomicExch(err, 1);
+            report_wait(err, a.gave_up);
         return;
     }
     pol.finish(a);

@@ -388,7 +388,7 @@ __global__ void __launch_bounds__(kWThreads, 8)
                 }
             }
             if (!ok)
-                atomicExch(err, 1);
+                report_wait(err, a.gave_up);
             __syncwarp();
         } else if (wp == 1 && run) {
             block_uniforms(a, ty * kWY, tx * kWX, t, U_s);
@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(kWThreads, 8)
                 }
             }
             if (!ok)
-                atomicExch(err, 1);
+                report_wait(err, a.gave_up);
             __syncwarp();
         } else if (wp == 1 || wp == 2) {   // 64 Philox calls: site rows of the phase
             const int i = (wp - 1) * 32 + lane;
